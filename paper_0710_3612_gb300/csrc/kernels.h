@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fixed.cuh"
+
 namespace mgk {
 
 // Kernel launches made by this library so far (counted at every launch site).
@@ -125,6 +127,7 @@ struct Epilogue {
   const void* W = nullptr;
   double* dot_ws = nullptr;
   double* dot_out = nullptr;     // <in, out> per rhs (fine stencil; needs <= 608 blocks)
+  bool dot_real = false;         // only Re<in, out> is read (the imaginary part may be zero)
   // with dot_out, instead of <in, out>: {Re<out, zq_q>, Re<zq_r, out>} per rhs,
   // zq_q and zq_r complex128 vectors shaped like out (the flexible-CG pair)
   const void* zq_q = nullptr;
@@ -133,13 +136,23 @@ struct Epilogue {
 
 // ---- fine Wilson operator ------------------------------------------------
 // U: [2][V] complex of precision R with the antiperiodic sign folded into the
-// t links at t = Lt - 1.  diag = 4 + m.
+// t links at t = Lt - 1.  diag = 4 + m.  W (FP64 vectors; may be null): the links of
+// fixed_links for this diag, which the integer kernel of fixed.cuh reads.
 template <typename R>
 cudaError_t wilson_D(const void* in, void* out, const void* U, double diag, int Lx, int Lt,
                      int nrhs, bool dagger, cudaStream_t s);
 template <typename R>
-cudaError_t wilson_A(const void* in, void* out, const void* U, double diag, int Lx, int Lt,
-                     int nrhs, const Epilogue& ep, cudaStream_t s);
+cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, double diag, int Lx,
+                     int Lt, int nrhs, const Epilogue& ep, cudaStream_t s);
+
+// A on FP64 vectors with the integer arithmetic of fixed.cuh, in tiles of tx x ty
+// sites (16 x 8, 32 x 8, 32 x 16; the results do not depend on the tile).
+// fixed_links fills W ([2][V] int4) for diag; wilson_A_fx_ok: whether the operator
+// and epilogue are ones the kernel takes.
+cudaError_t fixed_links(const void* U64, void* W, double diag, int Lx, int Lt, cudaStream_t s);
+bool wilson_A_fx_ok(const void* W, double diag, const Epilogue& ep);
+cudaError_t wilson_A_fx(int tx, int ty, const void* in, void* out, const void* U64, const void* W,
+                        double diag, int Lx, int Lt, int nrhs, const Epilogue& ep, cudaStream_t s);
 
 // out = sigma_3 in for V fine two-spinors (FP64); out may alias in.
 cudaError_t sigma3_mul(const void* in, void* out, long long V, cudaStream_t s);
@@ -160,13 +173,14 @@ struct StencilTuning {
 // device int); later wilson_A launches without the dot epilogue use the
 // fastest admitted shape.
 template <typename R>
-cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, double diag,
-                          int Lx, int Lt, int nrhs, int* dflag, cudaStream_t s);
+cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, const void* W,
+                          double diag, int Lx, int Lt, int nrhs, int* dflag, cudaStream_t s);
 // Copies up to max tuned shapes into out; returns how many exist.
 int stencil_tunings(StencilTuning* out, int max);
-// Thread blocks wilson_A launches per right-hand side (the fused <x, A x>
-// needs at most 608).
+// Thread blocks of the floating-point kernels per right-hand side with the fused
+// <x, A x> (which needs at most 608), and whether a fused launch fits at all.
 int wilson_A_ctas(int Lx, int Lt, bool f64);
+bool wilson_A_dot_fits(int Lx, int Lt, bool f64, double diag);
 // links: gauge complex128 [2][V] -> folded links of precision R
 template <typename R>
 cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s);

@@ -11,32 +11,10 @@
 #include <mutex>
 #include <tuple>
 
-#include "common.cuh"
 #include "kernels.h"
+#include "wilson.cuh"
 
 namespace mgk {
-
-template <typename R, bool DAG>
-__device__ __forceinline__ void wilson_site(const cplx_t<R>* __restrict__ in,
-                                            const cplx_t<R>* __restrict__ U, R diag, int x, int t,
-                                            int Lx, int Lt, cplx_t<R>& o0, cplx_t<R>& o1) {
-  using C = cplx_t<R>;
-  const int V = Lx * Lt;
-  const int site = x + Lx * t;
-  const int xp = (x + 1 == Lx) ? site - x : site + 1;
-  const int xm = (x == 0) ? site + Lx - 1 : site - 1;
-  const int tp = (t + 1 == Lt) ? x : site + Lx;
-  const int tm = (t == 0) ? site + (Lt - 1) * Lx : site - Lx;
-  const R sf = DAG ? (R)-1 : (R)1;   // projector sign of the forward hop
-  C a0 = mk((R)0, (R)0), a1 = mk((R)0, (R)0);
-  hop_x<R>(a0, a1, U[site], in[2 * xp], in[2 * xp + 1], sf);
-  hop_x<R>(a0, a1, cconj(U[xm]), in[2 * xm], in[2 * xm + 1], -sf);
-  hop_t<R>(a0, a1, U[V + site], in[2 * tp], in[2 * tp + 1], sf);
-  hop_t<R>(a0, a1, cconj(U[V + tm]), in[2 * tm], in[2 * tm + 1], -sf);
-  C p0 = in[2 * site], p1 = in[2 * site + 1];
-  o0 = mk(diag * p0.x - (R)0.5 * a0.x, diag * p0.y - (R)0.5 * a0.y);
-  o1 = mk(diag * p1.x - (R)0.5 * a1.x, diag * p1.y - (R)0.5 * a1.y);
-}
 
 template <typename R, bool DAG>
 __global__ void __launch_bounds__(256) k_wilson_D(const cplx_t<R>* __restrict__ in,
@@ -80,37 +58,6 @@ cudaError_t wilson_D(const void* in, void* out, const void* U, double diag, int 
 // memory below 48 KB); lattices with fewer than two tiles per SM use 16 x 8
 // tiles so that every SM gets work.
 
-template <typename R> struct spinor_t;              // both spin components of a site
-template <> struct spinor_t<float> { using type = float4; };
-template <> struct spinor_t<double> { using type = double4_32a; };
-
-__device__ __forceinline__ void split(const float4& v, float2& a, float2& b) {
-  a = make_float2(v.x, v.y);
-  b = make_float2(v.z, v.w);
-}
-__device__ __forceinline__ void split(const double4_32a& v, double2& a, double2& b) {
-  a = make_double2(v.x, v.y);
-  b = make_double2(v.z, v.w);
-}
-__device__ __forceinline__ float4 join(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
-__device__ __forceinline__ double4_32a join(double2 a, double2 b) {
-  double4_32a r;
-  r.x = a.x; r.y = a.y; r.z = b.x; r.w = b.y;
-  return r;
-}
-__device__ __forceinline__ float4 ld_spinor(const float2* p) { return *(const float4*)p; }
-__device__ __forceinline__ double4_32a ld_spinor(const double2* p) {
-  const double2 a = p[0], b = p[1];
-  return join(a, b);
-}
-__device__ __forceinline__ void st_spinor(float2* p, float4 v) { *(float4*)p = v; }
-__device__ __forceinline__ void st_spinor(double2* p, double4_32a v) {
-  p[0] = make_double2(v.x, v.y);
-  p[1] = make_double2(v.z, v.w);
-}
-
-__device__ __forceinline__ int wrap(int g, int L) { return g < 0 ? g + L : (g >= L ? g - L : g); }
-
 template <typename R, int TX, int TY, int RPT>
 __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict__ in,
                                                      cplx_t<R>* out,
@@ -130,11 +77,11 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
   const long long off = (long long)blockIdx.z * V * 2;
   const int tid = threadIdx.x;
   for (int q = tid; q < PH * PW; q += TX * TY) {
-    const int gx = wrap(x0 + q % PW - 2, Lx), gt = wrap(t0 + q / PW - 2, Lt);
+    const int gx = wrap_tile(x0 + q % PW - 2, Lx), gt = wrap_tile(t0 + q / PW - 2, Lt);
     sp[q] = ld_spinor(in + off + 2LL * (gx + Lx * gt));
   }
   for (int q = tid; q < UH * UW; q += TX * TY) {
-    const int gx = wrap(x0 + q % UW - 2, Lx), gt = wrap(t0 + q / UW - 2, Lt);
+    const int gx = wrap_tile(x0 + q % UW - 2, Lx), gt = wrap_tile(t0 + q / UW - 2, Lt);
     const int g = gx + Lx * gt;
     su[q][0] = U[g];
     su[q][1] = U[V + g];
@@ -282,17 +229,6 @@ __device__ __forceinline__ void dslash_row(cplx_t<R> f0, cplx_t<R> f1, cplx_t<R>
 // own spinor and links of a future row into a per-warp ring of SNB slots in
 // shared memory (cp.async), SNB - 1 iterations ahead of use.
 static constexpr int SNB = 4;
-
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem, int bytes) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  if (bytes == 16)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
 template <typename R>
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 3) k_wilson_A_stream(
@@ -446,16 +382,44 @@ static int wilson_default_variant(int Lx, int Lt, bool dot) {
   return f64 ? WV_32x8 : WV_32x8x2;
 }
 
+// FP64 vectors whose operator the integer kernel takes (wilson_A_fx_ok): its tiles
+// by the number of sites in the launch.  Measured (us, 16 x 8 / 32 x 8 / 32 x 16):
+// 128^2 6.2 / 6.3 / 8.3, 256^2 8.2 / 8.2 / 8.3, 512^2 18.2 / 16.4 / 16.5, 256^2 x 64
+// 237 / 191 / 172; with the fused dot 256^2 12.4 / 11.3 / 12.4, 210 x 90 x 12
+// 25.0 / 21.7 / 22.5, 256^2 x 64 325 / 251 / 207.  Small tiles spread few sites over
+// the SMs, large ones repeat less of the halo.  The fused dot takes at most 608 tiles.
+static int wilson_fx_variant(int Lx, int Lt, int nrhs, bool dot) {
+  const long long sites = (long long)Lx * Lt * nrhs;
+  int v = sites < (1 << 16) ? WV_16x8 : sites < (1 << 18) ? WV_32x8 : WV_32x8x2;
+  auto tiles = [&](int k) {
+    const int ty = WV_SHAPE[k][1] * WV_SHAPE[k][2];
+    return ((Lx + WV_SHAPE[k][0] - 1) / WV_SHAPE[k][0]) * ((Lt + ty - 1) / ty);
+  };
+  while (dot && tiles(v) > 608 && v != WV_32x8x2) v = v == WV_16x8 ? WV_32x8 : WV_32x8x2;
+  return v;
+}
+
+bool wilson_A_dot_fits(int Lx, int Lt, bool f64, double diag) {
+  if (f64 && fixed_diag_ok(diag)) return ((Lx + 31) / 32) * ((Lt + 15) / 16) <= 608;
+  return wilson_A_ctas(Lx, Lt, f64) <= 608;
+}
+
 template <typename R>
-static bool wilson_variant_ok(int v, int Lx, int Lt) {
+static bool wilson_variant_ok(int v, int Lx, int Lt, bool fx) {
+  if (fx) return v == WV_16x8 || v == WV_32x8 || v == WV_32x8x2;
   if (v == WV_STREAM) return wilson_A_streamed(Lx, Lt);
   if (sizeof(R) == 8 && (v == WV_32x8x2 || v == WV_64x4x2)) return false;   // shared memory
   return true;
 }
 
+// W: the fixed-point links when the integer kernel runs the launch, else null.
 template <typename R>
-static void launch_variant(int v, const void* in, void* out, const void* U, double diag, int Lx,
-                           int Lt, int nrhs, const Epilogue& ep, cudaStream_t s) {
+static cudaError_t launch_variant(int v, const void* in, void* out, const void* U, const void* W,
+                                  double diag, int Lx, int Lt, int nrhs, const Epilogue& ep,
+                                  cudaStream_t s) {
+  if (W)
+    return wilson_A_fx(WV_SHAPE[v][0], WV_SHAPE[v][1] * WV_SHAPE[v][2], in, out, U, W, diag, Lx, Lt,
+                       nrhs, ep, s);
   switch (v) {
     case WV_STREAM: {
       const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
@@ -474,21 +438,23 @@ static void launch_variant(int v, const void* in, void* out, const void* U, doub
       }
       break;
   }
+  return cudaGetLastError();
 }
 
 struct TuneKey {
   int prec, Lx, Lt, nrhs;
+  bool fx;
   bool operator<(const TuneKey& o) const {
-    return std::tie(prec, Lx, Lt, nrhs) < std::tie(o.prec, o.Lx, o.Lt, o.nrhs);
+    return std::tie(prec, Lx, Lt, nrhs, fx) < std::tie(o.prec, o.Lx, o.Lt, o.nrhs, o.fx);
   }
 };
 static std::mutex g_tune_mu;
 static std::map<TuneKey, StencilTuning> g_tune;
 
 template <typename R>
-static int tuned_variant(int Lx, int Lt, int nrhs) {
+static int tuned_variant(int Lx, int Lt, int nrhs, bool fx) {
   std::lock_guard<std::mutex> g(g_tune_mu);
-  auto it = g_tune.find({(int)sizeof(R), Lx, Lt, nrhs});
+  auto it = g_tune.find({(int)sizeof(R), Lx, Lt, nrhs, fx});
   return it == g_tune.end() ? -1 : it->second.variant;
 }
 
@@ -500,15 +466,16 @@ __global__ void k_count_diff(const unsigned long long* __restrict__ a,
 }
 
 template <typename R>
-cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, double diag,
-                          int Lx, int Lt, int nrhs, int* dflag, cudaStream_t s) {
-  const TuneKey key{(int)sizeof(R), Lx, Lt, nrhs};
+cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, const void* W,
+                          double diag, int Lx, int Lt, int nrhs, int* dflag, cudaStream_t s) {
+  const Epilogue none{};
+  if (!(sizeof(R) == 8 && wilson_A_fx_ok(W, diag, none))) W = nullptr;
+  const TuneKey key{(int)sizeof(R), Lx, Lt, nrhs, W != nullptr};
   {
     std::lock_guard<std::mutex> g(g_tune_mu);
     if (g_tune.count(key)) return cudaSuccess;
   }
-  const Epilogue none{};
-  const int def = wilson_default_variant<R>(Lx, Lt, false);
+  const int def = W ? wilson_fx_variant(Lx, Lt, nrhs, false) : wilson_default_variant<R>(Lx, Lt, false);
   const long long words = (long long)Lx * Lt * nrhs * 2 * sizeof(cplx_t<R>) / 8;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -518,11 +485,11 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, d
   t.Lx = Lx; t.Lt = Lt; t.nrhs = nrhs;
   t.variant = def;
   float best = 0.f;
-  launch_variant<R>(def, in, ref, U, diag, Lx, Lt, nrhs, none, s);
+  launch_variant<R>(def, in, ref, U, W, diag, Lx, Lt, nrhs, none, s);
   for (int v = 0; v < WV_COUNT; ++v) {
-    if (!wilson_variant_ok<R>(v, Lx, Lt)) continue;
+    if (!wilson_variant_ok<R>(v, Lx, Lt, W != nullptr)) continue;
     ++t.tried;
-    launch_variant<R>(v, in, out, U, diag, Lx, Lt, nrhs, none, s);
+    launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     int diff = 0;
     cudaMemsetAsync(dflag, 0, sizeof(int), s);
     k_count_diff<<<152, 256, 0, s>>>((const unsigned long long*)out,
@@ -536,10 +503,10 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, d
     }
     if (diff) continue;                                    // not bit-identical: never used
     ++t.admitted;
-    for (int w = 0; w < 2; ++w) launch_variant<R>(v, in, out, U, diag, Lx, Lt, nrhs, none, s);
+    for (int w = 0; w < 2; ++w) launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     constexpr int REPS = 10;
     cudaEventRecord(e0, s);
-    for (int w = 0; w < REPS; ++w) launch_variant<R>(v, in, out, U, diag, Lx, Lt, nrhs, none, s);
+    for (int w = 0; w < REPS; ++w) launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     cudaEventRecord(e1, s);
     cudaEventSynchronize(e1);
     float ms = 0.f;
@@ -581,15 +548,17 @@ int stencil_tunings(StencilTuning* out, int max) {
 }
 
 template <typename R>
-cudaError_t wilson_A(const void* in, void* out, const void* U, double diag, int Lx, int Lt,
-                     int nrhs, const Epilogue& ep, cudaStream_t s) {
+cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, double diag, int Lx,
+                     int Lt, int nrhs, const Epilogue& ep, cudaStream_t s) {
   const bool dot = ep.dot_out != nullptr;
-  if (dot && (nrhs > 64 || wilson_A_ctas(Lx, Lt, sizeof(R) == 8) > 608)) return cudaErrorInvalidValue;
-  int v = dot ? -1 : tuned_variant<R>(Lx, Lt, nrhs);
-  if (v < 0) v = wilson_default_variant<R>(Lx, Lt, dot);
-  launch_variant<R>(v, in, out, U, diag, Lx, Lt, nrhs, ep, s);
+  if (!(sizeof(R) == 8 && wilson_A_fx_ok(W, diag, ep))) W = nullptr;
+  if (dot && (nrhs > 64 || !wilson_A_dot_fits(Lx, Lt, sizeof(R) == 8, W ? diag : 0.0)))
+    return cudaErrorInvalidValue;
+  int v = dot ? -1 : tuned_variant<R>(Lx, Lt, nrhs, W != nullptr);
+  if (v < 0) v = W ? wilson_fx_variant(Lx, Lt, nrhs, dot) : wilson_default_variant<R>(Lx, Lt, dot);
+  const cudaError_t e = launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, ep, s);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 // out = sigma_3 in on V two-spinors (FP64): spin component 1 negated.
@@ -655,10 +624,10 @@ cudaError_t link_unitarity(const void* gauge, long long count, double* out, cuda
 #define INST(R)                                                                               \
   template cudaError_t wilson_D<R>(const void*, void*, const void*, double, int, int, int,    \
                                    bool, cudaStream_t);                                       \
-  template cudaError_t wilson_A<R>(const void*, void*, const void*, double, int, int, int,    \
-                                   const Epilogue&, cudaStream_t);                            \
-  template cudaError_t wilson_A_tune<R>(const void*, void*, void*, const void*, double, int,   \
-                                        int, int, int*, cudaStream_t);                        \
+  template cudaError_t wilson_A<R>(const void*, void*, const void*, const void*, double, int,   \
+                                   int, int, const Epilogue&, cudaStream_t);                  \
+  template cudaError_t wilson_A_tune<R>(const void*, void*, void*, const void*, const void*,   \
+                                        double, int, int, int, int*, cudaStream_t);           \
   template cudaError_t fold_links<R>(const void*, void*, int, int, cudaStream_t);
 INST(double)
 INST(float)

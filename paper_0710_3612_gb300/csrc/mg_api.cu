@@ -53,6 +53,7 @@ struct mg_handle {
   std::vector<Level> lv;
   double2* U64 = nullptr;
   float2* U32 = nullptr;
+  void* Wfx = nullptr;          // fixed-point links of the current mass (fixed_links)
   // coarsest level
   int Nc = 0, ldc = 0;
   float2* Binv = nullptr;
@@ -207,7 +208,7 @@ void apply_level(mg_handle* h, int l, const void* in, void* out, int nrhs, int w
   if (l == 0) {
     const double diag = 4.0 + h->mass;
     const void* U = sizeof(R) == 8 ? (const void*)h->U64 : (const void*)h->U32;
-    ck(h, wilson_A<R>(in, out, U, diag, L.Lx, L.Lt, nrhs, ep, h->s), "wilson_A");
+    ck(h, wilson_A<R>(in, out, U, h->Wfx, diag, L.Lx, L.Lt, nrhs, ep, h->s), "wilson_A");
   } else {
     const void* A = weights == W_F64 ? (const void*)L.A64
                     : weights == W_F32 ? (const void*)L.A32 : L.A16;
@@ -631,9 +632,16 @@ void drop_graphs(mg_handle* h) {
     }
 }
 
+// The mass of the operator and the fixed-point links that go with it.
+void set_operator_mass(mg_handle* h, double mass) {
+  h->mass = mass;
+  if (fixed_diag_ok(4.0 + mass))
+    ck(h, fixed_links(h->U64, h->Wfx, 4.0 + mass, h->lv[0].Lx, h->lv[0].Lt, h->s), "fixed links");
+}
+
 void set_mass_internal(mg_handle* h, double mass) {
   drop_graphs(h);
-  h->mass = mass;
+  set_operator_mass(h, mass);
   build_coarse_ops(h);
   for (int l = 0; l + 1 < h->L; ++l)
     smoother_coefficients(h, l, h->lv[l].w64[3], h->lv[l].w64[2]);
@@ -803,7 +811,7 @@ void apply_pq(mg_handle* h, int nrhs, int pmode) {
   const Level& F = h->lv[0];
   Epilogue ep;
   if (pmode == 3) {
-    if (wilson_A_ctas(F.Lx, F.Lt, false) <= 608) {
+    if (wilson_A_dot_fits(F.Lx, F.Lt, false, 0.0)) {
       ep.dot_ws = h->partials;
       ep.dot_out = slot(h, S_PQ);
     }
@@ -812,9 +820,10 @@ void apply_pq(mg_handle* h, int nrhs, int pmode) {
       ck(h, rdot(h->sv32[0], h->sv32[2], n, nrhs, h->partials, slot(h, S_PQ), h->s), "dot");
     return;
   }
-  if (wilson_A_ctas(F.Lx, F.Lt, true) <= 608) {
+  if (wilson_A_dot_fits(F.Lx, F.Lt, true, 4.0 + h->mass)) {
     ep.dot_ws = h->partials;
     ep.dot_out = slot(h, S_PQ);
+    ep.dot_real = true;
   }
   apply_level<double>(h, 0, h->sv64[2], h->sv64[3], nrhs, W_F64, ep);
   if (!ep.dot_out)
@@ -861,7 +870,7 @@ void pcg_direction(mg_handle* h, int pmode, int nrhs) {
     tail.dot_out = slot(h, S_T0);
     tail.zq_q = q;
     tail.zq_r = r;
-    const bool fused = nrhs > 1 && wilson_A_ctas(F.Lx, F.Lt, false) <= 608;
+    const bool fused = nrhs > 1 && wilson_A_dot_fits(F.Lx, F.Lt, false, 0.0);
     vcycle<float>(h, 0, h->sv32[1], h->sv32[4], nrhs, fused ? &tail : nullptr);
     if (!fused)
       ck(h, dot2_zq_rz(h->sv32[4], q, r, n, nrhs, h->partials, slot(h, S_T0), h->s), "dot2");
@@ -1219,6 +1228,7 @@ void allocate_storage(mg_handle* h) {
   const long long V = h->lv[0].V;
   h->U64 = dalloc<double2>(h, 2 * V * sizeof(double2));
   h->U32 = dalloc<float2>(h, 2 * V * sizeof(float2));
+  h->Wfx = dalloc(h, 2 * V * sizeof(int4));
   // per-level storage
   for (int l = 0; l < h->L; ++l) {
     Level& L = h->lv[l];
@@ -1547,9 +1557,9 @@ void autotune_fine(mg_handle* h) {
                           cudaMemcpyDeviceToDevice, h->s), "tune input");
   ck(h, convert_f64_f32(h->sv64[0], h->sv32[0], c * h->R, h->s), "tune input");
   for (int nrhs : {1, h->R}) {
-    ck(h, wilson_A_tune<double>(h->sv64[0], h->sv64[1], h->sv64[2], h->U64, diag, F.Lx, F.Lt,
+    ck(h, wilson_A_tune<double>(h->sv64[0], h->sv64[1], h->sv64[2], h->U64, h->Wfx, diag, F.Lx, F.Lt,
                                 nrhs, h->dflag, h->s), "tune f64");
-    ck(h, wilson_A_tune<float>(h->sv32[0], h->sv32[1], h->sv32[2], h->U32, diag, F.Lx, F.Lt,
+    ck(h, wilson_A_tune<float>(h->sv32[0], h->sv32[1], h->sv32[2], h->U32, nullptr, diag, F.Lx, F.Lt,
                                nrhs, h->dflag, h->s), "tune f32");
     if (h->R == 1) break;
   }
@@ -1722,13 +1732,13 @@ mg_status refine_core(mg_handle* src, int lr, const void* e0, int ncycles, const
     set_geometry(h);
     init_runtime(h);
     allocate_storage(h);
-    h->mass = src->mass;
     const long long V = h->lv[0].V;
     auto copy = [&](void* d, const void* sp, size_t bytes) {
       ck(h, cudaMemcpyAsync(d, sp, bytes, cudaMemcpyDeviceToDevice, h->s), "refine copy");
     };
     copy(h->U64, src->U64, 2 * V * sizeof(double2));
     copy(h->U32, src->U32, 2 * V * sizeof(float2));
+    set_operator_mass(h, src->mass);
     size_t pos = 0;
     for (int l = 0; l + 1 < h->L; ++l) {
       Level& L = h->lv[l];
@@ -1843,7 +1853,7 @@ mg_status mg_setup(const void* gauge, double mass, const mg_params* params, void
     if (!(dev <= 1e-12)) fail(h, MG_ERR_ARG, "gauge links are not unit modulus (|U|-1 = " + std::to_string(dev) + ")");
     ck(h, fold_links<double>(gauge, h->U64, P.Lx, P.Lt, h->s), "fold");
     ck(h, fold_links<float>(gauge, h->U32, P.Lx, P.Lt, h->s), "fold");
-    h->mass = mass;
+    set_operator_mass(h, mass);
     // adaptive setup, level by level (Sec. 3)
     const double2* noise = (const double2*)P.setup_noise;
     size_t pos = 0;
@@ -2355,7 +2365,7 @@ extern "C" mg_status mg_apply_A_dot_noalloc(mg_handle* h, const void* in, void* 
     Epilogue ep;
     ep.dot_ws = ws;
     ep.dot_out = xAx;
-    ck(h, wilson_A<double>(in, out, h->U64, 4.0 + h->mass, F.Lx, F.Lt, 1, ep, h->s), "wilson_A");
+    ck(h, wilson_A<double>(in, out, h->U64, h->Wfx, 4.0 + h->mass, F.Lx, F.Lt, 1, ep, h->s), "wilson_A");
   });
 }
 
