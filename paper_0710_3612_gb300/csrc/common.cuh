@@ -76,40 +76,49 @@ __device__ __forceinline__ void hop_t(cplx_t<R>& a0, cplx_t<R>& a1, cplx_t<R> u,
 
 __device__ __forceinline__ float2 bf2_to_f2(__nv_bfloat162 v) { return __bfloat1622float2(v); }
 
-// Fixed-order block reduction of (a, b) pairs held one per thread.
-__device__ __forceinline__ void block_sum2(double& a, double& b, double* sh) {
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_down_sync(0xffffffffu, a, o);
-    b += __shfl_down_sync(0xffffffffu, b, o);
-  }
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) { sh[2 * w] = a; sh[2 * w + 1] = b; }
+// Fixed-order block sums of one double per thread (N = 1) or two (N = 2), returned in
+// thread 0.  sh holds N * blockDim doubles.  Each lane of warp 0 (and of warp 1 for the
+// second number) first adds the entries of its column, so a 256-thread block issues 12
+// FP64 additions per number where shuffles in every warp would issue 45: the FP64 pipe
+// takes 16 clocks for each, and small reductions were bound by it.
+template <int N>
+__device__ __forceinline__ void block_sum(double& a, double& b, double* sh) {
+  const int n = blockDim.x, w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  sh[threadIdx.x] = a;
+  if (N == 2) sh[n + threadIdx.x] = b;
   __syncthreads();
-  if (w == 0) {
-    const int nw = blockDim.x >> 5;
-    a = l < nw ? sh[2 * l] : 0.0;
-    b = l < nw ? sh[2 * l + 1] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_down_sync(0xffffffffu, a, o);
-      b += __shfl_down_sync(0xffffffffu, b, o);
-    }
+  if (w < N && (N == 1 || n > 32)) {
+    double v = 0.0;
+    for (int i = l; i < n; i += 32) v += sh[w * n + i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    __syncwarp();
+    if (l == 0) sh[w * n] = v;
   }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a = sh[0];
+    if (N == 2) b = sh[n];
+  }
+  __syncthreads();
 }
 
 // Single-pass deterministic reduction.  Every block writes its partial sum;
 // the last block to finish (found with an atomic ticket) adds the partials in
 // a fixed order and resets the ticket.  ws = [64 tickets (as doubles)][partials].
-// rhs selects the output and ticket; blk in [0, G) is this block's slot.
+// rhs selects the output and ticket; blk in [0, G) is this block's slot; sh holds
+// N * blockDim doubles (at least 64 threads for N = 2).  N = 1: the real part alone,
+// the imaginary sum is written as zero.
 // Returns true in the block that wrote the sum (all its threads).
+template <int N>
 __device__ __forceinline__ bool finish_reduction_g(double re, double im, double* ws, double* out,
                                                    double* sh, int rhs, int blk, int G) {
   unsigned* tickets = (unsigned*)ws;
   double* partials = ws + 64;
   __shared__ bool last;
-  block_sum2(re, im, sh);
+  block_sum<N>(re, im, sh);
   if (threadIdx.x == 0) {
     partials[2 * ((long long)rhs * G + blk)] = re;
-    partials[2 * ((long long)rhs * G + blk) + 1] = im;
+    if (N == 2) partials[2 * ((long long)rhs * G + blk) + 1] = im;
     __threadfence();
     last = atomicAdd(&tickets[rhs], 1u) == (unsigned)(G - 1);
   }
@@ -120,60 +129,21 @@ __device__ __forceinline__ bool finish_reduction_g(double re, double im, double*
   im = 0.0;
   for (int i = threadIdx.x; i < G; i += blockDim.x) {
     re += __ldcg(&partials[2 * ((long long)rhs * G + i)]);
-    im += __ldcg(&partials[2 * ((long long)rhs * G + i) + 1]);
+    if (N == 2) im += __ldcg(&partials[2 * ((long long)rhs * G + i) + 1]);
   }
-  __syncthreads();
-  block_sum2(re, im, sh);
+  block_sum<N>(re, im, sh);
   if (threadIdx.x == 0) {
     out[2 * rhs] = re;
-    out[2 * rhs + 1] = im;
+    out[2 * rhs + 1] = N == 2 ? im : 0.0;
     tickets[rhs] = 0u;
   }
   return true;
 }
 
-// The real part alone (the imaginary sum is written as zero): half the FP64 additions.
-__device__ __forceinline__ bool finish_reduction_re(double re, double* ws, double* out, double* sh,
-                                                    int rhs, int blk, int G) {
-  unsigned* tickets = (unsigned*)ws;
-  double* partials = ws + 64;
-  __shared__ bool last_re;
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
-  auto block_sum = [&](double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    if (w == 0) {
-      v = l < nw ? sh[l] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    }
-    return v;
-  };
-  re = block_sum(re);
-  if (threadIdx.x == 0) {
-    partials[2 * ((long long)rhs * G + blk)] = re;
-    __threadfence();
-    last_re = atomicAdd(&tickets[rhs], 1u) == (unsigned)(G - 1);
-  }
-  __syncthreads();
-  if (!last_re) return false;
-  __threadfence();
-  re = 0.0;
-  for (int i = threadIdx.x; i < G; i += blockDim.x)
-    re += __ldcg(&partials[2 * ((long long)rhs * G + i)]);
-  __syncthreads();
-  re = block_sum(re);
-  if (threadIdx.x == 0) {
-    out[2 * rhs] = re;
-    out[2 * rhs + 1] = 0.0;
-    tickets[rhs] = 0u;
-  }
-  return true;
-}
-
+template <int N>
 __device__ __forceinline__ bool finish_reduction(double re, double im, double* ws, double* out,
                                                  double* sh) {
-  return finish_reduction_g(re, im, ws, out, sh, blockIdx.y, blockIdx.x, gridDim.x);
+  return finish_reduction_g<N>(re, im, ws, out, sh, blockIdx.y, blockIdx.x, gridDim.x);
 }
 
 // Block map of the geometric blocking S_j: coarse site and in-block offset.

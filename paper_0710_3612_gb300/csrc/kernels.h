@@ -18,8 +18,8 @@ void count_launch();
 void add_launches(long long n);
 
 // ---- deterministic reductions -------------------------------------------
-// Number of partial sums a reduction over `count` complex entries produces.
-int reduce_blocks(long long count);
+// Number of partial sums a reduction over `count` complex entries of each of nrhs vectors produces.
+int reduce_blocks(long long count, int nrhs);
 // Reductions take a workspace ws of (64 + 2 * 608 * nrhs) doubles whose first
 // 64 doubles (tickets) are zero before the first call (they are left zero);
 // nrhs <= 64.  One launch: the last block adds the partials in fixed order.

@@ -15,23 +15,36 @@ void add_launches(long long n) { g_launches.fetch_add((unsigned long long)n, std
 
 static constexpr int RT = 256;   // threads per reduction block
 
-int reduce_blocks(long long count) {
-  long long g = (count + RT - 1) / RT;           // one entry per thread until 608 blocks
-
-  if (g < 1) g = 1;
-  if (g > 608) g = 608;           // 4 x 152 SMs
+// Blocks per right-hand side: one entry per thread as long as the whole launch stays
+// below 8 blocks per SM, up to 16 entries per thread beyond (a block's sum and its
+// scalar division cost as many FP64 issue slots as 16 entries per thread do; with one
+// entry each, cg_xr on 131072 x 64 entries took 361 us, 129 us of it HBM time).
+int reduce_blocks(long long count, int nrhs) {
+  long long g = (count + RT - 1) / RT;
+  g = g < 1 ? 1 : g > 608 ? 608 : g;           // 4 x 152 SMs
+  while (g * nrhs > 8 * 152 && count < 8 * g * RT) g = (g + 1) / 2;
   return (int)g;
+}
+
+// num / den of the right-hand side, divided once per block (0 when den = 0)
+__device__ __forceinline__ double block_ratio(double num, double den) {
+  __shared__ double ratio;
+  if (threadIdx.x == 0) ratio = den != 0.0 ? num / den : 0.0;
+  __syncthreads();
+  return ratio;
 }
 
 template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT) k_dot(const cplx_t<R>* __restrict__ a,
                                             const cplx_t<R>* __restrict__ b, long long count,
                                             double* ws, double* out) {
-  __shared__ double sh[2 * RT / 32];
+  constexpr int N = NORM ? 1 : 2;
+  __shared__ double sh[N * RT];
   const int rhs = blockIdx.y;
   const cplx_t<R>* pa = a + (long long)rhs * count;
   const cplx_t<R>* pb = NORM ? pa : b + (long long)rhs * count;
   double re = 0.0, im = 0.0;
+#pragma unroll 4
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     cplx_t<R> u = pa[i];
@@ -46,14 +59,14 @@ __global__ void __launch_bounds__(RT) k_dot(const cplx_t<R>* __restrict__ a,
       im = fma(-(double)u.y, (double)v.x, im);
     }
   }
-  finish_reduction(re, im, ws, out, sh);
+  finish_reduction<N>(re, im, ws, out, sh);
 }
 
 template <typename R>
 cudaError_t dot(const void* a, const void* b, long long count, int nrhs, double* partials,
                 double* out, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  int g = reduce_blocks(count);
+  const int g = reduce_blocks(count, nrhs);
   k_dot<R, false><<<dim3(g, nrhs), RT, 0, s>>>((const cplx_t<R>*)a, (const cplx_t<R>*)b, count,
                                                partials, out);
   count_launch();
@@ -64,7 +77,7 @@ template <typename R>
 cudaError_t norm2(const void* a, long long count, int nrhs, double* partials, double* out,
                   cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  int g = reduce_blocks(count);
+  const int g = reduce_blocks(count, nrhs);
   k_dot<R, true><<<dim3(g, nrhs), RT, 0, s>>>((const cplx_t<R>*)a, nullptr, count, partials, out);
   count_launch();
   return cudaGetLastError();
@@ -123,13 +136,13 @@ __global__ void __launch_bounds__(RT) k_cg_xr(cplx_t<R>* __restrict__ x, cplx_t<
                                               const double* pq, const int* frozen,
                                               long long count, double* ws, double* rr,
                                               float2* __restrict__ r32, CgControl cc) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
-  const double d = pq[2 * rhs];
-  const R alpha = (d != 0.0 && !skip) ? (R)(rz[2 * rhs] / d) : (R)0;
+  const R alpha = (R)block_ratio(rz[2 * rhs], pq[2 * rhs]);
   double acc = 0.0;
   const long long base = (long long)rhs * count;
+#pragma unroll 2
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     const long long k = base + i;
@@ -144,7 +157,7 @@ __global__ void __launch_bounds__(RT) k_cg_xr(cplx_t<R>* __restrict__ x, cplx_t<
     acc = fma((double)rv.x, (double)rv.x, acc);
     acc = fma((double)rv.y, (double)rv.y, acc);
   }
-  const bool done = finish_reduction(acc, 0.0, ws, rr, sh);
+  const bool done = finish_reduction<1>(acc, 0.0, ws, rr, sh);
   // loop control in the block that completes the last right-hand side's sum
   if (cc.ctrl && done && threadIdx.x == 0) {
     __threadfence();
@@ -161,7 +174,7 @@ cudaError_t cg_xr(void* x, void* r, const void* p, const void* q, const double* 
                   const double* pq, const int* frozen, long long count, int nrhs, double* ws,
                   double* rr, cudaStream_t s, void* r32, const CgControl* cc) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  int g = reduce_blocks(count);
+  const int g = reduce_blocks(count, nrhs);
   k_cg_xr<R><<<dim3(g, nrhs), RT, 0, s>>>((cplx_t<R>*)x, (cplx_t<R>*)r, (const cplx_t<R>*)p,
                                           (const cplx_t<R>*)q, rz, pq, frozen, count, ws, rr,
                                           (float2*)r32, cc ? *cc : CgControl{});
@@ -170,24 +183,27 @@ cudaError_t cg_xr(void* x, void* r, const void* p, const void* q, const double* 
 }
 
 template <typename R>
-__global__ void k_cg_p(cplx_t<R>* __restrict__ p, const cplx_t<R>* __restrict__ z,
-                       const double* rz_new, const double* rz_old, const int* frozen,
-                       long long count) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(RT) k_cg_p(cplx_t<R>* __restrict__ p, const cplx_t<R>* __restrict__ z,
+                                             const double* rz_new, const double* rz_old,
+                                             const int* frozen, long long count) {
   const int rhs = blockIdx.y;
-  if (i >= count || (frozen && frozen[rhs])) return;
-  const double d = rz_old[2 * rhs];
-  const R beta = d != 0.0 ? (R)(rz_new[2 * rhs] / d) : (R)0;
-  i += (long long)rhs * count;
-  cplx_t<R> pv = p[i], zv = z[i];
-  p[i] = mk(fma(beta, pv.x, zv.x), fma(beta, pv.y, zv.y));
+  if (frozen && frozen[rhs]) return;
+  const R beta = (R)block_ratio(rz_new[2 * rhs], rz_old[2 * rhs]);
+  const long long base = (long long)rhs * count;
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
+       i += (long long)gridDim.x * RT) {
+    const cplx_t<R> pv = p[base + i], zv = z[base + i];
+    p[base + i] = mk(fma(beta, pv.x, zv.x), fma(beta, pv.y, zv.y));
+  }
 }
 
 template <typename R>
 cudaError_t cg_p(void* p, const void* z, const double* rz_new, const double* rz_old,
                  const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_cg_p<R><<<grid1(count, nrhs), RT, 0, s>>>((cplx_t<R>*)p, (const cplx_t<R>*)z, rz_new, rz_old,
-                                               frozen, count); count_launch();
+  k_cg_p<R><<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+      (cplx_t<R>*)p, (const cplx_t<R>*)z, rz_new, rz_old, frozen, count);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -272,9 +288,10 @@ __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
                                                    const double2* __restrict__ q,
                                                    const double2* __restrict__ r, long long count,
                                                    double* ws, double* zr) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   double a = 0.0, b = 0.0;
+#pragma unroll 4
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     const float2 zv = z[base + i];
@@ -284,13 +301,13 @@ __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
     b = fma(rv.x, (double)zv.x, b);
     b = fma(rv.y, (double)zv.y, b);
   }
-  finish_reduction(a, b, ws, zr, sh);
+  finish_reduction<2>(a, b, ws, zr, sh);
 }
 
 cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long count, int nrhs,
                        double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_dot2_zq_rz<<<dim3(reduce_blocks(count), nrhs), RT, 0, s>>>(
+  k_dot2_zq_rz<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
       (const float2*)z32, (const double2*)q, (const double2*)r, count, ws, zr);
   count_launch();
   return cudaGetLastError();
@@ -298,28 +315,30 @@ cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long 
 
 // beta = -zr[0] / Re(pq); p = z32 + beta p; rz <- {zr[1], 0}; per rhs, frozen
 // right-hand sides untouched.
-__global__ void k_cg_p_pr(double2* __restrict__ p, const float2* __restrict__ z, const double* zr,
-                          const double* pq, double* rz, const int* frozen, long long count) {
+__global__ void __launch_bounds__(RT) k_cg_p_pr(double2* __restrict__ p, const float2* __restrict__ z,
+                                                const double* zr, const double* pq, double* rz,
+                                                const int* frozen, long long count) {
   const int rhs = blockIdx.y;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (frozen && frozen[rhs]) return;
-  if (i == 0) {
+  const double beta = block_ratio(-zr[2 * rhs], pq[2 * rhs]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     rz[2 * rhs] = zr[2 * rhs + 1];
     rz[2 * rhs + 1] = 0.0;
   }
-  if (i >= count) return;
-  const double d = pq[2 * rhs];
-  const double beta = d != 0.0 ? -zr[2 * rhs] / d : 0.0;
-  const long long k = (long long)rhs * count + i;
-  const double2 pv = p[k];
-  const float2 zv = z[k];
-  p[k] = make_double2(fma(beta, pv.x, (double)zv.x), fma(beta, pv.y, (double)zv.y));
+  const long long base = (long long)rhs * count;
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
+       i += (long long)gridDim.x * RT) {
+    const double2 pv = p[base + i];
+    const float2 zv = z[base + i];
+    p[base + i] = make_double2(fma(beta, pv.x, (double)zv.x), fma(beta, pv.y, (double)zv.y));
+  }
 }
 
 cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq, double* rz,
                     const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_cg_p_pr<<<grid1(count, nrhs), RT, 0, s>>>((double2*)p, (const float2*)z32, zr, pq, rz, frozen,
-                                               count);
+  k_cg_p_pr<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+      (double2*)p, (const float2*)z32, zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -335,7 +354,7 @@ cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq
 __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
                                              const float2* __restrict__ b, long long count,
                                              double* ws, double* out) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float re = 0.f, im = 0.f;
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
@@ -344,13 +363,13 @@ __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
     re = fmaf(u.x, v.x, fmaf(u.y, v.y, re));
     im = fmaf(u.x, v.y, fmaf(-u.y, v.x, im));
   }
-  finish_reduction((double)re, (double)im, ws, out, sh);
+  finish_reduction<2>((double)re, (double)im, ws, out, sh);
 }
 
 cudaError_t rdot(const void* a, const void* b, long long count, int nrhs, double* ws, double* out,
                  cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rdot<<<dim3(reduce_blocks(count), nrhs), RT, 0, s>>>((const float2*)a, (const float2*)b,
+  k_rdot<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>((const float2*)a, (const float2*)b,
                                                          count, ws, out);
   count_launch();
   return cudaGetLastError();
@@ -364,11 +383,10 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
                                                const float2* __restrict__ q, const double* rz,
                                                const double* pq, const int* frozen,
                                                long long count, double* ws, double* rr) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
-  const double d = pq[2 * rhs];
-  const float alpha = (d != 0.0 && !skip) ? (float)(rz[2 * rhs] / d) : 0.f;
+  const float alpha = (float)block_ratio(rz[2 * rhs], pq[2 * rhs]);
   float acc = 0.f;
   const long long base = (long long)rhs * count;
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
@@ -383,14 +401,14 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
     }
     acc = fmaf(rv.x, rv.x, fmaf(rv.y, rv.y, acc));
   }
-  finish_reduction((double)acc, 0.0, ws, rr, sh);
+  finish_reduction<1>((double)acc, 0.0, ws, rr, sh);
 }
 
 cudaError_t rcg_xr(void* x32, void* r32, const void* p32, const void* q32, const double* rz,
                    const double* pq, const int* frozen, long long count, int nrhs, double* ws,
                    double* rr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rcg_xr<<<dim3(reduce_blocks(count), nrhs), RT, 0, s>>>(
+  k_rcg_xr<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
       (float2*)x32, (float2*)r32, (const float2*)p32, (const float2*)q32, rz, pq, frozen, count,
       ws, rr);
   count_launch();
@@ -402,7 +420,7 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
                                                     const float2* __restrict__ q,
                                                     const float2* __restrict__ r, long long count,
                                                     double* ws, double* zr) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float a = 0.f, b = 0.f;
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
@@ -411,40 +429,41 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
     a = fmaf(zv.x, qv.x, fmaf(zv.y, qv.y, a));
     b = fmaf(rv.x, zv.x, fmaf(rv.y, zv.y, b));
   }
-  finish_reduction((double)a, (double)b, ws, zr, sh);
+  finish_reduction<2>((double)a, (double)b, ws, zr, sh);
 }
 
 cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long long count,
                         int nrhs, double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rdot2_zq_rz<<<dim3(reduce_blocks(count), nrhs), RT, 0, s>>>(
+  k_rdot2_zq_rz<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
       (const float2*)z32, (const float2*)q32, (const float2*)r32, count, ws, zr);
   count_launch();
   return cudaGetLastError();
 }
 
 // beta = -zr[0] / Re(pq); p = z + beta p (FP32); rz <- {zr[1], 0}.
-__global__ void k_rcg_p(float2* __restrict__ p, const float2* __restrict__ z, const double* zr,
-                        const double* pq, double* rz, const int* frozen, long long count) {
+__global__ void __launch_bounds__(RT) k_rcg_p(float2* __restrict__ p, const float2* __restrict__ z,
+                                              const double* zr, const double* pq, double* rz,
+                                              const int* frozen, long long count) {
   const int rhs = blockIdx.y;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (frozen && frozen[rhs]) return;
-  if (i == 0) {
+  const float beta = (float)block_ratio(-zr[2 * rhs], pq[2 * rhs]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
     rz[2 * rhs] = zr[2 * rhs + 1];
     rz[2 * rhs + 1] = 0.0;
   }
-  if (i >= count) return;
-  const double d = pq[2 * rhs];
-  const float beta = d != 0.0 ? (float)(-zr[2 * rhs] / d) : 0.f;
-  const long long k = (long long)rhs * count + i;
-  const float2 pv = p[k], zv = z[k];
-  p[k] = make_float2(fmaf(beta, pv.x, zv.x), fmaf(beta, pv.y, zv.y));
+  const long long base = (long long)rhs * count;
+  for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
+       i += (long long)gridDim.x * RT) {
+    const float2 pv = p[base + i], zv = z[base + i];
+    p[base + i] = make_float2(fmaf(beta, pv.x, zv.x), fmaf(beta, pv.y, zv.y));
+  }
 }
 
 cudaError_t rcg_p(void* p32, const void* z32, const double* zr, const double* pq, double* rz,
                   const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_rcg_p<<<grid1(count, nrhs), RT, 0, s>>>((float2*)p32, (const float2*)z32, zr, pq, rz, frozen,
-                                             count);
+  k_rcg_p<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+      (float2*)p32, (const float2*)z32, zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -496,7 +515,7 @@ cudaError_t ru_fold(void* x64, void* x32, long long count, cudaStream_t s) {
 __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ r,
                                                     float2* __restrict__ r32, long long count,
                                                     double* ws, double* rr) {
-  __shared__ double sh[2 * RT / 32];
+  __shared__ double sh[RT];
   const long long base = (long long)blockIdx.y * count;
   double acc = 0.0;
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
@@ -505,7 +524,7 @@ __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ 
     r32[base + i] = make_float2((float)v.x, (float)v.y);
     acc = fma(v.x, v.x, fma(v.y, v.y, acc));
   }
-  finish_reduction(acc, 0.0, ws, rr, sh);
+  finish_reduction<1>(acc, 0.0, ws, rr, sh);
 }
 
 __global__ void k_copy_slots(const double* src, double* dst, int n2) {
@@ -516,7 +535,7 @@ __global__ void k_copy_slots(const double* src, double* dst, int n2) {
 cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, double* ws,
                         double* rr, double* rmax, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_ru_residual<<<dim3(reduce_blocks(count), nrhs), RT, 0, s>>>((const double2*)r64, (float2*)r32,
+  k_ru_residual<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>((const double2*)r64, (float2*)r32,
                                                                 count, ws, rr);
   count_launch();
   if (rmax) {

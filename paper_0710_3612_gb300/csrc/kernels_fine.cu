@@ -166,14 +166,15 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
     st_spinor(out + g, join(y0, y1));
   }
   if (ep.dot_out) {
-    __shared__ double sh[64];
-    if (ep.zq_q) {
-      finish_reduction_g(zq, rz, ep.dot_ws, ep.dot_out, sh, blockIdx.z,
-                         blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
-      return;
+    // the tile's shared memory is free again: it holds the block sums
+    static_assert(sizeof(sp) >= 2 * TX * TY * sizeof(double), "room for the block sums");
+    if (!ep.zq_q) {
+      zq = (double)dre;
+      rz = (double)dim;
     }
-    finish_reduction_g((double)dre, (double)dim, ep.dot_ws, ep.dot_out, sh, blockIdx.z,
-                       blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
+    __syncthreads();
+    finish_reduction_g<2>(zq, rz, ep.dot_ws, ep.dot_out, (double*)sp, blockIdx.z,
+                          blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   }
 }
 
@@ -372,12 +373,14 @@ enum { WV_STREAM = 0, WV_16x8, WV_32x8, WV_32x8x2, WV_16x16, WV_64x4, WV_64x4x2,
 static const int WV_SHAPE[WV_COUNT][3] = {{0, 0, 0}, {16, 8, 1}, {32, 8, 1}, {32, 8, 2},
                                           {16, 16, 1}, {64, 4, 1}, {64, 4, 2}};
 
-// The default shape (the choice made before any tuning).
+// The default shape (the choice made before any tuning).  A fused dot keeps its tile
+// whatever the tuner finds, so batches of it count all their tiles.
 template <typename R>
-static int wilson_default_variant(int Lx, int Lt, bool dot) {
+static int wilson_default_variant(int Lx, int Lt, int nrhs, bool dot) {
   const bool f64 = sizeof(R) == 8;
   if (!dot && wilson_A_streamed(Lx, Lt)) return WV_STREAM;
-  const bool big = ((Lx + 31) / 32) * ((Lt + (f64 ? 7 : 15)) / (f64 ? 8 : 16)) >= 2 * 152;
+  const long long tiles = (long long)((Lx + 31) / 32) * ((Lt + (f64 ? 7 : 15)) / (f64 ? 8 : 16));
+  const bool big = tiles * (dot ? nrhs : 1) >= 2 * 152;
   if (!big) return WV_16x8;
   return f64 ? WV_32x8 : WV_32x8x2;
 }
@@ -475,7 +478,7 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
     std::lock_guard<std::mutex> g(g_tune_mu);
     if (g_tune.count(key)) return cudaSuccess;
   }
-  const int def = W ? wilson_fx_variant(Lx, Lt, nrhs, false) : wilson_default_variant<R>(Lx, Lt, false);
+  const int def = W ? wilson_fx_variant(Lx, Lt, nrhs, false) : wilson_default_variant<R>(Lx, Lt, nrhs, false);
   const long long words = (long long)Lx * Lt * nrhs * 2 * sizeof(cplx_t<R>) / 8;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -555,7 +558,7 @@ cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, do
   if (dot && (nrhs > 64 || !wilson_A_dot_fits(Lx, Lt, sizeof(R) == 8, W ? diag : 0.0)))
     return cudaErrorInvalidValue;
   int v = dot ? -1 : tuned_variant<R>(Lx, Lt, nrhs, W != nullptr);
-  if (v < 0) v = W ? wilson_fx_variant(Lx, Lt, nrhs, dot) : wilson_default_variant<R>(Lx, Lt, dot);
+  if (v < 0) v = W ? wilson_fx_variant(Lx, Lt, nrhs, dot) : wilson_default_variant<R>(Lx, Lt, nrhs, dot);
   const cudaError_t e = launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, ep, s);
   count_launch();
   return e;

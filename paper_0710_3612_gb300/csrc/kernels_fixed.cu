@@ -191,12 +191,10 @@ __global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a) {
     fx_output<MODE>(a, y, gx, gt, off, dre, dim);
   }
   if (MODE >= FX_DOT_RE) {
-    __shared__ double sh[64];
-    const int blk = blockIdx.y * gridDim.x + blockIdx.x, G = gridDim.x * gridDim.y;
-    if (MODE == FX_DOT_RE)
-      finish_reduction_re(dre, a.ep.dot_ws, a.ep.dot_out, sh, blockIdx.z, blk, G);
-    else
-      finish_reduction_g(dre, dim, a.ep.dot_ws, a.ep.dot_out, sh, blockIdx.z, blk, G);
+    constexpr int N = MODE == FX_DOT ? 2 : 1;
+    __shared__ double sh[N * TX * TY];
+    finish_reduction_g<N>(dre, dim, a.ep.dot_ws, a.ep.dot_out, sh, blockIdx.z,
+                          blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   }
 }
 
