@@ -193,6 +193,15 @@ cudaError_t link_unitarity(const void* gauge, long long count, double* out, cuda
 enum CoarseWeights { W_F64 = 0, W_F32 = 1, W_BF16 = 2 };
 cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, int Lx, int Lt,
                          int n, int nrhs, const Epilogue& ep, cudaStream_t s);
+// The FP64 apply by integer arithmetic (fixed.cuh) from the blocks' words;
+// coarse_words_bytes: their size, 0 where the apply takes coarse_apply instead (n > 32).
+long long coarse_words_bytes(long long sites, int n);
+cudaError_t coarse_apply_fx(const void* in, void* out, const void* A64, const void* words, int Lx, int Lt,
+                            int n, int nrhs, const Epilogue& ep, cudaStream_t s);
+// The FP32 and BF16 copies and the words (may be null) of the blocks A64; with G0, first
+// A64 = G0 + m G1 + m^2 I.
+cudaError_t coarse_finish(const void* G0, const void* G1, double m, void* A64, void* A32, void* A16,
+                          void* words, long long sites, int n, cudaStream_t s);
 // Multi-RHS BF16 coarse apply on tcgen05 tensor cores (TMEM accumulator):
 // n in {16, 24}, 1 <= nrhs <= 64, FP32 vectors [nrhs][V][n], bf16x2 blocks.
 bool coarse_apply_tcgen05_ok(int n, int nrhs);
@@ -204,12 +213,9 @@ cudaError_t coarse_tc_take_error(int* flag);
 // Tensor-core kernel of coarse_apply for BF16 blocks and >= 8 right-hand
 // sides: 0 = tcgen05 where the shape allows it (default), 1 = mma.sync.
 void set_coarse_tensor_kernel(int kind);
-// A (complex128) -> float2 or bf16x2 copy
 // out = a X + b Y + c I for coarse operators of `sites` sites and n dof (FP64).
 cudaError_t coarse_lincomb(double a, const void* X, double b, const void* Y, double c, void* out,
                            long long sites, int n, cudaStream_t s);
-cudaError_t coarse_convert(const void* A64, void* out, int weights, long long count,
-                           cudaStream_t s);
 
 // ---- column probing (smoothed Galerkin products) ---------------------------
 // Probe vectors: out[s][j][r] = 1 if r == s and site j has colour (cx, ct) =

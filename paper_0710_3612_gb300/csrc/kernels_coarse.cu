@@ -293,24 +293,6 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
   return cudaGetLastError();
 }
 
-__global__ void k_coarse_convert(const double2* __restrict__ a, void* out, int weights,
-                                 long long count) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  double2 v = a[i];
-  if (weights == W_F32)
-    ((float2*)out)[i] = make_float2((float)v.x, (float)v.y);
-  else
-    ((__nv_bfloat162*)out)[i] = __floats2bfloat162_rn((float)v.x, (float)v.y);
-}
-
-cudaError_t coarse_convert(const void* A64, void* out, int weights, long long count,
-                           cudaStream_t s) {
-  k_coarse_convert<<<(unsigned)((count + 255) / 256), 256, 0, s>>>((const double2*)A64, out,
-                                                                   weights, count); count_launch();
-  return cudaGetLastError();
-}
-
 // out = a X + b Y + c I on 9-point block stencils [site][d][r][s] (I: the
 // identity blocks of the d = 4 displacement); out may alias X or Y.
 __global__ void k_coarse_lincomb(double a, const double2* X, double b, const double2* Y, double c,

@@ -30,6 +30,7 @@ struct Level {
   double2* A64 = nullptr;
   float2* A32 = nullptr;
   void* A16 = nullptr;
+  void* Afx = nullptr;                   // the FP64 blocks as integer words (coarse_finish)
   double2* G0 = nullptr;                 // A(m) = G0 + m G1 + m^2 I (remass_quadratic)
   double2* G1 = nullptr;
   // transfer to the next level
@@ -210,6 +211,10 @@ void apply_level(mg_handle* h, int l, const void* in, void* out, int nrhs, int w
     const void* U = sizeof(R) == 8 ? (const void*)h->U64 : (const void*)h->U32;
     ck(h, wilson_A<R>(in, out, U, h->Wfx, diag, L.Lx, L.Lt, nrhs, ep, h->s), "wilson_A");
   } else {
+    if (weights == W_F64 && L.Afx) {
+      ck(h, coarse_apply_fx(in, out, L.A64, L.Afx, L.Lx, L.Lt, L.n, nrhs, ep, h->s), "coarse_apply");
+      return;
+    }
     const void* A = weights == W_F64 ? (const void*)L.A64
                     : weights == W_F32 ? (const void*)L.A32 : L.A16;
     ck(h, coarse_apply(in, out, A, weights, L.Lx, L.Lt, L.n, nrhs, ep, h->s), "coarse_apply");
@@ -403,6 +408,12 @@ void build_quadratic(mg_handle* h) {
 
 void galerkin_next(mg_handle* h, int l);
 
+// The copies and words of level l's FP64 blocks.
+void finish_level(mg_handle* h, int l) {
+  Level& C = h->lv[l];
+  ck(h, coarse_finish(nullptr, nullptr, 0.0, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "level copies");
+}
+
 void build_coarse_ops(mg_handle* h) {
   if (h->p.remass_quadratic) {
     if (!h->g_built) build_quadratic(h);
@@ -410,21 +421,13 @@ void build_coarse_ops(mg_handle* h) {
     for (int l = 1; l < h->L; ++l) {
       Level& C = h->lv[l];
       ProfScope prof(h, MG_KF_GALERKIN);
-      ck(h, coarse_lincomb(1.0, C.G0, m, C.G1, m * m, C.A64, C.V, C.n, h->s), "A(m)");
-      const long long cnt = (long long)C.V * 9 * C.n * C.n;
-      ck(h, coarse_convert(C.A64, C.A32, W_F32, cnt, h->s), "convert f32");
-      ck(h, coarse_convert(C.A64, C.A16, W_BF16, cnt, h->s), "convert bf16");
+      ck(h, coarse_finish(C.G0, C.G1, m, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "A(m)");
     }
     return;
   }
   for (int l = 0; l + 1 < h->L; ++l) {
-    Level& L = h->lv[l];
-    Level& C = h->lv[l + 1];
     ProfScope prof(h, MG_KF_GALERKIN);
     galerkin_next(h, l);
-    const long long cnt = (long long)C.V * 9 * C.n * C.n;
-    ck(h, coarse_convert(C.A64, C.A32, W_F32, cnt, h->s), "convert f32");
-    ck(h, coarse_convert(C.A64, C.A16, W_BF16, cnt, h->s), "convert bf16");
   }
 }
 
@@ -1242,6 +1245,8 @@ void allocate_storage(mg_handle* h) {
       L.A64 = dalloc<double2>(h, ab * sizeof(double2));
       L.A32 = dalloc<float2>(h, ab * sizeof(float2));
       L.A16 = dalloc(h, ab * 4);
+      const long long wb = coarse_words_bytes(L.V, L.n);
+      if (wb) L.Afx = dalloc(h, (size_t)wb);
       if (h->p.remass_quadratic) {
         L.G0 = dalloc<double2>(h, ab * sizeof(double2));
         L.G1 = dalloc<double2>(h, ab * sizeof(double2));
@@ -1365,6 +1370,7 @@ void smoothed_combination(mg_handle* h, double2* const G[3], double omega) {
   Level& C = h->lv[1];
   ck(h, coarse_lincomb(1.0, G[0], -2.0 * omega, G[1], 0.0, C.A64, C.V, C.n, h->s), "A_c(omega)");
   ck(h, coarse_lincomb(1.0, C.A64, omega * omega, G[2], 0.0, C.A64, C.V, C.n, h->s), "A_c(omega)");
+  finish_level(h, 1);
 }
 
 // Largest eigenvalue of a Hermitian positive operator on n entries by
@@ -1482,7 +1488,7 @@ void galerkin_smoothed(mg_handle* h) {
   h->bytes -= 3LL * (long long)ab;
 }
 
-// Galerkin operator of level l + 1 from the vectors of level l (FP64 master only).
+// Galerkin operator of level l + 1 from the vectors of level l, with its copies.
 void galerkin_next(mg_handle* h, int l) {
   Level& L = h->lv[l];
   Level& C = h->lv[l + 1];
@@ -1492,6 +1498,7 @@ void galerkin_next(mg_handle* h, int l) {
     ck(h, galerkin_fine(h->U64, 4.0 + h->mass, L.Vst64, h->Wbuf, C.A64, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin_fine");
   else
     ck(h, galerkin_coarse(L.A64, L.Vst64, C.A64, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin_coarse");
+  finish_level(h, l + 1);
 }
 
 // One level of the adaptive setup (Sec. 3): with E = NULL, Nv random starts
