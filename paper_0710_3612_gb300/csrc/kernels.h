@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "fixed.cuh"
 
 namespace mgk {
@@ -255,17 +257,34 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
 // the stencil (complex128); rows/columns N..ld-1 are set to the identity.
 cudaError_t coarse_to_dense_f32(const void* A, void* dense, int Lx, int Lt, int n, long long ld,
                                 cudaStream_t s);
-// In-place blocked Gauss-Jordan inversion of a Hermitian positive definite
-// complex64 N x N matrix (N multiple of 64), lower triangle kept (the upper
-// halves of diagonal 64 x 64 tiles are rebuilt by pack_hermitian).
-// work: 3 * N * 64 + 2 * 64 * 64 complex64.  Launch sequence: begin (inverts
-// the first pivot block), then for k = 0 .. N/64 - 1: panel(k), update(k).
+// In-place Gauss-Jordan inversion of a Hermitian positive definite complex64 ld x ld
+// matrix (ld a multiple of 64) holding a 9-point stencil of Lx x Lt sites with n dof,
+// lower triangle of 64 x 64 tiles kept (the upper halves of diagonal tiles are rebuilt
+// by pack_hermitian).  inverse_plan: order and grouping of the pivot blocks (host only);
+// data: its int array on the device; work: inverse_work_entries(ld) complex64.  Launch
+// sequence: inverse_first, then for each group its panels (update = false) and tiles.
+struct InversePlan {
+  struct Group {
+    int npiv, nnext, nact, npanels;              // counts
+    int panels, piv, next, act, mask, slot;      // offsets into data
+  };
+  std::vector<Group> groups;
+  std::vector<int> data;
+  int first = 0;                                 // offset of the first group's pivots
+};
+InversePlan inverse_plan(int Lx, int Lt, int n, int ld);
+size_t inverse_work_entries(int ld);
+cudaError_t inverse_first(void* M, int ld, const InversePlan& plan, const int* data, void* work,
+                          cudaStream_t s);
+cudaError_t inverse_group(void* M, int ld, const InversePlan& plan, const int* data, int group,
+                          void* work, bool update, cudaStream_t s);
+// The same inversion, every pivot in order and every tile (mg_params.coarsest_gj_tcgen05):
+// the updates on tcgen05 tensor cores (TMEM accumulator).  N a multiple of 64; work: 3 * N *
+// 64 + 2 * 64 * 64 complex64, then an int error flag (16 bytes), zero before the first call,
+// set if a completion wait runs out (the inverse is then invalid).  Launch sequence: begin
+// (inverts the first pivot block), then for k = 0 .. N/64 - 1: panel(k), update_tc(k).
 cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s);
 cudaError_t gauss_jordan_panel(void* M, int N, int k, void* work, cudaStream_t s);
-cudaError_t gauss_jordan_update(void* M, int N, int k, void* work, cudaStream_t s);
-// The same update on tcgen05 tensor cores (TMEM accumulator); needs 16 more
-// bytes of work: an int error flag after the row panel, zero before the first
-// call, set if a completion wait runs out (the inverse is then invalid).
 cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream_t s);
 // y = B x, or y += B x when accumulate (complex64 B, leading dimension ld);
 // x complex128 (N) -> y complex128 (N); FP32 products and accumulation, result

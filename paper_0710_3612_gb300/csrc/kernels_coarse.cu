@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "mma_tf32.cuh"
 
 namespace mgk {
 
@@ -1065,161 +1066,8 @@ __global__ void __launch_bounds__(256) k_gj_panel(const float2* __restrict__ M, 
   }
 }
 
-// Lower tiles (I, J) for pivot block k: M_IJ -= Cold_I R_J for I, J != k, and
-// the sweep's write-back: M_kJ = R_J (J < k), M_Ik = -Cn_I (I > k), M_kk = P.
-// CTA 0 takes tile (k+1, k+1) and, after updating it, inverts it into Pnext
-// (the next pivot block), overlapping that sweep with the other tiles.
-//
-// The complex product runs on the tensor cores as a real GEMM: with complex
-// entries interleaved (re, im), Out (64 x 128) = C (64 x 128) B (128 x 128),
-// where B realifies R: B[2k][2j] = Re R_kj, B[2k][2j+1] = Im R_kj,
-// B[2k+1][2j] = -Im R_kj, B[2k+1][2j+1] = Re R_kj.  mma.sync m16n8k8 TF32 with
-// each operand split x = hi + lo (hi = tf32(x), lo = tf32(x - hi)) and three
-// products hi hi + hi lo + lo hi, FP32 accumulation: about FP32 accuracy.
-// 8 warps in a 2 x 4 grid, 32 x 32 real outputs each; lane (g, t) = (lane/4,
-// lane%4) holds complex outputs (row g or g + 8, column t) of each 16 x 4
-// complex sub-tile, so the epilogue works on whole complex numbers.
-static constexpr int GJC = 66;                   // sC row stride (float2), conflict-free A loads
-static constexpr int GJR = 68;                   // sR row stride (float2), conflict-free B loads
-
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-  asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(hi) : "f"(x));
-  const float r = x - __uint_as_float(hi);
-  asm("cvt.rna.tf32.f32 %0, %1;\n" : "=r"(lo) : "f"(r));
-}
-
-__device__ __forceinline__ void mma_tf32(float* d, const uint32_t* a, const uint32_t* b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__global__ void __launch_bounds__(256) k_gj_update(float2* __restrict__ M, int N, int k,
-                                                   const float2* __restrict__ P,
-                                                   float2* __restrict__ Pnext,
-                                                   const float2* __restrict__ Cold,
-                                                   const float2* __restrict__ Cn,
-                                                   const float2* __restrict__ Rp) {
-  extern __shared__ float2 gsm[];
-  const int nt = N / GJB;
-  // tile index: CTA 0 -> (k+1, k+1) if it exists; the rest in order, skipping it
-  const long long kp = (k + 1 < nt) ? (long long)(k + 1) * (k + 2) / 2 + (k + 1) : -1;
-  long long t = blockIdx.x;
-  if (kp >= 0) t = (t == 0) ? kp : (t <= kp ? t - 1 : t);
-  int I = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while ((long long)(I + 1) * (I + 2) / 2 <= t) ++I;
-  while ((long long)I * (I + 1) / 2 > t) --I;
-  const int J = (int)(t - (long long)I * (I + 1) / 2);
-  const int tid = threadIdx.x;
-  float2* tile = M + (long long)I * GJB * N + J * GJB;
-  if (I == k || J == k) {                              // pivot row / column / block
-    for (int q = tid; q < GJB * GJB; q += 256) {
-      const int r = q / GJB, c = q % GJB;
-      float2 v;
-      if (I == k && J == k) {
-        v = P[q];
-      } else if (I == k) {
-        v = Rp[(long long)r * N + J * GJB + c];
-      } else {
-        const float2 w = Cn[(long long)(I * GJB + r) * GJB + c];
-        v = make_float2(-w.x, -w.y);
-      }
-      tile[(long long)r * N + c] = v;
-    }
-    return;
-  }
-  float2* sC = gsm;                                    // Cold_I [64][GJC]
-  float2* sR = gsm + GJB * GJC;                        // R_J    [64][GJR]
-  {                                                    // two complex per 16-byte load,
-    float4 vc[8], vr[8];                               // all 16 loads in flight first
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = tid + 256 * u, r = q / (GJB / 2), c = 2 * (q % (GJB / 2));
-      vc[u] = *(const float4*)&Cold[(long long)(I * GJB + r) * GJB + c];
-      vr[u] = *(const float4*)&Rp[(long long)r * N + J * GJB + c];
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int q = tid + 256 * u, r = q / (GJB / 2), c = 2 * (q % (GJB / 2));
-      *(float4*)&sC[r * GJC + c] = vc[u];
-      *(float4*)&sR[r * GJR + c] = vr[u];
-    }
-  }
-  __syncthreads();
-  const int warp = tid >> 5, lane = tid & 31, g = lane >> 2, tq = lane & 3;
-  const int wm = warp >> 2, wn = warp & 3;             // rows 32 wm.., complex cols 16 wn..
-  const float* sCf = (const float*)sC;
-  float acc[2][4][4];
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[mt][n][e] = 0.f;
-#pragma unroll 2
-  for (int kk = 0; kk < 2 * GJB / 8; ++kk) {           // 16 real k-steps of 8
-    uint32_t ah[2][4], al[2][4], bh[4][2], bl[4][2];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      const int row = 32 * wm + 16 * mt + g;
-      const float* r0 = sCf + row * 2 * GJC + 8 * kk;
-      const float* r8 = r0 + 8 * 2 * GJC;
-      split_tf32(r0[tq], ah[mt][0], al[mt][0]);
-      split_tf32(r8[tq], ah[mt][1], al[mt][1]);
-      split_tf32(r0[tq + 4], ah[mt][2], al[mt][2]);
-      split_tf32(r8[tq + 4], ah[mt][3], al[mt][3]);
-    }
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      // B[8kk + tq][8n' + g] and B[8kk + tq + 4][8n' + g], n' = 4 wn + n
-      const int j = 16 * wn + 4 * n + (g >> 1), d = g & 1;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int kr = 8 * kk + tq + 4 * h;            // real row of B
-        const float2 v = sR[(kr >> 1) * GJR + j];
-        const float x = (kr & 1) ? (d ? v.x : -v.y) : (d ? v.y : v.x);
-        split_tf32(x, bh[n][h], bl[n][h]);
-      }
-    }
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        mma_tf32(acc[mt][n], al[mt], bh[n]);
-        mma_tf32(acc[mt][n], ah[mt], bl[n]);
-        mma_tf32(acc[mt][n], ah[mt], bh[n]);
-      }
-  }
-  const bool next_pivot = (long long)t == kp;
-  if (next_pivot) __syncthreads();                     // sC is reused for the new tile
-  float2 old[2][4][2];                                 // all tile loads before the stores
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        old[mt][n][h] = tile[(long long)(32 * wm + 16 * mt + g + 8 * h) * N + 16 * wn + 4 * n + tq];
-#pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = 32 * wm + 16 * mt + g + 8 * h, c = 16 * wn + 4 * n + tq;
-        const float2 o = old[mt][n][h];
-        const float2 nv = make_float2(o.x - acc[mt][n][2 * h], o.y - acc[mt][n][2 * h + 1]);
-        tile[(long long)r * N + c] = nv;
-        if (next_pivot) sC[r * GJS + c] = nv;
-      }
-  if (next_pivot) {
-    __syncthreads();
-    sweep_block64(sC, sR);
-    for (int q = tid; q < GJB * GJB; q += 256) Pnext[q] = sC[(q / GJB) * GJS + q % GJB];
-  }
-}
+static constexpr int GJC = 66;                   // tile row stride (float2), conflict-free A loads
+static constexpr int GJR = 68;                   // vector row stride (float2), conflict-free B loads
 
 // ---- tcgen05 variant of the update ---------------------------------------
 // The same update, M_IJ -= Cold_I R_J, on the 5th-generation tensor cores:
@@ -1502,8 +1350,6 @@ cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s) {
   if (!attr) {
     cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)(2 * GJB * GJS * sizeof(float2)));
-    cudaFuncSetAttribute(k_gj_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(GJB * (GJC + GJR) * sizeof(float2)));
     attr = true;
   }
   k_gj_pivot0<<<1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s>>>((const float2*)M, N, Pb[0]);
@@ -1544,18 +1390,6 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
   return cudaGetLastError();
 }
 
-cudaError_t gauss_jordan_update(void* M, int N, int k, void* work, cudaStream_t s) {
-  float2 *Pb[2], *Cold, *Cn, *Rp;
-  gj_work_split(work, N, Pb, &Cold, &Cn, &Rp);
-  const int nb = N / GJB;
-  k_gj_update<<<nb * (nb + 1) / 2, 256, GJB * (GJC + GJR) * sizeof(float2), s>>>(
-      (float2*)M, N, k, Pb[k & 1], Pb[(k + 1) & 1], Cold, Cn, Rp);
-  count_launch();
-  return cudaGetLastError();
-}
-
-// y = B x: one warp per row, FP32 products and accumulation, result widened.
-// B has leading dimension ld (even, >= N); xtmp holds ld complex64, zero beyond N.
 __global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ xf, int N, int ld) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < ld) xf[i] = i < N ? make_float2((float)x[i].x, (float)x[i].y) : make_float2(0.f, 0.f);

@@ -59,6 +59,8 @@ struct mg_handle {
   int Nc = 0, ldc = 0;
   float2* Binv = nullptr;
   float2* gj_work = nullptr;
+  InversePlan inv_plan;         // order of the inversion's pivots, and its device copy
+  int* inv_data = nullptr;
   float2* gemv_x = nullptr;
   float2* Bpk = nullptr;        // packed Hermitian tiles of the inverse
   float2* gemv_part = nullptr;  // partial products of the packed GEMV
@@ -563,17 +565,15 @@ void build_coarsest(mg_handle* h, bool remass = false) {
   ck(h, coarse_to_dense_f32(L.A64, h->Binv, L.Lx, L.Lt, L.n, h->ldc, h->s), "dense");
   {
     ProfScope prof(h, MG_KF_INVERSE);
-    const bool tc = h->p.coarsest_gj_tcgen05 != 0;
-    int* gj_err = (int*)(h->gj_work + (size_t)3 * h->ldc * 64 + 2 * 64 * 64);
-    if (tc) ck(h, cudaMemsetAsync(gj_err, 0, sizeof(int), h->s), "memset");
-    ck(h, gauss_jordan_begin(h->Binv, h->ldc, h->gj_work, h->s), "gauss-jordan");
-    for (int k = 0; k < h->ldc / 64; ++k) {
-      ck(h, gauss_jordan_panel(h->Binv, h->ldc, k, h->gj_work, h->s), "gauss-jordan panel");
-      ProfScope pu(h, MG_KF_GJ_UPDATE);
-      ck(h, tc ? gauss_jordan_update_tc(h->Binv, h->ldc, k, h->gj_work, h->s)
-               : gauss_jordan_update(h->Binv, h->ldc, k, h->gj_work, h->s), "gauss-jordan update");
-    }
-    if (tc) {
+    if (h->p.coarsest_gj_tcgen05) {
+      int* gj_err = (int*)(h->gj_work + (size_t)3 * h->ldc * 64 + 2 * 64 * 64);
+      ck(h, cudaMemsetAsync(gj_err, 0, sizeof(int), h->s), "memset");
+      ck(h, gauss_jordan_begin(h->Binv, h->ldc, h->gj_work, h->s), "gauss-jordan");
+      for (int k = 0; k < h->ldc / 64; ++k) {
+        ck(h, gauss_jordan_panel(h->Binv, h->ldc, k, h->gj_work, h->s), "gauss-jordan panel");
+        ProfScope pu(h, MG_KF_GJ_UPDATE);
+        ck(h, gauss_jordan_update_tc(h->Binv, h->ldc, k, h->gj_work, h->s), "gauss-jordan update");
+      }
       int e = 0;
       ck(h, cudaMemcpyAsync(&e, gj_err, sizeof(int), cudaMemcpyDeviceToHost, h->s), "read");
       sync(h);
@@ -582,6 +582,14 @@ void build_coarsest(mg_handle* h, bool remass = false) {
         // later result of this handle can be trusted
         h->poisoned = true;
         fail(h, MG_ERR_TIMEOUT, "tensor-core Gauss-Jordan update: completion wait ran out");
+      }
+    } else {
+      const InversePlan& pl = h->inv_plan;
+      ck(h, inverse_first(h->Binv, h->ldc, pl, h->inv_data, h->gj_work, h->s), "inverse");
+      for (int q = 0; q < (int)pl.groups.size(); ++q) {
+        ck(h, inverse_group(h->Binv, h->ldc, pl, h->inv_data, q, h->gj_work, false, h->s), "inverse panels");
+        ProfScope pu(h, MG_KF_GJ_UPDATE);
+        ck(h, inverse_group(h->Binv, h->ldc, pl, h->inv_data, q, h->gj_work, true, h->s), "inverse update");
       }
     }
     ck(h, pack_hermitian(h->Binv, h->Bpk, h->ldc, h->s), "pack");
@@ -1275,7 +1283,14 @@ void allocate_storage(mg_handle* h) {
     h->dense = h->Nc <= P.coarsest_dense_max;
     if (h->dense) {
       h->Binv = dalloc<float2>(h, (size_t)h->ldc * h->ldc * sizeof(float2));
-      h->gj_work = dalloc<float2>(h, ((size_t)3 * h->ldc * 64 + 2 * 64 * 64 + 2) * sizeof(float2));
+      const size_t tcw = (size_t)3 * h->ldc * 64 + 2 * 64 * 64 + 2;
+      h->gj_work = dalloc<float2>(h, std::max(inverse_work_entries(h->ldc), tcw) * sizeof(float2));
+      h->inv_plan = inverse_plan(C.Lx, C.Lt, C.n, h->ldc);
+      const size_t pb = h->inv_plan.data.size() * sizeof(int);
+      h->inv_data = dalloc<int>(h, pb);
+      if (!h->dry)                             // the plan lives in the handle: a plain copy
+        ck(h, cudaMemcpyAsync(h->inv_data, h->inv_plan.data.data(), pb, cudaMemcpyHostToDevice, h->s),
+           "upload plan");
       h->gemv_x = dalloc<float2>(h, (size_t)h->ldc * h->R * sizeof(float2));
       const size_t nt = h->ldc / 64, ntiles = nt * (nt + 1) / 2;
       h->Bpk = dalloc<float2>(h, ntiles * 64 * 64 * sizeof(float2));
