@@ -17,7 +17,7 @@
 // blocks without a common coupling in one pair of launches.  At 16 x 16 sites of 16
 // dof (64 blocks) 25,840 tile products in 28 groups are left of 129,024 in 64 steps,
 // at 32 x 32 sites a tenth.  Skipped products are with zero blocks: the arithmetic on
-// the rest is unchanged.  4096 unknowns: 8.0 -> 2.1 ms (the update of every tile in order
+// the rest is unchanged.  4096 unknowns: 8.0 -> 1.85 ms (the update of every tile in order
 // took 64 x 101 us, its panels 64 x 24 us).
 #include <algorithm>
 #include <numeric>
@@ -39,51 +39,39 @@ static constexpr int TILE = B * B;
 static constexpr int GMAX = 8;                   // pivots per group
 
 // In-place inversion of the Hermitian positive definite 64 x 64 block a[][LA] in shared
-// memory by 256 threads: four 16 x 16 sub-pivots K.  One warp sweeps the sub-pivot in
-// registers (lane (half, c) holds rows 8 half .. 8 half + 7 of column c), then all threads
-// form the row panel T = P a_Kx and the rank-16 update of the other 48 x 48 entries, 3 x 3
-// per thread; the column panel follows from T by the sign rule.  tmp: [16][48] complex.
-// 36 us (a barrier-per-element sweep of the sub-pivots: 42 us), the length of a small group.
+// memory by 256 threads: four 16 x 16 sub-pivots K, each swept with one entry per thread (in
+// a register; the rows and columns others need go through two alternating buffers, one barrier
+// a step), then the row panel T = P a_Kx and the rank-16 update of the other 48 x 48 entries,
+// 3 x 3 per thread; the column panel follows from T by the sign rule.  The diagonal of a
+// Hermitian block is real, so a pivot is inverted by one division.  tmp: [16][48] complex.
+// With its launch 28 us (36 with the sub-pivot in one warp's registers: 16 unrolled steps of
+// cold instructions; 42 with two barriers and a complex division a step).
 __device__ void invert64(float2* a, float2* tmp) {
   const int tid = threadIdx.x, ti = tid >> 4, tj = tid & 15;
+#pragma unroll 1
   for (int K = 0; K < 4; ++K) {
     const int k0 = 16 * K;
-    if (tid < 32) {
-      const int c = tid & 15, half = tid >> 4;
-      float2 v[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) v[i] = a[(k0 + 8 * half + i) * LA + k0 + c];
-#pragma unroll
-      for (int p = 0; p < 16; ++p) {
-        const int ph = p >> 3, pi = p & 7;
-        const float2 piv = make_float2(__shfl_sync(0xffffffffu, v[pi].x, p + 16 * ph),
-                                       __shfl_sync(0xffffffffu, v[pi].y, p + 16 * ph));
-        const float2 rowp = make_float2(__shfl_sync(0xffffffffu, v[pi].x, c + 16 * ph),
-                                        __shfl_sync(0xffffffffu, v[pi].y, c + 16 * ph));
-        const float den = piv.x * piv.x + piv.y * piv.y;
-        const float2 inv = make_float2(piv.x / den, -piv.y / den);
-        const float2 f = cmul(inv, rowp);          // inv * a_pc
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float2 colp = make_float2(__shfl_sync(0xffffffffu, v[i].x, p + 16 * half),
-                                          __shfl_sync(0xffffffffu, v[i].y, p + 16 * half));
-          const bool rp = half == ph && i == pi;
-          float2 w;
-          if (c == p) {
-            const float2 z = cmul(colp, inv);
-            w = rp ? inv : make_float2(-z.x, -z.y);
-          } else {
-            w = rp ? f : csub(v[i], cmul(colp, f));
-          }
-          v[i] = w;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) a[(k0 + 8 * half + i) * LA + k0 + c] = v[i];
+    float2 v = a[(k0 + ti) * LA + k0 + tj];
+    tmp[ti * 17 + tj] = v;
+    __syncthreads();
+#pragma unroll 2
+    for (int p = 0; p < 16; ++p) {
+      const float2* s = tmp + (p & 1) * 16 * 17;
+      const float inv = 1.f / s[p * 17 + p].x;
+      const float2 rp = s[p * 17 + tj], cp = s[ti * 17 + p];
+      const float2 f = make_float2(inv * rp.x, inv * rp.y);
+      if (tj == p)
+        v = ti == p ? make_float2(inv, 0.f) : make_float2(-inv * cp.x, -inv * cp.y);
+      else
+        v = ti == p ? f : csub(v, cmul(cp, f));
+      tmp[((p + 1) & 1) * 16 * 17 + ti * 17 + tj] = v;
+      __syncthreads();
     }
+    a[(k0 + ti) * LA + k0 + tj] = v;
     __syncthreads();
     {                                              // T[q][x], q = ti, x = tj + 16 u
       float2 acc[3] = {};
+#pragma unroll 4
       for (int s = 0; s < 16; ++s) {
         const float2 p = a[(k0 + ti) * LA + k0 + s];
 #pragma unroll
@@ -104,6 +92,7 @@ __device__ void invert64(float2* a, float2* tmp) {
         const int xi = ti + 16 * u, xj = tj + 16 * w;
         nv[u][w] = a[(xi < k0 ? xi : xi + 16) * LA + (xj < k0 ? xj : xj + 16)];
       }
+#pragma unroll 2
     for (int s = 0; s < 16; ++s) {
       float2 cv[3], rv[3];
 #pragma unroll
@@ -159,68 +148,74 @@ __global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M,
   for (int q = threadIdx.x; q < TILE; q += 256) g.Pnext[blockIdx.x * TILE + q] = a[(q / B) * LA + q % B];
 }
 
-// Panels of a group, one CTA of 512 threads per (block, pivot): C_b = M_bk from the stored
-// lower tile, N_b = C_b P, and the swept tile written back in place (M_bk <- -N_b, or M_kb <-
-// s_b N_b^H when the stored tile is (k, b)); the pivot tile itself becomes P.
-__global__ void __launch_bounds__(512) k_gji_panel(float2* __restrict__ M, int ld, GroupArgs g) {
-  extern __shared__ float2 psm[];
-  float2* sP = psm;                              // [64][LD]
-  float2* sX = psm + B * LD;
+// Panels of a group: C_b = M_bk from the stored lower tile, N_b = C_b P, and the swept tile
+// written back in place (M_bk <- -N_b, or M_kb <- s_b N_b^H when the stored tile is (k, b));
+// the pivot tile itself becomes P.  Four CTAs per (block, pivot), 16 rows of C_b each: they
+// read and write only their own rows (or columns) of the stored tile.  A group has 20 to 72
+// panels, too few to fill the GPU with one CTA each (12 us; four 7 to 10 us).
+__global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int ld, GroupArgs g) {
+  __shared__ __align__(16) float2 sP[B * B];
+  __shared__ __align__(16) float2 sX[16 * (B + 1)];
   const int3 e = g.panels[blockIdx.x];
-  const int b = e.x, k = g.piv[e.y], tid = threadIdx.x;
+  const int b = e.x, k = g.piv[e.y], tid = threadIdx.x, r0 = 16 * blockIdx.y;
   const float2* P = g.P + e.y * TILE;
   if (b == k) {
-    for (int q = tid; q < TILE; q += 512) M[((long long)k * B + q / B) * ld + k * B + q % B] = P[q];
+    for (int q = tid; q < 16 * B; q += 256)
+      M[((long long)k * B + r0 + q / B) * ld + k * B + q % B] = P[r0 * B + q];
     return;
   }
   const bool lower = b > k;                      // the stored tile is (b, k)
   float2* tile = M + (long long)(lower ? b : k) * B * ld + (long long)(lower ? k : b) * B;
   const float sg = e.z ? -1.f : 1.f;
+  float4 p[8];
+  float2 v[4];
 #pragma unroll
-  for (int u = 0; u < TILE / 2 / 512; ++u) {     // two complex per load
-    const int q = 2 * (tid + 512 * u), r = q / B, c = q % B;
-    const float4 p = *(const float4*)(P + q), v = *(const float4*)(tile + (long long)r * ld + c);
-    *(float4*)&sP[r * LD + c] = p;
-    if (lower) {
-      *(float4*)&sX[r * LD + c] = v;
-    } else {                                     // M_bk = s_b M_kb^H
-      sX[c * LD + r] = make_float2(sg * v.x, -sg * v.y);
-      sX[(c + 1) * LD + r] = make_float2(sg * v.z, -sg * v.w);
-    }
+  for (int u = 0; u < 8; ++u) p[u] = ((const float4*)P)[tid + 256 * u];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {                  // lower: row r0 + q / 64; else column r0 + q % 16
+    const int q = tid + 256 * u;
+    v[u] = lower ? tile[(long long)(r0 + q / B) * ld + q % B] : tile[(long long)(q / 16) * ld + r0 + q % 16];
+  }
+#pragma unroll
+  for (int u = 0; u < 8; ++u) ((float4*)sP)[tid + 256 * u] = p[u];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int q = tid + 256 * u;
+    if (lower)
+      sX[(q / B) * (B + 1) + q % B] = v[u];
+    else                                         // M_bk = s_b M_kb^H
+      sX[(q % 16) * (B + 1) + q / 16] = make_float2(sg * v[u].x, -sg * v[u].y);
   }
   __syncthreads();
-  const int r0 = 2 * (tid >> 4), c0 = tid & 15;  // rows r0, r0 + 1; columns c0 + 16 u
-  float2 acc[2][4] = {};
-#pragma unroll 4
+  const int r = tid >> 4, c0 = tid & 15;         // row r0 + r, columns c0 + 16 u
+  float2 acc[4] = {};
+#pragma unroll 8
   for (int q = 0; q < B; ++q) {
-    const float2 x0 = sX[r0 * LD + q], x1 = sX[(r0 + 1) * LD + q];
+    const float2 x = sX[r * (B + 1) + q];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const float2 p = sP[q * LD + c0 + 16 * u];
-      cfma(acc[0][u], x0, p);
-      cfma(acc[1][u], x1, p);
-    }
+    for (int u = 0; u < 4; ++u) cfma(acc[u], x, sP[q * B + c0 + 16 * u]);
   }
-  float2* C = g.C + (long long)blockIdx.x * TILE;
-  float2* N = g.N + (long long)blockIdx.x * TILE;
+  float2* C = g.C + (long long)blockIdx.x * TILE + (r0 + r) * B;
+  float2* N = g.N + (long long)blockIdx.x * TILE + (r0 + r) * B;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int r = r0 + i, c = c0 + 16 * u;
-      const float2 w = acc[i][u];
-      C[r * B + c] = sX[r * LD + c];
-      N[r * B + c] = w;
-      if (lower) tile[(long long)r * ld + c] = make_float2(-w.x, -w.y);
-    }
+  for (int u = 0; u < 4; ++u) {
+    const int c = c0 + 16 * u;
+    const float2 w = acc[u];
+    C[c] = sX[r * (B + 1) + c];
+    N[c] = w;
+    if (lower) tile[(long long)(r0 + r) * ld + c] = make_float2(-w.x, -w.y);
+  }
   if (!lower) {                                  // s_b N_b^H, transposed through shared memory
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) sX[(c0 + 16 * u) * LD + r0 + i] = make_float2(sg * acc[i][u].x, -sg * acc[i][u].y);
+    for (int u = 0; u < 4; ++u)
+      sX[r * (B + 1) + c0 + 16 * u] = make_float2(sg * acc[u].x, -sg * acc[u].y);
     __syncthreads();
-    for (int q = tid; q < TILE; q += 512) tile[(long long)(q / B) * ld + q % B] = sX[(q / B) * LD + q % B];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = tid + 256 * u;
+      tile[(long long)(q / 16) * ld + r0 + q % 16] = sX[(q % 16) * (B + 1) + q / 16];
+    }
   }
 }
 
@@ -450,10 +445,8 @@ size_t inverse_work_entries(int ld) { return (size_t)2 * ld * B + (size_t)2 * GM
 cudaError_t inverse_first(void* M, int ld, const InversePlan& plan, const int* data, void* work,
                           cudaStream_t s) {
   static const cudaError_t e0 = cudaFuncSetAttribute(
-      k_gji_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * B * LD * sizeof(float2)));
-  static const cudaError_t e1 = cudaFuncSetAttribute(
       k_gji_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * B * LD * sizeof(float2)));
-  if (e0 != cudaSuccess || e1 != cudaSuccess) return e0 != cudaSuccess ? e0 : e1;
+  if (e0 != cudaSuccess) return e0;
   GroupArgs g{};
   g.next = data + plan.first;
   g.Pnext = (float2*)work + (size_t)2 * ld * B;
@@ -472,7 +465,7 @@ cudaError_t inverse_group(void* M, int ld, const InversePlan& plan, const int* d
               (float2*)work, (float2*)work + (size_t)ld * B};
   const size_t smem = 2 * B * LD * sizeof(float2);
   if (!update) {
-    k_gji_panel<<<G.npanels, 512, smem, s>>>((float2*)M, ld, g);
+    k_gji_panel<<<dim3(G.npanels, B / 16), 256, 0, s>>>((float2*)M, ld, g);
   } else {
     const int grid = G.nnext + G.nact * (G.nact + 1) / 2;
     if (grid == 0) return cudaSuccess;

@@ -505,8 +505,11 @@ void build_coarsest_cg(mg_handle* h) {
 // Refinement with the FP32 inverse in hand on the current coarsest operator,
 // one step at a time: x = B b, then x += B (b - A x) until every test vector
 // reaches coarsest_tol within kmax steps.  On success *steps and *inner are the
-// largest step counts that reached coarsest_tol and 1e-6.
-bool refinement_test(mg_handle* h, int kmax, int* steps, int* inner, double* worst_rel) {
+// largest step counts that reached coarsest_tol and 1e-6; *worst_rel is the largest
+// residual reached (on a miss, the one of the vector that missed).
+enum RefineTest { REFINE_OK, REFINE_MISSED, REFINE_NONFINITE };
+
+RefineTest refinement_test(mg_handle* h, int kmax, int* steps, int* inner, double* worst_rel) {
   *steps = 0;
   *inner = 0;
   *worst_rel = 0.0;
@@ -525,11 +528,14 @@ bool refinement_test(mg_handle* h, int kmax, int* steps, int* inner, double* wor
       apply_level<double>(h, h->L - 1, h->cx, h->cr, 1, W_F64, ep_lincomb(-1.0, h->cb, 1.0));
       ck(h, norm2<double>(h->cr, h->Nc, 1, h->partials, slot(h, S_T0), h->s), "norm");
       const double rr = read_scalar(h, S_T0);
-      if (!(rr == rr)) return false;
+      if (!(rr == rr)) return REFINE_NONFINITE;
       rel = std::sqrt(rr / bn);
       if (s6 < 0 && rel <= 1e-6) s6 = s;
       if (rel <= h->p.coarsest_tol) break;
-      if (s == kmax) return false;
+      if (s == kmax) {
+        *worst_rel = rel;
+        return REFINE_MISSED;
+      }
       ck(h, hermitian_gemv_tiles(h->Bpk, h->cr, h->Nc, h->ldc, 1, h->gemv_part, h->s), "gemv");
       ck(h, hermitian_gemv_reduce(h->gemv_part, h->cx, h->Nc, h->ldc, 1, true, h->s), "gemv");
     }
@@ -537,7 +543,7 @@ bool refinement_test(mg_handle* h, int kmax, int* steps, int* inner, double* wor
     *inner = std::max(*inner, s6);
     *worst_rel = std::max(*worst_rel, rel);
   }
-  return true;
+  return REFINE_OK;
 }
 
 // remass: called for a new mass of an existing hierarchy (mg_set_mass).
@@ -551,7 +557,7 @@ void build_coarsest(mg_handle* h, bool remass = false) {
     int steps = 0, inner = 0;
     double rel = 0.0;
     const int kmax = std::min(h->p.coarsest_reuse, h->p.coarsest_refine_max - 1);
-    if (refinement_test(h, kmax, &steps, &inner, &rel)) {
+    if (refinement_test(h, kmax, &steps, &inner, &rel) == REFINE_OK) {
       h->coarsest_test_res = rel;
       h->n_refine = std::min(steps + 1, h->p.coarsest_refine_max);
       h->n_inner = std::max(h->p.inner_coarsest_refine, inner);
@@ -599,36 +605,18 @@ void build_coarsest(mg_handle* h, bool remass = false) {
   // If a test vector does not get there within coarsest_refine_max steps the
   // FP32 inverse is too inaccurate for this operator (condition number near
   // 1/eps_FP32): MG_ERR_NOCONV, with the residual reached in the message.
-  int worst = 0;
-  for (int tv = 0; tv < COARSEST_TEST_VECTORS; ++tv) {
-    std::vector<double2> tvec = coarsest_test_vector(h->Nc, (uint64_t)tv + 1);
-    ck(h, cudaMemcpyAsync(h->cb, tvec.data(), sizeof(double2) * h->Nc, cudaMemcpyHostToDevice,
-                          h->s),
-       "upload");
-    ck(h, norm2<double>(h->cb, h->Nc, 1, h->partials, slot(h, S_T1), h->s), "norm");
-    const double bn = read_scalar(h, S_T1);
-    int steps = 0;
-    double rel = 0.0;
-    for (; steps <= h->p.coarsest_refine_max; ++steps) {
-      coarsest_solve64(h, h->cb, h->cx, steps, 1);
-      apply_level<double>(h, h->L - 1, h->cx, h->cr, 1, W_F64);
-      ck(h, sub_from<double>(h->cb, h->cr, h->Nc, h->s), "residual");
-      ck(h, norm2<double>(h->cr, h->Nc, 1, h->partials, slot(h, S_T0), h->s), "norm");
-      const double rr = read_scalar(h, S_T0);
-      if (!(rr == rr)) fail(h, MG_ERR_BREAKDOWN, "coarsest inverse is not finite");
-      rel = std::sqrt(rr / bn);
-      if (rel <= h->p.coarsest_tol) break;
-    }
-    h->coarsest_test_res = std::max(h->coarsest_test_res, rel);
-    if (steps > h->p.coarsest_refine_max) {
-      char msg[200];
-      std::snprintf(msg, sizeof msg,
-                    "coarsest solve: FP64 refinement of the FP32 inverse reached %.3g, not "
-                    "coarsest_tol %.3g, in %d steps (operator too ill-conditioned for FP32)",
-                    rel, h->p.coarsest_tol, h->p.coarsest_refine_max);
-      fail(h, MG_ERR_NOCONV, msg);
-    }
-    worst = std::max(worst, steps);
+  int worst = 0, inner = 0;
+  double rel = 0.0;
+  const RefineTest t = refinement_test(h, h->p.coarsest_refine_max, &worst, &inner, &rel);
+  h->coarsest_test_res = rel;
+  if (t == REFINE_NONFINITE) fail(h, MG_ERR_BREAKDOWN, "coarsest inverse is not finite");
+  if (t == REFINE_MISSED) {
+    char msg[200];
+    std::snprintf(msg, sizeof msg,
+                  "coarsest solve: FP64 refinement of the FP32 inverse reached %.3g, not "
+                  "coarsest_tol %.3g, in %d steps (operator too ill-conditioned for FP32)",
+                  rel, h->p.coarsest_tol, h->p.coarsest_refine_max);
+    fail(h, MG_ERR_NOCONV, msg);
   }
   h->n_refine = std::min(worst + 1, h->p.coarsest_refine_max);
   h->n_inner = h->p.inner_coarsest_refine;
