@@ -240,6 +240,12 @@ template <typename R>
 cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, int Lt, int bx,
                        int bt, int h, int Nv, int nrhs, bool accumulate, cudaStream_t s);
 
+// FP32 transfers with the block vectors in registers, for the blockings (and 16-byte aligned
+// coarse vectors) of transfer_reg_ok (restrict_op and prolong_op use them).
+bool transfer_reg_ok(const void* coarse, int bx, int bt, int h, int Nv);
+cudaError_t transfer_reg(const void* in, void* out, const void* Vst, int Lx, int Lt, int bx, int bt,
+                         int h, int Nv, int nrhs, bool prolong, bool accumulate, cudaStream_t s);
+
 // ---- setup ---------------------------------------------------------------
 // Chirality-split block modified Gram-Schmidt (two passes) of Nv relaxed
 // vectors E [Nv][V_f][n] (complex128) into Vst [V_f][2][Nv][h] (complex128).

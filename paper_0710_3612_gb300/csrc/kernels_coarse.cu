@@ -524,6 +524,8 @@ static size_t transfer_multi_smem(int bx, int bt, int h, int Nv, int nrhs, size_
 template <typename R>
 cudaError_t restrict_op(const void* fine, void* coarse, const void* Vst, int Lx, int Lt, int bx,
                         int bt, int h, int Nv, int nrhs, cudaStream_t s) {
+  if (sizeof(R) == 4 && transfer_reg_ok(coarse, bx, bt, h, Nv))
+    return transfer_reg(fine, coarse, Vst, Lx, Lt, bx, bt, h, Nv, nrhs, false, false, s);
   const size_t sm = transfer_multi_smem(bx, bt, h, Nv, nrhs, sizeof(cplx_t<R>), true);
   if (sm <= 96 * 1024) {
     static bool attr = false;
@@ -566,6 +568,8 @@ __global__ void k_prolong(const cplx_t<R>* __restrict__ coarse, cplx_t<R>* __res
 template <typename R>
 cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, int Lt, int bx,
                        int bt, int h, int Nv, int nrhs, bool accumulate, cudaStream_t s) {
+  if (sizeof(R) == 4 && transfer_reg_ok(coarse, bx, bt, h, Nv))
+    return transfer_reg(coarse, fine, Vst, Lx, Lt, bx, bt, h, Nv, nrhs, true, accumulate, s);
   const size_t sm = transfer_multi_smem(bx, bt, h, Nv, nrhs, sizeof(cplx_t<R>), false);
   if (sm <= 96 * 1024) {
     static bool attr = false;
