@@ -143,9 +143,10 @@ typedef struct {
                                            is bit-identical to the default
                                            shape's (1)                          */
   int remass_quadratic;                 /* nonzero: keep G0_l and G1_l with
-                                           A_l(m) = G0_l + m G1_l + m^2 I on
-                                           every coarse level (A(m) = A0 +
-                                           m (D0 + D0^dagger) + m^2 and
+                                           A_l(m) = G0_l + d G1_l + d^2 I, d =
+                                           m - (set-up mass), on every coarse
+                                           level (A(m + d) = A(m) +
+                                           d (D + D^dagger) + d^2 and
                                            P^dagger P = I), so a new mass is one
                                            combination per level instead of the
                                            Galerkin products; two more FP64

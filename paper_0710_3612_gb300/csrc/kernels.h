@@ -186,7 +186,7 @@ bool wilson_A_dot_fits(int Lx, int Lt, bool f64, double diag);
 // links: gauge complex128 [2][V] -> folded links of precision R
 template <typename R>
 cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s);
-// max_i ||U_i| - 1| into *out (device double), single block reduction
+// max_i ||U_i| - 1| into *out (device double)
 cudaError_t link_unitarity(const void* gauge, long long count, double* out, cudaStream_t s);
 
 // ---- coarse operator -----------------------------------------------------
@@ -201,7 +201,7 @@ long long coarse_words_bytes(long long sites, int n);
 cudaError_t coarse_apply_fx(const void* in, void* out, const void* A64, const void* words, int Lx, int Lt,
                             int n, int nrhs, const Epilogue& ep, cudaStream_t s);
 // The FP32 and BF16 copies and the words (may be null) of the blocks A64; with G0, first
-// A64 = G0 + m G1 + m^2 I.
+// A64 = G0 + m G1 + m^2 I (m: the distance from the mass of G0).
 cudaError_t coarse_finish(const void* G0, const void* G1, double m, void* A64, void* A32, void* A16,
                           void* words, long long sites, int n, cudaStream_t s);
 // Multi-RHS BF16 coarse apply on tcgen05 tensor cores (TMEM accumulator):
@@ -253,8 +253,9 @@ cudaError_t transfer_reg(const void* in, void* out, const void* Vst, int Lx, int
 cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx, int bt, int h,
                                int Nv, double breakdown_tol, int* flag, cudaStream_t s);
 // Level-1 Galerkin: W = D P on the extended blocks, then A_c = W^dagger W
-// overlaps.  Wbuf: [Vc][2Nv][(bx+2)(bt+2)][2] complex128 scratch.
-cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* Wbuf, void* Ac,
+// overlaps.  Wbuf: [Vc][2Nv][(bx+2)(bt+2)][2] complex128 scratch.  G1 (optional) receives
+// P^dagger W + W^dagger P: A_c(m + d) = A_c + d G1 + d^2 I.
+cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* Wbuf, void* Ac, void* G1,
                           int Lx, int Lt, int bx, int bt, int Nv, cudaStream_t s);
 // Level >= 2 Galerkin: A_{l+1}[j][d] = sum P(i)^dagger A_l[i][e] P(i+e).
 cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, int Lt, int bx,

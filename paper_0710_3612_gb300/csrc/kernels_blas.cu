@@ -107,12 +107,17 @@ cudaError_t axpby(double a, const void* x, double b, void* y, long long count, i
 }
 
 template <typename R>
-__global__ void k_scale_inv_sqrt(const cplx_t<R>* __restrict__ x, cplx_t<R>* __restrict__ y,
-                                 const double* nrm, long long count) {
+__global__ void __launch_bounds__(RT) k_scale_inv_sqrt(const cplx_t<R>* x, cplx_t<R>* y,
+                                                       const double* nrm, long long count) {
+  __shared__ double ssc;                             // one root and division per block
+  if (threadIdx.x == 0) {
+    const double n2 = nrm[2 * blockIdx.y];
+    ssc = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
+  }
+  __syncthreads();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
-  const double n2 = nrm[2 * blockIdx.y];
-  const R sc = n2 > 0.0 ? (R)(1.0 / sqrt(n2)) : (R)0;
+  const R sc = (R)ssc;
   i += (long long)blockIdx.y * count;
   cplx_t<R> u = x[i];
   y[i] = mk(u.x * sc, u.y * sc);

@@ -591,99 +591,111 @@ cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, 
 }
 
 // ---------------------------------------------------------------------------
-// Chirality-split block modified Gram-Schmidt, one warp per (block, chirality).
-// The m = bx*bt*h entries of a block vector are spread over the 32 lanes
-// (entry e = lane + 32 q); orthonormalised vectors are kept in shared memory.
+// Chirality-split block modified Gram-Schmidt (two passes), LPB lanes per (block,
+// chirality): the m = bx*bt*h entries of a block vector are spread over them (entry e =
+// lane + LPB q, q < NQ); orthonormalised vectors are kept in shared memory.  Bound by FP64
+// issue: NQ and LPB are compile-time so that no slot goes to entries past m (eight
+// predicated entries a lane for every size took 837 us for 2048 blocks of 16 entries
+// and 8 vectors, 248 us for 512 of 32; 92 and 74 us here).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+template <int LPB>
+__device__ __forceinline__ double lanes_sum(double v) {
+#pragma unroll
+  for (int o = LPB / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-static constexpr int GS_MAXQ = 8;   // up to 256 entries per block vector
-
+template <int LPB, int NQ>
 __global__ void __launch_bounds__(32) k_block_gs(const double2* __restrict__ E,
                                                  double2* __restrict__ Vst, int Lx, int Lt,
                                                  int bx, int bt, int h, int Nv, double tol,
-                                                 int* flag) {
-  extern __shared__ double2 Q[];   // [Nv][m]
+                                                 int* flag, int nblocks) {
+  extern __shared__ double2 Qs[];   // [32 / LPB][Nv][m]
   const int V = Lx * Lt, nf = 2 * h, Lxc = Lx / bx;
-  const int j = blockIdx.x >> 1, c = blockIdx.x & 1, lane = threadIdx.x;
-  const int m = bx * bt * h, nq = (m + 31) / 32;
+  const int sub = threadIdx.x / LPB, lane = threadIdx.x % LPB;
+  const int blk = blockIdx.x * (32 / LPB) + sub;
+  const bool on = blk < nblocks;
+  const int j = blk >> 1, c = blk & 1;
+  const int m = bx * bt * h;
+  double2* Q = Qs + sub * Nv * m;
+  long long at[NQ];                 // entry e of the block: site * 2 h + c h + a, or -1
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const int e = lane + LPB * q;
+    at[q] = on && e < m ? (long long)block_site(j, e / h, Lxc, Lx, bx, bt) * nf + c * h + e % h : -1;
+  }
   for (int k = 0; k < Nv; ++k) {
-    double2 u[GS_MAXQ];
+    double2 u[NQ];
     double n0 = 0.0;
 #pragma unroll
-    for (int q = 0; q < GS_MAXQ; ++q) {
-      u[q] = make_double2(0.0, 0.0);
-      const int e = lane + 32 * q;
-      if (q < nq && e < m) {
-        const int o = e / h, a = e % h;
-        const int i = block_site(j, o, Lxc, Lx, bx, bt);
-        u[q] = E[((long long)k * V + i) * nf + c * h + a];
-        n0 += u[q].x * u[q].x + u[q].y * u[q].y;
-      }
+    for (int q = 0; q < NQ; ++q) {
+      u[q] = at[q] >= 0 ? E[(long long)k * V * nf + at[q]] : make_double2(0.0, 0.0);
+      n0 += u[q].x * u[q].x + u[q].y * u[q].y;
     }
-    n0 = warp_sum(n0);
+    n0 = lanes_sum<LPB>(n0);
     for (int pass = 0; pass < 2; ++pass) {
       for (int kk = 0; kk < k; ++kk) {
+        double2 w[NQ];
         double re = 0.0, im = 0.0;
 #pragma unroll
-        for (int q = 0; q < GS_MAXQ; ++q) {
-          const int e = lane + 32 * q;
-          if (q < nq && e < m) {
-            double2 w = Q[kk * m + e];
-            re += w.x * u[q].x + w.y * u[q].y;
-            im += w.x * u[q].y - w.y * u[q].x;
-          }
+        for (int q = 0; q < NQ; ++q) {
+          w[q] = at[q] >= 0 ? Q[kk * m + lane + LPB * q] : make_double2(0.0, 0.0);
+          re += w[q].x * u[q].x + w[q].y * u[q].y;
+          im += w[q].x * u[q].y - w[q].y * u[q].x;
         }
-        re = warp_sum(re);
-        im = warp_sum(im);
+        re = lanes_sum<LPB>(re);
+        im = lanes_sum<LPB>(im);
 #pragma unroll
-        for (int q = 0; q < GS_MAXQ; ++q) {
-          const int e = lane + 32 * q;
-          if (q < nq && e < m) {
-            double2 w = Q[kk * m + e];
-            u[q].x -= re * w.x - im * w.y;
-            u[q].y -= re * w.y + im * w.x;
-          }
+        for (int q = 0; q < NQ; ++q) {
+          u[q].x -= re * w[q].x - im * w[q].y;
+          u[q].y -= re * w[q].y + im * w[q].x;
         }
       }
     }
     double n1 = 0.0;
 #pragma unroll
-    for (int q = 0; q < GS_MAXQ; ++q)
-      if (q < nq) n1 += u[q].x * u[q].x + u[q].y * u[q].y;
-    n1 = warp_sum(n1);
+    for (int q = 0; q < NQ; ++q) n1 += u[q].x * u[q].x + u[q].y * u[q].y;
+    n1 = lanes_sum<LPB>(n1);
     if (!(n1 > tol * tol * n0)) {
-      if (lane == 0) atomicExch(flag, 1);
+      if (on && lane == 0) atomicExch(flag, 1);
       n1 = n1 > 0.0 ? n1 : 1.0;
     }
     const double inv = 1.0 / sqrt(n1);
 #pragma unroll
-    for (int q = 0; q < GS_MAXQ; ++q) {
-      const int e = lane + 32 * q;
-      if (q < nq && e < m) {
-        double2 w = make_double2(u[q].x * inv, u[q].y * inv);
+    for (int q = 0; q < NQ; ++q)
+      if (at[q] >= 0) {
+        const int e = lane + LPB * q, a = e % h;
+        const double2 w = make_double2(u[q].x * inv, u[q].y * inv);
         Q[k * m + e] = w;
-        const int o = e / h, a = e % h;
-        const int i = block_site(j, o, Lxc, Lx, bx, bt);
-        Vst[(((long long)i * 2 + c) * Nv + k) * h + a] = w;
+        const long long i = (at[q] - c * h - a) / nf;
+        Vst[((i * 2 + c) * Nv + k) * h + a] = w;
       }
-    }
     __syncwarp();
   }
 }
 
 cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx, int bt, int h,
                                int Nv, double breakdown_tol, int* flag, cudaStream_t s) {
-  const int m = bx * bt * h;
-  if (m > 32 * GS_MAXQ) return cudaErrorInvalidValue;
-  const int Vc = (Lx / bx) * (Lt / bt);
-  const size_t smem = (size_t)Nv * m * sizeof(double2);
-  k_block_gs<<<2 * Vc, 32, smem, s>>>((const double2*)E, (double2*)Vst, Lx, Lt, bx, bt, h, Nv,
-                                     breakdown_tol, flag); count_launch();
-  return cudaGetLastError();
+  const int m = bx * bt * h, nb = 2 * (Lx / bx) * (Lt / bt);
+  if (m > 256) return cudaErrorInvalidValue;
+  auto go = [&](auto lpb, auto nq) {
+    constexpr int LPB = decltype(lpb)::value, NQ = decltype(nq)::value;
+    const int per = 32 / LPB;
+    const size_t smem = (size_t)per * Nv * m * sizeof(double2);   // at most 128 KB (m = 256, Nv = 32)
+    static const cudaError_t e = cudaFuncSetAttribute(
+        k_block_gs<LPB, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    if (e != cudaSuccess) return e;
+    k_block_gs<LPB, NQ><<<(nb + per - 1) / per, 32, smem, s>>>((const double2*)E, (double2*)Vst, Lx, Lt, bx,
+                                                              bt, h, Nv, breakdown_tol, flag, nb);
+    count_launch();
+    return cudaGetLastError();
+  };
+  using std::integral_constant;
+  if (m <= 16) return go(integral_constant<int, 16>(), integral_constant<int, 1>());
+  if (m <= 32) return go(integral_constant<int, 32>(), integral_constant<int, 1>());
+  if (m <= 64) return go(integral_constant<int, 32>(), integral_constant<int, 2>());
+  if (m <= 128) return go(integral_constant<int, 32>(), integral_constant<int, 4>());
+  return go(integral_constant<int, 32>(), integral_constant<int, 8>());
 }
 
 // ---------------------------------------------------------------------------
@@ -743,43 +755,96 @@ __global__ void k_galerkin_W(const double2* __restrict__ U, double diag,
   Wbuf[2 * idx + 1] = w1;
 }
 
-__global__ void k_galerkin_WW(const double2* __restrict__ Wbuf, double2* __restrict__ Ac, int Lx,
-                              int Lt, int bx, int bt, int Nv) {
-  const int Lxc = Lx / bx, Ltc = Lt / bt, Vc = Lxc * Ltc, nc = 2 * Nv;
-  const int ex_w = bx + 2, E = (bx + 2) * (bt + 2);
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)Vc * 9 * nc * nc) return;
-  const int sc = (int)(idx % nc);
-  const int r = (int)((idx / nc) % nc);
-  const int d = (int)((idx / (nc * nc)) % 9);
-  const int j = (int)(idx / (9LL * nc * nc));
+// A_c = W^dagger W, or (G1) the derivative in the mass: W(m + d) = W + d P gives
+// A_c(m + d) = W^dagger W + d (P^dagger W + W^dagger P) + d^2.  Hermitian, so only
+// displacements 4 (its lower half) .. 8 are summed and their mirror images written too: the
+// sums are FP64-bound (51,200 complex products per site, 375 us for 1024 sites of 16 dof;
+// 26,800 and 181 us with the symmetry, the derivative 69 us).
+// Entries are numbered with all centres first, then edges, then corners: the threads of a
+// warp run sums of one length.
+template <bool G1>
+__global__ void k_galerkin_WW(const double2* __restrict__ Wbuf, const double2* __restrict__ Vst,
+                              double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt, int Nv) {
+  const int Lxc = Lx / bx, Ltc = Lt / bt, nc = 2 * Nv;
+  const long long Vc = (long long)Lxc * Ltc;
+  const int ex_w = bx + 2, E = (bx + 2) * (bt + 2), tri = nc * (nc + 1) / 2;
+  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  int d, r, sc, j;
+  if (idx < Vc * tri) {
+    const int t = (int)(idx % tri);
+    j = (int)(idx / tri);
+    r = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+    while ((r + 1) * (r + 2) / 2 <= t) ++r;
+    while (r * (r + 1) / 2 > t) --r;
+    sc = t - r * (r + 1) / 2;
+    d = 4;
+  } else {
+    idx -= Vc * tri;
+    const int g = (int)(idx / (2 * Vc * nc * nc));          // 0: edges 5, 7; 1: corners 6, 8
+    if (g > 1) return;
+    idx -= (long long)g * 2 * Vc * nc * nc;
+    sc = (int)(idx % nc);
+    r = (int)((idx / nc) % nc);
+    d = 5 + g + 2 * (int)((idx / (nc * nc)) % 2);
+    j = (int)(idx / (2LL * nc * nc));
+  }
   const int dx = d % 3 - 1, dt = d / 3 - 1;
   const int jx = j % Lxc, jt = j / Lxc;
   const int j2 = ((jx + dx + Lxc) % Lxc) + Lxc * ((jt + dt + Ltc) % Ltc);
-  const int x0 = max(-1, dx * bx - 1), x1 = min(bx, dx * bx + bx);
-  const int t0 = max(-1, dt * bt - 1), t1 = min(bt, dt * bt + bt);
   const double2* Wa = Wbuf + ((long long)j * nc + r) * E * 2;
   const double2* Wb = Wbuf + ((long long)j2 * nc + sc) * E * 2;
   double2 acc = make_double2(0.0, 0.0);
-  for (int lt = t0; lt <= t1; ++lt)
-    for (int lx = x0; lx <= x1; ++lx) {
-      const int e1 = (lt + 1) * ex_w + (lx + 1);
-      const int e2 = (lt - dt * bt + 1) * ex_w + (lx - dx * bx + 1);
-      cfmac(acc, Wa[2 * e1], Wb[2 * e2]);
-      cfmac(acc, Wa[2 * e1 + 1], Wb[2 * e2 + 1]);
-    }
+  if (!G1) {
+    const int x0 = max(-1, dx * bx - 1), x1 = min(bx, dx * bx + bx);
+    const int t0 = max(-1, dt * bt - 1), t1 = min(bt, dt * bt + bt);
+    for (int lt = t0; lt <= t1; ++lt)
+      for (int lx = x0; lx <= x1; ++lx) {
+        const int e1 = (lt + 1) * ex_w + (lx + 1);
+        const int e2 = (lt - dt * bt + 1) * ex_w + (lx - dx * bx + 1);
+        cfmac(acc, Wa[2 * e1], Wb[2 * e2]);
+        cfmac(acc, Wa[2 * e1 + 1], Wb[2 * e2 + 1]);
+      }
+  } else if (d % 2 == 0 && d != 4) {
+    // no hop reaches across a corner: zero
+  } else {
+    const int cr = r / Nv, kr = r % Nv, cs = sc / Nv, ks = sc % Nv;
+    // sites of block j (local coordinates) within one of block j + d, and vice versa
+    const int ax0 = max(0, dx * bx - 1), ax1 = min(bx - 1, dx * bx + bx);
+    const int at0 = max(0, dt * bt - 1), at1 = min(bt - 1, dt * bt + bt);
+    for (int lt = at0; lt <= at1; ++lt)
+      for (int lx = ax0; lx <= ax1; ++lx) {                 // conj(P_j,r) W_{j+d,s}
+        const int e2 = (lt - dt * bt + 1) * ex_w + (lx - dx * bx + 1);
+        const long long i = (jx * bx + lx) + (long long)Lx * (jt * bt + lt);
+        cfmac(acc, Vst[(i * 2 + cr) * Nv + kr], Wb[2 * e2 + cr]);
+      }
+    const int kx = j2 % Lxc, kt = j2 / Lxc;
+    const int bx0 = max(0, -dx * bx - 1), bx1 = min(bx - 1, -dx * bx + bx);
+    const int bt0 = max(0, -dt * bt - 1), bt1 = min(bt - 1, -dt * bt + bt);
+    for (int lt = bt0; lt <= bt1; ++lt)
+      for (int lx = bx0; lx <= bx1; ++lx) {                 // conj(W_j,r) P_{j+d,s}
+        const int e1 = (lt + dt * bt + 1) * ex_w + (lx + dx * bx + 1);
+        const long long i = (kx * bx + lx) + (long long)Lx * (kt * bt + lt);
+        cfmac(acc, Wa[2 * e1 + cs], Vst[(i * 2 + cs) * Nv + ks]);
+      }
+  }
+  if (d == 4 && r == sc) acc.y = 0.0;
   Ac[(((long long)j * 9 + d) * nc + r) * nc + sc] = acc;
+  if (d != 4 || r != sc) Ac[(((long long)j2 * 9 + 8 - d) * nc + sc) * nc + r] = cconj(acc);
 }
 
-cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* Wbuf, void* Ac,
+cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* Wbuf, void* Ac, void* G1,
                           int Lx, int Lt, int bx, int bt, int Nv, cudaStream_t s) {
   const long long Vc = (long long)(Lx / bx) * (Lt / bt), nc = 2 * Nv;
   const long long nW = Vc * nc * (bx + 2) * (bt + 2);
   k_galerkin_W<<<(unsigned)((nW + 255) / 256), 256, 0, s>>>(
       (const double2*)U64, diag, (const double2*)Vst, (double2*)Wbuf, Lx, Lt, bx, bt, Nv); count_launch();
-  const long long nA = Vc * 9 * nc * nc;
-  k_galerkin_WW<<<(unsigned)((nA + 255) / 256), 256, 0, s>>>((const double2*)Wbuf,
-                                                              (double2*)Ac, Lx, Lt, bx, bt, Nv); count_launch();
+  const long long nA = Vc * (nc * (nc + 1) / 2 + 4 * nc * nc);
+  k_galerkin_WW<false><<<(unsigned)((nA + 255) / 256), 256, 0, s>>>(
+      (const double2*)Wbuf, (const double2*)Vst, (double2*)Ac, Lx, Lt, bx, bt, Nv); count_launch();
+  if (G1) {
+    k_galerkin_WW<true><<<(unsigned)((nA + 255) / 256), 256, 0, s>>>(
+        (const double2*)Wbuf, (const double2*)Vst, (double2*)G1, Lx, Lt, bx, bt, Nv); count_launch();
+  }
   return cudaGetLastError();
 }
 
@@ -787,7 +852,9 @@ cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* W
 // Level >= 2 Galerkin, one CTA per coarse site j; the CTA accumulates the 9
 // blocks of A_{l+1}[j] in shared memory.  For each fine site i of S_j and
 // each fine displacement e: T = A_l[i][e] P(i+e) (nf x nc), then
-// A_{l+1}[j][disp(i,e)] += P(i)^dagger T, disp = floor((o_i + e) / b).
+// A_{l+1}[j][disp(i,e)] += P(i)^dagger T, disp = floor((o_i + e) / b).  The operator is
+// Hermitian: displacements 4 .. 8 are summed (26 of the 36 products of a 2 x 2 block) and
+// their mirror images written; FP64-bound.
 // ---------------------------------------------------------------------------
 __global__ void k_galerkin_coarse(const double2* __restrict__ Af, const double2* __restrict__ Vst,
                                   double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt,
@@ -811,6 +878,7 @@ __global__ void k_galerkin_coarse(const double2* __restrict__ Af, const double2*
       const int ddx = (ox + ex < 0) ? -1 : ((ox + ex >= bx) ? 1 : 0);
       const int ddt = (ot + et < 0) ? -1 : ((ot + et >= bt) ? 1 : 0);
       const int d = (ddx + 1) + 3 * (ddt + 1);
+      if (d < 4) continue;
       const double2* Ablk = Af + ((long long)i * 9 + e) * nf * nf;
       // T[a][s] = sum_b A[a][c_s h + b] V_{k_s}(i2)[c_s h + b]
       for (int q = threadIdx.x; q < nf * nc; q += blockDim.x) {
@@ -833,8 +901,15 @@ __global__ void k_galerkin_coarse(const double2* __restrict__ Af, const double2*
       __syncthreads();
     }
   }
-  for (int q = threadIdx.x; q < 9 * nc * nc; q += blockDim.x)
-    Ac[(long long)j * 9 * nc * nc + q] = acc[q];
+  const int Lxc2 = Lx / bx, Ltc = Lt / bt;
+  for (int q = threadIdx.x + 4 * nc * nc; q < 9 * nc * nc; q += blockDim.x) {
+    const int d = q / (nc * nc), r = q / nc % nc, sc = q % nc;
+    const double2 v = acc[q];
+    Ac[(long long)j * 9 * nc * nc + q] = v;
+    if (d == 4) continue;                            // summed in full
+    const int j2 = (jx + d % 3 - 1 + Lxc2) % Lxc2 + Lxc2 * ((jt + d / 3 - 1 + Ltc) % Ltc);
+    Ac[(((long long)j2 * 9 + 8 - d) * nc + sc) * nc + r] = cconj(v);
+  }
 }
 
 cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, int Lt, int bx,

@@ -598,29 +598,26 @@ cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t 
   return cudaGetLastError();
 }
 
-__global__ void k_link_unitarity(const double2* __restrict__ g, long long count, double* out) {
-  double m = 0.0;
-  for (long long i = threadIdx.x; i < count; i += blockDim.x) {
-    double2 u = g[i];
-    double d = fabs(sqrt(u.x * u.x + u.y * u.y) - 1.0);
-    m = (d > m || d != d) ? d : m;   // NaN propagates
+// Non-negative doubles (and NaN above them) order like their bit patterns.
+__global__ void __launch_bounds__(256) k_link_unitarity(const double2* __restrict__ g, long long count,
+                                                        unsigned long long* out) {
+  unsigned long long m = 0;
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < count; i += 256LL * gridDim.x) {
+    const double2 u = g[i];
+    const double d = fabs(sqrt(u.x * u.x + u.y * u.y) - 1.0);
+    m = max(m, (unsigned long long)__double_as_longlong(d));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    double v = __shfl_down_sync(0xffffffffu, m, o);
-    m = (v > m || v != v) ? v : m;
-  }
-  __shared__ double sh[32];
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r = (sh[w] > r || sh[w] != sh[w]) ? sh[w] : r;
-    *out = r;
-  }
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
 }
 
 cudaError_t link_unitarity(const void* gauge, long long count, double* out, cudaStream_t s) {
-  k_link_unitarity<<<1, 1024, 0, s>>>((const double2*)gauge, count, out); count_launch();
+  const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), s);
+  if (e != cudaSuccess) return e;
+  const long long g = (count + 255) / 256;
+  k_link_unitarity<<<(unsigned)(g < 1216 ? g : 1216), 256, 0, s>>>((const double2*)gauge, count,
+                                                                 (unsigned long long*)out);
+  count_launch();
   return cudaGetLastError();
 }
 

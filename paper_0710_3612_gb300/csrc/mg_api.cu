@@ -31,7 +31,7 @@ struct Level {
   float2* A32 = nullptr;
   void* A16 = nullptr;
   void* Afx = nullptr;                   // the FP64 blocks as integer words (coarse_finish)
-  double2* G0 = nullptr;                 // A(m) = G0 + m G1 + m^2 I (remass_quadratic)
+  double2* G0 = nullptr;                 // A(m) = G0 + d G1 + d^2 I, d = m - g_mass (remass_quadratic)
   double2* G1 = nullptr;
   // transfer to the next level
   int bx = 0, bt = 0, Nv = 0;
@@ -102,6 +102,8 @@ struct mg_handle {
   double* hscal = nullptr;      // pinned host mirror
   int* dflag = nullptr;
   std::vector<void*> allocs;
+  char* slab = nullptr;         // one allocation behind everything allocate_storage hands out
+  size_t slab_left = 0;
   long long bytes = 0;          // device bytes currently allocated by the handle
   long long peak_bytes = 0;     // largest value of `bytes` so far
   bool dry = false;             // size-only pass: dalloc counts bytes, allocates nothing
@@ -109,6 +111,7 @@ struct mg_handle {
   long long fine_applies = 0, vcycles = 0;
   std::vector<double> refine_rho;   // rho of each adaptive pass made by mg_setup
   bool g_built = false;             // G0, G1 of every coarse level hold the current vectors
+  double g_mass = 0.0;              // the mass at which G0 is the operator
   // optional per-family event timing
   bool prof_on = false;
   std::vector<cudaEvent_t> prof_ev[MG_KF_COUNT];
@@ -142,10 +145,17 @@ void ck(mg_handle* h, cudaError_t e, const char* what) {
 template <typename T = void>
 T* dalloc(mg_handle* h, size_t bytes) {
   void* p = nullptr;
-  if (bytes == 0) bytes = 16;
+  bytes = (bytes + 255) / 256 * 256;
+  if (bytes == 0) bytes = 256;
   h->bytes += (long long)bytes;
   h->peak_bytes = std::max(h->peak_bytes, h->bytes);
   if (h->dry) return (T*)(uintptr_t)256;        // never dereferenced in a size-only pass
+  if (bytes <= h->slab_left) {
+    p = h->slab;
+    h->slab += bytes;
+    h->slab_left -= bytes;
+    return (T*)p;
+  }
   cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -154,6 +164,14 @@ T* dalloc(mg_handle* h, size_t bytes) {
   }
   h->allocs.push_back(p);
   return (T*)p;
+}
+
+// Frees one dalloc made outside allocate_storage.
+void dfree(mg_handle* h, void* q, size_t bytes) {
+  for (auto& a : h->allocs)
+    if (a == q) a = nullptr;
+  cudaFree(q);
+  h->bytes -= (long long)((bytes + 255) / 256 * 256);
 }
 
 void sync(mg_handle* h) { ck(h, cudaStreamSynchronize(h->s), "stream synchronize"); }
@@ -352,18 +370,31 @@ void vcycle(mg_handle* h, int l, const void* b, void* x, int nrhs = 1,
 }
 
 // ----- setup pieces ---------------------------------------------------------
+// Rayleigh quotient after power_iters applications.  The iterate is normalised only every
+// POWER_NORM steps for ordinary masses (a scale does not change the quotient, and the 16th
+// power of A < 2^14 is within the exponents the kernels take): a norm and a scaling per step
+// were two of its three launches (set-up of the 128^2 workload: 0.7 ms).
+constexpr int POWER_NORM = 16;
+
 double power_lambda_max(mg_handle* h, int l, const double2* start, void* v, void* w) {
   Level& L = h->lv[l];
   const long long n = L.count();
   ck(h, norm2<double>(start, n, 1, h->partials, slot(h, S_T0), h->s), "norm");
   ck(h, scale_inv_sqrt<double>(start, v, slot(h, S_T0), n, 1, h->s), "scale");
-  for (int it = 0; it < h->p.power_iters; ++it) {
+  const int every = fixed_diag_ok(4.0 + h->mass) ? POWER_NORM : 1;
+  for (int it = 0; it < h->p.power_iters - 1; ++it) {
     apply_level<double>(h, l, v, w, 1, W_F64);
-    if (it == h->p.power_iters - 1) ck(h, dot<double>(v, w, n, 1, h->partials, slot(h, S_T1), h->s), "dot");
-    ck(h, norm2<double>(w, n, 1, h->partials, slot(h, S_T0), h->s), "norm");
-    ck(h, scale_inv_sqrt<double>(w, v, slot(h, S_T0), n, 1, h->s), "scale");
+    std::swap(v, w);
+    if ((it + 1) % every == 0) {
+      ck(h, norm2<double>(v, n, 1, h->partials, slot(h, S_T0), h->s), "norm");
+      ck(h, scale_inv_sqrt<double>(v, v, slot(h, S_T0), n, 1, h->s), "scale");
+    }
   }
-  return read_scalar(h, S_T1);
+  apply_level<double>(h, l, v, w, 1, W_F64);
+  ck(h, dot<double>(v, w, n, 1, h->partials, slot(h, S_T1), h->s), "dot");
+  ck(h, norm2<double>(v, n, 1, h->partials, slot(h, S_T0), h->s), "norm");
+  const double num = read_scalar(h, S_T1), den = read_scalar(h, S_T0);
+  return num / den;
 }
 
 void smoother_coefficients(mg_handle* h, int l, void* q, void* r1) {
@@ -388,26 +419,6 @@ void smoother_coefficients(mg_handle* h, int l, void* q, void* r1) {
   L.c1 = -om * om * a0 * a1;
 }
 
-// G0 and G1 of every coarse level from the vectors: on level 2, G0 = the
-// Galerkin product at m = 0 and G1 = (the product at m = 1) - G0 - I; below,
-// both pass through P^dagger . P like the operator itself.
-void build_quadratic(mg_handle* h) {
-  for (int l = 0; l + 1 < h->L; ++l) {
-    Level& L = h->lv[l];
-    Level& C = h->lv[l + 1];
-    ProfScope prof(h, MG_KF_GALERKIN);
-    if (l == 0) {
-      ck(h, galerkin_fine(h->U64, 4.0, L.Vst64, h->Wbuf, C.G0, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin G0");
-      ck(h, galerkin_fine(h->U64, 5.0, L.Vst64, h->Wbuf, C.G1, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin A(1)");
-      ck(h, coarse_lincomb(1.0, C.G1, -1.0, C.G0, -1.0, C.G1, C.V, C.n, h->s), "G1");
-    } else {
-      ck(h, galerkin_coarse(L.G0, L.Vst64, C.G0, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin G0");
-      ck(h, galerkin_coarse(L.G1, L.Vst64, C.G1, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin G1");
-    }
-  }
-  h->g_built = true;
-}
-
 void galerkin_next(mg_handle* h, int l);
 
 // The copies and words of level l's FP64 blocks.
@@ -416,21 +427,21 @@ void finish_level(mg_handle* h, int l) {
   ck(h, coarse_finish(nullptr, nullptr, 0.0, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "level copies");
 }
 
+// Level l's operator at the handle's mass from G0 and G1, with its copies.
+void combine_level(mg_handle* h, int l) {
+  Level& C = h->lv[l];
+  ck(h, coarse_finish(C.G0, C.G1, h->mass - h->g_mass, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "A(m)");
+}
+
 void build_coarse_ops(mg_handle* h) {
-  if (h->p.remass_quadratic) {
-    if (!h->g_built) build_quadratic(h);
-    const double m = h->mass;
-    for (int l = 1; l < h->L; ++l) {
-      Level& C = h->lv[l];
-      ProfScope prof(h, MG_KF_GALERKIN);
-      ck(h, coarse_finish(C.G0, C.G1, m, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "A(m)");
-    }
-    return;
-  }
   for (int l = 0; l + 1 < h->L; ++l) {
     ProfScope prof(h, MG_KF_GALERKIN);
-    galerkin_next(h, l);
+    if (h->p.remass_quadratic && h->g_built)
+      combine_level(h, l + 1);
+    else
+      galerkin_next(h, l);
   }
+  h->g_built = h->p.remass_quadratic != 0;
 }
 
 // Test vectors of the coarsest solve's set-up: complex Gaussian entries (Re,
@@ -648,6 +659,15 @@ void set_mass_internal(mg_handle* h, double mass) {
   sync(h);
 }
 
+// After the levels have been built at the handle's mass: smoothers and coarsest solve.
+void finish_setup(mg_handle* h) {
+  h->g_built = h->p.remass_quadratic != 0;
+  for (int l = 0; l + 1 < h->L; ++l)
+    smoother_coefficients(h, l, h->lv[l].w64[3], h->lv[l].w64[2]);
+  if (h->L > 1) build_coarsest(h);
+  sync(h);
+}
+
 // Adaptive passes asked for by p (refine_levels up to the first 0).
 // Parameters as the handle uses them: smoothed aggregation probes every mass
 // anew, so it keeps no quadratic re-mass coefficients.
@@ -792,7 +812,6 @@ void free_all(mg_handle* h) {
   h->allocs.clear();
   if (h->hscal) cudaFreeHost(h->hscal);
   h->hscal = nullptr;
-  if (h->hctrl) cudaFreeHost(h->hctrl);
   h->hctrl = nullptr;
 }
 
@@ -1273,7 +1292,7 @@ void allocate_storage(mg_handle* h) {
       h->Binv = dalloc<float2>(h, (size_t)h->ldc * h->ldc * sizeof(float2));
       const size_t tcw = (size_t)3 * h->ldc * 64 + 2 * 64 * 64 + 2;
       h->gj_work = dalloc<float2>(h, std::max(inverse_work_entries(h->ldc), tcw) * sizeof(float2));
-      h->inv_plan = inverse_plan(C.Lx, C.Lt, C.n, h->ldc);
+      if (h->inv_plan.groups.empty()) h->inv_plan = inverse_plan(C.Lx, C.Lt, C.n, h->ldc);
       const size_t pb = h->inv_plan.data.size() * sizeof(int);
       h->inv_data = dalloc<int>(h, pb);
       if (!h->dry)                             // the plan lives in the handle: a plain copy
@@ -1293,10 +1312,32 @@ void allocate_storage(mg_handle* h) {
   }
 }
 
+// The handle's storage from one cudaMalloc, sized by a size-only pass (75 allocations and
+// frees took 2.1 of the 11.4 ms of a 128^2 set-up with its destruction).
+void allocate_handle(mg_handle* h) {
+  const long long b0 = h->bytes, p0 = h->peak_bytes;
+  h->dry = true;
+  allocate_storage(h);
+  h->dry = false;
+  const size_t total = (size_t)(h->bytes - b0);
+  h->bytes = b0;
+  h->peak_bytes = p0;
+  h->partial_rhs = 0;
+  void* p = nullptr;
+  if (cudaMalloc(&p, total) != cudaSuccess) {
+    cudaGetLastError();
+    fail(h, MG_ERR_NOMEM, "cudaMalloc of " + std::to_string(total) + " bytes failed");
+  }
+  h->allocs.push_back(p);
+  h->slab = (char*)p;
+  h->slab_left = total;
+  allocate_storage(h);
+}
+
 // Pinned host mirrors, the internal graph stream and its fences.
 void init_runtime(mg_handle* h) {
-  ck(h, cudaMallocHost((void**)&h->hscal, 64 * sizeof(double)), "pinned alloc");
-  ck(h, cudaMallocHost((void**)&h->hctrl, (4 + 2 * h->R) * sizeof(int)), "pinned alloc");
+  ck(h, cudaMallocHost((void**)&h->hscal, 64 * sizeof(double) + (4 + 2 * h->R) * sizeof(int)), "pinned alloc");
+  h->hctrl = (int*)(h->hscal + 64);
   ck(h, cudaStreamCreateWithFlags(&h->gs, cudaStreamNonBlocking), "stream create");
   ck(h, cudaEventCreateWithFlags(&h->fence[0], cudaEventDisableTiming), "event create");
   ck(h, cudaEventCreateWithFlags(&h->fence[1], cudaEventDisableTiming), "event create");
@@ -1308,13 +1349,13 @@ void init_runtime(mg_handle* h) {
 long long setup_temp_bytes(const mg_handle* h) {
   long long t = 0;
   for (int l = 0; l + 1 < h->L; ++l)
-    t = std::max(t, 2LL * h->lv[l].Nv * h->lv[l].count() * (long long)sizeof(double2));
+    t = std::max(t, 2LL * h->lv[l].Nv * h->lv[l].count() * (long long)sizeof(double2) + 256);
   if (h->p.smooth_omega != 0.0 && h->L > 1) {   // column probing of the smoothed level 2
     const Level& L = h->lv[0];
     const Level& C = h->lv[1];
     const long long nc = 2LL * L.Nv;
     t = std::max(t, (3 * nc * L.count() + 2 * nc * C.count() + 3LL * C.V * 9 * C.n * C.n) *
-                        (long long)sizeof(double2));
+                        (long long)sizeof(double2) + 8 * 256);
   }
   return t;
 }
@@ -1361,12 +1402,8 @@ void smoothed_products(mg_handle* h, double2* G[3]) {
       }
     }
   sync(h);
-  for (void* q : {W, T1, T2, E, Y}) {
-    for (auto& a : h->allocs)
-      if (a == q) a = nullptr;
-    cudaFree(q);
-  }
-  h->bytes -= (3LL * nc * c + 2LL * nc * cc) * (long long)sizeof(double2);
+  for (void* q : {W, T1, T2}) dfree(h, q, (size_t)nc * c * sizeof(double2));
+  for (void* q : {E, Y}) dfree(h, q, (size_t)nc * cc * sizeof(double2));
 }
 
 void smoothed_combination(mg_handle* h, double2* const G[3], double omega) {
@@ -1483,22 +1520,32 @@ void galerkin_smoothed(mg_handle* h) {
   }
   smoothed_combination(h, G, h->smooth);
   sync(h);
-  for (double2* q : G) {
-    for (auto& a : h->allocs)
-      if (a == q) a = nullptr;
-    cudaFree(q);
-  }
-  h->bytes -= 3LL * (long long)ab;
+  for (double2* q : G) dfree(h, q, ab);
 }
 
-// Galerkin operator of level l + 1 from the vectors of level l, with its copies.
+// Galerkin operator of level l + 1 from the vectors of level l, with its copies.  With
+// remass_quadratic through its mass coefficients about the current mass: on level 2 both come
+// from one W = D P (G0 = W^dagger W, G1 = P^dagger W + W^dagger P), below both pass through
+// P^dagger . P like the operator itself; the operator at this mass is G0, at others their
+// combination.  Three products (at this mass, at 0 and at 1) took 2.3 of an 18.7 ms set-up.
 void galerkin_next(mg_handle* h, int l) {
   Level& L = h->lv[l];
   Level& C = h->lv[l + 1];
+  if (h->p.remass_quadratic) {
+    if (l == 0) {
+      h->g_mass = h->mass;
+      ck(h, galerkin_fine(h->U64, 4.0 + h->mass, L.Vst64, h->Wbuf, C.G0, C.G1, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin G0");
+    } else {
+      ck(h, galerkin_coarse(L.G0, L.Vst64, C.G0, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin G0");
+      ck(h, galerkin_coarse(L.G1, L.Vst64, C.G1, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin G1");
+    }
+    combine_level(h, l + 1);
+    return;
+  }
   if (l == 0 && h->p.smooth_omega != 0.0)
     galerkin_smoothed(h);
   else if (l == 0)
-    ck(h, galerkin_fine(h->U64, 4.0 + h->mass, L.Vst64, h->Wbuf, C.A64, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin_fine");
+    ck(h, galerkin_fine(h->U64, 4.0 + h->mass, L.Vst64, h->Wbuf, C.A64, nullptr, L.Lx, L.Lt, L.bx, L.bt, L.Nv, h->s), "galerkin_fine");
   else
     ck(h, galerkin_coarse(L.A64, L.Vst64, C.A64, L.Lx, L.Lt, L.bx, L.bt, L.n, L.Nv, h->s), "galerkin_coarse");
   finish_level(h, l + 1);
@@ -1515,6 +1562,7 @@ void build_level(mg_handle* h, int l, const double2* noise, const void* Egiven) 
   const long long c = L.count();
   void* E = nullptr;
   void* T = nullptr;
+  void* scratch = nullptr;          // holds E and T
   if (!Egiven) {
     const double2* starts = noise;
     const double2* pw = noise + (size_t)L.Nv * c;
@@ -1524,12 +1572,13 @@ void build_level(mg_handle* h, int l, const double2* noise, const void* Egiven) 
     if (!(L.lambda_max > 0.0)) fail(h, MG_ERR_BREAKDOWN, "power iteration gave lambda_max <= 0");
     L.omega_relax = 1.0 / L.lambda_max;
     // Eq. relax: e <- (1 - omega A) e, nu sweeps, all Nv vectors at once
-    E = dalloc(h, (size_t)L.Nv * c * sizeof(double2));
-    T = dalloc(h, (size_t)L.Nv * c * sizeof(double2));
+    E = dalloc(h, 2 * (size_t)L.Nv * c * sizeof(double2));
+    T = (double2*)E + (size_t)L.Nv * c;
+    scratch = E;
     ck(h, cudaMemcpyAsync(E, starts, (size_t)L.Nv * c * sizeof(double2), cudaMemcpyDeviceToDevice, h->s), "copy");
     for (int sw = 0; sw < h->p.setup_sweeps; ++sw) {
-      apply_level<double>(h, l, E, T, L.Nv, W_F64);
-      ck(h, axpby<double>(-L.omega_relax, T, 1.0, E, c, L.Nv, h->s), "relax");
+      apply_level<double>(h, l, E, T, L.Nv, W_F64, ep_lincomb(-L.omega_relax, E, 1.0));
+      std::swap(E, T);
     }
   }
   // chirality split + block Gram-Schmidt (FP64)
@@ -1545,13 +1594,7 @@ void build_level(mg_handle* h, int l, const double2* noise, const void* Egiven) 
   // Galerkin operator of the next level (needed before relaxing on it)
   galerkin_next(h, l);
   sync(h);
-  if (E) {
-    for (auto& a : h->allocs)
-      if (a == E || a == T) a = nullptr;
-    cudaFree(E);
-    cudaFree(T);
-    h->bytes -= 2LL * L.Nv * c * (long long)sizeof(double2);
-  }
+  if (scratch) dfree(h, scratch, 2 * (size_t)L.Nv * c * sizeof(double2));
 }
 
 // Autotuning of the fused fine A for this handle's launches (FP32 and FP64,
@@ -1741,7 +1784,7 @@ mg_status refine_core(mg_handle* src, int lr, const void* e0, int ncycles, const
   st = guarded(h, [&]() {
     set_geometry(h);
     init_runtime(h);
-    allocate_storage(h);
+    allocate_handle(h);
     const long long V = h->lv[0].V;
     auto copy = [&](void* d, const void* sp, size_t bytes) {
       ck(h, cudaMemcpyAsync(d, sp, bytes, cudaMemcpyDeviceToDevice, h->s), "refine copy");
@@ -1770,7 +1813,7 @@ mg_status refine_core(mg_handle* src, int lr, const void* e0, int ncycles, const
         pos += (size_t)(L.Nv + 2) * L.count();
       }
     }
-    set_mass_internal(h, src->mass);
+    finish_setup(h);
   });
   cudaFree(E);
   if (st != MG_OK) {
@@ -1855,7 +1898,7 @@ mg_status mg_setup(const void* gauge, double mass, const mg_params* params, void
     const mg_params& P = h->p;
     set_geometry(h);
     init_runtime(h);
-    allocate_storage(h);
+    allocate_handle(h);
     // links
     const long long V = h->lv[0].V;
     ck(h, link_unitarity(gauge, 2 * V, slot(h, S_T0), h->s), "unitarity");
@@ -1871,7 +1914,7 @@ mg_status mg_setup(const void* gauge, double mass, const mg_params* params, void
       build_level(h, l, noise + pos, nullptr);
       pos += (size_t)(h->lv[l].Nv + 2) * h->lv[l].count();
     }
-    set_mass_internal(h, mass);
+    finish_setup(h);
     // adaptive passes (Sec. 3), each replacing the hierarchy in place
     std::vector<double> rhos;
     const int np = refine_count(params);
@@ -1958,7 +2001,7 @@ mg_status mg_clone(const mg_handle* src, double mass, void* stream, mg_handle** 
   mg_status st = guarded(h, [&]() {
     set_geometry(h);
     init_runtime(h);
-    allocate_storage(h);
+    allocate_handle(h);
     const long long V = h->lv[0].V;
     auto copy = [&](void* d, const void* sp, size_t bytes) {
       ck(h, cudaMemcpyAsync(d, sp, bytes, cudaMemcpyDeviceToDevice, h->s), "clone copy");
@@ -1984,6 +2027,7 @@ mg_status mg_clone(const mg_handle* src, double mass, void* stream, mg_handle** 
         copy(h->lv[l].G1, src->lv[l].G1, ab);
       }
       h->g_built = true;
+      h->g_mass = src->g_mass;
     }
     set_mass_internal(h, mass);
   });
