@@ -178,7 +178,8 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
   }
 }
 
-// Register-streaming A = D^dagger D for large lattices.  A warp owns a strip
+// Register-streaming A = D^dagger D on FP64 vectors for large lattices (masses the integer
+// kernel does not take).  A warp owns a strip
 // of 32 consecutive x sites (lanes 2..29 produce output, lanes 0, 1, 30, 31
 // are halo) and marches along t over SROWS output rows, keeping three rows of
 // psi, two rows of D psi and the needed link rows in registers; x neighbours
@@ -231,12 +232,12 @@ __device__ __forceinline__ void dslash_row(cplx_t<R> f0, cplx_t<R> f1, cplx_t<R>
 // shared memory (cp.async), SNB - 1 iterations ahead of use.
 static constexpr int SNB = 4;
 
-template <typename R>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 3) k_wilson_A_stream(
-    const cplx_t<R>* __restrict__ in, cplx_t<R>* out, const cplx_t<R>* __restrict__ U, R diag,
-    int Lx, int Lt, Epilogue ep) {
-  using C = cplx_t<R>;
-  using S = typename spinor_t<R>::type;
+__global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __restrict__ in, double2* out,
+                                                           const double2* __restrict__ U, double diag,
+                                                           int Lx, int Lt, Epilogue ep) {
+  using R = double;
+  using C = double2;
+  using S = double4_32a;
   __shared__ S ring_psi[4][SNB][32];           // [warp][slot][lane]
   __shared__ C ring_u[4][SNB][32][2];
   const int V = Lx * Lt;
@@ -266,15 +267,11 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 3) k_wilson_A_stream
       const int slot = (r - t0 + 1 + SNB) % SNB;
       const C* ps = in + off + 2LL * (x + Lx * wrap(r + 2, Lt));
       char* dst = (char*)&ring_psi[wl][slot][lane];
-      if (sizeof(S) == 16) {
-        cp_async(dst, ps, 16);
-      } else {
-        cp_async(dst, ps, 16);
-        cp_async(dst + 16, ps + 1, 16);
-      }
+      cp_async(dst, ps, 16);
+      cp_async(dst + 16, ps + 1, 16);
       const int g = x + Lx * wrap(r + 1, Lt);
-      cp_async(&ring_u[wl][slot][lane][0], U + g, (int)sizeof(C));
-      cp_async(&ring_u[wl][slot][lane][1], U + V + g, (int)sizeof(C));
+      cp_async(&ring_u[wl][slot][lane][0], U + g, 16);
+      cp_async(&ring_u[wl][slot][lane][1], U + V + g, 16);
     }
     cp_commit();
   };
@@ -335,10 +332,196 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 7 : 3) k_wilson_A_stream
   cp_wait<0>();
 }
 
-// The streaming kernel serves lattices with enough strips to fill the GPU.
-bool wilson_A_streamed(int Lx, int Lt) {
+// Register-streaming A on FP32 vectors, two sites per lane.  Both sites of a lane go through
+// every operation together as packed pairs (fma.rn.f32x2: one issue slot for two FMAs), so a
+// row step takes 40 packed operations for two sites where k_wilson_A_stream takes 88, and
+// only one shuffle per component and direction; a warp owns 64 sites of a row, 60 of them
+// outputs.  Computed as -2 D and -2 D^dagger (r = -2 diag psi + sum of hops), the factor 4
+// removed with the epilogue's scale: powers of two, so nothing rounds differently.  The
+// t-backward product of a row is formed when the row is current and carried.  Bound by FMA
+// issue (72% of the heavy pipe) and HBM: 4096^2 128 us (0.93 of the copy bandwidth; 144 us with
+// one site per lane), 1024^2 x 16 119 (146), 256^2 x 64 40 (68 with tiles).
+using P2 = unsigned long long;                       // two floats, low = first site
+
+__device__ __forceinline__ P2 p2(float a, float b) {
+  P2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float lo(P2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return a;
+}
+__device__ __forceinline__ float hi(P2 v) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+  return b;
+}
+__device__ __forceinline__ P2 fma2(P2 a, P2 b, P2 c) {
+  P2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ P2 mul2(P2 a, P2 b) {
+  P2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ P2 add2(P2 a, P2 b) {
+  P2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ P2 sub2(P2 a, P2 b) { return fma2(b, 0xBF800000BF800000ull, a); }
+
+struct C2 { P2 x, y; };                              // complex numbers of two sites
+struct S2 { C2 a, b; };                              // their spinors
+struct L2 { P2 x, y, n; };                           // their links: re, im, -im
+
+__device__ __forceinline__ C2 add2(C2 a, C2 b) { return {add2(a.x, b.x), add2(a.y, b.y)}; }
+__device__ __forceinline__ C2 sub2(C2 a, C2 b) { return {sub2(a.x, b.x), sub2(a.y, b.y)}; }
+__device__ __forceinline__ C2 mul2(const L2& u, C2 h) {
+  return {fma2(u.n, h.y, mul2(u.x, h.x)), fma2(u.y, h.x, mul2(u.x, h.y))};
+}
+__device__ __forceinline__ C2 mulc2(const L2& u, C2 h) {   // conj(u) h
+  return {fma2(u.y, h.y, mul2(u.x, h.x)), fma2(u.n, h.x, mul2(u.x, h.y))};
+}
+__device__ __forceinline__ S2 spinors(float4 p, float4 q) {
+  return {{p2(p.x, q.x), p2(p.y, q.y)}, {p2(p.z, q.z), p2(p.w, q.w)}};
+}
+__device__ __forceinline__ L2 links(float4 u) {
+  const P2 y = p2(u.y, u.w);
+  return {p2(u.x, u.z), y, y ^ 0x8000000080000000ull};
+}
+// f0 + i s f1
+template <int S>
+__device__ __forceinline__ C2 proj_t(const S2& f) {
+  return S > 0 ? C2{sub2(f.a.x, f.b.y), add2(f.a.y, f.b.x)} : C2{add2(f.a.x, f.b.y), sub2(f.a.y, f.b.x)};
+}
+// the pair one site to the right / left of each site's value
+__device__ __forceinline__ P2 from_right(P2 v) { return p2(hi(v), __shfl_down_sync(0xffffffffu, lo(v), 1)); }
+__device__ __forceinline__ P2 from_left(P2 v) { return p2(__shfl_up_sync(0xffffffffu, hi(v), 1), lo(v)); }
+
+// -2 D (S = 1) or -2 D^dagger (S = -1) of one row; f the row, up the next one, tb the
+// t-backward product, m2d = -2 diag.
+template <int S>
+__device__ __forceinline__ S2 row2(const S2& f, const S2& up, const L2& ux, const L2& ut, C2 tb, P2 m2d) {
+  const C2 q = S > 0 ? sub2(f.a, f.b) : add2(f.a, f.b);
+  const C2 g = mulc2(ux, S > 0 ? add2(f.a, f.b) : sub2(f.a, f.b));
+  const C2 X = mul2(ux, C2{from_right(q.x), from_right(q.y)});
+  const C2 Y = {from_left(g.x), from_left(g.y)};
+  const C2 Z = mul2(ut, proj_t<S>(up));
+  const C2 s = add2(add2(add2(X, Y), Z), tb);
+  const C2 d = S > 0 ? sub2(Y, X) : sub2(X, Y), e = S > 0 ? sub2(Z, tb) : sub2(tb, Z);
+  return {{fma2(m2d, f.a.x, s.x), fma2(m2d, f.a.y, s.y)},
+          {fma2(m2d, f.b.x, add2(d.x, e.y)), fma2(m2d, f.b.y, sub2(d.y, e.x))}};
+}
+
+static constexpr int SOUT2 = 60;           // output sites per warp
+
+__global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __restrict__ in, float2* out,
+                                                             const float2* __restrict__ U, float diag,
+                                                             int Lx, int Lt, int rows, Epilogue ep) {
+  __shared__ float4 ring_psi[4][SNB][2][32];           // [warp][slot][site][lane]
+  __shared__ float4 ring_u[4][SNB][2][32];             // [warp][slot][direction][lane]
+  const int V = Lx * Lt;
+  const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+  const int strips = (Lx + SOUT2 - 1) / SOUT2, row_blocks = (Lt + rows - 1) / rows;
+  const int w = blockIdx.x * 4 + wl;
+  if (w >= strips * row_blocks) return;                // whole warp
+  const int strip = w % strips, t0 = (w / strips) * rows, t1 = min(t0 + rows, Lt);
+  const int xu = strip * SOUT2 - 2 + 2 * lane;
+  const int x = min(wrap(xu, Lx), Lx - 2);             // Lx is even: both sites wrap together
+  const bool writer = lane >= 1 && lane < 31 && xu < Lx;
+  const long long off = (long long)blockIdx.y * V * 2;
+  const float2* col = in + off + 2 * x;
+  auto issue = [&](int r) {                            // psi(r + 2) and links(r + 1) for step r
+    if (r < t1) {
+      const int slot = (r - t0 + 1 + SNB) % SNB;
+      const float2* ps = col + 2LL * Lx * wrap(r + 2, Lt);
+      cp_async(&ring_psi[wl][slot][0][lane], ps, 16);
+      cp_async(&ring_psi[wl][slot][1][lane], ps + 2, 16);
+      const float2* pu = U + x + Lx * wrap(r + 1, Lt);
+      cp_async(&ring_u[wl][slot][0][lane], pu, 16);
+      cp_async(&ring_u[wl][slot][1][lane], pu + V, 16);
+    }
+    cp_commit();
+  };
+  auto ld_psi = [&](int t) {
+    const float4* p = (const float4*)(col + 2LL * Lx * wrap(t, Lt));
+    return spinors(p[0], p[1]);
+  };
+  auto ld_u = [&](int mu, int t) { return links(*(const float4*)(U + mu * V + x + Lx * wrap(t, Lt))); };
+  for (int k = 0; k < SNB - 1; ++k) issue(t0 - 1 + k);
+  const P2 m2d = p2(-2.f * diag, -2.f * diag);
+  C2 tb = mulc2(ld_u(1, t0 - 2), proj_t<-1>(ld_psi(t0 - 2)));
+  S2 pc = ld_psi(t0 - 1), pp = ld_psi(t0), dc = {{0, 0}, {0, 0}};
+  L2 ux = ld_u(0, t0 - 1), ut = ld_u(1, t0 - 1), uxo = {0, 0, 0}, uto = {0, 0, 0};
+  C2 db = {0, 0};
+  const float ca = 0.25f * (float)ep.ca, cu = (float)ep.cu, cw = (float)ep.cw;
+  const float2 *EU = (const float2*)ep.U, *EW = (const float2*)ep.W;
+#pragma unroll 2                                       // the row window rotates by renaming
+  for (int r = t0 - 1; r <= t1; ++r) {
+    const S2 e = row2<1>(pc, pp, ux, ut, tb, m2d);     // -2 D psi at row r
+    if (r > t0) {                                      // output row r - 1
+      const S2 y = row2<-1>(dc, e, uxo, uto, db, m2d);
+      if (writer) {
+        const long long g = off + 2LL * (x + Lx * (r - 1));
+        const P2 c = p2(ca, ca);
+        S2 o = {{mul2(c, y.a.x), mul2(c, y.a.y)}, {mul2(c, y.b.x), mul2(c, y.b.y)}};
+        auto axpy = [&](float k, const float2* v) {
+          const float4* p = (const float4*)(v + g);
+          const S2 u = spinors(p[0], p[1]);
+          const P2 kk = p2(k, k);
+          o = {{fma2(kk, u.a.x, o.a.x), fma2(kk, u.a.y, o.a.y)}, {fma2(kk, u.b.x, o.b.x), fma2(kk, u.b.y, o.b.y)}};
+        };
+        if (EU) axpy(cu, EU);
+        if (EW) axpy(cw, EW);
+        float4* po = (float4*)(out + g);
+        po[0] = make_float4(lo(o.a.x), lo(o.a.y), lo(o.b.x), lo(o.b.y));
+        po[1] = make_float4(hi(o.a.x), hi(o.a.y), hi(o.b.x), hi(o.b.y));
+      }
+    }
+    db = mulc2(uto, proj_t<1>(dc));                    // into D^dagger's row r
+    tb = mulc2(ut, proj_t<-1>(pc));                    // into D's row r + 1
+    dc = e;
+    uxo = ux;
+    uto = ut;
+    pc = pp;
+    if (r < t1) {                                      // psi(r + 2), links(r + 1)
+      cp_wait<SNB - 2>();
+      const int slot = (r - t0 + 1 + SNB) % SNB;
+      pp = spinors(ring_psi[wl][slot][0][lane], ring_psi[wl][slot][1][lane]);
+      ux = links(ring_u[wl][slot][0][lane]);
+      ut = links(ring_u[wl][slot][1][lane]);
+    }
+    issue(r + SNB - 1);
+  }
+  cp_wait<0>();
+}
+
+// The FP64 streaming kernel serves lattices with enough strips to fill the GPU.
+static bool streamed64(int Lx, int Lt) {
   const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
   return Lx >= 64 && Lt >= 2 * SROWS && warps >= 4LL * 152;
+}
+
+// The FP32 one: launches with 12 warps per SM at 8 rows each (at 256^2 x 16 it takes 16.4 us
+// against 18.6 with tiles, at 512^2 x 4 14.1 against 18.5, at 512^2 8.2 against 8.3), then the
+// most rows per warp that leave two rounds of 16 warps per SM: more rows repeat less of the
+// 4-row halo (1024^2 x 16: 133, 121, 119 us with 8, 16, 32), fewer fill the GPU (256^2 x 64:
+// 41, 40, 43 us).
+static long long stream32_warps(int Lx, int Lt, int nrhs, int rows) {
+  return (long long)((Lx + SOUT2 - 1) / SOUT2) * ((Lt + rows - 1) / rows) * nrhs;
+}
+static bool streamed32(int Lx, int Lt, int nrhs) {
+  return Lx >= 64 && Lt >= 16 && stream32_warps(Lx, Lt, nrhs, 8) >= 12LL * 152;
+}
+static int stream32_rows(int Lx, int Lt, int nrhs) {
+  int rows = 32;
+  while (rows > 8 && stream32_warps(Lx, Lt, nrhs, rows) < 2LL * 16 * 152) rows /= 2;
+  return rows;
 }
 
 // Tile choice of the fused kernel: 32 x 8 (FP64) or 32 x 16 (FP32) when that
@@ -378,7 +561,7 @@ static const int WV_SHAPE[WV_COUNT][3] = {{0, 0, 0}, {16, 8, 1}, {32, 8, 1}, {32
 template <typename R>
 static int wilson_default_variant(int Lx, int Lt, int nrhs, bool dot) {
   const bool f64 = sizeof(R) == 8;
-  if (!dot && wilson_A_streamed(Lx, Lt)) return WV_STREAM;
+  if (!dot && (f64 ? streamed64(Lx, Lt) : streamed32(Lx, Lt, nrhs))) return WV_STREAM;
   const long long tiles = (long long)((Lx + 31) / 32) * ((Lt + (f64 ? 7 : 15)) / (f64 ? 8 : 16));
   const bool big = tiles * (dot ? nrhs : 1) >= 2 * 152;
   if (!big) return WV_16x8;
@@ -408,9 +591,9 @@ bool wilson_A_dot_fits(int Lx, int Lt, bool f64, double diag) {
 }
 
 template <typename R>
-static bool wilson_variant_ok(int v, int Lx, int Lt, bool fx) {
+static bool wilson_variant_ok(int v, int Lx, int Lt, int nrhs, bool fx) {
   if (fx) return v == WV_16x8 || v == WV_32x8 || v == WV_32x8x2;
-  if (v == WV_STREAM) return wilson_A_streamed(Lx, Lt);
+  if (v == WV_STREAM) return sizeof(R) == 8 ? streamed64(Lx, Lt) : streamed32(Lx, Lt, nrhs);
   if (sizeof(R) == 8 && (v == WV_32x8x2 || v == WV_64x4x2)) return false;   // shared memory
   return true;
 }
@@ -425,9 +608,16 @@ static cudaError_t launch_variant(int v, const void* in, void* out, const void* 
                        nrhs, ep, s);
   switch (v) {
     case WV_STREAM: {
-      const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
-      k_wilson_A_stream<R><<<dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s>>>(
-          (const cplx_t<R>*)in, (cplx_t<R>*)out, (const cplx_t<R>*)U, (R)diag, Lx, Lt, ep);
+      if constexpr (sizeof(R) == 4) {
+        const int rows = stream32_rows(Lx, Lt, nrhs);
+        const long long warps = stream32_warps(Lx, Lt, 1, rows);
+        k_wilson_A_stream2<<<dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s>>>(
+            (const float2*)in, (float2*)out, (const float2*)U, (float)diag, Lx, Lt, rows, ep);
+      } else {
+        const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
+        k_wilson_A_stream<<<dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s>>>(
+            (const double2*)in, (double2*)out, (const double2*)U, diag, Lx, Lt, ep);
+      }
       break;
     }
     case WV_16x8: launch_wilson_A<R, 16, 8, 1>(in, out, U, diag, Lx, Lt, nrhs, ep, s); break;
@@ -490,7 +680,7 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
   float best = 0.f;
   launch_variant<R>(def, in, ref, U, W, diag, Lx, Lt, nrhs, none, s);
   for (int v = 0; v < WV_COUNT; ++v) {
-    if (!wilson_variant_ok<R>(v, Lx, Lt, W != nullptr)) continue;
+    if (!wilson_variant_ok<R>(v, Lx, Lt, nrhs, W != nullptr)) continue;
     ++t.tried;
     launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     int diff = 0;
