@@ -18,8 +18,8 @@
 // accumulation); the blocks are the stored BF16 copy of the operator, so only
 // they round.
 //
-// Sliding window.  A CTA walks strips of consecutive sites along x (one
-// row t, up to SL sites).  The X operand is staged per coarse site as a
+// Sliding window.  A CTA walks its share of the sites in strips of consecutive
+// sites along x (one row t).  The X operand is staged per coarse site as a
 // block of 128 rows x 2n (the hi / lo rows of 64 right-hand sides, Re and Im
 // halves along K), K-major without swizzle (8 rows x 16 bytes per core
 // matrix).  A ring of NCOL columns x 3 rows of blocks holds the neighbourhood
@@ -32,8 +32,8 @@
 // row is 128 bytes, so that the conversion reads are free of bank conflicts)
 // and one bulk copy of the blocks, all completing on the slot's mbarrier.
 //
-// Roles, synchronised through mbarriers only: warps 0-7 convert and write
-// outputs, warp 8 issues the MMAs, warp 9 issues the loads.  The loader fills
+// Roles, synchronised through mbarriers only: warps 0-7 convert, warp 8 issues the
+// MMAs, warp 9 issues the loads, warps 10-13 write the outputs.  The loader fills
 // raw slot q % R with load q once the converting threads have released the
 // slot's previous load (empty[q % R]); the load completes rawbar[q % R].
 // When a site's operands are in place the 256 converting threads arrive on
@@ -41,10 +41,17 @@
 // K-steps into accumulator g % 2 of tensor memory (each K-step reading its
 // neighbour's staged block through its own descriptor) and commits them to
 // done[g % 2].  The converting threads wait on done before they overwrite a
-// ring slot or B buffer the MMAs may still read, and before they read an
-// accumulator (tcgen05.ld) to write the outputs.  Every wait is bounded: one
+// ring slot or B buffer the MMAs may still read.  The output warps load their
+// epilogue operands, wait on done, read the accumulator (tcgen05.ld), release it
+// through accfree[g % 2] (which warp 8 awaits before site g + 2) and store; with the
+// outputs written by the converting warps, conversion and output of a site ran one
+// after the other.  4096 sites of 16 dof, 64 right-hand sides: 58 -> 55 us, in the V-cycle
+// (whose epilogue operands are then loaded ahead) 8% of the batched solve; 47 us with even
+// shares of sites.  Every wait is bounded: one
 // that runs out sets the flag read by coarse_tc_take_error, and the CTA
 // frees its tensor memory and returns.
+#include <algorithm>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -73,7 +80,8 @@ struct CoarseTC {
   static constexpr int FIXED = 2 * (3 * NCOL * XBLK + NB * BELEM);   // operand bytes
   static constexpr int TCOLS = 2 * NC <= 64 ? 64 : 128;  // tensor-memory columns (2 accumulators)
   static constexpr int PRODUCERS = 256;                  // warps 0-7
-  static constexpr int THREADS = PRODUCERS + 64;         // + the MMA warp and the load warp
+  static constexpr int WRITERS = 128;                    // warps 10-13
+  static constexpr int THREADS = PRODUCERS + 64 + WRITERS;   // + the MMA warp and the load warp
   static constexpr int C8 = n / 8;                       // 8-column groups of a block row
   static constexpr int P = n / 2;                        // 16-byte chunks per raw X row
   static constexpr bool SWZ = n == 16;                   // raw X rows of 128 bytes, swizzled
@@ -131,20 +139,21 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* m) {
 }
 
 template <int NDOF>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(448, 1)
     k_coarse_apply_tc(const __grid_constant__ CUtensorMap xmap, float2* out,
-                      const __nv_bfloat162* __restrict__ A, int Lx, int Lt, int nrhs, int SL,
-                      int R, Epilogue ep) {
+                      const __nv_bfloat162* __restrict__ A, int Lx, int Lt, int nrhs, int R,
+                      Epilogue ep) {
   using C = CoarseTC<NDOF>;
   constexpr int n = C::n, KB = C::KB, KA = C::KA, C8 = C::C8, P = C::P, NCOL = C::NCOL;
   extern __shared__ __align__(16) unsigned char dyn[];
-  __shared__ __align__(8) uint64_t full[2], done[2], rawbar[4], empty[4];
+  __shared__ __align__(8) uint64_t full[2], done[2], accfree[2], rawbar[4], empty[4];
   __shared__ uint32_t tmem_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int V = Lx * Lt;
   const int NR = (nrhs + 7) & ~7;                        // raw rows per column row
-  const int spr = (Lx + SL - 1) / SL;                    // strips per row
-  const int NS = spr * Lt;
+  // this CTA's sites, in row order; a strip is the part of them within one row
+  const int p0 = (int)((long long)V * blockIdx.x / gridDim.x);
+  const int p1 = (int)((long long)V * (blockIdx.x + 1) / gridDim.x);
   unsigned char* xs = dyn + ((1024u - (tc::saddr(dyn) & 1023u)) & 1023u);
   unsigned char* bs = xs + 2 * 3 * NCOL * C::XBLK;       // NB B buffers
   unsigned char* raw = bs + 2 * C::NB * C::BELEM;        // R raw slots
@@ -158,6 +167,8 @@ __global__ void __launch_bounds__(320, 1)
     tc::mbar_init(&full[1], C::PRODUCERS);
     tc::mbar_init(&done[0], 1);
     tc::mbar_init(&done[1], 1);
+    tc::mbar_init(&accfree[0], C::WRITERS);
+    tc::mbar_init(&accfree[1], C::WRITERS);
     for (int q = 0; q < 4; ++q) {
       tc::mbar_init(&rawbar[q], 1);
       tc::mbar_init(&empty[q], C::PRODUCERS);
@@ -173,10 +184,12 @@ __global__ void __launch_bounds__(320, 1)
   if (warp == 8) {
     // ---- MMA warp: the sites of this CTA in order
     int g = 0;
-    for (int sidx = blockIdx.x; sidx < NS && ok; sidx += gridDim.x) {
-      const int len = min(SL, Lx - (sidx % spr) * SL);
+    for (int p = p0, len; p < p1 && ok; p += len) {
+      len = min(Lx - p % Lx, p1 - p);
       for (int i = 0; i < len; ++i, ++g) {
         ok = tc::mbar_wait(&full[g & 1], (uint32_t)((g >> 1) & 1), &g_coarse_tc_err);
+        if (ok && g >= 2)            // the accumulator of site g - 2 has been read
+          ok = tc::mbar_wait(&accfree[g & 1], (uint32_t)((g / 2 - 1) & 1), &g_coarse_tc_err);
         if (!ok) break;
         if (lane == 0) {
           tc::fence_after_sync();
@@ -204,9 +217,9 @@ __global__ void __launch_bounds__(320, 1)
     // the blocks of site x0 + k - 2.  Load q uses raw slot q % R.
     if (lane == 0) {
       int q = 0;
-      for (int sidx = blockIdx.x; sidx < NS && ok; sidx += gridDim.x) {
-        const int t = sidx / spr, x0 = (sidx % spr) * SL;
-        const int len = min(SL, Lx - x0);
+      for (int p = p0, len; p < p1 && ok; p += len) {
+        const int t = p / Lx, x0 = p % Lx;
+        len = min(Lx - x0, p1 - p);
         for (int k = 0; k < len + 2; ++k, ++q) {
           const int slot = q % R;
           if (q >= R) {              // the converting threads are done with load q - R
@@ -230,6 +243,66 @@ __global__ void __launch_bounds__(320, 1)
       }
     }
     __syncwarp();
+  } else if (warp >= 10) {
+    // ---- output warps: warp w reads rows 32 (w % 4) .. + 31 of the accumulators, the
+    // (hi, lo) rows of 16 right-hand sides; of a pair's n outputs the even lane writes
+    // the first half, the odd lane the second
+    constexpr int H = n / 2;
+    const int qd = warp & 3, r = 16 * qd + (lane >> 1), half = lane & 1;
+    const float ca = (float)ep.ca, cu = (float)ep.cu, cw = (float)ep.cw;
+    int g = 0;
+    for (int p = p0, len; p < p1 && ok; p += len) {
+      const int t = p / Lx, x0 = p % Lx;
+      len = min(Lx - x0, p1 - p);
+      for (int i = 0; i < len; ++i, ++g) {
+        const long long o = ((long long)r * V + x0 + i + Lx * t) * n + half * H;
+        float4 y[H / 2];
+#pragma unroll
+        for (int q = 0; q < H / 2; ++q) y[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < nrhs) {
+          if (ep.U) {
+#pragma unroll
+            for (int q = 0; q < H / 2; ++q) {
+              const float4 w = *(const float4*)((const float2*)ep.U + o + 2 * q);
+              y[q] = make_float4(cu * w.x, cu * w.y, cu * w.z, cu * w.w);
+            }
+          }
+          if (ep.W) {
+#pragma unroll
+            for (int q = 0; q < H / 2; ++q) {
+              const float4 w = *(const float4*)((const float2*)ep.W + o + 2 * q);
+              y[q] = make_float4(y[q].x + cw * w.x, y[q].y + cw * w.y, y[q].z + cw * w.z, y[q].w + cw * w.w);
+            }
+          }
+        }
+        ok = tc::mbar_wait(&done[g & 1], (uint32_t)((g >> 1) & 1), &g_coarse_tc_err);
+        if (!ok) break;
+        tc::fence_after_sync();
+        const uint32_t tb = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)((g & 1) * C::NC);
+        float vre[n], vim[n];
+#pragma unroll
+        for (int q = 0; q < n; q += 8) {
+          tc::tmem_ld8(tb + q, vre + q);
+          tc::tmem_ld8(tb + n + q, vim + q);
+        }
+        tc::tmem_wait_ld();
+        tc::fence_before_sync();
+        mbar_arrive(&accfree[g & 1]);
+#pragma unroll
+        for (int q = 0; q < H; ++q) {  // hi + lo of this lane's half; the other half goes to the partner
+          const float sr = half ? vre[q] : vre[H + q], si = half ? vim[q] : vim[H + q];
+          vre[q] = (half ? vre[H + q] : vre[q]) + __shfl_xor_sync(0xffffffffu, sr, 1);
+          vim[q] = (half ? vim[H + q] : vim[q]) + __shfl_xor_sync(0xffffffffu, si, 1);
+        }
+        if (r < nrhs) {
+#pragma unroll
+          for (int q = 0; q < H / 2; ++q)
+            *(float4*)(out + o + 2 * q) =
+                make_float4(y[q].x + ca * vre[2 * q], y[q].y + ca * vim[2 * q],
+                            y[q].z + ca * vre[2 * q + 1], y[q].w + ca * vim[2 * q + 1]);
+        }
+      }
+    }
   } else {
     // conversion of a raw column into ring column `slot`.  X item e: r = 4 (..)
     // + (e & 3), combo = (tr, 8-column group); lanes 4k..4k+3 write the high
@@ -299,59 +372,15 @@ __global__ void __launch_bounds__(320, 1)
         *(uint4*)(p + lower + n * 16) = make_uint4(re[0], re[1], re[2], re[3]);
       }
     };
-    // outputs of site j from accumulator buf (its MMAs have completed)
-    auto epilogue = [&](int j, int buf) {
-      tc::fence_after_sync();
-      constexpr int H = n / 2;                     // block rows of this warp's half
-      const int qd = warp & 3, hh = warp >> 2;
-      const uint32_t tb = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(buf * C::NC + hh * H);
-      float vre[H], vim[H];
-      tc::tmem_ld8(tb, vre);
-      tc::tmem_ld8(tb + n, vim);
-      if constexpr (H == 12) {
-        tc::tmem_ld4(tb + 8, vre + 8);
-        tc::tmem_ld4(tb + n + 8, vim + 8);
-      }
-      tc::tmem_wait_ld();
-      tc::fence_before_sync();
-#pragma unroll
-      for (int i = 0; i < H; ++i) {
-        vre[i] += __shfl_xor_sync(0xffffffffu, vre[i], 1);   // hi + lo rows
-        vim[i] += __shfl_xor_sync(0xffffffffu, vim[i], 1);
-      }
-      // the even lane writes the first half of the row's H outputs, the odd lane the second
-      const int r = 16 * qd + (lane >> 1), half = lane & 1;
-      if (r < nrhs) {
-        const long long o = ((long long)r * V + j) * n + hh * H + half * (H / 2);
-        const float ca = (float)ep.ca, cu = (float)ep.cu, cw = (float)ep.cw;
-#pragma unroll
-        for (int i = 0; i < H / 2; i += 2) {      // two complex outputs per 16-byte store
-          float4 y;
-          y.x = ca * (half ? vre[H / 2 + i] : vre[i]);
-          y.y = ca * (half ? vim[H / 2 + i] : vim[i]);
-          y.z = ca * (half ? vre[H / 2 + i + 1] : vre[i + 1]);
-          y.w = ca * (half ? vim[H / 2 + i + 1] : vim[i + 1]);
-          if (ep.U) {
-            const float4 w = *(const float4*)((const float2*)ep.U + o + i);
-            y.x += cu * w.x; y.y += cu * w.y; y.z += cu * w.z; y.w += cu * w.w;
-          }
-          if (ep.W) {
-            const float4 w = *(const float4*)((const float2*)ep.W + o + i);
-            y.x += cw * w.x; y.y += cw * w.y; y.z += cw * w.z; y.w += cw * w.w;
-          }
-          *(float4*)(out + o + i) = y;
-        }
-      }
-    };
     auto wait_done = [&](int site) -> bool {
       return tc::mbar_wait(&done[site & 1], (uint32_t)((site >> 1) & 1), &g_coarse_tc_err);
     };
 
     int g = 0;                     // sites handed to the MMA warp; site g uses accumulator g & 1
     int q = 0;                     // loads consumed
-    for (int sidx = blockIdx.x; sidx < NS && ok; sidx += gridDim.x) {
-      const int t = sidx / spr, x0 = (sidx % spr) * SL;
-      const int len = min(SL, Lx - x0);
+    for (int p = p0, len; p < p1 && ok; p += len) {
+      const int t = p / Lx, x0 = p % Lx;
+      len = min(Lx - x0, p1 - p);
       for (int k = 0; k < len + 2; ++k, ++q) {
         // the MMAs that may still read the ring slot (and B buffer) about to be
         // replaced: at a strip's first load every earlier site, then the site
@@ -369,16 +398,7 @@ __global__ void __launch_bounds__(320, 1)
           tc::fence_proxy_async();
           mbar_arrive(&full[g & 1]);   // operands of site g in place
         }
-        if (k >= 3) {                // outputs of the previous site of this strip
-          ok = wait_done(g - 1);
-          if (!ok) break;
-          epilogue(x0 + k - 3 + Lx * t, (g - 1) & 1);
-        }
         if (k >= 2) ++g;
-      }
-      if (ok && len > 0) {           // the strip's last site
-        ok = wait_done(g - 1);
-        if (ok) epilogue(x0 + len - 1 + Lx * t, (g - 1) & 1);
       }
     }
   }
@@ -449,15 +469,12 @@ cudaError_t launch_tc(const void* in, void* out, const void* A, int Lx, int Lt, 
   R = R > 4 ? 4 : R;
   if (R < 1) return cudaErrorInvalidValue;
   const int smem = C::FIXED + R * C::raw_bytes(NR) + 1024;
-  // one CTA per SM; strips of SL sites, short enough that every CTA gets one, at most 8
-  int SL = (int)((V + sms - 1) / sms);
-  SL = SL < 2 ? 2 : (SL > 8 ? 8 : SL);
-  if (SL > Lx) SL = Lx;
-  const long long NS = (long long)((Lx + SL - 1) / SL) * Lt;
-  const int grid = (int)(NS < sms ? NS : sms);
-  k_coarse_apply_tc<NDOF><<<grid, C::THREADS, smem, s>>>(map, (float2*)out,
-                                                        (const __nv_bfloat162*)A, Lx, Lt, nrhs, SL,
-                                                        R, ep);
+  // one CTA per SM, an even share of the sites each, at least two (a strip loads two
+  // columns before its first site).  Strips of at most 8 sites dealt out in turn left a
+  // quarter of the SM time idle at 4096 sites (4 strips for some CTAs, 3 for others).
+  const int grid = (int)std::max(1LL, std::min((long long)sms, V / 2));
+  k_coarse_apply_tc<NDOF><<<grid, C::THREADS, smem, s>>>(map, (float2*)out, (const __nv_bfloat162*)A, Lx,
+                                                        Lt, nrhs, R, ep);
   count_launch();
   return cudaGetLastError();
 }

@@ -696,14 +696,20 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
     }
     if (diff) continue;                                    // not bit-identical: never used
     ++t.admitted;
+    // the best of three rounds of 20: one round of 10 is off by up to 40% on launches of 5 us
+    // (32 CTAs of 64 x 4 x 2 were once chosen for 128^2, 7.6 us against 5.7 in the solve)
+    constexpr int REPS = 20;
     for (int w = 0; w < 2; ++w) launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
-    constexpr int REPS = 10;
-    cudaEventRecord(e0, s);
-    for (int w = 0; w < REPS; ++w) launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
-    cudaEventRecord(e1, s);
-    cudaEventSynchronize(e1);
     float ms = 0.f;
-    cudaEventElapsedTime(&ms, e0, e1);
+    for (int round = 0; round < 3; ++round) {
+      cudaEventRecord(e0, s);
+      for (int w = 0; w < REPS; ++w) launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
+      cudaEventRecord(e1, s);
+      cudaEventSynchronize(e1);
+      float one = 0.f;
+      cudaEventElapsedTime(&one, e0, e1);
+      if (round == 0 || one < ms) ms = one;
+    }
     const double us = 1000.0 * ms / REPS;
     if (v == def) t.us_default = us;
     if (t.admitted == 1 || ms < best) {
