@@ -314,6 +314,15 @@ cudaError_t hermitian_gemv_f32(const void* P, const void* x, void* y, int N, int
 // products run on tensor cores from an FP32 copy of x held there.
 cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, int nrhs,
                                  void* part, cudaStream_t s, void* xscratch = nullptr);
+// FP32 copy xs [nrhs][ld] of x [nrhs][N], zero beyond N
+cudaError_t to_f32_padded(const void* x, void* xs, int N, int ld, int nrhs, cudaStream_t s);
+// The whole product for 16 to 64 vectors on tcgen05 (TF32 hi + lo operands, FP32
+// accumulation).  xscratch: nrhs * ld complex64; part as above; y32 as below.
+bool hermitian_gemv_tc_ok(int ld, int nrhs);
+cudaError_t hermitian_gemv_tc(const void* P, const void* x, void* y, int N, int ld, int nrhs,
+                              void* xscratch, void* part, bool accumulate, void* y32, cudaStream_t s);
+// *flag = 1 if a bounded wait of k_hgemv_tc ran out since the last call
+cudaError_t gemv_tc_take_error(int* flag);
 // hermitian_gemv_tiles for 1 to 4 vectors given in FP32 (x32, complex64
 // [nrhs][N]); the diagonal tiles also write the exact FP64 copy of x32 into
 // x64 (complex128 [nrhs][N]).

@@ -1612,7 +1612,8 @@ __device__ __forceinline__ void hgemv_mma_item(const float2* sT, const float2* s
       }
 }
 
-// Tensor-core variant for 16..64 right-hand sides: per stored tile T (64 x 64
+// Tensor-core variant for 16..64 right-hand sides on smaller levels (hermitian_gemv_tc_ok
+// has the line): per stored tile T (64 x 64
 // complex) the row products T X_J and, off the diagonal, the column products
 // T^H X_I, as realified GEMMs on mma.sync m16n8k8 TF32 with three products per
 // FP32-accurate product (the layout and fragment mapping of k_gj_update: A =
@@ -1891,15 +1892,20 @@ __global__ void __launch_bounds__(256) k_hgemv_reduce(const float2* __restrict__
   }
 }
 
+cudaError_t to_f32_padded(const void* x, void* xs, int N, int ld, int nrhs, cudaStream_t s) {
+  const long long n = (long long)ld * nrhs;
+  k_x32_pad<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)x, (float2*)xs, N, ld, nrhs);
+  count_launch();
+  return cudaGetLastError();
+}
+
 cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, int nrhs,
                                  void* part, cudaStream_t s, void* xscratch) {
   if (ld % HT || ld < N) return cudaErrorInvalidValue;
   const int nt = ld / HT, ntiles = nt * (nt + 1) / 2;
   if (nrhs >= 16 && nrhs <= 64 && xscratch) {   // tensor cores
-    const long long n = (long long)ld * nrhs;
-    k_x32_pad<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)x, (float2*)xscratch, N,
-                                                        ld, nrhs);
-    count_launch();
+    const cudaError_t e = to_f32_padded(x, xscratch, N, ld, nrhs, s);
+    if (e != cudaSuccess) return e;
     const size_t sm = (size_t)HT * (GJC + 2 * GJR) * sizeof(float2);
     static bool attr = false;
     if (!attr) {

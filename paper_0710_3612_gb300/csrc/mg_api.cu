@@ -292,6 +292,12 @@ void coarsest_solve64(mg_handle* h, const double2* b, double2* x, int steps, int
     return;
   }
   auto gemv = [&](const double2* in, bool accumulate, void* out32) {
+    if (hermitian_gemv_tc_ok(h->ldc, nrhs)) {
+      ProfScope pd(h, MG_KF_DENSE);
+      ck(h, hermitian_gemv_tc(h->Bpk, in, x, h->Nc, h->ldc, nrhs, h->gemv_x, h->gemv_part, accumulate,
+                              out32, h->s), "coarsest gemv");
+      return;
+    }
     {
       ProfScope pd(h, MG_KF_DENSE);
       if (in32 && in == b)
@@ -2219,6 +2225,12 @@ void check_device_waits(mg_handle* h) {
   if (flag) {
     h->poisoned = true;
     fail(h, MG_ERR_TIMEOUT, "tcgen05 coarse apply: a completion wait ran out (results invalid)");
+  }
+  if (h->R < 16) return;                               // smaller batches never take the kernel
+  ck(h, gemv_tc_take_error(&flag), "read the wait flag");
+  if (flag) {
+    h->poisoned = true;
+    fail(h, MG_ERR_TIMEOUT, "tcgen05 coarsest GEMV: a completion wait ran out (results invalid)");
   }
 }
 
