@@ -37,7 +37,8 @@ __device__ __forceinline__ double block_ratio(double num, double den) {
 template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT) k_dot(const cplx_t<R>* __restrict__ a,
                                             const cplx_t<R>* __restrict__ b, long long count,
-                                            double* ws, double* out) {
+                                            double* ws, double* out, int dependent) {
+  pdl_wait(dependent);
   constexpr int N = NORM ? 1 : 2;
   __shared__ double sh[N * RT];
   const int rhs = blockIdx.y;
@@ -67,7 +68,7 @@ cudaError_t dot(const void* a, const void* b, long long count, int nrhs, double*
                 double* out, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
   const int g = reduce_blocks(count, nrhs);
-  k_dot<R, false><<<dim3(g, nrhs), RT, 0, s>>>((const cplx_t<R>*)a, (const cplx_t<R>*)b, count,
+  launch_after(k_dot<R, false>, dim3(g, nrhs), RT, 0, s, (const cplx_t<R>*)a, (const cplx_t<R>*)b, count,
                                                partials, out);
   count_launch();
   return cudaGetLastError();
@@ -78,7 +79,7 @@ cudaError_t norm2(const void* a, long long count, int nrhs, double* partials, do
                   cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
   const int g = reduce_blocks(count, nrhs);
-  k_dot<R, true><<<dim3(g, nrhs), RT, 0, s>>>((const cplx_t<R>*)a, nullptr, count, partials, out);
+  launch_after(k_dot<R, true>, dim3(g, nrhs), RT, 0, s, (const cplx_t<R>*)a, nullptr, count, partials, out);
   count_launch();
   return cudaGetLastError();
 }
@@ -90,7 +91,8 @@ static inline dim3 grid1(long long count, int nrhs) {
 
 template <typename R>
 __global__ void k_axpby(R a, const cplx_t<R>* __restrict__ x, R b, cplx_t<R>* __restrict__ y,
-                        long long count) {
+                        long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   i += (long long)blockIdx.y * count;
@@ -101,14 +103,15 @@ __global__ void k_axpby(R a, const cplx_t<R>* __restrict__ x, R b, cplx_t<R>* __
 template <typename R>
 cudaError_t axpby(double a, const void* x, double b, void* y, long long count, int nrhs,
                   cudaStream_t s) {
-  k_axpby<R><<<grid1(count, nrhs), RT, 0, s>>>((R)a, (const cplx_t<R>*)x, (R)b, (cplx_t<R>*)y,
+  launch_after(k_axpby<R>, grid1(count, nrhs), RT, 0, s, (R)a, (const cplx_t<R>*)x, (R)b, (cplx_t<R>*)y,
                                                 count); count_launch();
   return cudaGetLastError();
 }
 
 template <typename R>
 __global__ void __launch_bounds__(RT) k_scale_inv_sqrt(const cplx_t<R>* x, cplx_t<R>* y,
-                                                       const double* nrm, long long count) {
+                                                       const double* nrm, long long count, int dependent) {
+  pdl_wait(dependent);
   __shared__ double ssc;                             // one root and division per block
   if (threadIdx.x == 0) {
     const double n2 = nrm[2 * blockIdx.y];
@@ -126,7 +129,7 @@ __global__ void __launch_bounds__(RT) k_scale_inv_sqrt(const cplx_t<R>* x, cplx_
 template <typename R>
 cudaError_t scale_inv_sqrt(const void* x, void* y, const double* nrm, long long count, int nrhs,
                            cudaStream_t s) {
-  k_scale_inv_sqrt<R><<<grid1(count, nrhs), RT, 0, s>>>((const cplx_t<R>*)x, (cplx_t<R>*)y, nrm,
+  launch_after(k_scale_inv_sqrt<R>, grid1(count, nrhs), RT, 0, s, (const cplx_t<R>*)x, (cplx_t<R>*)y, nrm,
                                                          count); count_launch();
   return cudaGetLastError();
 }
@@ -140,7 +143,8 @@ __global__ void __launch_bounds__(RT) k_cg_xr(cplx_t<R>* __restrict__ x, cplx_t<
                                               const cplx_t<R>* __restrict__ q, const double* rz,
                                               const double* pq, const int* frozen,
                                               long long count, double* ws, double* rr,
-                                              float2* __restrict__ r32, CgControl cc) {
+                                              float2* __restrict__ r32, CgControl cc, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
@@ -180,7 +184,7 @@ cudaError_t cg_xr(void* x, void* r, const void* p, const void* q, const double* 
                   double* rr, cudaStream_t s, void* r32, const CgControl* cc) {
   if (nrhs > 64) return cudaErrorInvalidValue;
   const int g = reduce_blocks(count, nrhs);
-  k_cg_xr<R><<<dim3(g, nrhs), RT, 0, s>>>((cplx_t<R>*)x, (cplx_t<R>*)r, (const cplx_t<R>*)p,
+  launch_after(k_cg_xr<R>, dim3(g, nrhs), RT, 0, s, (cplx_t<R>*)x, (cplx_t<R>*)r, (const cplx_t<R>*)p,
                                           (const cplx_t<R>*)q, rz, pq, frozen, count, ws, rr,
                                           (float2*)r32, cc ? *cc : CgControl{});
   count_launch();
@@ -190,7 +194,8 @@ cudaError_t cg_xr(void* x, void* r, const void* p, const void* q, const double* 
 template <typename R>
 __global__ void __launch_bounds__(RT) k_cg_p(cplx_t<R>* __restrict__ p, const cplx_t<R>* __restrict__ z,
                                              const double* rz_new, const double* rz_old,
-                                             const int* frozen, long long count) {
+                                             const int* frozen, long long count, int dependent) {
+  pdl_wait(dependent);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const R beta = (R)block_ratio(rz_new[2 * rhs], rz_old[2 * rhs]);
@@ -206,7 +211,7 @@ __global__ void __launch_bounds__(RT) k_cg_p(cplx_t<R>* __restrict__ p, const cp
 template <typename R>
 cudaError_t cg_p(void* p, const void* z, const double* rz_new, const double* rz_old,
                  const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_cg_p<R><<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_cg_p<R>, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (cplx_t<R>*)p, (const cplx_t<R>*)z, rz_new, rz_old, frozen, count);
   count_launch();
   return cudaGetLastError();
@@ -251,14 +256,15 @@ __device__ void cg_control_step(const double* rr, const double* pq, const double
 }
 
 __global__ void k_cg_control(const double* rr, const double* pq, const double* stop, int* ctrl,
-                             cudaGraphConditionalHandle cond) {
+                             cudaGraphConditionalHandle cond, int dependent) {
+  pdl_wait(dependent);
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   cg_control_step(rr, pq, stop, ctrl, cond);
 }
 
 cudaError_t cg_control(const double* rr, const double* pq, const double* stop, int* ctrl,
                        cudaGraphConditionalHandle cond, cudaStream_t s) {
-  k_cg_control<<<1, 32, 0, s>>>(rr, pq, stop, ctrl, cond);
+  launch_after(k_cg_control, 1, 32, 0, s, rr, pq, stop, ctrl, cond);
   count_launch();
   return cudaGetLastError();
 }
@@ -266,7 +272,8 @@ cudaError_t cg_control(const double* rr, const double* pq, const double* stop, i
 // Initialises ctrl and stop[rhs] = tol2 * bn[rhs]; right-hand sides with
 // b = 0 start frozen (x = 0 is exact).
 __global__ void k_set_control(int* ctrl, int maxiter, int nrhs, const double* bn, double tol2,
-                              double* stop) {
+                              double* stop, int dependent) {
+  pdl_wait(dependent);
   if (threadIdx.x != 0) return;
   ctrl[0] = 0;
   ctrl[1] = 0;
@@ -282,7 +289,7 @@ __global__ void k_set_control(int* ctrl, int maxiter, int nrhs, const double* bn
 
 cudaError_t set_control(int* ctrl, int maxiter, int nrhs, const double* bn, double tol2,
                         double* stop, cudaStream_t s) {
-  k_set_control<<<1, 32, 0, s>>>(ctrl, maxiter, nrhs, bn, tol2, stop);
+  launch_after(k_set_control, 1, 32, 0, s, ctrl, maxiter, nrhs, bn, tol2, stop);
   count_launch();
   return cudaGetLastError();
 }
@@ -292,7 +299,8 @@ cudaError_t set_control(int* ctrl, int maxiter, int nrhs, const double* bn, doub
 __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
                                                    const double2* __restrict__ q,
                                                    const double2* __restrict__ r, long long count,
-                                                   double* ws, double* zr) {
+                                                   double* ws, double* zr, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   double a = 0.0, b = 0.0;
@@ -312,7 +320,7 @@ __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
 cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long count, int nrhs,
                        double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_dot2_zq_rz<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_dot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (const float2*)z32, (const double2*)q, (const double2*)r, count, ws, zr);
   count_launch();
   return cudaGetLastError();
@@ -322,7 +330,8 @@ cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long 
 // right-hand sides untouched.
 __global__ void __launch_bounds__(RT) k_cg_p_pr(double2* __restrict__ p, const float2* __restrict__ z,
                                                 const double* zr, const double* pq, double* rz,
-                                                const int* frozen, long long count) {
+                                                const int* frozen, long long count, int dependent) {
+  pdl_wait(dependent);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const double beta = block_ratio(-zr[2 * rhs], pq[2 * rhs]);
@@ -342,7 +351,7 @@ __global__ void __launch_bounds__(RT) k_cg_p_pr(double2* __restrict__ p, const f
 
 cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq, double* rz,
                     const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_cg_p_pr<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_cg_p_pr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (double2*)p, (const float2*)z32, zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
@@ -358,7 +367,8 @@ cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq
 // ab[rhs] = <a, b> of FP32 vectors.
 __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
                                              const float2* __restrict__ b, long long count,
-                                             double* ws, double* out) {
+                                             double* ws, double* out, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float re = 0.f, im = 0.f;
@@ -374,7 +384,7 @@ __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
 cudaError_t rdot(const void* a, const void* b, long long count, int nrhs, double* ws, double* out,
                  cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rdot<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>((const float2*)a, (const float2*)b,
+  launch_after(k_rdot, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (const float2*)a, (const float2*)b,
                                                          count, ws, out);
   count_launch();
   return cudaGetLastError();
@@ -387,7 +397,8 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
                                                const float2* __restrict__ p,
                                                const float2* __restrict__ q, const double* rz,
                                                const double* pq, const int* frozen,
-                                               long long count, double* ws, double* rr) {
+                                               long long count, double* ws, double* rr, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
@@ -413,7 +424,7 @@ cudaError_t rcg_xr(void* x32, void* r32, const void* p32, const void* q32, const
                    const double* pq, const int* frozen, long long count, int nrhs, double* ws,
                    double* rr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rcg_xr<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_rcg_xr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (float2*)x32, (float2*)r32, (const float2*)p32, (const float2*)q32, rz, pq, frozen, count,
       ws, rr);
   count_launch();
@@ -424,7 +435,8 @@ cudaError_t rcg_xr(void* x32, void* r32, const void* p32, const void* q32, const
 __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z,
                                                     const float2* __restrict__ q,
                                                     const float2* __restrict__ r, long long count,
-                                                    double* ws, double* zr) {
+                                                    double* ws, double* zr, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float a = 0.f, b = 0.f;
@@ -440,7 +452,7 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
 cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long long count,
                         int nrhs, double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_rdot2_zq_rz<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_rdot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (const float2*)z32, (const float2*)q32, (const float2*)r32, count, ws, zr);
   count_launch();
   return cudaGetLastError();
@@ -449,7 +461,8 @@ cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long 
 // beta = -zr[0] / Re(pq); p = z + beta p (FP32); rz <- {zr[1], 0}.
 __global__ void __launch_bounds__(RT) k_rcg_p(float2* __restrict__ p, const float2* __restrict__ z,
                                               const double* zr, const double* pq, double* rz,
-                                              const int* frozen, long long count) {
+                                              const int* frozen, long long count, int dependent) {
+  pdl_wait(dependent);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const float beta = (float)block_ratio(-zr[2 * rhs], pq[2 * rhs]);
@@ -467,7 +480,7 @@ __global__ void __launch_bounds__(RT) k_rcg_p(float2* __restrict__ p, const floa
 
 cudaError_t rcg_p(void* p32, const void* z32, const double* zr, const double* pq, double* rz,
                   const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  k_rcg_p<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>(
+  launch_after(k_rcg_p, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
       (float2*)p32, (const float2*)z32, zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
@@ -477,7 +490,8 @@ cudaError_t rcg_p(void* p32, const void* z32, const double* zr, const double* pq
 // rmax = max(rmax, rr); an update is due when some rr < delta^2 rmax.  Sets
 // *due (and the IF condition of the enclosing graph node when cond_set).
 __global__ void k_ru_check(const double* rr, double* rmax, const int* ctrl, double delta2,
-                           int* due, int* count, cudaGraphConditionalHandle cond, int cond_set) {
+                           int* due, int* count, cudaGraphConditionalHandle cond, int cond_set, int dependent) {
+  pdl_wait(dependent);
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int nrhs = ctrl[3];
   const int* frozen = ctrl + 4;
@@ -495,13 +509,14 @@ __global__ void k_ru_check(const double* rr, double* rmax, const int* ctrl, doub
 
 cudaError_t ru_check(const double* rr, double* rmax, const int* ctrl, double delta2, int* due,
                      int* count, cudaGraphConditionalHandle cond, bool cond_set, cudaStream_t s) {
-  k_ru_check<<<1, 32, 0, s>>>(rr, rmax, ctrl, delta2, due, count, cond, cond_set ? 1 : 0);
+  launch_after(k_ru_check, 1, 32, 0, s, rr, rmax, ctrl, delta2, due, count, cond, cond_set ? 1 : 0);
   count_launch();
   return cudaGetLastError();
 }
 
 // x64 += x32, x32 = 0 (the FP32 increment folded into the FP64 solution).
-__global__ void k_ru_fold(double2* __restrict__ x, float2* __restrict__ x32, long long count) {
+__global__ void k_ru_fold(double2* __restrict__ x, float2* __restrict__ x32, long long count, int dependent) {
+  pdl_wait(dependent);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float2 v = x32[i];
@@ -511,7 +526,7 @@ __global__ void k_ru_fold(double2* __restrict__ x, float2* __restrict__ x32, lon
 }
 
 cudaError_t ru_fold(void* x64, void* x32, long long count, cudaStream_t s) {
-  k_ru_fold<<<grid1(count, 1), RT, 0, s>>>((double2*)x64, (float2*)x32, count);
+  launch_after(k_ru_fold, grid1(count, 1), RT, 0, s, (double2*)x64, (float2*)x32, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -519,7 +534,8 @@ cudaError_t ru_fold(void* x64, void* x32, long long count, cudaStream_t s) {
 // r32 = (float) r64 and rr = rmax = |r64|^2 (FP64) per right-hand side.
 __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ r,
                                                     float2* __restrict__ r32, long long count,
-                                                    double* ws, double* rr) {
+                                                    double* ws, double* rr, int dependent) {
+  pdl_wait(dependent);
   __shared__ double sh[RT];
   const long long base = (long long)blockIdx.y * count;
   double acc = 0.0;
@@ -532,7 +548,8 @@ __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ 
   finish_reduction<1>(acc, 0.0, ws, rr, sh);
 }
 
-__global__ void k_copy_slots(const double* src, double* dst, int n2) {
+__global__ void k_copy_slots(const double* src, double* dst, int n2, int dependent) {
+  pdl_wait(dependent);
   const int i = threadIdx.x;
   if (i < n2) dst[i] = src[i];
 }
@@ -540,18 +557,20 @@ __global__ void k_copy_slots(const double* src, double* dst, int n2) {
 cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, double* ws,
                         double* rr, double* rmax, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  k_ru_residual<<<dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s>>>((const double2*)r64, (float2*)r32,
+  launch_after(k_ru_residual, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
+               (const double2*)r64, (float2*)r32,
                                                                 count, ws, rr);
   count_launch();
   if (rmax) {
-    k_copy_slots<<<1, 128, 0, s>>>(rr, rmax, 2 * nrhs);
+    launch_after(k_copy_slots, 1, 128, 0, s, rr, rmax, 2 * nrhs);
     count_launch();
   }
   return cudaGetLastError();
 }
 
 __global__ void k_f64_to_f32_scaled(const double2* __restrict__ in, float2* __restrict__ out,
-                                    const double* nrm, long long count) {
+                                    const double* nrm, long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const double n2 = nrm[2 * blockIdx.y];
@@ -563,13 +582,14 @@ __global__ void k_f64_to_f32_scaled(const double2* __restrict__ in, float2* __re
 
 cudaError_t f64_to_f32_scaled(const void* in, void* out, const double* nrm, long long count,
                               int nrhs, cudaStream_t s) {
-  k_f64_to_f32_scaled<<<grid1(count, nrhs), RT, 0, s>>>((const double2*)in, (float2*)out, nrm,
+  launch_after(k_f64_to_f32_scaled, grid1(count, nrhs), RT, 0, s, (const double2*)in, (float2*)out, nrm,
                                                          count); count_launch();
   return cudaGetLastError();
 }
 
 __global__ void k_f32_acc_scaled(const float2* __restrict__ in, double2* __restrict__ x,
-                                 const double* nrm, long long count) {
+                                 const double* nrm, long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const double sc = nrm ? sqrt(nrm[2 * blockIdx.y]) : 1.0;
@@ -581,32 +601,37 @@ __global__ void k_f32_acc_scaled(const float2* __restrict__ in, double2* __restr
 
 cudaError_t f32_accumulate_scaled(const void* in, void* x, const double* nrm, long long count,
                                   int nrhs, cudaStream_t s) {
-  k_f32_acc_scaled<<<grid1(count, nrhs), RT, 0, s>>>((const float2*)in, (double2*)x, nrm, count); count_launch();
+  launch_after(k_f32_acc_scaled, grid1(count, nrhs), RT, 0, s,
+               (const float2*)in, (double2*)x, nrm, count);
+  count_launch();
   return cudaGetLastError();
 }
 
 __global__ void k_cvt_64_32(const double2* __restrict__ in, float2* __restrict__ out,
-                            long long count) {
+                            long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 __global__ void k_cvt_32_64(const float2* __restrict__ in, double2* __restrict__ out,
-                            long long count) {
+                            long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) out[i] = make_double2(in[i].x, in[i].y);
 }
 cudaError_t convert_f64_f32(const void* in, void* out, long long count, cudaStream_t s) {
-  k_cvt_64_32<<<grid1(count, 1), RT, 0, s>>>((const double2*)in, (float2*)out, count); count_launch();
+  launch_after(k_cvt_64_32, grid1(count, 1), RT, 0, s, (const double2*)in, (float2*)out, count); count_launch();
   return cudaGetLastError();
 }
 cudaError_t convert_f32_f64(const void* in, void* out, long long count, cudaStream_t s) {
-  k_cvt_32_64<<<grid1(count, 1), RT, 0, s>>>((const float2*)in, (double2*)out, count); count_launch();
+  launch_after(k_cvt_32_64, grid1(count, 1), RT, 0, s, (const float2*)in, (double2*)out, count); count_launch();
   return cudaGetLastError();
 }
 
 template <typename R>
 __global__ void k_lincomb(cplx_t<R>* out, R a, const cplx_t<R>* u, R b, const cplx_t<R>* v, R c,
-                          const cplx_t<R>* w, long long count) {
+                          const cplx_t<R>* w, long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   i += (long long)blockIdx.y * count;
@@ -623,7 +648,7 @@ __global__ void k_lincomb(cplx_t<R>* out, R a, const cplx_t<R>* u, R b, const cp
 template <typename R>
 cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v, double c,
                     const void* w, long long count, int nrhs, cudaStream_t s) {
-  k_lincomb<R><<<grid1(count, nrhs), RT, 0, s>>>((cplx_t<R>*)out, (R)a, (const cplx_t<R>*)u, (R)b,
+  launch_after(k_lincomb<R>, grid1(count, nrhs), RT, 0, s, (cplx_t<R>*)out, (R)a, (const cplx_t<R>*)u, (R)b,
                                                   (const cplx_t<R>*)v, (R)c,
                                                   (const cplx_t<R>*)w, count); count_launch();
   return cudaGetLastError();
@@ -631,13 +656,16 @@ cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v,
 
 template <typename R>
 __global__ void k_sub_from(const cplx_t<R>* __restrict__ b, cplx_t<R>* __restrict__ r,
-                           long long count) {
+                           long long count, int dependent) {
+  pdl_wait(dependent);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) r[i] = csub(b[i], r[i]);
 }
 template <typename R>
 cudaError_t sub_from(const void* b, void* r, long long count, cudaStream_t s) {
-  k_sub_from<R><<<grid1(count, 1), RT, 0, s>>>((const cplx_t<R>*)b, (cplx_t<R>*)r, count); count_launch();
+  launch_after(k_sub_from<R>, grid1(count, 1), RT, 0, s,
+               (const cplx_t<R>*)b, (cplx_t<R>*)r, count);
+  count_launch();
   return cudaGetLastError();
 }
 

@@ -70,7 +70,8 @@ template <typename R, typename WT>
 __global__ void __launch_bounds__(576, 2) k_coarse_apply(const cplx_t<R>* __restrict__ in,
                                                       cplx_t<R>* out,
                                                       const WT* __restrict__ A, int Lx, int Lt,
-                                                      int n, Epilogue ep) {
+                                                      int n, Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ unsigned char smraw[];
   cplx_t<R>* xs = (cplx_t<R>*)smraw;            // [9][n] neighbour vectors
   cplx_t<R>* part = xs + 9 * n;                 // [9][n] partial row products
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(576, 2) k_coarse_apply(const cplx_t<R>* __rest
   if constexpr (kBf16) {
     if (pre && threadIdx.x < 9 * n) {
       const int d = threadIdx.x / n, r = threadIdx.x % n;
-      const uint4* row4 = (const uint4*)(A + (((long long)j * 9 + d) * n + r) * n);
+      const uint4* row4 = pdl_ordered((const uint4*)(A + (((long long)j * 9 + d) * n + r) * n));
 #pragma unroll
       for (int k = 0; k < PRE; ++k)
         if (k < n / 4) rv[k] = __ldg(row4 + k);
@@ -178,7 +179,8 @@ static constexpr int MMA_RC = 16;            // right-hand sides per CTA
 __global__ void __launch_bounds__(64) k_coarse_apply_mma(const float2* __restrict__ in, float2* out,
                                                          const __nv_bfloat162* __restrict__ A,
                                                          int Lx, int Lt, int n, int nrhs,
-                                                         Epilogue ep) {
+                                                         Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ __nv_bfloat162 Xs[];
   constexpr int RS = MMA_RC + 8;             // padded row: conflict-free fragment loads
   const int V = Lx * Lt;
@@ -274,7 +276,7 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
       attr = true;
     }
     dim3 grid(Lx * Lt, (nrhs + MMA_RC - 1) / MMA_RC);
-    k_coarse_apply_mma<<<grid, 64, smem, s>>>((const float2*)in, (float2*)out,
+    launch_after(k_coarse_apply_mma, grid, 64, smem, s, (const float2*)in, (float2*)out,
                                               (const __nv_bfloat162*)A, Lx, Lt, n, nrhs, ep);
     count_launch();
     return cudaGetLastError();
@@ -282,13 +284,13 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
   dim3 grid(Lx * Lt, nrhs);
   const int threads = (9 * n + 31) / 32 * 32;
   if (weights == W_F64)
-    k_coarse_apply<double, double2><<<grid, threads, 18 * n * sizeof(double2), s>>>(
+    launch_after(k_coarse_apply<double, double2>, grid, threads, 18 * n * sizeof(double2), s,
         (const double2*)in, (double2*)out, (const double2*)A, Lx, Lt, n, ep);
   else if (weights == W_F32)
-    k_coarse_apply<float, float2><<<grid, threads, 18 * n * sizeof(float2), s>>>(
+    launch_after(k_coarse_apply<float, float2>, grid, threads, 18 * n * sizeof(float2), s,
         (const float2*)in, (float2*)out, (const float2*)A, Lx, Lt, n, ep);
   else
-    k_coarse_apply<float, __nv_bfloat162><<<grid, threads, 18 * n * sizeof(float2), s>>>(
+    launch_after(k_coarse_apply<float, __nv_bfloat162>, grid, threads, 18 * n * sizeof(float2), s,
         (const float2*)in, (float2*)out, (const __nv_bfloat162*)A, Lx, Lt, n, ep);
   count_launch();
   return cudaGetLastError();
@@ -297,7 +299,8 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
 // out = a X + b Y + c I on 9-point block stencils [site][d][r][s] (I: the
 // identity blocks of the d = 4 displacement); out may alias X or Y.
 __global__ void k_coarse_lincomb(double a, const double2* X, double b, const double2* Y, double c,
-                                 double2* out, long long count, int n) {
+                                 double2* out, long long count, int n, int dependent) {
+  pdl_wait(dependent);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int q = (int)(i % ((long long)9 * n * n));
@@ -311,7 +314,7 @@ __global__ void k_coarse_lincomb(double a, const double2* X, double b, const dou
 cudaError_t coarse_lincomb(double a, const void* X, double b, const void* Y, double c, void* out,
                            long long sites, int n, cudaStream_t s) {
   const long long count = sites * 9 * n * n;
-  k_coarse_lincomb<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(
+  launch_after(k_coarse_lincomb, (unsigned)((count + 255) / 256), 256, 0, s,
       a, (const double2*)X, b, (const double2*)Y, c, (double2*)out, count, n);
   count_launch();
   return cudaGetLastError();
@@ -324,7 +327,8 @@ cudaError_t coarse_lincomb(double a, const void* X, double b, const void* Y, dou
 // sites of one colour are never within one block of the same site.
 // ---------------------------------------------------------------------------
 __global__ void k_probe_vectors(double2* __restrict__ out, int Lxc, int Ltc, int nc, int Kx, int Kt,
-                                int cx, int ct) {
+                                int cx, int ct, int dependent) {
+  pdl_wait(dependent);
   const long long Vc = (long long)Lxc * Ltc;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)nc * Vc * nc) return;
@@ -335,7 +339,8 @@ __global__ void k_probe_vectors(double2* __restrict__ out, int Lxc, int Ltc, int
 }
 
 __global__ void k_probe_scatter(const double2* __restrict__ y, double2* __restrict__ Ac, int Lxc,
-                                int Ltc, int nc, int Kx, int Kt, int cx, int ct) {
+                                int Ltc, int nc, int Kx, int Kt, int cx, int ct, int dependent) {
+  pdl_wait(dependent);
   const long long Vc = (long long)Lxc * Ltc;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= Vc * 9 * nc * nc) return;
@@ -348,7 +353,7 @@ __global__ void k_probe_scatter(const double2* __restrict__ y, double2* __restri
 cudaError_t probe_vectors(void* out, int Lxc, int Ltc, int nc, int Kx, int Kt, int cx, int ct,
                           cudaStream_t s) {
   const long long n = (long long)nc * Lxc * Ltc * nc;
-  k_probe_vectors<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((double2*)out, Lxc, Ltc, nc, Kx, Kt,
+  launch_after(k_probe_vectors, (unsigned)((n + 255) / 256), 256, 0, s, (double2*)out, Lxc, Ltc, nc, Kx, Kt,
                                                             cx, ct);
   count_launch();
   return cudaGetLastError();
@@ -357,7 +362,7 @@ cudaError_t probe_vectors(void* out, int Lxc, int Ltc, int nc, int Kx, int Kt, i
 cudaError_t probe_scatter(const void* y, void* Ac, int Lxc, int Ltc, int nc, int Kx, int Kt, int cx,
                           int ct, cudaStream_t s) {
   const long long n = (long long)Lxc * Ltc * 9 * nc * nc;
-  k_probe_scatter<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)y, (double2*)Ac, Lxc,
+  launch_after(k_probe_scatter, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)y, (double2*)Ac, Lxc,
                                                             Ltc, nc, Kx, Kt, cx, ct);
   count_launch();
   return cudaGetLastError();
@@ -379,7 +384,8 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_restrict(const cplx_t<R>* __restrict__ fine,
                                                   cplx_t<R>* __restrict__ coarse,
                                                   const cplx_t<R>* __restrict__ Vst, int Lx,
-                                                  int Lt, int bx, int bt, int h, int Nv) {
+                                                  int Lt, int bx, int bt, int h, int Nv, int dependent) {
+  pdl_wait(dependent);
   const int Lxc = Lx / bx, Vc = Lxc * (Lt / bt), nc = 2 * Nv, nf = 2 * h;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w >= Vc * nc) return;
@@ -428,7 +434,8 @@ __global__ void __launch_bounds__(256) k_restrict_multi(const cplx_t<R>* __restr
                                                         cplx_t<R>* __restrict__ coarse,
                                                         const cplx_t<R>* __restrict__ Vst, int Lx,
                                                         int Lt, int bx, int bt, int h, int Nv,
-                                                        int nrhs, int G) {
+                                                        int nrhs, int G, int dependent) {
+  pdl_wait(dependent);
   using C = cplx_t<R>;
   extern __shared__ unsigned char smraw[];
   const int b2 = bx * bt, nf = 2 * h, nc = 2 * Nv, T = b2 * h, Lxc = Lx / bx, Vc = Lxc * (Lt / bt);
@@ -470,7 +477,8 @@ __global__ void __launch_bounds__(256) k_prolong_multi(const cplx_t<R>* __restri
                                                        cplx_t<R>* __restrict__ fine,
                                                        const cplx_t<R>* __restrict__ Vst, int Lx,
                                                        int Lt, int bx, int bt, int h, int Nv,
-                                                       int nrhs, bool accumulate, int G) {
+                                                       int nrhs, bool accumulate, int G, int dependent) {
+  pdl_wait(dependent);
   using C = cplx_t<R>;
   extern __shared__ unsigned char smraw[];
   const int b2 = bx * bt, nf = 2 * h, nc = 2 * Nv, Lxc = Lx / bx, Vc = Lxc * (Lt / bt);
@@ -533,14 +541,14 @@ cudaError_t restrict_op(const void* fine, void* coarse, const void* Vst, int Lx,
       cudaFuncSetAttribute(k_restrict_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
       attr = true;
     }
-    k_restrict_multi<R><<<(Lx / bx) * (Lt / bt), 256, sm, s>>>(
+    launch_after(k_restrict_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
         (const cplx_t<R>*)fine, (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
         nrhs, transfer_group(nrhs * 2 * Nv, bx * bt * h));
     count_launch();
     return cudaGetLastError();
   }
   const int warps = (Lx / bx) * (Lt / bt) * 2 * Nv;
-  k_restrict<R><<<dim3((warps + 7) / 8, nrhs), 256, 0, s>>>(
+  launch_after(k_restrict<R>, dim3((warps + 7) / 8, nrhs), 256, 0, s,
       (const cplx_t<R>*)fine, (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv);
   count_launch();
   return cudaGetLastError();
@@ -549,7 +557,8 @@ cudaError_t restrict_op(const void* fine, void* coarse, const void* Vst, int Lx,
 template <typename R>
 __global__ void k_prolong(const cplx_t<R>* __restrict__ coarse, cplx_t<R>* __restrict__ fine,
                           const cplx_t<R>* __restrict__ Vst, int Lx, int Lt, int bx, int bt, int h,
-                          int Nv, bool accumulate) {
+                          int Nv, bool accumulate, int dependent) {
+  pdl_wait(dependent);
   const int V = Lx * Lt, nf = 2 * h, nc = 2 * Nv;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= V * nf) return;
@@ -577,14 +586,14 @@ cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, 
       cudaFuncSetAttribute(k_prolong_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
       attr = true;
     }
-    k_prolong_multi<R><<<(Lx / bx) * (Lt / bt), 256, sm, s>>>(
+    launch_after(k_prolong_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
         (const cplx_t<R>*)coarse, (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
         nrhs, accumulate, transfer_group(nrhs * bx * bt * 2 * h, Nv));
     count_launch();
     return cudaGetLastError();
   }
   const int tot = Lx * Lt * 2 * h;
-  k_prolong<R><<<dim3((tot + 255) / 256, nrhs), 256, 0, s>>>(
+  launch_after(k_prolong<R>, dim3((tot + 255) / 256, nrhs), 256, 0, s,
       (const cplx_t<R>*)coarse, (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
       accumulate); count_launch();
   return cudaGetLastError();
@@ -609,7 +618,8 @@ template <int LPB, int NQ>
 __global__ void __launch_bounds__(32) k_block_gs(const double2* __restrict__ E,
                                                  double2* __restrict__ Vst, int Lx, int Lt,
                                                  int bx, int bt, int h, int Nv, double tol,
-                                                 int* flag, int nblocks) {
+                                                 int* flag, int nblocks, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ double2 Qs[];   // [32 / LPB][Nv][m]
   const int V = Lx * Lt, nf = 2 * h, Lxc = Lx / bx;
   const int sub = threadIdx.x / LPB, lane = threadIdx.x % LPB;
@@ -685,7 +695,8 @@ cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx,
     static const cudaError_t e = cudaFuncSetAttribute(
         k_block_gs<LPB, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
     if (e != cudaSuccess) return e;
-    k_block_gs<LPB, NQ><<<(nb + per - 1) / per, 32, smem, s>>>((const double2*)E, (double2*)Vst, Lx, Lt, bx,
+    launch_after(k_block_gs<LPB, NQ>, (nb + per - 1) / per, 32, smem, s,
+                 (const double2*)E, (double2*)Vst, Lx, Lt, bx,
                                                               bt, h, Nv, breakdown_tol, flag, nb);
     count_launch();
     return cudaGetLastError();
@@ -707,7 +718,8 @@ cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx,
 // ---------------------------------------------------------------------------
 __global__ void k_galerkin_W(const double2* __restrict__ U, double diag,
                              const double2* __restrict__ Vst, double2* __restrict__ Wbuf, int Lx,
-                             int Lt, int bx, int bt, int Nv) {
+                             int Lt, int bx, int bt, int Nv, int dependent) {
+  pdl_wait(dependent);
   const int Lxc = Lx / bx, Vc = Lxc * (Lt / bt), nc = 2 * Nv;
   const int ex_w = bx + 2, E = (bx + 2) * (bt + 2);
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -764,7 +776,8 @@ __global__ void k_galerkin_W(const double2* __restrict__ U, double diag,
 // warp run sums of one length.
 template <bool G1>
 __global__ void k_galerkin_WW(const double2* __restrict__ Wbuf, const double2* __restrict__ Vst,
-                              double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt, int Nv) {
+                              double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt, int Nv, int dependent) {
+  pdl_wait(dependent);
   const int Lxc = Lx / bx, Ltc = Lt / bt, nc = 2 * Nv;
   const long long Vc = (long long)Lxc * Ltc;
   const int ex_w = bx + 2, E = (bx + 2) * (bt + 2), tri = nc * (nc + 1) / 2;
@@ -836,13 +849,13 @@ cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* W
                           int Lx, int Lt, int bx, int bt, int Nv, cudaStream_t s) {
   const long long Vc = (long long)(Lx / bx) * (Lt / bt), nc = 2 * Nv;
   const long long nW = Vc * nc * (bx + 2) * (bt + 2);
-  k_galerkin_W<<<(unsigned)((nW + 255) / 256), 256, 0, s>>>(
+  launch_after(k_galerkin_W, (unsigned)((nW + 255) / 256), 256, 0, s,
       (const double2*)U64, diag, (const double2*)Vst, (double2*)Wbuf, Lx, Lt, bx, bt, Nv); count_launch();
   const long long nA = Vc * (nc * (nc + 1) / 2 + 4 * nc * nc);
-  k_galerkin_WW<false><<<(unsigned)((nA + 255) / 256), 256, 0, s>>>(
+  launch_after(k_galerkin_WW<false>, (unsigned)((nA + 255) / 256), 256, 0, s,
       (const double2*)Wbuf, (const double2*)Vst, (double2*)Ac, Lx, Lt, bx, bt, Nv); count_launch();
   if (G1) {
-    k_galerkin_WW<true><<<(unsigned)((nA + 255) / 256), 256, 0, s>>>(
+    launch_after(k_galerkin_WW<true>, (unsigned)((nA + 255) / 256), 256, 0, s,
         (const double2*)Wbuf, (const double2*)Vst, (double2*)G1, Lx, Lt, bx, bt, Nv); count_launch();
   }
   return cudaGetLastError();
@@ -858,7 +871,8 @@ cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* W
 // ---------------------------------------------------------------------------
 __global__ void k_galerkin_coarse(const double2* __restrict__ Af, const double2* __restrict__ Vst,
                                   double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt,
-                                  int nf, int Nv) {
+                                  int nf, int Nv, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ double2 sm[];
   const int nc = 2 * Nv, h = nf / 2, Lxc = Lx / bx;
   double2* acc = sm;                  // [9][nc][nc]
@@ -923,7 +937,7 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
     attr_set = true;
   }
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  k_galerkin_coarse<<<Vc, 256, smem, s>>>((const double2*)Af, (const double2*)Vst, (double2*)Ac,
+  launch_after(k_galerkin_coarse, Vc, 256, smem, s, (const double2*)Af, (const double2*)Vst, (double2*)Ac,
                                           Lx, Lt, bx, bt, nf, Nv); count_launch();
   return cudaGetLastError();
 }
@@ -932,7 +946,8 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
 // Coarsest level: dense matrix, FP32 Gauss-Jordan inverse, GEMV.
 // ---------------------------------------------------------------------------
 __global__ void k_coarse_to_dense(const double2* __restrict__ A, float2* __restrict__ M, int Lx,
-                                  int Lt, int n, long long ld) {
+                                  int Lt, int n, long long ld, int dependent) {
+  pdl_wait(dependent);
   const int V = Lx * Lt;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)V * n * n) return;
@@ -948,7 +963,8 @@ __global__ void k_coarse_to_dense(const double2* __restrict__ A, float2* __restr
   }
 }
 
-__global__ void k_pad_identity(float2* __restrict__ M, long long N, long long ld) {
+__global__ void k_pad_identity(float2* __restrict__ M, long long N, long long ld, int dependent) {
+  pdl_wait(dependent);
   const long long i = N + (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < ld) M[i * ld + i] = make_float2(1.f, 0.f);
 }
@@ -960,10 +976,10 @@ cudaError_t coarse_to_dense_f32(const void* A, void* dense, int Lx, int Lt, int 
   cudaError_t e = cudaMemsetAsync(dense, 0, (size_t)(ld * ld * sizeof(float2)), s);
   if (e != cudaSuccess) return e;
   const long long tot = (long long)Lx * Lt * n * n;
-  k_coarse_to_dense<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>((const double2*)A,
+  launch_after(k_coarse_to_dense, (unsigned)((tot + 255) / 256), 256, 0, s, (const double2*)A,
                                                                   (float2*)dense, Lx, Lt, n, ld); count_launch();
   if (ld > N) {
-    k_pad_identity<<<(unsigned)((ld - N + 255) / 256), 256, 0, s>>>((float2*)dense, N, ld);
+    launch_after(k_pad_identity, (unsigned)((ld - N + 255) / 256), 256, 0, s, (float2*)dense, N, ld);
     count_launch();
   }
   return cudaGetLastError();
@@ -1066,7 +1082,8 @@ __device__ void sweep_block64(float2* a, float2* tmp) {
 
 // Inverts the first pivot block: P = M_00^{-1}.
 __global__ void __launch_bounds__(256) k_gj_pivot0(const float2* __restrict__ M, int N,
-                                                   float2* __restrict__ P) {
+                                                   float2* __restrict__ P, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ float2 gsm[];
   for (int q = threadIdx.x; q < GJB * GJB; q += 256)
     gsm[(q / GJB) * GJS + q % GJB] = M[(long long)(q / GJB) * N + q % GJB];
@@ -1083,7 +1100,8 @@ __global__ void __launch_bounds__(256) k_gj_panel(const float2* __restrict__ M, 
                                                   const float2* __restrict__ P,
                                                   float2* __restrict__ Cold,
                                                   float2* __restrict__ Cn,
-                                                  float2* __restrict__ Rp) {
+                                                  float2* __restrict__ Rp, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ float2 gsm[];
   float2* sP = gsm;
   float2* sX = gsm + GJB * GJS;
@@ -1240,7 +1258,8 @@ __global__ void __launch_bounds__(256, 2) k_gj_update_tc(float2* __restrict__ M,
                                                          const float2* __restrict__ Cold,
                                                          const float2* __restrict__ Cn,
                                                          const float2* __restrict__ Rp,
-                                                         int* __restrict__ err) {
+                                                         int* __restrict__ err, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ __align__(16) unsigned char tc_dyn[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_sh;
@@ -1431,7 +1450,7 @@ cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s) {
                          (int)(2 * GJB * GJS * sizeof(float2)));
     attr = true;
   }
-  k_gj_pivot0<<<1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s>>>((const float2*)M, N, Pb[0]);
+  launch_after(k_gj_pivot0, 1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s, (const float2*)M, N, Pb[0]);
   count_launch();
   return cudaGetLastError();
 }
@@ -1440,7 +1459,7 @@ cudaError_t gauss_jordan_panel(void* M, int N, int k, void* work, cudaStream_t s
   float2 *Pb[2], *Cold, *Cn, *Rp;
   gj_work_split(work, N, Pb, &Cold, &Cn, &Rp);
   const int nb = N / GJB;
-  k_gj_panel<<<dim3(2 * nb, GJB / 16), 256, 2 * GJB * GJS * sizeof(float2), s>>>(
+  launch_after(k_gj_panel, dim3(2 * nb, GJB / 16), 256, 2 * GJB * GJS * sizeof(float2), s,
       (const float2*)M, N, k, Pb[k & 1], Cold, Cn, Rp);
   count_launch();
   return cudaGetLastError();
@@ -1463,13 +1482,14 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
     cudaFuncSetAttribute(k_gj_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     attr = true;
   }
-  k_gj_update_tc<<<tc_tile_count(nb), 256, sm, s>>>((float2*)M, N, k, Pb[k & 1], Pb[(k + 1) & 1],
+  launch_after(k_gj_update_tc, tc_tile_count(nb), 256, sm, s, (float2*)M, N, k, Pb[k & 1], Pb[(k + 1) & 1],
                                                     Cold, Cn, Rp, (int*)(Rp + (long long)GJB * N));
   count_launch();
   return cudaGetLastError();
 }
 
-__global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ xf, int N, int ld) {
+__global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ xf, int N, int ld, int dependent) {
+  pdl_wait(dependent);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < ld) xf[i] = i < N ? make_float2((float)x[i].x, (float)x[i].y) : make_float2(0.f, 0.f);
 }
@@ -1477,7 +1497,8 @@ __global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ x
 __global__ void __launch_bounds__(256) k_gemv(const float2* __restrict__ B,
                                               const float2* __restrict__ xf,
                                               double2* __restrict__ y, int N, int ld,
-                                              bool accumulate) {
+                                              bool accumulate, int dependent) {
+  pdl_wait(dependent);
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= N) return;
   const float4* b4 = (const float4*)(B + (long long)row * ld);
@@ -1502,8 +1523,10 @@ __global__ void __launch_bounds__(256) k_gemv(const float2* __restrict__ B,
 cudaError_t dense_gemv_f32(const void* B, const void* x, void* y, int N, int ld, void* xtmp,
                            bool accumulate, cudaStream_t s) {
   if (ld % 2 || ld < N) return cudaErrorInvalidValue;
-  k_x_to_f32<<<(ld + 255) / 256, 256, 0, s>>>((const double2*)x, (float2*)xtmp, N, ld); count_launch();
-  k_gemv<<<(N + 7) / 8, 256, 0, s>>>((const float2*)B, (const float2*)xtmp, (double2*)y, N, ld,
+  launch_after(k_x_to_f32, (ld + 255) / 256, 256, 0, s,
+               (const double2*)x, (float2*)xtmp, N, ld);
+  count_launch();
+  launch_after(k_gemv, (N + 7) / 8, 256, 0, s, (const float2*)B, (const float2*)xtmp, (double2*)y, N, ld,
                                      accumulate); count_launch();
   return cudaGetLastError();
 }
@@ -1516,7 +1539,8 @@ cudaError_t dense_gemv_f32(const void* B, const void* x, void* y, int N, int ld,
 static constexpr int HT = 64;
 
 
-__global__ void k_pack_hermitian(const float2* __restrict__ M, float2* __restrict__ P, int ld) {
+__global__ void k_pack_hermitian(const float2* __restrict__ M, float2* __restrict__ P, int ld, int dependent) {
+  pdl_wait(dependent);
   const int k = blockIdx.x;
   int I = (int)((sqrtf(8.f * k + 1.f) - 1.f) * 0.5f);
   while ((I + 1) * (I + 2) / 2 <= k) ++I;
@@ -1538,7 +1562,7 @@ __global__ void k_pack_hermitian(const float2* __restrict__ M, float2* __restric
 cudaError_t pack_hermitian(const void* M, void* P, int ld, cudaStream_t s) {
   if (ld % HT) return cudaErrorInvalidValue;
   const int nt = ld / HT;
-  k_pack_hermitian<<<nt * (nt + 1) / 2, 256, 0, s>>>((const float2*)M, (float2*)P, ld);
+  launch_after(k_pack_hermitian, nt * (nt + 1) / 2, 256, 0, s, (const float2*)M, (float2*)P, ld);
   count_launch();
   return cudaGetLastError();
 }
@@ -1625,7 +1649,8 @@ __device__ __forceinline__ void hgemv_mma_item(const float2* sT, const float2* s
 __global__ void __launch_bounds__(256) k_hgemv_mma(const float2* __restrict__ P,
                                                    const float2* __restrict__ xs, int ld,
                                                    int ntiles, int nrhs,
-                                                   float2* __restrict__ part) {
+                                                   float2* __restrict__ part, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ float2 hsm[];
   float2* sT = hsm;                                      // [64][GJC]
   float2* sXJ = sT + HT * GJC;                           // [64 k][GJR]: X_J[k][rhs]
@@ -1675,7 +1700,8 @@ __global__ void __launch_bounds__(256) k_hgemv_mma(const float2* __restrict__ P,
 }
 
 __global__ void k_x32_pad(const double2* __restrict__ x, float2* __restrict__ xs, int N, int ld,
-                          int nrhs) {
+                          int nrhs, int dependent) {
+  pdl_wait(dependent);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)ld * nrhs) return;
   const int r = (int)(i / ld), c = (int)(i % ld);
@@ -1685,7 +1711,8 @@ __global__ void k_x32_pad(const double2* __restrict__ x, float2* __restrict__ xs
 
 __global__ void __launch_bounds__(256) k_hgemv_tiles(const float2* __restrict__ P,
                                                      const double2* __restrict__ x, int N,
-                                                     int nrhs, float2* __restrict__ part) {
+                                                     int nrhs, float2* __restrict__ part, int dependent) {
+  pdl_wait(dependent);
   __shared__ float2 T[HT][HT + 1];
   __shared__ float2 xi[HT], xj[HT];
   __shared__ float2 red[4][HT];
@@ -1773,7 +1800,8 @@ __global__ void __launch_bounds__(64) k_hgemv_warp(const float2* __restrict__ P,
                                                    const XT* __restrict__ x, int N,
                                                    int ntiles, int nrhs,
                                                    float2* __restrict__ part,
-                                                   double2* __restrict__ x64) {
+                                                   double2* __restrict__ x64, int dependent) {
+  pdl_wait(dependent);
   __shared__ float4 colsum[NR][32];                      // column partials of warp 1
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int k = blockIdx.x;                              // one tile, rows split by warp
@@ -1781,7 +1809,7 @@ __global__ void __launch_bounds__(64) k_hgemv_warp(const float2* __restrict__ P,
   while ((I + 1) * (I + 2) / 2 <= k) ++I;
   while (I * (I + 1) / 2 > k) --I;
   const int J = k - I * (I + 1) / 2;
-  const float4* src = (const float4*)(P + (long long)k * HT * HT) + lane;
+  const float4* src = pdl_ordered((const float4*)(P + (long long)k * HT * HT)) + lane;
   for (int q0 = 0; q0 < nrhs; q0 += NR) {
     float2 xj0[NR], xj1[NR], xi0[NR], xi1[NR], ac0[NR], ac1[NR];
 #pragma unroll
@@ -1865,7 +1893,8 @@ __global__ void __launch_bounds__(64) k_hgemv_warp(const float2* __restrict__ P,
 __global__ void __launch_bounds__(256) k_hgemv_reduce(const float2* __restrict__ part,
                                                       double2* __restrict__ y, int N, int nt,
                                                       bool accumulate,
-                                                      float2* __restrict__ y32) {
+                                                      float2* __restrict__ y32, int dependent) {
+  pdl_wait(dependent);
   __shared__ float2 red[4][HT];
   const int I = blockIdx.x, rr = threadIdx.x % HT, g = threadIdx.x / HT;
   part += (long long)blockIdx.y * (nt * (nt + 1) / 2) * 2 * HT;
@@ -1894,7 +1923,7 @@ __global__ void __launch_bounds__(256) k_hgemv_reduce(const float2* __restrict__
 
 cudaError_t to_f32_padded(const void* x, void* xs, int N, int ld, int nrhs, cudaStream_t s) {
   const long long n = (long long)ld * nrhs;
-  k_x32_pad<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((const double2*)x, (float2*)xs, N, ld, nrhs);
+  launch_after(k_x32_pad, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)x, (float2*)xs, N, ld, nrhs);
   count_launch();
   return cudaGetLastError();
 }
@@ -1912,7 +1941,7 @@ cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, in
       cudaFuncSetAttribute(k_hgemv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
       attr = true;
     }
-    k_hgemv_mma<<<ntiles, 256, sm, s>>>((const float2*)P, (const float2*)xscratch, ld, ntiles,
+    launch_after(k_hgemv_mma, ntiles, 256, sm, s, (const float2*)P, (const float2*)xscratch, ld, ntiles,
                                         nrhs, (float2*)part);
     count_launch();
     return cudaGetLastError();
@@ -1920,16 +1949,16 @@ cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, in
   if (nrhs <= 4) {                               // streamed from global, one warp per tile
     const dim3 grid(ntiles);
     if (nrhs == 1)
-      k_hgemv_warp<1><<<grid, 64, 0, s>>>((const float2*)P, (const double2*)x, N, ntiles, nrhs,
+      launch_after(k_hgemv_warp<1>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
                                            (float2*)part, nullptr);
     else if (nrhs == 2)
-      k_hgemv_warp<2><<<grid, 64, 0, s>>>((const float2*)P, (const double2*)x, N, ntiles, nrhs,
+      launch_after(k_hgemv_warp<2>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
                                            (float2*)part, nullptr);
     else
-      k_hgemv_warp<4><<<grid, 64, 0, s>>>((const float2*)P, (const double2*)x, N, ntiles, nrhs,
+      launch_after(k_hgemv_warp<4>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
                                            (float2*)part, nullptr);
   } else {
-    k_hgemv_tiles<<<ntiles, 256, 0, s>>>((const float2*)P, (const double2*)x, N, nrhs,
+    launch_after(k_hgemv_tiles, ntiles, 256, 0, s, (const float2*)P, (const double2*)x, N, nrhs,
                                          (float2*)part);
   }
   count_launch();
@@ -1940,7 +1969,7 @@ cudaError_t hermitian_gemv_reduce(const void* part, void* y, int N, int ld, int 
                                   bool accumulate, cudaStream_t s, void* y32) {
   if (ld % HT || ld < N) return cudaErrorInvalidValue;
   const int nt = ld / HT;
-  k_hgemv_reduce<<<dim3(nt, nrhs), 256, 0, s>>>((const float2*)part, (double2*)y, N, nt,
+  launch_after(k_hgemv_reduce, dim3(nt, nrhs), 256, 0, s, (const float2*)part, (double2*)y, N, nt,
                                                 accumulate, (float2*)y32);
   count_launch();
   return cudaGetLastError();
@@ -1954,13 +1983,13 @@ cudaError_t hermitian_gemv_tiles_f32in(const void* P, const void* x32, int N, in
   const int nt = ld / HT, ntiles = nt * (nt + 1) / 2;
   const dim3 grid(ntiles);
   if (nrhs == 1)
-    k_hgemv_warp<1, float2><<<grid, 64, 0, s>>>((const float2*)P, (const float2*)x32, N, ntiles,
+    launch_after(k_hgemv_warp<1, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
                                                  nrhs, (float2*)part, (double2*)x64);
   else if (nrhs == 2)
-    k_hgemv_warp<2, float2><<<grid, 64, 0, s>>>((const float2*)P, (const float2*)x32, N, ntiles,
+    launch_after(k_hgemv_warp<2, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
                                                  nrhs, (float2*)part, (double2*)x64);
   else
-    k_hgemv_warp<4, float2><<<grid, 64, 0, s>>>((const float2*)P, (const float2*)x32, N, ntiles,
+    launch_after(k_hgemv_warp<4, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
                                                  nrhs, (float2*)part, (double2*)x64);
   count_launch();
   return cudaGetLastError();
@@ -1973,7 +2002,8 @@ cudaError_t hermitian_gemv_f32(const void* P, const void* x, void* y, int N, int
   return hermitian_gemv_reduce(part, y, N, ld, nrhs, accumulate, s);
 }
 
-__global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset) {
+__global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset, int dependent) {
+  pdl_wait(dependent);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Lx * Lt) return;
   const int x = i % Lx, t = i / Lx;
@@ -1983,7 +2013,7 @@ __global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int
 
 cudaError_t block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset,
                       cudaStream_t s) {
-  k_block_map<<<(Lx * Lt + 255) / 256, 256, 0, s>>>(Lx, Lt, bx, bt, coarse, offset); count_launch();
+  launch_after(k_block_map, (Lx * Lt + 255) / 256, 256, 0, s, Lx, Lt, bx, bt, coarse, offset); count_launch();
   return cudaGetLastError();
 }
 

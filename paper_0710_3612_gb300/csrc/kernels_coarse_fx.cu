@@ -120,7 +120,8 @@ __global__ void __launch_bounds__(256) k_coarse_finish(const double2* __restrict
                                                        const double2* __restrict__ G1, double m,
                                                        double2* __restrict__ A64, float2* __restrict__ A32,
                                                        __nv_bfloat162* __restrict__ A16, int4* __restrict__ W,
-                                                       int* __restrict__ E, int n, int P) {
+                                                       int* __restrict__ E, int n, int P, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ int4 wsm[];                      // [9 n][n | 1]
   const int NR = 9 * n, LD = n | 1;
   const int c = threadIdx.x & (P - 1), step = 256 / P;
@@ -165,7 +166,8 @@ __global__ void __launch_bounds__(256) k_coarse_finish(const double2* __restrict
 template <int RG>
 __global__ void __launch_bounds__(288, RG == 1 ? 1 : 2) k_coarse_fx(const double2* __restrict__ in, double2* out, const double2* __restrict__ A,
                             const int4* __restrict__ W, const int* __restrict__ E, int Lx, int Lt, int n,
-                            int nrhs, int rpc, Epilogue ep) {
+                            int nrhs, int rpc, Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ __align__(16) unsigned char csm[];
   const int NR = 9 * n;
   longlong2* sp = (longlong2*)csm;                   // [RG][NR] row sums
@@ -258,7 +260,7 @@ cudaError_t launch(const double2* x, double2* y, const double2* A, const int4* W
   static const cudaError_t e =
       cudaFuncSetAttribute(k_coarse_fx<RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
   if (e != cudaSuccess) return e;
-  k_coarse_fx<RG><<<dim3(Lx * Lt, (nrhs + rpc - 1) / rpc), (NR + 31) & ~31, smem, s>>>(
+  launch_after(k_coarse_fx<RG>, dim3(Lx * Lt, (nrhs + rpc - 1) / rpc), (NR + 31) & ~31, smem, s,
       x, y, A, W, E, Lx, Lt, n, nrhs, rpc, ep);
   return cudaGetLastError();
 }
@@ -283,11 +285,12 @@ cudaError_t coarse_finish(const void* G0, const void* G1, double m, void* A64, v
       k_coarse_finish<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
   if (e0 != cudaSuccess || e1 != cudaSuccess) return e0 != cudaSuccess ? e0 : e1;
   if (G0)
-    k_coarse_finish<true><<<(unsigned)sites, 256, smem, s>>>((const double2*)G0, (const double2*)G1, m,
+    launch_after(k_coarse_finish<true>, (unsigned)sites, 256, smem, s,
+                 (const double2*)G0, (const double2*)G1, m,
                                                              (double2*)A64, (float2*)A32,
                                                              (__nv_bfloat162*)A16, W, E, n, P);
   else
-    k_coarse_finish<false><<<(unsigned)sites, 256, smem, s>>>(nullptr, nullptr, 0.0, (double2*)A64,
+    launch_after(k_coarse_finish<false>, (unsigned)sites, 256, smem, s, nullptr, nullptr, 0.0, (double2*)A64,
                                                               (float2*)A32, (__nv_bfloat162*)A16, W, E, n,
                                                               P);
   count_launch();

@@ -142,7 +142,8 @@ template <int NDOF>
 __global__ void __launch_bounds__(448, 1)
     k_coarse_apply_tc(const __grid_constant__ CUtensorMap xmap, float2* out,
                       const __nv_bfloat162* __restrict__ A, int Lx, int Lt, int nrhs, int R,
-                      Epilogue ep) {
+                      Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   using C = CoarseTC<NDOF>;
   constexpr int n = C::n, KB = C::KB, KA = C::KA, C8 = C::C8, P = C::P, NCOL = C::NCOL;
   extern __shared__ __align__(16) unsigned char dyn[];
@@ -473,7 +474,8 @@ cudaError_t launch_tc(const void* in, void* out, const void* A, int Lx, int Lt, 
   // columns before its first site).  Strips of at most 8 sites dealt out in turn left a
   // quarter of the SM time idle at 4096 sites (4 strips for some CTAs, 3 for others).
   const int grid = (int)std::max(1LL, std::min((long long)sms, V / 2));
-  k_coarse_apply_tc<NDOF><<<grid, C::THREADS, smem, s>>>(map, (float2*)out, (const __nv_bfloat162*)A, Lx,
+  launch_after(k_coarse_apply_tc<NDOF>, grid, C::THREADS, smem, s,
+               map, (float2*)out, (const __nv_bfloat162*)A, Lx,
                                                         Lt, nrhs, R, ep);
   count_launch();
   return cudaGetLastError();

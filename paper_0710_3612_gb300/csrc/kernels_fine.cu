@@ -20,7 +20,8 @@ template <typename R, bool DAG>
 __global__ void __launch_bounds__(256) k_wilson_D(const cplx_t<R>* __restrict__ in,
                                                   cplx_t<R>* __restrict__ out,
                                                   const cplx_t<R>* __restrict__ U, R diag, int Lx,
-                                                  int Lt) {
+                                                  int Lt, int dependent) {
+  pdl_wait(dependent);
   const int V = Lx * Lt;
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   if (site >= V) return;
@@ -37,10 +38,10 @@ cudaError_t wilson_D(const void* in, void* out, const void* U, double diag, int 
   const int V = Lx * Lt;
   dim3 grid((V + 255) / 256, nrhs);
   if (dagger)
-    k_wilson_D<R, true><<<grid, 256, 0, s>>>((const cplx_t<R>*)in, (cplx_t<R>*)out,
+    launch_after(k_wilson_D<R, true>, grid, 256, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
                                              (const cplx_t<R>*)U, (R)diag, Lx, Lt);
   else
-    k_wilson_D<R, false><<<grid, 256, 0, s>>>((const cplx_t<R>*)in, (cplx_t<R>*)out,
+    launch_after(k_wilson_D<R, false>, grid, 256, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
                                               (const cplx_t<R>*)U, (R)diag, Lx, Lt);
   count_launch();
   return cudaGetLastError();
@@ -62,7 +63,8 @@ template <typename R, int TX, int TY, int RPT>
 __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict__ in,
                                                      cplx_t<R>* out,
                                                      const cplx_t<R>* __restrict__ U, R diag,
-                                                     int Lx, int Lt, Epilogue ep) {
+                                                     int Lx, int Lt, Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   constexpr int TT = TY * RPT;
   constexpr int PW = TX + 4, PH = TT + 4;     // psi region [-2, TX+1] x [-2, TT+1]
   constexpr int DW = TX + 2, DH = TT + 2;     // D psi region [-1, TX] x [-1, TT]
@@ -234,7 +236,8 @@ static constexpr int SNB = 4;
 
 __global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __restrict__ in, double2* out,
                                                            const double2* __restrict__ U, double diag,
-                                                           int Lx, int Lt, Epilogue ep) {
+                                                           int Lx, int Lt, Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   using R = double;
   using C = double2;
   using S = double4_32a;
@@ -422,7 +425,8 @@ static constexpr int SOUT2 = 60;           // output sites per warp
 
 __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __restrict__ in, float2* out,
                                                              const float2* __restrict__ U, float diag,
-                                                             int Lx, int Lt, int rows, Epilogue ep) {
+                                                             int Lx, int Lt, int rows, Epilogue ep, int dependent) {
+  pdl_wait(dependent);
   __shared__ float4 ring_psi[4][SNB][2][32];           // [warp][slot][site][lane]
   __shared__ float4 ring_u[4][SNB][2][32];             // [warp][slot][direction][lane]
   const int V = Lx * Lt;
@@ -539,7 +543,7 @@ static void launch_wilson_A(const void* in, void* out, const void* U, double dia
                         sizeof(R) * 4 * (TY * RPT + 3) * (TX + 3) <= 48 * 1024,
                 "tile above the static shared-memory limit");
   dim3 grid((Lx + TX - 1) / TX, (Lt + TY * RPT - 1) / (TY * RPT), nrhs);
-  k_wilson_A<R, TX, TY, RPT><<<grid, TX * TY, 0, s>>>((const cplx_t<R>*)in, (cplx_t<R>*)out,
+  launch_after(k_wilson_A<R, TX, TY, RPT>, grid, TX * TY, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
                                                       (const cplx_t<R>*)U, (R)diag, Lx, Lt, ep);
 }
 
@@ -611,11 +615,11 @@ static cudaError_t launch_variant(int v, const void* in, void* out, const void* 
       if constexpr (sizeof(R) == 4) {
         const int rows = stream32_rows(Lx, Lt, nrhs);
         const long long warps = stream32_warps(Lx, Lt, 1, rows);
-        k_wilson_A_stream2<<<dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s>>>(
+        launch_after(k_wilson_A_stream2, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
             (const float2*)in, (float2*)out, (const float2*)U, (float)diag, Lx, Lt, rows, ep);
       } else {
         const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
-        k_wilson_A_stream<<<dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s>>>(
+        launch_after(k_wilson_A_stream, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
             (const double2*)in, (double2*)out, (const double2*)U, diag, Lx, Lt, ep);
       }
       break;
@@ -652,7 +656,8 @@ static int tuned_variant(int Lx, int Lt, int nrhs, bool fx) {
 }
 
 __global__ void k_count_diff(const unsigned long long* __restrict__ a,
-                             const unsigned long long* __restrict__ b, long long n, int* diff) {
+                             const unsigned long long* __restrict__ b, long long n, int* diff, int dependent) {
+  pdl_wait(dependent);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     if (a[i] != b[i]) atomicAdd(diff, 1);
@@ -685,7 +690,7 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
     launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     int diff = 0;
     cudaMemsetAsync(dflag, 0, sizeof(int), s);
-    k_count_diff<<<152, 256, 0, s>>>((const unsigned long long*)out,
+    launch_after(k_count_diff, 152, 256, 0, s, (const unsigned long long*)out,
                                      (const unsigned long long*)ref, words, dflag);
     cudaMemcpyAsync(&diff, dflag, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t err = cudaStreamSynchronize(s);
@@ -761,7 +766,8 @@ cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, do
 }
 
 // out = sigma_3 in on V two-spinors (FP64): spin component 1 negated.
-__global__ void k_sigma3(const double2* __restrict__ in, double2* out, long long V) {
+__global__ void k_sigma3(const double2* __restrict__ in, double2* out, long long V, int dependent) {
+  pdl_wait(dependent);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V) return;
   const double2 a = in[2 * i], b = in[2 * i + 1];
@@ -770,14 +776,15 @@ __global__ void k_sigma3(const double2* __restrict__ in, double2* out, long long
 }
 
 cudaError_t sigma3_mul(const void* in, void* out, long long V, cudaStream_t s) {
-  k_sigma3<<<(unsigned)((V + 255) / 256), 256, 0, s>>>((const double2*)in, (double2*)out, V);
+  launch_after(k_sigma3, (unsigned)((V + 255) / 256), 256, 0, s, (const double2*)in, (double2*)out, V);
   count_launch();
   return cudaGetLastError();
 }
 
 template <typename R>
 __global__ void k_fold_links(const double2* __restrict__ g, cplx_t<R>* __restrict__ U, int Lx,
-                             int Lt) {
+                             int Lt, int dependent) {
+  pdl_wait(dependent);
   const int V = Lx * Lt;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * V) return;
@@ -790,13 +797,16 @@ __global__ void k_fold_links(const double2* __restrict__ g, cplx_t<R>* __restric
 template <typename R>
 cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s) {
   const int n = 2 * Lx * Lt;
-  k_fold_links<R><<<(n + 255) / 256, 256, 0, s>>>((const double2*)gauge, (cplx_t<R>*)U, Lx, Lt); count_launch();
+  launch_after(k_fold_links<R>, (n + 255) / 256, 256, 0, s,
+               (const double2*)gauge, (cplx_t<R>*)U, Lx, Lt);
+  count_launch();
   return cudaGetLastError();
 }
 
 // Non-negative doubles (and NaN above them) order like their bit patterns.
 __global__ void __launch_bounds__(256) k_link_unitarity(const double2* __restrict__ g, long long count,
-                                                        unsigned long long* out) {
+                                                        unsigned long long* out, int dependent) {
+  pdl_wait(dependent);
   unsigned long long m = 0;
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < count; i += 256LL * gridDim.x) {
     const double2 u = g[i];
@@ -811,7 +821,7 @@ cudaError_t link_unitarity(const void* gauge, long long count, double* out, cuda
   const cudaError_t e = cudaMemsetAsync(out, 0, sizeof(double), s);
   if (e != cudaSuccess) return e;
   const long long g = (count + 255) / 256;
-  k_link_unitarity<<<(unsigned)(g < 1216 ? g : 1216), 256, 0, s>>>((const double2*)gauge, count,
+  launch_after(k_link_unitarity, (unsigned)(g < 1216 ? g : 1216), 256, 0, s, (const double2*)gauge, count,
                                                                  (unsigned long long*)out);
   count_launch();
   return cudaGetLastError();

@@ -151,7 +151,8 @@ struct FxTile {
 // 10.2 us, 210 x 90 x 12 14.4 against 71.6 us; with the fused dot 207 against 1254 us.
 // A warp-streaming form (rows in registers, shuffles along x) took 260 us there.
 template <int TX, int TY, int RPT, int MINB, int MODE>
-__global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a) {
+__global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a, int dependent) {
+  pdl_wait(dependent);
   using T = FxTile<TX, TY, RPT>;
   extern __shared__ __align__(16) unsigned char fsm[];
   longlong2* p16 = (longlong2*)fsm;
@@ -207,7 +208,8 @@ __device__ __forceinline__ long long fx_link_word(double u, double diag) {
   return w;
 }
 
-__global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ W, double diag, int n) {
+__global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ W, double diag, int n, int dependent) {
+  pdl_wait(dependent);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double2 u = U[i];
@@ -223,7 +225,7 @@ cudaError_t launch_mode(const FxArgs& a, int nrhs, cudaStream_t s) {
                            cudaFuncAttributeMaxDynamicSharedMemorySize, T::BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.Lx + TX - 1) / TX, (a.Lt + T::TT - 1) / T::TT, nrhs);
-  k_wilson_A_fx<TX, TY, RPT, MINB, MODE><<<grid, TX * TY, T::BYTES, s>>>(a);
+  launch_after(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>, grid, TX * TY, T::BYTES, s, a);
   return cudaGetLastError();
 }
 
@@ -253,7 +255,7 @@ FxScale make_scale(double ca, double diag) {
 
 cudaError_t fixed_links(const void* U64, void* W, double diag, int Lx, int Lt, cudaStream_t s) {
   const int n = 2 * Lx * Lt;
-  k_fixed_links<<<(n + 255) / 256, 256, 0, s>>>((const double2*)U64, (int4*)W, diag, n);
+  launch_after(k_fixed_links, (n + 255) / 256, 256, 0, s, (const double2*)U64, (int4*)W, diag, n);
   count_launch();
   return cudaGetLastError();
 }

@@ -39,7 +39,8 @@ __device__ __forceinline__ double uniform53(unsigned hi, unsigned lo) {
 // given parity (they share no plaquette).  theta: [2][Lt][Lx] angles.
 __global__ void k_metropolis_half(double* __restrict__ theta, int Lx, int Lt, double beta,
                                   double eps, int mu, int parity, unsigned long long half,
-                                  uint2 key, unsigned long long* accepted) {
+                                  uint2 key, unsigned long long* accepted, int dependent) {
+  pdl_wait(dependent);
   constexpr double PI = 3.141592653589793, TWO_PI = 6.283185307179586;
   const int n = Lx * Lt / 2;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -100,7 +101,8 @@ __global__ void k_metropolis_half(double* __restrict__ theta, int Lx, int Lt, do
 }
 
 __global__ void k_links_from_angles(const double* __restrict__ theta, double2* __restrict__ U,
-                                    long long n) {
+                                    long long n, int dependent) {
+  pdl_wait(dependent);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s, c;
@@ -116,7 +118,7 @@ cudaError_t gauge_metropolis(double* theta, int Lx, int Lt, double beta, double 
   for (long long sw = first_sweep; sw < first_sweep + sweeps; ++sw)
     for (int mu = 0; mu < 2; ++mu)
       for (int parity = 0; parity < 2; ++parity) {
-        k_metropolis_half<<<(n + 255) / 256, 256, 0, s>>>(
+        launch_after(k_metropolis_half, (n + 255) / 256, 256, 0, s,
             theta, Lx, Lt, beta, eps, mu, parity, (unsigned long long)(4 * sw + 2 * mu + parity),
             key, accepted);
         count_launch();
@@ -125,7 +127,7 @@ cudaError_t gauge_metropolis(double* theta, int Lx, int Lt, double beta, double 
 }
 
 cudaError_t links_from_angles(const double* theta, void* U, long long n, cudaStream_t s) {
-  k_links_from_angles<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(theta, (double2*)U, n);
+  launch_after(k_links_from_angles, (unsigned)((n + 255) / 256), 256, 0, s, theta, (double2*)U, n);
   count_launch();
   return cudaGetLastError();
 }

@@ -87,7 +87,8 @@ __device__ __forceinline__ void gt_copy8(uint32_t dst, const void* src) {
 
 __global__ void __launch_bounds__(GT_THREADS, 1)
     k_hgemv_tc(const float2* __restrict__ P, const float2* __restrict__ xs, int ld, int nt, int nrhs,
-               float* __restrict__ part) {
+               float* __restrict__ part, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ __align__(16) unsigned char gt_dyn[];
   __shared__ __align__(8) uint64_t full[GT_SLOTS], empty[GT_SLOTS], done[2], accfree[2];
   __shared__ uint32_t tmem_sh;
@@ -261,7 +262,8 @@ __global__ void __launch_bounds__(GT_THREADS, 1)
 // The column shares of a row added in order.
 __global__ void __launch_bounds__(128) k_hgemv_tc_sum(const float* __restrict__ part, double2* __restrict__ y,
                                                       int N, int ld, int splits, bool accumulate,
-                                                      float2* __restrict__ y32) {
+                                                      float2* __restrict__ y32, int dependent) {
+  pdl_wait(dependent);
   const int row = blockIdx.x * 128 + threadIdx.x, r = blockIdx.y, nrhs = gridDim.y;
   if (row >= N) return;
   float2 a = make_float2(0.f, 0.f);
@@ -312,9 +314,11 @@ cudaError_t hermitian_gemv_tc(const void* P, const void* x, void* y, int N, int 
   const cudaError_t ex = to_f32_padded(x, xscratch, N, ld, nrhs, s);
   if (ex != cudaSuccess) return ex;
   const int nt = ld / GT_T, splits = gt_splits(nt);
-  k_hgemv_tc<<<dim3((nt + 1) / 2, splits), GT_THREADS, GT_SMEM, s>>>((const float2*)P, (const float2*)xscratch,
+  launch_after(k_hgemv_tc, dim3((nt + 1) / 2, splits), GT_THREADS, GT_SMEM, s,
+               (const float2*)P, (const float2*)xscratch,
                                                                      ld, nt, nrhs, (float*)part);
-  k_hgemv_tc_sum<<<dim3((N + 127) / 128, nrhs), 128, 0, s>>>((const float*)part, (double2*)y, N, ld, splits,
+  launch_after(k_hgemv_tc_sum, dim3((N + 127) / 128, nrhs), 128, 0, s,
+               (const float*)part, (double2*)y, N, ld, splits,
                                                              accumulate, (float2*)y32);
   count_launch();
   count_launch();

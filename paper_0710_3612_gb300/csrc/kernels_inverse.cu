@@ -139,7 +139,8 @@ struct GroupArgs {
   float2 *C, *N;                                 // panel tiles per slot
 };
 
-__global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M, int ld, GroupArgs g) {
+__global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
+  pdl_wait(dependent);
   __shared__ float2 a[B * LA], tmp[16 * 48];
   const long long k = g.next[blockIdx.x];
   for (int q = threadIdx.x; q < TILE; q += 256) a[(q / B) * LA + q % B] = M[(k * B + q / B) * ld + k * B + q % B];
@@ -153,7 +154,8 @@ __global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M,
 // the pivot tile itself becomes P.  Four CTAs per (block, pivot), 16 rows of C_b each: they
 // read and write only their own rows (or columns) of the stored tile.  A group has 20 to 72
 // panels, too few to fill the GPU with one CTA each (12 us; four 7 to 10 us).
-__global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int ld, GroupArgs g) {
+__global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
+  pdl_wait(dependent);
   __shared__ __align__(16) float2 sP[B * B];
   __shared__ __align__(16) float2 sX[16 * (B + 1)];
   const int3 e = g.panels[blockIdx.x];
@@ -228,7 +230,8 @@ __global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int l
 // (-im, re) for d = 1; m16n8k8 TF32 with three products per FP32-accurate product.  8 warps
 // in a 2 x 4 grid, 32 x 32 real outputs each; lane (g, t) holds complex outputs (row g or
 // g + 8, column t) of each 16 x 4 complex sub-tile.
-__global__ void __launch_bounds__(256, 3) k_gji_update(float2* __restrict__ M, int ld, GroupArgs g) {
+__global__ void __launch_bounds__(256, 3) k_gji_update(float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
+  pdl_wait(dependent);
   extern __shared__ float2 usm[];
   float2* sC = usm;                              // C_I [64][LD]
   float2* sN = usm + B * LD;                     // N_J [64][LD]
@@ -450,7 +453,7 @@ cudaError_t inverse_first(void* M, int ld, const InversePlan& plan, const int* d
   GroupArgs g{};
   g.next = data + plan.first;
   g.Pnext = (float2*)work + (size_t)2 * ld * B;
-  k_gji_first<<<plan.groups[0].npiv, 256, 0, s>>>((const float2*)M, ld, g);
+  launch_after(k_gji_first, plan.groups[0].npiv, 256, 0, s, (const float2*)M, ld, g);
   count_launch();
   return cudaGetLastError();
 }
@@ -465,11 +468,11 @@ cudaError_t inverse_group(void* M, int ld, const InversePlan& plan, const int* d
               (float2*)work, (float2*)work + (size_t)ld * B};
   const size_t smem = 2 * B * LD * sizeof(float2);
   if (!update) {
-    k_gji_panel<<<dim3(G.npanels, B / 16), 256, 0, s>>>((float2*)M, ld, g);
+    launch_after(k_gji_panel, dim3(G.npanels, B / 16), 256, 0, s, (float2*)M, ld, g);
   } else {
     const int grid = G.nnext + G.nact * (G.nact + 1) / 2;
     if (grid == 0) return cudaSuccess;
-    k_gji_update<<<grid, 256, smem, s>>>((float2*)M, ld, g);
+    launch_after(k_gji_update, grid, 256, smem, s, (float2*)M, ld, g);
   }
   count_launch();
   return cudaGetLastError();

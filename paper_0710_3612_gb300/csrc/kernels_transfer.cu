@@ -63,7 +63,8 @@ struct Lane {
 };
 
 template <int ROWS, int NV, int H2, int BXW>
-__global__ void __launch_bounds__(128) k_restrict_reg(const TransferArgs t) {
+__global__ void __launch_bounds__(128) k_restrict_reg(const TransferArgs t, int dependent) {
+  pdl_wait(dependent);
   using G = Geo<ROWS, NV, H2, BXW>;
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const int run = w % t.runs, jt = w / t.runs;
@@ -137,7 +138,8 @@ __global__ void __launch_bounds__(128) k_restrict_reg(const TransferArgs t) {
 }
 
 template <int ROWS, int NV, int H2, int BXW, bool ACC>
-__global__ void __launch_bounds__(128) k_prolong_reg(const TransferArgs t) {
+__global__ void __launch_bounds__(128) k_prolong_reg(const TransferArgs t, int dependent) {
+  pdl_wait(dependent);
   const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int run = w % t.runs, jt = w / t.runs;
   if (jt >= t.Lt / t.bt) return;
@@ -194,11 +196,11 @@ cudaError_t launch(TransferArgs t, bool prolong, bool acc, cudaStream_t s) {
   t.chunk = chunk_of(warps, t.nrhs);
   const dim3 grid((unsigned)((warps + 3) / 4), (t.nrhs + t.chunk - 1) / t.chunk);
   if (!prolong)
-    k_restrict_reg<ROWS, NV, H2, BXW><<<grid, 128, 0, s>>>(t);
+    launch_after(k_restrict_reg<ROWS, NV, H2, BXW>, grid, 128, 0, s, t);
   else if (acc)
-    k_prolong_reg<ROWS, NV, H2, BXW, true><<<grid, 128, 0, s>>>(t);
+    launch_after(k_prolong_reg<ROWS, NV, H2, BXW, true>, grid, 128, 0, s, t);
   else
-    k_prolong_reg<ROWS, NV, H2, BXW, false><<<grid, 128, 0, s>>>(t);
+    launch_after(k_prolong_reg<ROWS, NV, H2, BXW, false>, grid, 128, 0, s, t);
   return cudaGetLastError();
 }
 
