@@ -47,7 +47,7 @@
 // outputs written by the converting warps, conversion and output of a site ran one
 // after the other.  4096 sites of 16 dof, 64 right-hand sides: 58 -> 55 us, in the V-cycle
 // (whose epilogue operands are then loaded ahead) 8% of the batched solve; 47 us with even
-// shares of sites.  Every wait is bounded: one
+// shares of sites (44 back to back with dependent launches).  Every wait is bounded: one
 // that runs out sets the flag read by coarse_tc_take_error, and the CTA
 // frees its tensor memory and returns.
 #include <algorithm>
