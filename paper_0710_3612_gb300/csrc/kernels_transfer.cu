@@ -12,6 +12,10 @@
 // shared-memory kernels (k_restrict_multi, k_prolong_multi) read two shared operands
 // for every complex product and keep one site per CTA in flight: 256^2, 64 right-hand
 // sides, 84 and 101 us against 36 and 36 us here (109 MB each, 3.0 TB/s).
+//
+// Rounding: sums run in short chains added pairwise (two halves of the rows, four chains
+// of the vectors), since one chain of Nv products was further from the exact result than
+// the shared-memory kernels' trees at one right-hand side (Nv = 12: 9.3e-8 against 6.5e-8).
 #include <type_traits>
 
 #include "common.cuh"
@@ -85,9 +89,11 @@ __global__ void __launch_bounds__(128) k_restrict_reg(const TransferArgs t, int 
     float2 acc[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
-      acc[k] = make_float2(0.f, 0.f);
+      float2 hi = make_float2(0.f, 0.f);               // the rows in two halves
+      acc[k] = hi;
 #pragma unroll
-      for (int q = 0; q < ROWS; ++q) cfmac(acc[k], v[q][k], r[q]);
+      for (int q = 0; q < ROWS; ++q) cfmac(q < ROWS / 2 ? acc[k] : hi, v[q][k], r[q]);
+      acc[k] = cadd(acc[k], hi);
     }
     int k0 = 0;
     bool writer = l.on || l.a >= t.h;                  // lanes past h hold sums of others too
@@ -164,12 +170,13 @@ __global__ void __launch_bounds__(128) k_prolong_reg(const TransferArgs t, int d
     float2 s[ROWS];
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) {
-      s[q] = make_float2(0.f, 0.f);
+      float2 p[4] = {};                                // four sums: see the rounding above
 #pragma unroll
       for (int k = 0; k < NV / 2; ++k) {
-        cfma(s[q], v[q][2 * k], make_float2(e[k].x, e[k].y));
-        cfma(s[q], v[q][2 * k + 1], make_float2(e[k].z, e[k].w));
+        cfma(p[2 * k % 4], v[q][2 * k], make_float2(e[k].x, e[k].y));
+        cfma(p[2 * k % 4 + 1], v[q][2 * k + 1], make_float2(e[k].z, e[k].w));
       }
+      s[q] = cadd(cadd(p[0], p[1]), cadd(p[2], p[3]));
     }
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) t.out[rhs * nf + l.off[q]] = ACC ? cadd(f[q], s[q]) : s[q];
