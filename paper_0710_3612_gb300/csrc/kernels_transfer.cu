@@ -11,10 +11,10 @@
 // Bound by HBM and latency: per right-hand side a fine entry is 8 bytes and 4 Nv FMAs.  The
 // shared-memory kernels (k_restrict_multi, k_prolong_multi) read two shared operands
 // for every complex product and keep one site per CTA in flight: 256^2, 64 right-hand
-// sides, 84 and 101 us against 36 and 36 us here (109 MB each, 3.0 TB/s).
+// sides, 84 and 101 us against 37 and 37 us here (109 MB each, 3.0 TB/s).
 //
-// Rounding: sums run in short chains added pairwise (two halves of the rows, four chains
-// of the vectors), since one chain of Nv products was further from the exact result than
+// Rounding: sums run in short chains added pairwise (two halves of the rows, four or
+// six chains of the vectors), since one chain of Nv products was further from the exact result than
 // the shared-memory kernels' trees at one right-hand side (Nv = 12: 9.3e-8 against 6.5e-8).
 #include <type_traits>
 
@@ -170,13 +170,15 @@ __global__ void __launch_bounds__(128) k_prolong_reg(const TransferArgs t, int d
     float2 s[ROWS];
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) {
-      float2 p[4] = {};                                // four sums: see the rounding above
+      constexpr int CH = NV == 12 ? 6 : 4;             // chains: see the rounding above
+      float2 p[CH] = {};
 #pragma unroll
       for (int k = 0; k < NV / 2; ++k) {
-        cfma(p[2 * k % 4], v[q][2 * k], make_float2(e[k].x, e[k].y));
-        cfma(p[2 * k % 4 + 1], v[q][2 * k + 1], make_float2(e[k].z, e[k].w));
+        cfma(p[2 * k % CH], v[q][2 * k], make_float2(e[k].x, e[k].y));
+        cfma(p[2 * k % CH + 1], v[q][2 * k + 1], make_float2(e[k].z, e[k].w));
       }
       s[q] = cadd(cadd(p[0], p[1]), cadd(p[2], p[3]));
+      if constexpr (CH == 6) s[q] = cadd(s[q], cadd(p[4], p[5]));
     }
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) t.out[rhs * nf + l.off[q]] = ACC ? cadd(f[q], s[q]) : s[q];
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(128) k_prolong_reg(const TransferArgs t, int d
 }
 
 // Right-hand sides per warp: enough chunks for 16 warps on every SM.  256^2 x 64, restriction
-// and prolongation together: 72 us; half as many right-hand sides per warp 84, a quarter 103
+// and prolongation together: 74 us; half as many right-hand sides per warp 84, a quarter 103
 // (the vectors are read again for each chunk), twice as many 68 but the solve 1% slower.
 int chunk_of(long long warps, int nrhs) {
   int chunk = nrhs;
