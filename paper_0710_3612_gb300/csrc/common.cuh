@@ -24,15 +24,24 @@ unsigned long long launch_count();
 // already: with the wait in every kernel the 64-source solve on 256^2 took 2% longer.
 static constexpr long long PDL_MAX_CTAS = 152 * 16;
 
-__device__ __forceinline__ void pdl_wait(int dependent) {
-  if (dependent) asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-// A pointer for read-only loads (__ldg), which a compiler may move past the wait's memory
-// clobber but not ahead of this.
+// A pointer whose loads may not be moved ahead of this.  A kernel's `const T* __restrict__`
+// argument and __ldg promise data that nobody writes while the kernel runs, which lets a
+// compiler move loads over the wait's memory clobber; behind a wait that promise holds only
+// from here on.  The pointer that comes out carries no such promise of its own; it is made
+// from a global address again, or its loads would be generic ones, which may meet the stores
+// to shared memory around them (one-source solve on 128^2 11.2 ms against 10.8 to 11.1).
 template <typename T>
-__device__ __forceinline__ const T* pdl_ordered(const T* p) {
-  asm volatile("" : "+l"(p)::"memory");
-  return p;
+__device__ __forceinline__ void pdl_ordered(T& p) {
+  size_t g = __cvta_generic_to_global((const void*)p);
+  asm volatile("" : "+l"(g)::"memory");
+  p = (T)__cvta_global_to_generic(g);
+}
+// p: every pointer argument of the kernel.  (Pointers inside structure arguments are not
+// declared restrict: their loads stay behind the clobber.)
+template <typename... T>
+__device__ __forceinline__ void pdl_wait(int dependent, T&... p) {
+  if (dependent) asm volatile("griddepcontrol.wait;" ::: "memory");
+  (pdl_ordered(p), ...);
 }
 
 // Launches kernel(args..., dependent).

@@ -38,7 +38,7 @@ template <typename R, bool NORM>
 __global__ void __launch_bounds__(RT) k_dot(const cplx_t<R>* __restrict__ a,
                                             const cplx_t<R>* __restrict__ b, long long count,
                                             double* ws, double* out, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, a, b, ws, out);
   constexpr int N = NORM ? 1 : 2;
   __shared__ double sh[N * RT];
   const int rhs = blockIdx.y;
@@ -92,7 +92,7 @@ static inline dim3 grid1(long long count, int nrhs) {
 template <typename R>
 __global__ void k_axpby(R a, const cplx_t<R>* __restrict__ x, R b, cplx_t<R>* __restrict__ y,
                         long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, y);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   i += (long long)blockIdx.y * count;
@@ -111,7 +111,7 @@ cudaError_t axpby(double a, const void* x, double b, void* y, long long count, i
 template <typename R>
 __global__ void __launch_bounds__(RT) k_scale_inv_sqrt(const cplx_t<R>* x, cplx_t<R>* y,
                                                        const double* nrm, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, y, nrm);
   __shared__ double ssc;                             // one root and division per block
   if (threadIdx.x == 0) {
     const double n2 = nrm[2 * blockIdx.y];
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(RT) k_cg_xr(cplx_t<R>* __restrict__ x, cplx_t<
                                               const double* pq, const int* frozen,
                                               long long count, double* ws, double* rr,
                                               float2* __restrict__ r32, CgControl cc, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, r, p, q, rz, pq, frozen, ws, rr, r32);
   __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
@@ -195,7 +195,7 @@ template <typename R>
 __global__ void __launch_bounds__(RT) k_cg_p(cplx_t<R>* __restrict__ p, const cplx_t<R>* __restrict__ z,
                                              const double* rz_new, const double* rz_old,
                                              const int* frozen, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, p, z, rz_new, rz_old, frozen);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const R beta = (R)block_ratio(rz_new[2 * rhs], rz_old[2 * rhs]);
@@ -257,7 +257,7 @@ __device__ void cg_control_step(const double* rr, const double* pq, const double
 
 __global__ void k_cg_control(const double* rr, const double* pq, const double* stop, int* ctrl,
                              cudaGraphConditionalHandle cond, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, rr, pq, stop, ctrl);
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   cg_control_step(rr, pq, stop, ctrl, cond);
 }
@@ -273,7 +273,7 @@ cudaError_t cg_control(const double* rr, const double* pq, const double* stop, i
 // b = 0 start frozen (x = 0 is exact).
 __global__ void k_set_control(int* ctrl, int maxiter, int nrhs, const double* bn, double tol2,
                               double* stop, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, ctrl, bn, stop);
   if (threadIdx.x != 0) return;
   ctrl[0] = 0;
   ctrl[1] = 0;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
                                                    const double2* __restrict__ q,
                                                    const double2* __restrict__ r, long long count,
                                                    double* ws, double* zr, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, z, q, r, ws, zr);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   double a = 0.0, b = 0.0;
@@ -331,7 +331,7 @@ cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long 
 __global__ void __launch_bounds__(RT) k_cg_p_pr(double2* __restrict__ p, const float2* __restrict__ z,
                                                 const double* zr, const double* pq, double* rz,
                                                 const int* frozen, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, p, z, zr, pq, rz, frozen);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const double beta = block_ratio(-zr[2 * rhs], pq[2 * rhs]);
@@ -368,7 +368,7 @@ cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq
 __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
                                              const float2* __restrict__ b, long long count,
                                              double* ws, double* out, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, a, b, ws, out);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float re = 0.f, im = 0.f;
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
                                                const float2* __restrict__ q, const double* rz,
                                                const double* pq, const int* frozen,
                                                long long count, double* ws, double* rr, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, r, p, q, rz, pq, frozen, ws, rr);
   __shared__ double sh[RT];
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
                                                     const float2* __restrict__ q,
                                                     const float2* __restrict__ r, long long count,
                                                     double* ws, double* zr, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, z, q, r, ws, zr);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
   float a = 0.f, b = 0.f;
@@ -462,7 +462,7 @@ cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long 
 __global__ void __launch_bounds__(RT) k_rcg_p(float2* __restrict__ p, const float2* __restrict__ z,
                                               const double* zr, const double* pq, double* rz,
                                               const int* frozen, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, p, z, zr, pq, rz, frozen);
   const int rhs = blockIdx.y;
   if (frozen && frozen[rhs]) return;
   const float beta = (float)block_ratio(-zr[2 * rhs], pq[2 * rhs]);
@@ -491,7 +491,7 @@ cudaError_t rcg_p(void* p32, const void* z32, const double* zr, const double* pq
 // *due (and the IF condition of the enclosing graph node when cond_set).
 __global__ void k_ru_check(const double* rr, double* rmax, const int* ctrl, double delta2,
                            int* due, int* count, cudaGraphConditionalHandle cond, int cond_set, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, rr, rmax, ctrl, due, count);
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const int nrhs = ctrl[3];
   const int* frozen = ctrl + 4;
@@ -516,7 +516,7 @@ cudaError_t ru_check(const double* rr, double* rmax, const int* ctrl, double del
 
 // x64 += x32, x32 = 0 (the FP32 increment folded into the FP64 solution).
 __global__ void k_ru_fold(double2* __restrict__ x, float2* __restrict__ x32, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, x32);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const float2 v = x32[i];
@@ -535,7 +535,7 @@ cudaError_t ru_fold(void* x64, void* x32, long long count, cudaStream_t s) {
 __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ r,
                                                     float2* __restrict__ r32, long long count,
                                                     double* ws, double* rr, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, r, r32, ws, rr);
   __shared__ double sh[RT];
   const long long base = (long long)blockIdx.y * count;
   double acc = 0.0;
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(RT) k_ru_residual(const double2* __restrict__ 
 }
 
 __global__ void k_copy_slots(const double* src, double* dst, int n2, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, src, dst);
   const int i = threadIdx.x;
   if (i < n2) dst[i] = src[i];
 }
@@ -570,7 +570,7 @@ cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, d
 
 __global__ void k_f64_to_f32_scaled(const double2* __restrict__ in, float2* __restrict__ out,
                                     const double* nrm, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, nrm);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const double n2 = nrm[2 * blockIdx.y];
@@ -589,7 +589,7 @@ cudaError_t f64_to_f32_scaled(const void* in, void* out, const double* nrm, long
 
 __global__ void k_f32_acc_scaled(const float2* __restrict__ in, double2* __restrict__ x,
                                  const double* nrm, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, x, nrm);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const double sc = nrm ? sqrt(nrm[2 * blockIdx.y]) : 1.0;
@@ -609,13 +609,13 @@ cudaError_t f32_accumulate_scaled(const void* in, void* x, const double* nrm, lo
 
 __global__ void k_cvt_64_32(const double2* __restrict__ in, float2* __restrict__ out,
                             long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 __global__ void k_cvt_32_64(const float2* __restrict__ in, double2* __restrict__ out,
                             long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) out[i] = make_double2(in[i].x, in[i].y);
 }
@@ -631,7 +631,7 @@ cudaError_t convert_f32_f64(const void* in, void* out, long long count, cudaStre
 template <typename R>
 __global__ void k_lincomb(cplx_t<R>* out, R a, const cplx_t<R>* u, R b, const cplx_t<R>* v, R c,
                           const cplx_t<R>* w, long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, out, u, v, w);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   i += (long long)blockIdx.y * count;
@@ -657,7 +657,7 @@ cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v,
 template <typename R>
 __global__ void k_sub_from(const cplx_t<R>* __restrict__ b, cplx_t<R>* __restrict__ r,
                            long long count, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, b, r);
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) r[i] = csub(b[i], r[i]);
 }

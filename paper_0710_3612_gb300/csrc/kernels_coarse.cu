@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(576, 2) k_coarse_apply(const cplx_t<R>* __rest
                                                       cplx_t<R>* out,
                                                       const WT* __restrict__ A, int Lx, int Lt,
                                                       int n, Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, A);
   extern __shared__ unsigned char smraw[];
   cplx_t<R>* xs = (cplx_t<R>*)smraw;            // [9][n] neighbour vectors
   cplx_t<R>* part = xs + 9 * n;                 // [9][n] partial row products
@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(576, 2) k_coarse_apply(const cplx_t<R>* __rest
   if constexpr (kBf16) {
     if (pre && threadIdx.x < 9 * n) {
       const int d = threadIdx.x / n, r = threadIdx.x % n;
-      const uint4* row4 = pdl_ordered((const uint4*)(A + (((long long)j * 9 + d) * n + r) * n));
+      const uint4* row4 = (const uint4*)(A + (((long long)j * 9 + d) * n + r) * n);
 #pragma unroll
       for (int k = 0; k < PRE; ++k)
         if (k < n / 4) rv[k] = __ldg(row4 + k);
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(64) k_coarse_apply_mma(const float2* __restric
                                                          const __nv_bfloat162* __restrict__ A,
                                                          int Lx, int Lt, int n, int nrhs,
                                                          Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, A);
   extern __shared__ __nv_bfloat162 Xs[];
   constexpr int RS = MMA_RC + 8;             // padded row: conflict-free fragment loads
   const int V = Lx * Lt;
@@ -300,7 +300,7 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
 // identity blocks of the d = 4 displacement); out may alias X or Y.
 __global__ void k_coarse_lincomb(double a, const double2* X, double b, const double2* Y, double c,
                                  double2* out, long long count, int n, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, X, Y, out);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int q = (int)(i % ((long long)9 * n * n));
@@ -328,7 +328,7 @@ cudaError_t coarse_lincomb(double a, const void* X, double b, const void* Y, dou
 // ---------------------------------------------------------------------------
 __global__ void k_probe_vectors(double2* __restrict__ out, int Lxc, int Ltc, int nc, int Kx, int Kt,
                                 int cx, int ct, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, out);
   const long long Vc = (long long)Lxc * Ltc;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)nc * Vc * nc) return;
@@ -340,7 +340,7 @@ __global__ void k_probe_vectors(double2* __restrict__ out, int Lxc, int Ltc, int
 
 __global__ void k_probe_scatter(const double2* __restrict__ y, double2* __restrict__ Ac, int Lxc,
                                 int Ltc, int nc, int Kx, int Kt, int cx, int ct, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, y, Ac);
   const long long Vc = (long long)Lxc * Ltc;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= Vc * 9 * nc * nc) return;
@@ -385,7 +385,7 @@ __global__ void __launch_bounds__(256) k_restrict(const cplx_t<R>* __restrict__ 
                                                   cplx_t<R>* __restrict__ coarse,
                                                   const cplx_t<R>* __restrict__ Vst, int Lx,
                                                   int Lt, int bx, int bt, int h, int Nv, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, fine, coarse, Vst);
   const int Lxc = Lx / bx, Vc = Lxc * (Lt / bt), nc = 2 * Nv, nf = 2 * h;
   const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (w >= Vc * nc) return;
@@ -435,7 +435,7 @@ __global__ void __launch_bounds__(256) k_restrict_multi(const cplx_t<R>* __restr
                                                         const cplx_t<R>* __restrict__ Vst, int Lx,
                                                         int Lt, int bx, int bt, int h, int Nv,
                                                         int nrhs, int G, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, fine, coarse, Vst);
   using C = cplx_t<R>;
   extern __shared__ unsigned char smraw[];
   const int b2 = bx * bt, nf = 2 * h, nc = 2 * Nv, T = b2 * h, Lxc = Lx / bx, Vc = Lxc * (Lt / bt);
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(256) k_prolong_multi(const cplx_t<R>* __restri
                                                        const cplx_t<R>* __restrict__ Vst, int Lx,
                                                        int Lt, int bx, int bt, int h, int Nv,
                                                        int nrhs, bool accumulate, int G, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, coarse, fine, Vst);
   using C = cplx_t<R>;
   extern __shared__ unsigned char smraw[];
   const int b2 = bx * bt, nf = 2 * h, nc = 2 * Nv, Lxc = Lx / bx, Vc = Lxc * (Lt / bt);
@@ -558,7 +558,7 @@ template <typename R>
 __global__ void k_prolong(const cplx_t<R>* __restrict__ coarse, cplx_t<R>* __restrict__ fine,
                           const cplx_t<R>* __restrict__ Vst, int Lx, int Lt, int bx, int bt, int h,
                           int Nv, bool accumulate, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, coarse, fine, Vst);
   const int V = Lx * Lt, nf = 2 * h, nc = 2 * Nv;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= V * nf) return;
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(32) k_block_gs(const double2* __restrict__ E,
                                                  double2* __restrict__ Vst, int Lx, int Lt,
                                                  int bx, int bt, int h, int Nv, double tol,
                                                  int* flag, int nblocks, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, E, Vst, flag);
   extern __shared__ double2 Qs[];   // [32 / LPB][Nv][m]
   const int V = Lx * Lt, nf = 2 * h, Lxc = Lx / bx;
   const int sub = threadIdx.x / LPB, lane = threadIdx.x % LPB;
@@ -719,7 +719,7 @@ cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx,
 __global__ void k_galerkin_W(const double2* __restrict__ U, double diag,
                              const double2* __restrict__ Vst, double2* __restrict__ Wbuf, int Lx,
                              int Lt, int bx, int bt, int Nv, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, U, Vst, Wbuf);
   const int Lxc = Lx / bx, Vc = Lxc * (Lt / bt), nc = 2 * Nv;
   const int ex_w = bx + 2, E = (bx + 2) * (bt + 2);
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -777,7 +777,7 @@ __global__ void k_galerkin_W(const double2* __restrict__ U, double diag,
 template <bool G1>
 __global__ void k_galerkin_WW(const double2* __restrict__ Wbuf, const double2* __restrict__ Vst,
                               double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt, int Nv, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, Wbuf, Vst, Ac);
   const int Lxc = Lx / bx, Ltc = Lt / bt, nc = 2 * Nv;
   const long long Vc = (long long)Lxc * Ltc;
   const int ex_w = bx + 2, E = (bx + 2) * (bt + 2), tri = nc * (nc + 1) / 2;
@@ -872,7 +872,7 @@ cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* W
 __global__ void k_galerkin_coarse(const double2* __restrict__ Af, const double2* __restrict__ Vst,
                                   double2* __restrict__ Ac, int Lx, int Lt, int bx, int bt,
                                   int nf, int Nv, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, Af, Vst, Ac);
   extern __shared__ double2 sm[];
   const int nc = 2 * Nv, h = nf / 2, Lxc = Lx / bx;
   double2* acc = sm;                  // [9][nc][nc]
@@ -947,7 +947,7 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
 // ---------------------------------------------------------------------------
 __global__ void k_coarse_to_dense(const double2* __restrict__ A, float2* __restrict__ M, int Lx,
                                   int Lt, int n, long long ld, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, A, M);
   const int V = Lx * Lt;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)V * n * n) return;
@@ -964,7 +964,7 @@ __global__ void k_coarse_to_dense(const double2* __restrict__ A, float2* __restr
 }
 
 __global__ void k_pad_identity(float2* __restrict__ M, long long N, long long ld, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M);
   const long long i = N + (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < ld) M[i * ld + i] = make_float2(1.f, 0.f);
 }
@@ -1083,7 +1083,7 @@ __device__ void sweep_block64(float2* a, float2* tmp) {
 // Inverts the first pivot block: P = M_00^{-1}.
 __global__ void __launch_bounds__(256) k_gj_pivot0(const float2* __restrict__ M, int N,
                                                    float2* __restrict__ P, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M, P);
   extern __shared__ float2 gsm[];
   for (int q = threadIdx.x; q < GJB * GJB; q += 256)
     gsm[(q / GJB) * GJS + q % GJB] = M[(long long)(q / GJB) * N + q % GJB];
@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(256) k_gj_panel(const float2* __restrict__ M, 
                                                   float2* __restrict__ Cold,
                                                   float2* __restrict__ Cn,
                                                   float2* __restrict__ Rp, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M, P, Cold, Cn, Rp);
   extern __shared__ float2 gsm[];
   float2* sP = gsm;
   float2* sX = gsm + GJB * GJS;
@@ -1259,7 +1259,7 @@ __global__ void __launch_bounds__(256, 2) k_gj_update_tc(float2* __restrict__ M,
                                                          const float2* __restrict__ Cn,
                                                          const float2* __restrict__ Rp,
                                                          int* __restrict__ err, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M, P, Pnext, Cold, Cn, Rp, err);
   extern __shared__ __align__(16) unsigned char tc_dyn[];
   __shared__ __align__(8) uint64_t mbar;
   __shared__ uint32_t tmem_sh;
@@ -1489,7 +1489,7 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
 }
 
 __global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ xf, int N, int ld, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, xf);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < ld) xf[i] = i < N ? make_float2((float)x[i].x, (float)x[i].y) : make_float2(0.f, 0.f);
 }
@@ -1498,7 +1498,7 @@ __global__ void __launch_bounds__(256) k_gemv(const float2* __restrict__ B,
                                               const float2* __restrict__ xf,
                                               double2* __restrict__ y, int N, int ld,
                                               bool accumulate, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, B, xf, y);
   const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (row >= N) return;
   const float4* b4 = (const float4*)(B + (long long)row * ld);
@@ -1540,7 +1540,7 @@ static constexpr int HT = 64;
 
 
 __global__ void k_pack_hermitian(const float2* __restrict__ M, float2* __restrict__ P, int ld, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M, P);
   const int k = blockIdx.x;
   int I = (int)((sqrtf(8.f * k + 1.f) - 1.f) * 0.5f);
   while ((I + 1) * (I + 2) / 2 <= k) ++I;
@@ -1650,7 +1650,7 @@ __global__ void __launch_bounds__(256) k_hgemv_mma(const float2* __restrict__ P,
                                                    const float2* __restrict__ xs, int ld,
                                                    int ntiles, int nrhs,
                                                    float2* __restrict__ part, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, P, xs, part);
   extern __shared__ float2 hsm[];
   float2* sT = hsm;                                      // [64][GJC]
   float2* sXJ = sT + HT * GJC;                           // [64 k][GJR]: X_J[k][rhs]
@@ -1701,7 +1701,7 @@ __global__ void __launch_bounds__(256) k_hgemv_mma(const float2* __restrict__ P,
 
 __global__ void k_x32_pad(const double2* __restrict__ x, float2* __restrict__ xs, int N, int ld,
                           int nrhs, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, x, xs);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)ld * nrhs) return;
   const int r = (int)(i / ld), c = (int)(i % ld);
@@ -1712,7 +1712,7 @@ __global__ void k_x32_pad(const double2* __restrict__ x, float2* __restrict__ xs
 __global__ void __launch_bounds__(256) k_hgemv_tiles(const float2* __restrict__ P,
                                                      const double2* __restrict__ x, int N,
                                                      int nrhs, float2* __restrict__ part, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, P, x, part);
   __shared__ float2 T[HT][HT + 1];
   __shared__ float2 xi[HT], xj[HT];
   __shared__ float2 red[4][HT];
@@ -1801,7 +1801,7 @@ __global__ void __launch_bounds__(64) k_hgemv_warp(const float2* __restrict__ P,
                                                    int ntiles, int nrhs,
                                                    float2* __restrict__ part,
                                                    double2* __restrict__ x64, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, P, x, part, x64);
   __shared__ float4 colsum[NR][32];                      // column partials of warp 1
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int k = blockIdx.x;                              // one tile, rows split by warp
@@ -1809,7 +1809,7 @@ __global__ void __launch_bounds__(64) k_hgemv_warp(const float2* __restrict__ P,
   while ((I + 1) * (I + 2) / 2 <= k) ++I;
   while (I * (I + 1) / 2 > k) --I;
   const int J = k - I * (I + 1) / 2;
-  const float4* src = pdl_ordered((const float4*)(P + (long long)k * HT * HT)) + lane;
+  const float4* src = (const float4*)(P + (long long)k * HT * HT) + lane;
   for (int q0 = 0; q0 < nrhs; q0 += NR) {
     float2 xj0[NR], xj1[NR], xi0[NR], xi1[NR], ac0[NR], ac1[NR];
 #pragma unroll
@@ -1894,7 +1894,7 @@ __global__ void __launch_bounds__(256) k_hgemv_reduce(const float2* __restrict__
                                                       double2* __restrict__ y, int N, int nt,
                                                       bool accumulate,
                                                       float2* __restrict__ y32, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, part, y, y32);
   __shared__ float2 red[4][HT];
   const int I = blockIdx.x, rr = threadIdx.x % HT, g = threadIdx.x / HT;
   part += (long long)blockIdx.y * (nt * (nt + 1) / 2) * 2 * HT;
@@ -2003,7 +2003,7 @@ cudaError_t hermitian_gemv_f32(const void* P, const void* x, void* y, int N, int
 }
 
 __global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, coarse, offset);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= Lx * Lt) return;
   const int x = i % Lx, t = i / Lx;

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256) k_coarse_finish(const double2* __restrict
                                                        double2* __restrict__ A64, float2* __restrict__ A32,
                                                        __nv_bfloat162* __restrict__ A16, int4* __restrict__ W,
                                                        int* __restrict__ E, int n, int P, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, G0, G1, A64, A32, A16, W, E);
   extern __shared__ int4 wsm[];                      // [9 n][n | 1]
   const int NR = 9 * n, LD = n | 1;
   const int c = threadIdx.x & (P - 1), step = 256 / P;
@@ -167,7 +167,7 @@ template <int RG>
 __global__ void __launch_bounds__(288, RG == 1 ? 1 : 2) k_coarse_fx(const double2* __restrict__ in, double2* out, const double2* __restrict__ A,
                             const int4* __restrict__ W, const int* __restrict__ E, int Lx, int Lt, int n,
                             int nrhs, int rpc, Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, A, W, E);
   extern __shared__ __align__(16) unsigned char csm[];
   const int NR = 9 * n;
   longlong2* sp = (longlong2*)csm;                   // [RG][NR] row sums

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(448, 1)
     k_coarse_apply_tc(const __grid_constant__ CUtensorMap xmap, float2* out,
                       const __nv_bfloat162* __restrict__ A, int Lx, int Lt, int nrhs, int R,
                       Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, out, A);
   using C = CoarseTC<NDOF>;
   constexpr int n = C::n, KB = C::KB, KA = C::KA, C8 = C::C8, P = C::P, NCOL = C::NCOL;
   extern __shared__ __align__(16) unsigned char dyn[];

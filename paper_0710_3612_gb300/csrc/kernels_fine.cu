@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(256) k_wilson_D(const cplx_t<R>* __restrict__ 
                                                   cplx_t<R>* __restrict__ out,
                                                   const cplx_t<R>* __restrict__ U, R diag, int Lx,
                                                   int Lt, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, U);
   const int V = Lx * Lt;
   const int site = blockIdx.x * blockDim.x + threadIdx.x;
   if (site >= V) return;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
                                                      cplx_t<R>* out,
                                                      const cplx_t<R>* __restrict__ U, R diag,
                                                      int Lx, int Lt, Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, U);
   constexpr int TT = TY * RPT;
   constexpr int PW = TX + 4, PH = TT + 4;     // psi region [-2, TX+1] x [-2, TT+1]
   constexpr int DW = TX + 2, DH = TT + 2;     // D psi region [-1, TX] x [-1, TT]
@@ -237,7 +237,7 @@ static constexpr int SNB = 4;
 __global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __restrict__ in, double2* out,
                                                            const double2* __restrict__ U, double diag,
                                                            int Lx, int Lt, Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, U);
   using R = double;
   using C = double2;
   using S = double4_32a;
@@ -426,7 +426,7 @@ static constexpr int SOUT2 = 60;           // output sites per warp
 __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __restrict__ in, float2* out,
                                                              const float2* __restrict__ U, float diag,
                                                              int Lx, int Lt, int rows, Epilogue ep, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out, U);
   __shared__ float4 ring_psi[4][SNB][2][32];           // [warp][slot][site][lane]
   __shared__ float4 ring_u[4][SNB][2][32];             // [warp][slot][direction][lane]
   const int V = Lx * Lt;
@@ -657,7 +657,7 @@ static int tuned_variant(int Lx, int Lt, int nrhs, bool fx) {
 
 __global__ void k_count_diff(const unsigned long long* __restrict__ a,
                              const unsigned long long* __restrict__ b, long long n, int* diff, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, a, b, diff);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     if (a[i] != b[i]) atomicAdd(diff, 1);
@@ -767,7 +767,7 @@ cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, do
 
 // out = sigma_3 in on V two-spinors (FP64): spin component 1 negated.
 __global__ void k_sigma3(const double2* __restrict__ in, double2* out, long long V, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, in, out);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V) return;
   const double2 a = in[2 * i], b = in[2 * i + 1];
@@ -784,7 +784,7 @@ cudaError_t sigma3_mul(const void* in, void* out, long long V, cudaStream_t s) {
 template <typename R>
 __global__ void k_fold_links(const double2* __restrict__ g, cplx_t<R>* __restrict__ U, int Lx,
                              int Lt, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, g, U);
   const int V = Lx * Lt;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * V) return;
@@ -806,7 +806,7 @@ cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t 
 // Non-negative doubles (and NaN above them) order like their bit patterns.
 __global__ void __launch_bounds__(256) k_link_unitarity(const double2* __restrict__ g, long long count,
                                                         unsigned long long* out, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, g, out);
   unsigned long long m = 0;
   for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < count; i += 256LL * gridDim.x) {
     const double2 u = g[i];

@@ -209,7 +209,7 @@ __device__ __forceinline__ long long fx_link_word(double u, double diag) {
 }
 
 __global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ W, double diag, int n, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, U, W);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double2 u = U[i];

@@ -40,7 +40,7 @@ __device__ __forceinline__ double uniform53(unsigned hi, unsigned lo) {
 __global__ void k_metropolis_half(double* __restrict__ theta, int Lx, int Lt, double beta,
                                   double eps, int mu, int parity, unsigned long long half,
                                   uint2 key, unsigned long long* accepted, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, theta, accepted);
   constexpr double PI = 3.141592653589793, TWO_PI = 6.283185307179586;
   const int n = Lx * Lt / 2;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -102,7 +102,7 @@ __global__ void k_metropolis_half(double* __restrict__ theta, int Lx, int Lt, do
 
 __global__ void k_links_from_angles(const double* __restrict__ theta, double2* __restrict__ U,
                                     long long n, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, theta, U);
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s, c;

@@ -88,7 +88,7 @@ __device__ __forceinline__ void gt_copy8(uint32_t dst, const void* src) {
 __global__ void __launch_bounds__(GT_THREADS, 1)
     k_hgemv_tc(const float2* __restrict__ P, const float2* __restrict__ xs, int ld, int nt, int nrhs,
                float* __restrict__ part, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, P, xs, part);
   extern __shared__ __align__(16) unsigned char gt_dyn[];
   __shared__ __align__(8) uint64_t full[GT_SLOTS], empty[GT_SLOTS], done[2], accfree[2];
   __shared__ uint32_t tmem_sh;
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(GT_THREADS, 1)
 __global__ void __launch_bounds__(128) k_hgemv_tc_sum(const float* __restrict__ part, double2* __restrict__ y,
                                                       int N, int ld, int splits, bool accumulate,
                                                       float2* __restrict__ y32, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, part, y, y32);
   const int row = blockIdx.x * 128 + threadIdx.x, r = blockIdx.y, nrhs = gridDim.y;
   if (row >= N) return;
   float2 a = make_float2(0.f, 0.f);

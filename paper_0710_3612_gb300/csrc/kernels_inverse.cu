@@ -140,7 +140,7 @@ struct GroupArgs {
 };
 
 __global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M);
   __shared__ float2 a[B * LA], tmp[16 * 48];
   const long long k = g.next[blockIdx.x];
   for (int q = threadIdx.x; q < TILE; q += 256) a[(q / B) * LA + q % B] = M[(k * B + q / B) * ld + k * B + q % B];
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(256) k_gji_first(const float2* __restrict__ M,
 // read and write only their own rows (or columns) of the stored tile.  A group has 20 to 72
 // panels, too few to fill the GPU with one CTA each (12 us; four 7 to 10 us).
 __global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M);
   __shared__ __align__(16) float2 sP[B * B];
   __shared__ __align__(16) float2 sX[16 * (B + 1)];
   const int3 e = g.panels[blockIdx.x];
@@ -231,7 +231,7 @@ __global__ void __launch_bounds__(256) k_gji_panel(float2* __restrict__ M, int l
 // in a 2 x 4 grid, 32 x 32 real outputs each; lane (g, t) holds complex outputs (row g or
 // g + 8, column t) of each 16 x 4 complex sub-tile.
 __global__ void __launch_bounds__(256, 3) k_gji_update(float2* __restrict__ M, int ld, GroupArgs g, int dependent) {
-  pdl_wait(dependent);
+  pdl_wait(dependent, M);
   extern __shared__ float2 usm[];
   float2* sC = usm;                              // C_I [64][LD]
   float2* sN = usm + B * LD;                     // N_J [64][LD]
