@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 namespace mgk {
 
 static constexpr int FX_BITS = 58;
@@ -127,12 +129,31 @@ __host__ __device__ __forceinline__ void fx_row(FxSpinor& r, const FxSpinor& c, 
   }
 }
 
-// Output scale: y * diag^2 as FP64.  sq = {lo, hi} of diag^2 * 2^sh, sq in [2^62, 2^63).
+// Output scale: y * ca * diag^2 as FP64, the factor as q * 2^(exp - 64) in split words.
 struct FxScale { int lo, hi; int exp; };             // exp: added to the site exponent
 __host__ __device__ __forceinline__ long long fx_scale(long long y, FxScale q) {
   const int yl = fx_lo(y), yh = fx_hi(y);
   const long long m = fx_mad(q.hi, yl, (long long)q.lo * yh);
   return fx_mad(q.hi, yh, m >> 32);
+}
+// factor = q * 2^(exp - 64), |q| about 2^62 .. 2^63 - 2^31: the carry of the low word has to fit
+// into the high one.  A q above that (ca diag^2 less than 2^-32 of itself below a power of
+// two, or rounded up to one) is halved.
+inline FxScale make_scale(double ca, double diag) {
+  int ex;
+  const double f = std::frexp(diag * diag, &ex);       // the product's rounding is recovered below
+  const double lo = std::ldexp(std::fma(diag, diag, -diag * diag), -ex);
+  int ec;
+  const double c = std::frexp(std::fabs(ca), &ec);
+  double ph = f * c, pl = std::fma(f, c, -ph) + lo * c;
+  if (ph < 0.5) { ph *= 2; pl *= 2; --ex; }
+  unsigned long long m = (unsigned long long)std::ldexp(ph, 63) + (long long)std::llrint(std::ldexp(pl, 63));
+  if (m >= (1ull << 63) - (1ull << 31)) {
+    m = (m + 1) >> 1;
+    ++ex;
+  }
+  const long long q = ca < 0 ? -(long long)m : (long long)m;
+  return FxScale{fx_lo(q), fx_hi(q), ex + ec + 1};
 }
 // v * 2^(e + shift) of an FP64-representable size
 __device__ __forceinline__ double fx_double(long long v, int e) {

@@ -238,19 +238,6 @@ cudaError_t launch_tile(const FxArgs& a, int nrhs, cudaStream_t s) {
                 : launch_mode<TX, TY, RPT, MINB, FX_PLAIN>(a, nrhs, s);
 }
 
-// factor = q * 2^(exp - 64) as a 63-bit mantissa in split words
-FxScale make_scale(double ca, double diag) {
-  int ex;
-  const double f = std::frexp(diag * diag, &ex);       // the product's rounding is recovered below
-  const double lo = std::ldexp(std::fma(diag, diag, -diag * diag), -ex);
-  int ec;
-  const double c = std::frexp(ca, &ec);
-  double ph = f * c, pl = std::fma(f, c, -ph) + lo * c;
-  if (std::fabs(ph) < 0.5) { ph *= 2; pl *= 2; --ex; }
-  const long long q = (long long)std::ldexp(ph, 63) + (long long)std::llrint(std::ldexp(pl, 63));
-  return FxScale{fx_lo(q), fx_hi(q), ex + ec + 1};
-}
-
 }  // namespace
 
 cudaError_t fixed_links(const void* U64, void* W, double diag, int Lx, int Lt, cudaStream_t s) {
