@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(288, RG == 1 ? 1 : 2) k_coarse_fx(const double
 #pragma unroll
     for (int g = 0; g < RG; ++g)                     // thread (d, r) loads component r of x(j + d)
       xv[g] = row && r0 + g < r1 ? in[(r0 + g) * V * n + nb + r] : make_double2(0.0, 0.0);
-    if (tid < RG * 9) kx[tid] = 0;
+    for (int i = tid; i < RG * 9; i += blockDim.x) kx[i] = 0;   // more than a warp; n = 2 has one
     __syncthreads();                                 // kx cleared; the previous group's sums are read
     if (tid < RG) bad[tid] = 0;
 #pragma unroll
