@@ -30,8 +30,12 @@ static constexpr int CF_BAD = 1 << 20;
 // range of a row's plus a vector's exponent whose product is a normal FP64 number
 static constexpr int CF_SMIN = 1300, CF_SMAX = 2800;
 
+// The larger exponent field; 1 for subnormal numbers, so that rows or vectors of those alone
+// are told from zeros (and lie outside the range).
 __device__ __forceinline__ uint32_t exp_field(double2 v) {
-  return max((uint32_t)__double2hiint(v.x) & 0x7ff00000u, (uint32_t)__double2hiint(v.y) & 0x7ff00000u);
+  const uint32_t hx = (uint32_t)__double2hiint(v.x) & 0x7fffffffu, hy = (uint32_t)__double2hiint(v.y) & 0x7fffffffu;
+  const uint32_t k = max(hx, hy) & 0x7ff00000u, lo = (uint32_t)__double2loint(v.x) | (uint32_t)__double2loint(v.y);
+  return k == 0 && (hx | hy | lo) ? 1u << 20 : k;
 }
 // exponent of a row or vector from the largest exponent field of its entries
 __device__ __forceinline__ int scale_of(uint32_t k) {
