@@ -247,9 +247,11 @@ cudaError_t fixed_links(const void* U64, void* W, double diag, int Lx, int Lt, c
   return cudaGetLastError();
 }
 
+// Factors ca of 2^-120 .. 2^120: a result's exponent field is at least 143 + q.exp (a site at
+// FX_EMIN, one unit left of its sum) and at most 1805 + q.exp, with q.exp within 14 of ca's.
 bool wilson_A_fx_ok(const void* W, double diag, const Epilogue& ep) {
-  return W && fixed_diag_ok(diag) && !ep.zq_q && ep.ca != 0.0 && std::fabs(ep.ca) < 1e100 &&
-         std::fabs(ep.ca) > 1e-100 && (ep.U || !ep.W) && !(ep.dot_out && (ep.U || ep.ca != 1.0));
+  return W && fixed_diag_ok(diag) && !ep.zq_q && std::fabs(ep.ca) <= 0x1p120 &&
+         std::fabs(ep.ca) >= 0x1p-120 && (ep.U || !ep.W) && !(ep.dot_out && (ep.U || ep.ca != 1.0));
 }
 
 cudaError_t wilson_A_fx(int tx, int ty, const void* in, void* out, const void* U64, const void* W,
