@@ -80,8 +80,8 @@ cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long 
                        double* ws, double* zr, cudaStream_t s);
 cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq, double* rz,
                     const int* frozen, long long count, int nrhs, cudaStream_t s);
-// Reliable-update flexible CG: every vector of the iteration in FP32 (per-
-// thread FP32 partial sums, FP64 across blocks); the solution increment x32
+// Reliable-update flexible CG: every vector of the iteration in FP32 (each
+// entry's products summed in FP32, entries in FP64); the solution increment x32
 // and the true residual are carried over to FP64 by ru_fold / ru_residual.
 cudaError_t rdot(const void* a, const void* b, long long count, int nrhs, double* ws, double* out,
                  cudaStream_t s);

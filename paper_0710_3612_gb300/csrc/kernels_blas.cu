@@ -359,9 +359,11 @@ cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq
 
 // ---------------------------------------------------------------------------
 // Reliable-update flexible CG (FP32 iteration, FP64 solution and true
-// residual).  Per-thread partial sums are kept in FP32 (a thread covers a few
-// entries) and the blocks are combined in FP64 by the deterministic
-// single-pass reduction, so no FP64 arithmetic runs per entry.
+// residual).  Each entry's products are summed in FP32 and added in FP64, one
+// conversion and one addition per number and entry (with FP32 chains over a
+// thread's entries, up to 16 in batches, the sums were less accurate than with
+// one entry per thread); the blocks are combined by the deterministic
+// single-pass reduction.
 // ---------------------------------------------------------------------------
 
 // ab[rhs] = <a, b> of FP32 vectors.
@@ -371,14 +373,15 @@ __global__ void __launch_bounds__(RT) k_rdot(const float2* __restrict__ a,
   pdl_wait(dependent, a, b, ws, out);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
-  float re = 0.f, im = 0.f;
+  double re = 0.0, im = 0.0;
+#pragma unroll 4
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     const float2 u = a[base + i], v = b[base + i];
-    re = fmaf(u.x, v.x, fmaf(u.y, v.y, re));
-    im = fmaf(u.x, v.y, fmaf(-u.y, v.x, im));
+    re += (double)fmaf(u.x, v.x, u.y * v.y);
+    im += (double)fmaf(u.x, v.y, -u.y * v.x);
   }
-  finish_reduction<2>((double)re, (double)im, ws, out, sh);
+  finish_reduction<2>(re, im, ws, out, sh);
 }
 
 cudaError_t rdot(const void* a, const void* b, long long count, int nrhs, double* ws, double* out,
@@ -403,8 +406,9 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
   const int rhs = blockIdx.y;
   const bool skip = frozen && frozen[rhs];
   const float alpha = (float)block_ratio(rz[2 * rhs], pq[2 * rhs]);
-  float acc = 0.f;
+  double acc = 0.0;
   const long long base = (long long)rhs * count;
+#pragma unroll 2
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     const long long k = base + i;
@@ -415,9 +419,9 @@ __global__ void __launch_bounds__(RT) k_rcg_xr(float2* __restrict__ x, float2* _
       rv = make_float2(fmaf(-alpha, qv.x, rv.x), fmaf(-alpha, qv.y, rv.y));
       r[k] = rv;
     }
-    acc = fmaf(rv.x, rv.x, fmaf(rv.y, rv.y, acc));
+    acc += (double)fmaf(rv.x, rv.x, rv.y * rv.y);
   }
-  finish_reduction<1>((double)acc, 0.0, ws, rr, sh);
+  finish_reduction<1>(acc, 0.0, ws, rr, sh);
 }
 
 cudaError_t rcg_xr(void* x32, void* r32, const void* p32, const void* q32, const double* rz,
@@ -439,14 +443,15 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
   pdl_wait(dependent, z, q, r, ws, zr);
   __shared__ double sh[2 * RT];
   const long long base = (long long)blockIdx.y * count;
-  float a = 0.f, b = 0.f;
+  double a = 0.0, b = 0.0;
+#pragma unroll 4
   for (long long i = (long long)blockIdx.x * RT + threadIdx.x; i < count;
        i += (long long)gridDim.x * RT) {
     const float2 zv = z[base + i], qv = q[base + i], rv = r[base + i];
-    a = fmaf(zv.x, qv.x, fmaf(zv.y, qv.y, a));
-    b = fmaf(rv.x, zv.x, fmaf(rv.y, zv.y, b));
+    a += (double)fmaf(zv.x, qv.x, zv.y * qv.y);
+    b += (double)fmaf(rv.x, zv.x, rv.y * zv.y);
   }
-  finish_reduction<2>((double)a, (double)b, ws, zr, sh);
+  finish_reduction<2>(a, b, ws, zr, sh);
 }
 
 cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long long count,

@@ -114,8 +114,7 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
   const R ca = (R)ep.ca, cu = (R)ep.cu, cw = (R)ep.cw;
   const C* EU = (const C*)ep.U;
   const C* EW = (const C*)ep.W;
-  R dre = (R)0, dim = (R)0;     // per-thread partials in the stencil's precision
-  double zq = 0.0, rz = 0.0;     // the flexible-CG pair (FP64 operands)
+  double zq = 0.0, rz = 0.0;     // the dot (a site's sum in the stencil's precision) or the flexible-CG pair
 #pragma unroll
   for (int k = 0; k < RPT; ++k) {
     const int lt = tid / TX + TY * k;
@@ -139,8 +138,8 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
     if (ep.dot_out && !ep.zq_q) {
       C p0, p1;
       split(sp[(lt + 2) * PW + (lx + 2)], p0, p1);
-      dre += p0.x * y0.x + p0.y * y0.y + p1.x * y1.x + p1.y * y1.y;
-      dim += p0.x * y0.y - p0.y * y0.x + p1.x * y1.y - p1.y * y1.x;
+      zq += (double)(p0.x * y0.x + p0.y * y0.y + p1.x * y1.x + p1.y * y1.y);
+      rz += (double)(p0.x * y0.y - p0.y * y0.x + p1.x * y1.y - p1.y * y1.x);
     }
     y0 = mk(ca * y0.x, ca * y0.y);
     y1 = mk(ca * y1.x, ca * y1.y);
@@ -170,10 +169,6 @@ __global__ void __launch_bounds__(TX* TY) k_wilson_A(const cplx_t<R>* __restrict
   if (ep.dot_out) {
     // the tile's shared memory is free again: it holds the block sums
     static_assert(sizeof(sp) >= 2 * TX * TY * sizeof(double), "room for the block sums");
-    if (!ep.zq_q) {
-      zq = (double)dre;
-      rz = (double)dim;
-    }
     __syncthreads();
     finish_reduction_g<2>(zq, rz, ep.dot_ws, ep.dot_out, (double*)sp, blockIdx.z,
                           blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
