@@ -138,8 +138,9 @@ struct Epilogue {
 
 // ---- fine Wilson operator ------------------------------------------------
 // U: [2][V] complex of precision R with the antiperiodic sign folded into the
-// t links at t = Lt - 1.  diag = 4 + m.  W (FP64 vectors; may be null): the links of
-// fixed_links for this diag, which the integer kernel of fixed.cuh reads.
+// t links at t = Lt - 1.  diag = 4 + m.  W: on FP64 vectors the links of fixed_links for
+// this diag, which the integer kernel of fixed.cuh reads, or null; on FP32 vectors U times
+// -1/2 (fold_links), which the streaming kernel reads (null only with the fused dot).
 template <typename R>
 cudaError_t wilson_D(const void* in, void* out, const void* U, double diag, int Lx, int Lt,
                      int nrhs, bool dagger, cudaStream_t s);
@@ -183,9 +184,9 @@ int stencil_tunings(StencilTuning* out, int max);
 // <x, A x> (which needs at most 608), and whether a fused launch fits at all.
 int wilson_A_ctas(int Lx, int Lt, bool f64);
 bool wilson_A_dot_fits(int Lx, int Lt, bool f64, double diag);
-// links: gauge complex128 [2][V] -> folded links of precision R
+// links: gauge complex128 [2][V] -> folded links of precision R, times factor
 template <typename R>
-cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s);
+cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s, double factor = 1.0);
 // max_i ||U_i| - 1| into *out (device double)
 cudaError_t link_unitarity(const void* gauge, long long count, double* out, cudaStream_t s);
 

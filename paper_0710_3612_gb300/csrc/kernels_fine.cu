@@ -334,9 +334,8 @@ __global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __res
 // every operation together as packed pairs (fma.rn.f32x2: one issue slot for two FMAs), so a
 // row step takes 40 packed operations for two sites where k_wilson_A_stream takes 88, and
 // only one shuffle per component and direction; a warp owns 64 sites of a row, 60 of them
-// outputs.  Computed as -2 D and -2 D^dagger (r = -2 diag psi + sum of hops), the factor 4
-// removed with the epilogue's scale: powers of two, so nothing rounds differently.  The
-// t-backward product of a row is formed when the row is current and carried.  Bound by FMA
+// outputs.  Its links are stored as -U / 2, so that D is diag psi + the sum of hops and nothing
+// leaves the range that the result has.  The t-backward product of a row is formed when the row is current and carried.  Bound by FMA
 // issue (72% of the heavy pipe) and HBM: 4096^2 128 us (0.93 of the copy bandwidth; 144 us with
 // one site per lane), 1024^2 x 16 119 (146), 256^2 x 64 40 (68 with tiles).
 using P2 = unsigned long long;                       // two floats, low = first site
@@ -401,10 +400,10 @@ __device__ __forceinline__ C2 proj_t(const S2& f) {
 __device__ __forceinline__ P2 from_right(P2 v) { return p2(hi(v), __shfl_down_sync(0xffffffffu, lo(v), 1)); }
 __device__ __forceinline__ P2 from_left(P2 v) { return p2(__shfl_up_sync(0xffffffffu, hi(v), 1), lo(v)); }
 
-// -2 D (S = 1) or -2 D^dagger (S = -1) of one row; f the row, up the next one, tb the
-// t-backward product, m2d = -2 diag.
+// D (S = 1) or D^dagger (S = -1) of one row; f the row, up the next one, tb the t-backward
+// product, ux and ut the links times -1/2.
 template <int S>
-__device__ __forceinline__ S2 row2(const S2& f, const S2& up, const L2& ux, const L2& ut, C2 tb, P2 m2d) {
+__device__ __forceinline__ S2 row2(const S2& f, const S2& up, const L2& ux, const L2& ut, C2 tb, P2 diag) {
   const C2 q = S > 0 ? sub2(f.a, f.b) : add2(f.a, f.b);
   const C2 g = mulc2(ux, S > 0 ? add2(f.a, f.b) : sub2(f.a, f.b));
   const C2 X = mul2(ux, C2{from_right(q.x), from_right(q.y)});
@@ -412,16 +411,16 @@ __device__ __forceinline__ S2 row2(const S2& f, const S2& up, const L2& ux, cons
   const C2 Z = mul2(ut, proj_t<S>(up));
   const C2 s = add2(add2(add2(X, Y), Z), tb);
   const C2 d = S > 0 ? sub2(Y, X) : sub2(X, Y), e = S > 0 ? sub2(Z, tb) : sub2(tb, Z);
-  return {{fma2(m2d, f.a.x, s.x), fma2(m2d, f.a.y, s.y)},
-          {fma2(m2d, f.b.x, add2(d.x, e.y)), fma2(m2d, f.b.y, sub2(d.y, e.x))}};
+  return {{fma2(diag, f.a.x, s.x), fma2(diag, f.a.y, s.y)},
+          {fma2(diag, f.b.x, add2(d.x, e.y)), fma2(diag, f.b.y, sub2(d.y, e.x))}};
 }
 
 static constexpr int SOUT2 = 60;           // output sites per warp
 
 __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __restrict__ in, float2* out,
-                                                             const float2* __restrict__ U, float diag,
+                                                             const float2* __restrict__ W, float diag,
                                                              int Lx, int Lt, int rows, Epilogue ep, int dependent) {
-  pdl_wait(dependent, in, out, U);
+  pdl_wait(dependent, in, out, W);
   __shared__ float4 ring_psi[4][SNB][2][32];           // [warp][slot][site][lane]
   __shared__ float4 ring_u[4][SNB][2][32];             // [warp][slot][direction][lane]
   const int V = Lx * Lt;
@@ -441,7 +440,7 @@ __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __res
       const float2* ps = col + 2LL * Lx * wrap(r + 2, Lt);
       cp_async(&ring_psi[wl][slot][0][lane], ps, 16);
       cp_async(&ring_psi[wl][slot][1][lane], ps + 2, 16);
-      const float2* pu = U + x + Lx * wrap(r + 1, Lt);
+      const float2* pu = W + x + Lx * wrap(r + 1, Lt);
       cp_async(&ring_u[wl][slot][0][lane], pu, 16);
       cp_async(&ring_u[wl][slot][1][lane], pu + V, 16);
     }
@@ -451,20 +450,20 @@ __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __res
     const float4* p = (const float4*)(col + 2LL * Lx * wrap(t, Lt));
     return spinors(p[0], p[1]);
   };
-  auto ld_u = [&](int mu, int t) { return links(*(const float4*)(U + mu * V + x + Lx * wrap(t, Lt))); };
+  auto ld_u = [&](int mu, int t) { return links(*(const float4*)(W + mu * V + x + Lx * wrap(t, Lt))); };
   for (int k = 0; k < SNB - 1; ++k) issue(t0 - 1 + k);
-  const P2 m2d = p2(-2.f * diag, -2.f * diag);
+  const P2 d2 = p2(diag, diag);
   C2 tb = mulc2(ld_u(1, t0 - 2), proj_t<-1>(ld_psi(t0 - 2)));
   S2 pc = ld_psi(t0 - 1), pp = ld_psi(t0), dc = {{0, 0}, {0, 0}};
   L2 ux = ld_u(0, t0 - 1), ut = ld_u(1, t0 - 1), uxo = {0, 0, 0}, uto = {0, 0, 0};
   C2 db = {0, 0};
-  const float ca = 0.25f * (float)ep.ca, cu = (float)ep.cu, cw = (float)ep.cw;
+  const float ca = (float)ep.ca, cu = (float)ep.cu, cw = (float)ep.cw;
   const float2 *EU = (const float2*)ep.U, *EW = (const float2*)ep.W;
 #pragma unroll 2                                       // the row window rotates by renaming
   for (int r = t0 - 1; r <= t1; ++r) {
-    const S2 e = row2<1>(pc, pp, ux, ut, tb, m2d);     // -2 D psi at row r
+    const S2 e = row2<1>(pc, pp, ux, ut, tb, d2);      // D psi at row r
     if (r > t0) {                                      // output row r - 1
-      const S2 y = row2<-1>(dc, e, uxo, uto, db, m2d);
+      const S2 y = row2<-1>(dc, e, uxo, uto, db, d2);
       if (writer) {
         const long long g = off + 2LL * (x + Lx * (r - 1));
         const P2 c = p2(ca, ca);
@@ -597,12 +596,13 @@ static bool wilson_variant_ok(int v, int Lx, int Lt, int nrhs, bool fx) {
   return true;
 }
 
-// W: the fixed-point links when the integer kernel runs the launch, else null.
+// W: FP64, the fixed-point links when the integer kernel runs the launch, else null; FP32, the
+// links times -1/2.
 template <typename R>
 static cudaError_t launch_variant(int v, const void* in, void* out, const void* U, const void* W,
                                   double diag, int Lx, int Lt, int nrhs, const Epilogue& ep,
                                   cudaStream_t s) {
-  if (W)
+  if (sizeof(R) == 8 && W)
     return wilson_A_fx(WV_SHAPE[v][0], WV_SHAPE[v][1] * WV_SHAPE[v][2], in, out, U, W, diag, Lx, Lt,
                        nrhs, ep, s);
   switch (v) {
@@ -611,7 +611,7 @@ static cudaError_t launch_variant(int v, const void* in, void* out, const void* 
         const int rows = stream32_rows(Lx, Lt, nrhs);
         const long long warps = stream32_warps(Lx, Lt, 1, rows);
         launch_after(k_wilson_A_stream2, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
-            (const float2*)in, (float2*)out, (const float2*)U, (float)diag, Lx, Lt, rows, ep);
+            (const float2*)in, (float2*)out, (const float2*)W, (float)diag, Lx, Lt, rows, ep);
       } else {
         const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
         launch_after(k_wilson_A_stream, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
@@ -662,13 +662,14 @@ template <typename R>
 cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, const void* W,
                           double diag, int Lx, int Lt, int nrhs, int* dflag, cudaStream_t s) {
   const Epilogue none{};
-  if (!(sizeof(R) == 8 && wilson_A_fx_ok(W, diag, none))) W = nullptr;
-  const TuneKey key{(int)sizeof(R), Lx, Lt, nrhs, W != nullptr};
+  const bool fx = sizeof(R) == 8 && wilson_A_fx_ok(W, diag, none);
+  if (sizeof(R) == 8 && !fx) W = nullptr;
+  const TuneKey key{(int)sizeof(R), Lx, Lt, nrhs, fx};
   {
     std::lock_guard<std::mutex> g(g_tune_mu);
     if (g_tune.count(key)) return cudaSuccess;
   }
-  const int def = W ? wilson_fx_variant(Lx, Lt, nrhs, false) : wilson_default_variant<R>(Lx, Lt, nrhs, false);
+  const int def = fx ? wilson_fx_variant(Lx, Lt, nrhs, false) : wilson_default_variant<R>(Lx, Lt, nrhs, false);
   const long long words = (long long)Lx * Lt * nrhs * 2 * sizeof(cplx_t<R>) / 8;
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
@@ -680,7 +681,7 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
   float best = 0.f;
   launch_variant<R>(def, in, ref, U, W, diag, Lx, Lt, nrhs, none, s);
   for (int v = 0; v < WV_COUNT; ++v) {
-    if (!wilson_variant_ok<R>(v, Lx, Lt, nrhs, W != nullptr)) continue;
+    if (!wilson_variant_ok<R>(v, Lx, Lt, nrhs, fx)) continue;
     ++t.tried;
     launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     int diff = 0;
@@ -750,11 +751,13 @@ template <typename R>
 cudaError_t wilson_A(const void* in, void* out, const void* U, const void* W, double diag, int Lx,
                      int Lt, int nrhs, const Epilogue& ep, cudaStream_t s) {
   const bool dot = ep.dot_out != nullptr;
-  if (!(sizeof(R) == 8 && wilson_A_fx_ok(W, diag, ep))) W = nullptr;
-  if (dot && (nrhs > 64 || !wilson_A_dot_fits(Lx, Lt, sizeof(R) == 8, W ? diag : 0.0)))
+  const bool fx = sizeof(R) == 8 && wilson_A_fx_ok(W, diag, ep);
+  if (sizeof(R) == 8 && !fx) W = nullptr;
+  if (sizeof(R) == 4 && !W && !dot) return cudaErrorInvalidValue;
+  if (dot && (nrhs > 64 || !wilson_A_dot_fits(Lx, Lt, sizeof(R) == 8, fx ? diag : 0.0)))
     return cudaErrorInvalidValue;
-  int v = dot ? -1 : tuned_variant<R>(Lx, Lt, nrhs, W != nullptr);
-  if (v < 0) v = W ? wilson_fx_variant(Lx, Lt, nrhs, dot) : wilson_default_variant<R>(Lx, Lt, nrhs, dot);
+  int v = dot ? -1 : tuned_variant<R>(Lx, Lt, nrhs, fx);
+  if (v < 0) v = fx ? wilson_fx_variant(Lx, Lt, nrhs, dot) : wilson_default_variant<R>(Lx, Lt, nrhs, dot);
   const cudaError_t e = launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, ep, s);
   count_launch();
   return e;
@@ -778,22 +781,22 @@ cudaError_t sigma3_mul(const void* in, void* out, long long V, cudaStream_t s) {
 
 template <typename R>
 __global__ void k_fold_links(const double2* __restrict__ g, cplx_t<R>* __restrict__ U, int Lx,
-                             int Lt, int dependent) {
+                             int Lt, double factor, int dependent) {
   pdl_wait(dependent, g, U);
   const int V = Lx * Lt;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= 2 * V) return;
   const int mu = i / V, site = i % V;
-  const double sg = (mu == 1 && site / Lx == Lt - 1) ? -1.0 : 1.0;
+  const double sg = (mu == 1 && site / Lx == Lt - 1) ? -factor : factor;
   double2 u = g[i];
   U[i] = mk((R)(sg * u.x), (R)(sg * u.y));
 }
 
 template <typename R>
-cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s) {
+cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s, double factor) {
   const int n = 2 * Lx * Lt;
   launch_after(k_fold_links<R>, (n + 255) / 256, 256, 0, s,
-               (const double2*)gauge, (cplx_t<R>*)U, Lx, Lt);
+               (const double2*)gauge, (cplx_t<R>*)U, Lx, Lt, factor);
   count_launch();
   return cudaGetLastError();
 }
@@ -829,7 +832,7 @@ cudaError_t link_unitarity(const void* gauge, long long count, double* out, cuda
                                    int, int, const Epilogue&, cudaStream_t);                  \
   template cudaError_t wilson_A_tune<R>(const void*, void*, void*, const void*, const void*,   \
                                         double, int, int, int, int*, cudaStream_t);           \
-  template cudaError_t fold_links<R>(const void*, void*, int, int, cudaStream_t);
+  template cudaError_t fold_links<R>(const void*, void*, int, int, cudaStream_t, double);
 INST(double)
 INST(float)
 #undef INST

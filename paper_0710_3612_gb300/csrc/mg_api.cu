@@ -54,6 +54,7 @@ struct mg_handle {
   std::vector<Level> lv;
   double2* U64 = nullptr;
   float2* U32 = nullptr;
+  float2* U32h = nullptr;       // times -1/2, for the streaming stencil
   void* Wfx = nullptr;          // fixed-point links of the current mass (fixed_links)
   // coarsest level
   int Nc = 0, ldc = 0;
@@ -229,7 +230,8 @@ void apply_level(mg_handle* h, int l, const void* in, void* out, int nrhs, int w
   if (l == 0) {
     const double diag = 4.0 + h->mass;
     const void* U = sizeof(R) == 8 ? (const void*)h->U64 : (const void*)h->U32;
-    ck(h, wilson_A<R>(in, out, U, h->Wfx, diag, L.Lx, L.Lt, nrhs, ep, h->s), "wilson_A");
+    const void* W = sizeof(R) == 8 ? h->Wfx : (const void*)h->U32h;
+    ck(h, wilson_A<R>(in, out, U, W, diag, L.Lx, L.Lt, nrhs, ep, h->s), "wilson_A");
   } else {
     if (weights == W_F64 && L.Afx) {
       ck(h, coarse_apply_fx(in, out, L.A64, L.Afx, L.Lx, L.Lt, L.n, nrhs, ep, h->s), "coarse_apply");
@@ -1252,6 +1254,7 @@ void allocate_storage(mg_handle* h) {
   const long long V = h->lv[0].V;
   h->U64 = dalloc<double2>(h, 2 * V * sizeof(double2));
   h->U32 = dalloc<float2>(h, 2 * V * sizeof(float2));
+  h->U32h = dalloc<float2>(h, 2 * V * sizeof(float2));
   h->Wfx = dalloc(h, 2 * V * sizeof(int4));
   // per-level storage
   for (int l = 0; l < h->L; ++l) {
@@ -1618,7 +1621,7 @@ void autotune_fine(mg_handle* h) {
   for (int nrhs : {1, h->R}) {
     ck(h, wilson_A_tune<double>(h->sv64[0], h->sv64[1], h->sv64[2], h->U64, h->Wfx, diag, F.Lx, F.Lt,
                                 nrhs, h->dflag, h->s), "tune f64");
-    ck(h, wilson_A_tune<float>(h->sv32[0], h->sv32[1], h->sv32[2], h->U32, nullptr, diag, F.Lx, F.Lt,
+    ck(h, wilson_A_tune<float>(h->sv32[0], h->sv32[1], h->sv32[2], h->U32, h->U32h, diag, F.Lx, F.Lt,
                                nrhs, h->dflag, h->s), "tune f32");
     if (h->R == 1) break;
   }
@@ -1797,6 +1800,7 @@ mg_status refine_core(mg_handle* src, int lr, const void* e0, int ncycles, const
     };
     copy(h->U64, src->U64, 2 * V * sizeof(double2));
     copy(h->U32, src->U32, 2 * V * sizeof(float2));
+    copy(h->U32h, src->U32h, 2 * V * sizeof(float2));
     set_operator_mass(h, src->mass);
     size_t pos = 0;
     for (int l = 0; l + 1 < h->L; ++l) {
@@ -1912,6 +1916,7 @@ mg_status mg_setup(const void* gauge, double mass, const mg_params* params, void
     if (!(dev <= 1e-12)) fail(h, MG_ERR_ARG, "gauge links are not unit modulus (|U|-1 = " + std::to_string(dev) + ")");
     ck(h, fold_links<double>(gauge, h->U64, P.Lx, P.Lt, h->s), "fold");
     ck(h, fold_links<float>(gauge, h->U32, P.Lx, P.Lt, h->s), "fold");
+    ck(h, fold_links<float>(gauge, h->U32h, P.Lx, P.Lt, h->s, -0.5), "fold");
     set_operator_mass(h, mass);
     // adaptive setup, level by level (Sec. 3)
     const double2* noise = (const double2*)P.setup_noise;
@@ -2014,6 +2019,7 @@ mg_status mg_clone(const mg_handle* src, double mass, void* stream, mg_handle** 
     };
     copy(h->U64, src->U64, 2 * V * sizeof(double2));
     copy(h->U32, src->U32, 2 * V * sizeof(float2));
+    copy(h->U32h, src->U32h, 2 * V * sizeof(float2));
     for (int l = 0; l + 1 < h->L; ++l) {
       Level& L = h->lv[l];
       const Level& S = src->lv[l];
