@@ -144,12 +144,15 @@ typedef struct {
                                            shape's (1)                          */
   int remass_quadratic;                 /* nonzero: keep G0_l and G1_l with
                                            A_l(m) = G0_l + d G1_l + d^2 I, d =
-                                           m - (set-up mass), on every coarse
+                                           m - (mass of G0), on every coarse
                                            level (A(m + d) = A(m) +
                                            d (D + D^dagger) + d^2 and
                                            P^dagger P = I), so a new mass is one
                                            combination per level instead of the
-                                           Galerkin products; two more FP64
+                                           Galerkin products (G0 is formed at
+                                           set-up, and again at a mass so far
+                                           from it that the terms would cancel
+                                           more than three bits); two more FP64
                                            copies of each coarse operator (1)   */
   double smooth_omega;                  /* smoothed aggregation of the first
                                            coarsening (Sec. 3): the columns of

@@ -441,7 +441,16 @@ void combine_level(mg_handle* h, int l) {
   ck(h, coarse_finish(C.G0, C.G1, h->mass - h->g_mass, C.A64, C.A32, C.A16, C.Afx, C.V, C.n, h->s), "A(m)");
 }
 
+// Size of the terms that make up A(mass) from G0 and G1 at mass `base`, over its own (hops: 4).
+double remass_growth(double base, double mass) {
+  const double b = 4.0 + base, d = mass - base, a = 4.0 + mass;
+  return (b * b + 2.0 * std::fabs(b * d) + d * d + 4.0) / (a * a + 4.0);
+}
+
+// A coarse operator far from the mass of G0 would cancel digits (60 -> -0.05: three): beyond
+// three bits, and beyond what expanding about m = 0 costs, both are formed anew at this mass.
 void build_coarse_ops(mg_handle* h) {
+  if (remass_growth(h->g_mass, h->mass) > std::max(8.0, remass_growth(0.0, h->mass))) h->g_built = false;
   for (int l = 0; l + 1 < h->L; ++l) {
     ProfScope prof(h, MG_KF_GALERKIN);
     if (h->p.remass_quadratic && h->g_built)
