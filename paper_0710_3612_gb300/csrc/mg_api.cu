@@ -380,8 +380,9 @@ void vcycle(mg_handle* h, int l, const void* b, void* x, int nrhs = 1,
 // ----- setup pieces ---------------------------------------------------------
 // Rayleigh quotient after power_iters applications.  The iterate is normalised only every
 // POWER_NORM steps for ordinary masses (a scale does not change the quotient, and the 16th
-// power of A < 2^14 is within the exponents the kernels take): a norm and a scaling per step
-// were two of its three launches (set-up of the 128^2 workload: 0.7 ms).
+// power of A < 2^14 is within the exponents the kernels take; below a smoothed coarsening A may
+// be larger): a norm and a scaling per step were two of its three launches (set-up of the 128^2
+// workload: 0.7 ms).
 constexpr int POWER_NORM = 16;
 
 double power_lambda_max(mg_handle* h, int l, const double2* start, void* v, void* w) {
@@ -389,7 +390,7 @@ double power_lambda_max(mg_handle* h, int l, const double2* start, void* v, void
   const long long n = L.count();
   ck(h, norm2<double>(start, n, 1, h->partials, slot(h, S_T0), h->s), "norm");
   ck(h, scale_inv_sqrt<double>(start, v, slot(h, S_T0), n, 1, h->s), "scale");
-  const int every = fixed_diag_ok(4.0 + h->mass) ? POWER_NORM : 1;
+  const int every = fixed_diag_ok(4.0 + h->mass) && (l == 0 || h->p.smooth_omega == 0.0) ? POWER_NORM : 1;
   for (int it = 0; it < h->p.power_iters - 1; ++it) {
     apply_level<double>(h, l, v, w, 1, W_F64);
     std::swap(v, w);
