@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 namespace mgk {
@@ -64,6 +65,24 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, siz
   cfg.numAttrs = dependent;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)..., dependent);
 }
+
+// A kernel's dynamic shared-memory limit belongs to a device: raised on its first launch on
+// each (a static of the launcher, one for every kernel; a failure is tried again).
+class SmemLimit {
+  std::atomic<unsigned long long> done_{0};            // bit per device
+ public:
+  template <typename K>
+  cudaError_t raise(K* kernel, int bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+    if (done_.load() & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done_.fetch_or(bit);
+    return e;
+  }
+};
 
 template <typename R> struct cplx_of;
 template <> struct cplx_of<double> { using type = double2; };

@@ -269,12 +269,9 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
     return coarse_apply_tcgen05(in, out, A, Lx, Lt, n, nrhs, ep, s);
   if (coarse_apply_tensor(weights, n, nrhs)) {
     const size_t smem = (size_t)2 * 9 * n * (MMA_RC + 8) * sizeof(__nv_bfloat162);
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_coarse_apply_mma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           64 * 1024);
-      attr = true;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_coarse_apply_mma, 64 * 1024);
+    if (e != cudaSuccess) return e;
     dim3 grid(Lx * Lt, (nrhs + MMA_RC - 1) / MMA_RC);
     launch_after(k_coarse_apply_mma, grid, 64, smem, s, (const float2*)in, (float2*)out,
                                               (const __nv_bfloat162*)A, Lx, Lt, n, nrhs, ep);
@@ -536,11 +533,9 @@ cudaError_t restrict_op(const void* fine, void* coarse, const void* Vst, int Lx,
     return transfer_reg(fine, coarse, Vst, Lx, Lt, bx, bt, h, Nv, nrhs, false, false, s);
   const size_t sm = transfer_multi_smem(bx, bt, h, Nv, nrhs, sizeof(cplx_t<R>), true);
   if (sm <= 96 * 1024) {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_restrict_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-      attr = true;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_restrict_multi<R>, 96 * 1024);
+    if (e != cudaSuccess) return e;
     launch_after(k_restrict_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
         (const cplx_t<R>*)fine, (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
         nrhs, transfer_group(nrhs * 2 * Nv, bx * bt * h));
@@ -581,11 +576,9 @@ cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, 
     return transfer_reg(coarse, fine, Vst, Lx, Lt, bx, bt, h, Nv, nrhs, true, accumulate, s);
   const size_t sm = transfer_multi_smem(bx, bt, h, Nv, nrhs, sizeof(cplx_t<R>), false);
   if (sm <= 96 * 1024) {
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_prolong_multi<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-      attr = true;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_prolong_multi<R>, 96 * 1024);
+    if (e != cudaSuccess) return e;
     launch_after(k_prolong_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
         (const cplx_t<R>*)coarse, (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
         nrhs, accumulate, transfer_group(nrhs * bx * bt * 2 * h, Nv));
@@ -692,8 +685,8 @@ cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx,
     constexpr int LPB = decltype(lpb)::value, NQ = decltype(nq)::value;
     const int per = 32 / LPB;
     const size_t smem = (size_t)per * Nv * m * sizeof(double2);   // at most 128 KB (m = 256, Nv = 32)
-    static const cudaError_t e = cudaFuncSetAttribute(
-        k_block_gs<LPB, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise(k_block_gs<LPB, NQ>, 160 * 1024);
     if (e != cudaSuccess) return e;
     launch_after(k_block_gs<LPB, NQ>, (nb + per - 1) / per, 32, smem, s,
                  (const double2*)E, (double2*)Vst, Lx, Lt, bx,
@@ -930,13 +923,10 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
                             int bt, int nf, int Nv, cudaStream_t s) {
   const int nc = 2 * Nv, Vc = (Lx / bx) * (Lt / bt);
   const size_t smem = (size_t)(9 * nc * nc + nf * nc) * sizeof(double2);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_galerkin_coarse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
-    attr_set = true;
-  }
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_galerkin_coarse, 200 * 1024);
+  if (e != cudaSuccess) return e;
   launch_after(k_galerkin_coarse, Vc, 256, smem, s, (const double2*)Af, (const double2*)Vst, (double2*)Ac,
                                           Lx, Lt, bx, bt, nf, Nv); count_launch();
   return cudaGetLastError();
@@ -1444,12 +1434,9 @@ cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s) {
   if (N % GJB != 0) return cudaErrorInvalidValue;
   float2 *Pb[2], *Cold, *Cn, *Rp;
   gj_work_split(work, N, Pb, &Cold, &Cn, &Rp);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(2 * GJB * GJS * sizeof(float2)));
-    attr = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_gj_panel, (int)(2 * GJB * GJS * sizeof(float2)));
+  if (e != cudaSuccess) return e;
   launch_after(k_gj_pivot0, 1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s, (const float2*)M, N, Pb[0]);
   count_launch();
   return cudaGetLastError();
@@ -1477,11 +1464,9 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
   gj_work_split(work, N, Pb, &Cold, &Cn, &Rp);
   const int nb = N / GJB;
   const size_t sm = 4 * TC_OPF * sizeof(float) + 1024;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_gj_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    attr = true;
-  }
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_gj_update_tc, (int)sm);
+  if (e != cudaSuccess) return e;
   launch_after(k_gj_update_tc, tc_tile_count(nb), 256, sm, s, (float2*)M, N, k, Pb[k & 1], Pb[(k + 1) & 1],
                                                     Cold, Cn, Rp, (int*)(Rp + (long long)GJB * N));
   count_launch();
@@ -1933,14 +1918,11 @@ cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, in
   if (ld % HT || ld < N) return cudaErrorInvalidValue;
   const int nt = ld / HT, ntiles = nt * (nt + 1) / 2;
   if (nrhs >= 16 && nrhs <= 64 && xscratch) {   // tensor cores
-    const cudaError_t e = to_f32_padded(x, xscratch, N, ld, nrhs, s);
-    if (e != cudaSuccess) return e;
     const size_t sm = (size_t)HT * (GJC + 2 * GJR) * sizeof(float2);
-    static bool attr = false;
-    if (!attr) {
-      cudaFuncSetAttribute(k_hgemv_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-      attr = true;
-    }
+    static SmemLimit limit;
+    cudaError_t e = limit.raise(k_hgemv_mma, (int)sm);
+    if (e == cudaSuccess) e = to_f32_padded(x, xscratch, N, ld, nrhs, s);
+    if (e != cudaSuccess) return e;
     launch_after(k_hgemv_mma, ntiles, 256, sm, s, (const float2*)P, (const float2*)xscratch, ld, ntiles,
                                         nrhs, (float2*)part);
     count_launch();

@@ -261,8 +261,8 @@ cudaError_t launch(const double2* x, double2* y, const double2* A, const int4* W
                    int Lt, int n, int nrhs, int rpc, const Epilogue& ep, cudaStream_t s) {
   const int NR = 9 * n;
   const size_t smem = (size_t)RG * (NR * (16 + 16 + 8 + 4) + 40);   // at most 51 KB
-  static const cudaError_t e =
-      cudaFuncSetAttribute(k_coarse_fx<RG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_coarse_fx<RG>, 64 * 1024);
   if (e != cudaSuccess) return e;
   launch_after(k_coarse_fx<RG>, dim3(Lx * Lt, (nrhs + rpc - 1) / rpc), (NR + 31) & ~31, smem, s,
       x, y, A, W, E, Lx, Lt, n, nrhs, rpc, ep);
@@ -283,11 +283,10 @@ cudaError_t coarse_finish(const void* G0, const void* G1, double m, void* A64, v
   int P = 2;
   while (P < n) P *= 2;
   if (P > 256) return cudaErrorInvalidValue;
-  static const cudaError_t e0 = cudaFuncSetAttribute(
-      k_coarse_finish<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-  static const cudaError_t e1 = cudaFuncSetAttribute(
-      k_coarse_finish<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-  if (e0 != cudaSuccess || e1 != cudaSuccess) return e0 != cudaSuccess ? e0 : e1;
+  static SmemLimit limit0, limit1;
+  const cudaError_t e = G0 ? limit1.raise(k_coarse_finish<true>, 160 * 1024)
+                           : limit0.raise(k_coarse_finish<false>, 160 * 1024);
+  if (e != cudaSuccess) return e;
   if (G0)
     launch_after(k_coarse_finish<true>, (unsigned)sites, 256, smem, s,
                  (const double2*)G0, (const double2*)G1, m,

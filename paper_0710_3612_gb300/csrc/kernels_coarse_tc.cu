@@ -429,15 +429,19 @@ template <int NDOF>
 cudaError_t launch_tc(const void* in, void* out, const void* A, int Lx, int Lt, int nrhs,
                       const Epilogue& ep, cudaStream_t s) {
   using C = CoarseTC<NDOF>;
-  static int sms = 0, dyn_max = 0;
-  if (!sms) {
+  struct Device { std::atomic<int> sms{0}, dyn_max{0}; };
+  static Device devices[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  Device& D = devices[dev & 63];
+  if (!D.sms.load()) {
     // the largest dynamic shared memory a block may opt in to, less the static part
-    int dev = 0, m = 0, optin = 0;
-    cudaGetDevice(&dev);
+    int m = 0, optin = 0;
     cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaFuncAttributes fa{};
-    cudaError_t e = cudaFuncGetAttributes(&fa, k_coarse_apply_tc<NDOF>);
+    e = cudaFuncGetAttributes(&fa, k_coarse_apply_tc<NDOF>);
     if (e != cudaSuccess) return e;
     const int dm = optin - (int)fa.sharedSizeBytes;
     e = cudaFuncSetAttribute(k_coarse_apply_tc<NDOF>, cudaFuncAttributeMaxDynamicSharedMemorySize, dm);
@@ -445,9 +449,10 @@ cudaError_t launch_tc(const void* in, void* out, const void* A, int Lx, int Lt, 
     e = cudaFuncSetAttribute(k_coarse_apply_tc<NDOF>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              (int)cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    dyn_max = dm;
-    sms = m > 0 ? m : 1;
+    D.dyn_max.store(dm);
+    D.sms.store(m > 0 ? m : 1);
   }
+  const int sms = D.sms.load(), dyn_max = D.dyn_max.load();
   EncodeTiled enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
   // X as a 2D FP32 tensor [nrhs][V * 2n]: a box is one site's nrhs rows (NR

@@ -220,9 +220,8 @@ __global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ 
 template <int TX, int TY, int RPT, int MINB, int MODE>
 cudaError_t launch_mode(const FxArgs& a, int nrhs, cudaStream_t s) {
   using T = FxTile<TX, TY, RPT>;
-  static const cudaError_t e =
-      cudaFuncSetAttribute(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, T::BYTES);
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>, T::BYTES);
   if (e != cudaSuccess) return e;
   const dim3 grid((a.Lx + TX - 1) / TX, (a.Lt + T::TT - 1) / T::TT, nrhs);
   launch_after(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>, grid, TX * TY, T::BYTES, s, a);

@@ -285,12 +285,9 @@ __global__ void __launch_bounds__(128) k_hgemv_tc_sum(const float* __restrict__ 
 
 // Column shares per row block: as many as fill the SMs once (one CTA each).
 int gt_splits(int nt) {
-  static const int sms = [] {
-    int dev = 0, m = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
-    return m > 0 ? m : 1;
-  }();
+  int dev = 0, sms = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   return std::max(1, std::min(nt, sms / ((nt + 1) / 2)));
 }
 
@@ -308,8 +305,8 @@ bool hermitian_gemv_tc_ok(int ld, int nrhs) {
 cudaError_t hermitian_gemv_tc(const void* P, const void* x, void* y, int N, int ld, int nrhs, void* xscratch,
                               void* part, bool accumulate, void* y32, cudaStream_t s) {
   if (ld % GT_T || ld < N || nrhs < 1 || nrhs > 64) return cudaErrorInvalidValue;
-  static const cudaError_t e =
-      cudaFuncSetAttribute(k_hgemv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, GT_SMEM);
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_hgemv_tc, GT_SMEM);
   if (e != cudaSuccess) return e;
   const cudaError_t ex = to_f32_padded(x, xscratch, N, ld, nrhs, s);
   if (ex != cudaSuccess) return ex;

@@ -447,8 +447,8 @@ size_t inverse_work_entries(int ld) { return (size_t)2 * ld * B + (size_t)2 * GM
 
 cudaError_t inverse_first(void* M, int ld, const InversePlan& plan, const int* data, void* work,
                           cudaStream_t s) {
-  static const cudaError_t e0 = cudaFuncSetAttribute(
-      k_gji_update, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(2 * B * LD * sizeof(float2)));
+  static SmemLimit limit;
+  const cudaError_t e0 = limit.raise(k_gji_update, (int)(2 * B * LD * sizeof(float2)));
   if (e0 != cudaSuccess) return e0;
   GroupArgs g{};
   g.next = data + plan.first;
