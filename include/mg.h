@@ -367,7 +367,11 @@ mg_status mg_apply_D(mg_handle* h, const void* in, void* out, int nrhs, int dagg
 mg_status mg_apply_A(mg_handle* h, const void* in, void* out, int nrhs, int precision);
 
 /* Coarse operator A_level (2 <= level <= nlevels) on nrhs level vectors
- * (Eq. Galerkin).  precision F64, F32 or BF16 (coarse blocks in bf16). */
+ * (Eq. Galerkin).  precision F64, F32 or BF16 (coarse blocks in bf16).  F64 on
+ * up to 32 components per site works in 64-bit integers: an entry of the
+ * result is exact to a few units of 2^-56 per product of the largest entry of
+ * its block row times the largest component of the vector there, and rows
+ * whose products are all small against that (2^-8) are formed in FP64. */
 mg_status mg_apply_coarse(mg_handle* h, int level, const void* in, void* out, int nrhs,
                           int precision);
 
