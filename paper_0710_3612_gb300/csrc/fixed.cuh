@@ -8,11 +8,12 @@
 // scale per site:
 //   value = v * 2^(e - FX_BIAS),  |v| < 2^FX_BITS,
 // e the largest biased FP64 exponent of the site's components.  A sum over
-// neighbours is formed at the largest exponent among them: each term is
-// computed at its own site's scale and shifted right by the difference.  The
-// absolute error of a result is then a few units of 2^-58 of the largest
-// neighbouring component, below the 2^-53 roundings of the same sum in FP64
-// (whose terms have that size too), whatever the range of the field elsewhere.
+// neighbours is formed at the largest exponent among its terms: each is
+// computed at its own site's scale and shifted right by the difference.  Hop
+// terms are smaller than their site by 2 diag: their coefficients are held times
+// 2^k and their exponents are e - k.  The absolute error of a result is then a few
+// units of 2^-58 of the largest term, below the 2^-53 roundings of the same sum in
+// FP64, whatever the range of the field elsewhere.
 // Results do not depend on the tiling.  Components below the FP64 normal range
 // count as zero next to larger ones; sites holding infinities or NaN, or whose
 // exponents lie outside [FX_EMIN, FX_EMAX] (sites of subnormals alone among them: the
@@ -103,8 +104,8 @@ __host__ __device__ __forceinline__ FxC fx_shr(FxC p, int s) { return {p.re >> s
 __host__ __device__ __forceinline__ int fx_gap(int f, int e) { return f - e > 63 ? 63 : f - e; }
 
 // Hop terms of the Wilson stencil from the spinor f, S = +1: projector (1 - sigma),
-// S = -1: (1 + sigma); w = link / (2 diag), CONJ for the backward hop.  Returned at
-// the scale of f (fx_hop_*), and added to the row sum (fx_add_*): with
+// S = -1: (1 + sigma); w = 2^k link / (2 diag), CONJ for the backward hop.  Returned at
+// the scale of f over 2^k (fx_hop_*), and added to the row sum (fx_add_*): with
 // D psi / diag = psi - sum w (1 -+ sigma) psi, the hops enter with a minus sign.
 template <int S, bool CONJ>
 __host__ __device__ __forceinline__ FxC fx_hop_x(int4 w, const FxSpinor& f) {
@@ -166,8 +167,14 @@ __device__ __forceinline__ double fx_double(long long v, int e) {
   return v == 0 ? 0.0 : __hiloint2double(__double2hiint(d) + (e << 20), __double2loint(d));
 }
 
-// The products stay in range for |diag| >= 1.5 (|w| <= 1/3); beyond 64 the words of w
-// would hold fewer than 57 bits.
+// k: the largest with |w| = 2^k / (2 |diag|) <= 1/3, where the products stay in range.  With 0
+// everywhere, fields that fall by 1 / diag per site kept 44 bits at |diag| = 64; below 6 they
+// keep 50 or more (two hops are 1 / (4 diag^2) of a site), and k stays 0.
+inline int fixed_shift(double diag) {
+  const double a = std::fabs(diag);
+  return a < 6.0 ? 0 : std::ilogb(a / 1.5);
+}
+// |diag| from 1.5 to 64 (k = 5).
 __host__ __device__ __forceinline__ bool fixed_diag_ok(double diag) {
   const double a = diag < 0 ? -diag : diag;
   return a >= 1.5 && a <= 64.0;

@@ -48,9 +48,11 @@ struct FxArgs {
   const int4* W;
   FxScale q;
   double diag;
+  int k;                                               // of the hop terms (fixed_shift)
   int Lx, Lt;
   Epilogue ep;
 };
+static constexpr int FX_BAD_SUM = FX_BAD / 2;          // sums inherit FX_BAD less 2 k at most
 
 // What follows the stencil at a site: nothing, out = ca y + cu U (+ cw W), or the dot
 // with psi (its real part, or both parts).  Separate kernels: a skipped FP64
@@ -65,7 +67,7 @@ __device__ __forceinline__ void fx_output(const FxArgs& a, const FxSpinor& y, in
                                           double& dre, double& dim) {
   const long long g = off + 2LL * (x + a.Lx * t);
   double2 y0, y1;
-  if (y.e >= FX_BAD) {
+  if (y.e >= FX_BAD_SUM) {
     double2 o[2];
     wilson_A_site64(a.in + off, a.U, a.diag, x, t, a.Lx, a.Lt, o);
     y0 = mk(a.ep.ca * o[0].x, a.ep.ca * o[0].y);
@@ -97,17 +99,17 @@ __device__ __forceinline__ void fx_output(const FxArgs& a, const FxSpinor& y, in
 }
 
 // One row sum of D (S = +1) or D^dagger (S = -1) from the site's spinor and the
-// four hop products, each with its own exponent.
+// four hop products, each with its own site's exponent (k above the product's).
 template <int S>
 __device__ __forceinline__ FxSpinor fx_sum(FxSpinor c, FxC xf, int exf, FxC xb, int exb, FxC tf, int etf,
-                                           FxC tb, int etb) {
+                                           FxC tb, int etb, int k) {
   FxSpinor r;
-  r.e = max(max(max(exf, exb), max(etf, etb)), c.e);
-  const int sc = fx_gap(r.e, c.e);
+  r.e = max(max(max(exf, exb), max(etf, etb)) - k, c.e);
+  const int sc = fx_gap(r.e, c.e), h = r.e + k;
   c.a = fx_shr(c.a, sc);
   c.b = fx_shr(c.b, sc);
-  fx_row<S>(r, c, fx_shr(xf, fx_gap(r.e, exf)), fx_shr(xb, fx_gap(r.e, exb)),
-            fx_shr(tf, fx_gap(r.e, etf)), fx_shr(tb, fx_gap(r.e, etb)));
+  fx_row<S>(r, c, fx_shr(xf, fx_gap(h, exf)), fx_shr(xb, fx_gap(h, exb)), fx_shr(tf, fx_gap(h, etf)),
+            fx_shr(tb, fx_gap(h, etb)));
   return r;
 }
 
@@ -129,10 +131,10 @@ struct FxField {
 
 template <int S>
 __device__ __forceinline__ FxSpinor fx_stencil(const FxField& f, int c, int row, const int4* wx,
-                                               const int4* wt, int u, int urow) {
+                                               const int4* wt, int u, int urow, int k) {
   const FxSpinor xp = f.get(c + 1), xm = f.get(c - 1), tp = f.get(c + row), tm = f.get(c - row);
   return fx_sum<S>(f.get(c), fx_hop_x<S, false>(wx[u], xp), xp.e, fx_hop_x<-S, true>(wx[u - 1], xm), xm.e,
-                   fx_hop_t<S, false>(wt[u], tp), tp.e, fx_hop_t<-S, true>(wt[u - urow], tm), tm.e);
+                   fx_hop_t<S, false>(wt[u], tp), tp.e, fx_hop_t<-S, true>(wt[u - urow], tm), tm.e, k);
 }
 
 template <int TX, int TY, int RPT>
@@ -149,8 +151,9 @@ struct FxTile {
 // masks, comparisons), 22 mad.wide per clock: bound by those two pipes.  256^2 x 64:
 // 166 us against 1024 us in FP64 (137 FP64 instructions per site), 128^2 4.2 against
 // 10.2 us, 210 x 90 x 12 12.6 against 71.6 us; with the fused dot 207 against 1254 us.
-// A warp-streaming form (rows in registers, shuffles along x) took 260 us there.
-template <int TX, int TY, int RPT, int MINB, int MODE>
+// A warp-streaming form (rows in registers, shuffles along x) took 260 us there.  SHIFT: hop
+// terms with k > 0 (1.1% more).
+template <int TX, int TY, int RPT, int MINB, int MODE, bool SHIFT>
 __global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a, int dependent) {
   pdl_wait(dependent);
   using T = FxTile<TX, TY, RPT>;
@@ -178,7 +181,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a, in
   __syncthreads();
   for (int q = tid; q < T::ND; q += TX * TY) {
     const int lx = q % T::DW + 1, lt = q / T::DW + 1;
-    fd.put(q, fx_stencil<1>(fp, lt * T::PW + lx, T::PW, wx, wt, lt * T::UW + lx, T::UW));
+    fd.put(q, fx_stencil<1>(fp, lt * T::PW + lx, T::PW, wx, wt, lt * T::UW + lx, T::UW, SHIFT ? a.k : 0));
   }
   __syncthreads();
   double dre = 0.0, dim = 0.0;
@@ -188,7 +191,7 @@ __global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a, in
     const int lt = tid / TX + TY * k, gt = t0 + lt;
     if (gx >= a.Lx || gt >= a.Lt) continue;
     const FxSpinor y = fx_stencil<-1>(fd, (lt + 1) * T::DW + lx + 1, T::DW, wx, wt,
-                                      (lt + 2) * T::UW + lx + 2, T::UW);
+                                      (lt + 2) * T::UW + lx + 2, T::UW, SHIFT ? a.k : 0);
     fx_output<MODE>(a, y, gx, gt, off, dre, dim);
   }
   if (MODE >= FX_DOT_RE) {
@@ -199,33 +202,40 @@ __global__ void __launch_bounds__(TX* TY, MINB) k_wilson_A_fx(const FxArgs a, in
   }
 }
 
-// Links over 2 diag as split 64-bit words.  The quotient is carried to 2^-106 by the
-// division's remainder, so a word is exact to one unit of 2^-63.
-__device__ __forceinline__ long long fx_link_word(double u, double diag) {
+// Links over 2 diag, times 2^k, as split 64-bit words; scale = 2^(63 + k).  The quotient is
+// carried to 2^-106 by the division's remainder, so a word is exact to one unit of 2^-63.
+__device__ __forceinline__ long long fx_link_word(double u, double diag, double scale) {
   const double q = u / diag, r = fma(-q, diag, u) / diag;
-  long long w = (long long)(q * 0x1p63) + __double2ll_rn(r * 0x1p63);
+  long long w = (long long)(q * scale) + __double2ll_rn(r * scale);
   if ((int)w == INT32_MIN) ++w;                        // the low word is negated for conj(w)
   return w;
 }
 
-__global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ W, double diag, int n, int dependent) {
+__global__ void k_fixed_links(const double2* __restrict__ U, int4* __restrict__ W, double diag, double scale, int n,
+                              int dependent) {
   pdl_wait(dependent, U, W);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double2 u = U[i];
-  const long long a = fx_link_word(u.x, diag), b = fx_link_word(u.y, diag);
+  const long long a = fx_link_word(u.x, diag, scale), b = fx_link_word(u.y, diag, scale);
   W[i] = make_int4(fx_lo(a), fx_hi(a), fx_lo(b), fx_hi(b));
+}
+
+template <int TX, int TY, int RPT, int MINB, int MODE, bool SHIFT>
+cudaError_t launch_shift(const FxArgs& a, int nrhs, cudaStream_t s) {
+  using T = FxTile<TX, TY, RPT>;
+  static SmemLimit limit;
+  const cudaError_t e = limit.raise(k_wilson_A_fx<TX, TY, RPT, MINB, MODE, SHIFT>, T::BYTES);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((a.Lx + TX - 1) / TX, (a.Lt + T::TT - 1) / T::TT, nrhs);
+  launch_after(k_wilson_A_fx<TX, TY, RPT, MINB, MODE, SHIFT>, grid, TX * TY, T::BYTES, s, a);
+  return cudaGetLastError();
 }
 
 template <int TX, int TY, int RPT, int MINB, int MODE>
 cudaError_t launch_mode(const FxArgs& a, int nrhs, cudaStream_t s) {
-  using T = FxTile<TX, TY, RPT>;
-  static SmemLimit limit;
-  const cudaError_t e = limit.raise(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>, T::BYTES);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((a.Lx + TX - 1) / TX, (a.Lt + T::TT - 1) / T::TT, nrhs);
-  launch_after(k_wilson_A_fx<TX, TY, RPT, MINB, MODE>, grid, TX * TY, T::BYTES, s, a);
-  return cudaGetLastError();
+  return a.k ? launch_shift<TX, TY, RPT, MINB, MODE, true>(a, nrhs, s)
+             : launch_shift<TX, TY, RPT, MINB, MODE, false>(a, nrhs, s);
 }
 
 template <int TX, int TY, int RPT, int MINB>
@@ -241,13 +251,14 @@ cudaError_t launch_tile(const FxArgs& a, int nrhs, cudaStream_t s) {
 
 cudaError_t fixed_links(const void* U64, void* W, double diag, int Lx, int Lt, cudaStream_t s) {
   const int n = 2 * Lx * Lt;
-  launch_after(k_fixed_links, (n + 255) / 256, 256, 0, s, (const double2*)U64, (int4*)W, diag, n);
+  launch_after(k_fixed_links, (n + 255) / 256, 256, 0, s, (const double2*)U64, (int4*)W, diag,
+               std::ldexp(1.0, 63 + fixed_shift(diag)), n);
   count_launch();
   return cudaGetLastError();
 }
 
-// Factors ca of 2^-120 .. 2^120: a result's exponent field is at least 143 + q.exp (a site at
-// FX_EMIN, one unit left of its sum) and at most 1805 + q.exp, with q.exp within 14 of ca's.
+// Factors ca of 2^-120 .. 2^120: a result's exponent field is at least 133 + q.exp (hops from a
+// site at FX_EMIN, one unit left of their sum) and at most 1805 + q.exp, with q.exp within 14 of ca's.
 bool wilson_A_fx_ok(const void* W, double diag, const Epilogue& ep) {
   return W && fixed_diag_ok(diag) && !ep.zq_q && std::fabs(ep.ca) <= 0x1p120 &&
          std::fabs(ep.ca) >= 0x1p-120 && (ep.U || !ep.W) && !(ep.dot_out && (ep.U || ep.ca != 1.0));
@@ -256,7 +267,7 @@ bool wilson_A_fx_ok(const void* W, double diag, const Epilogue& ep) {
 cudaError_t wilson_A_fx(int tx, int ty, const void* in, void* out, const void* U64, const void* W,
                         double diag, int Lx, int Lt, int nrhs, const Epilogue& ep, cudaStream_t s) {
   const FxArgs a{(const double2*)in, (double2*)out, (const double2*)U64, (const int4*)W,
-                 make_scale(ep.ca, diag), diag, Lx, Lt, ep};
+                 make_scale(ep.ca, diag), diag, fixed_shift(diag), Lx, Lt, ep};
   if (tx == 16 && ty == 8) return launch_tile<16, 8, 1, 4>(a, nrhs, s);
   if (tx == 32 && ty == 8) return launch_tile<32, 8, 1, 3>(a, nrhs, s);
   if (tx == 32 && ty == 16) return launch_tile<32, 8, 2, 3>(a, nrhs, s);
