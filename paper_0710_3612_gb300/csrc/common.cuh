@@ -102,11 +102,6 @@ template <typename C> __device__ __forceinline__ C cmulc(C a, C b) {
   return {a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x};
 }
 template <typename C> __device__ __forceinline__ C cconj(C a) { return {a.x, -a.y}; }
-// i * a
-template <typename C> __device__ __forceinline__ C ci(C a) { return {-a.y, a.x}; }
-template <typename C, typename R> __device__ __forceinline__ C cscale(C a, R s) {
-  return {a.x * s, a.y * s};
-}
 // acc += a * b
 template <typename C> __device__ __forceinline__ void cfma(C& acc, C a, C b) {
   acc.x = fma(a.x, b.x, acc.x);

@@ -101,12 +101,6 @@ cudaError_t ru_fold(void* x64, void* x32, long long count, cudaStream_t s);
 // r32 = (float) r64, rr = |r64|^2 per rhs, and rmax = rr when rmax is given.
 cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, double* ws,
                         double* rr, double* rmax, cudaStream_t s);
-// out(FP32) = in(FP64) * (1/sqrt(nrm[rhs].x)) ; in==0 norm -> 0.
-cudaError_t f64_to_f32_scaled(const void* in, void* out, const double* nrm, long long count,
-                              int nrhs, cudaStream_t s);
-// x(FP64) += in(FP32) * sqrt(nrm[rhs].x)   (scale 1 when nrm is null)
-cudaError_t f32_accumulate_scaled(const void* in, void* x, const double* nrm, long long count,
-                                  int nrhs, cudaStream_t s);
 // out = in (precision convert, no scaling)
 cudaError_t convert_f64_f32(const void* in, void* out, long long count, cudaStream_t s);
 cudaError_t convert_f32_f64(const void* in, void* out, long long count, cudaStream_t s);
@@ -114,10 +108,6 @@ cudaError_t convert_f32_f64(const void* in, void* out, long long count, cudaStre
 template <typename R>
 cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v, double c,
                     const void* w, long long count, int nrhs, cudaStream_t s);
-// r = b - r  (in place: r holds A x on entry)
-template <typename R>
-cudaError_t sub_from(const void* b, void* r, long long count, cudaStream_t s);
-
 // ---- fused epilogue of the operator kernels -------------------------------
 // out = ca * (Op x) + cu * U + cw * W (U, W optional, same precision and layout
 // as out; out may alias W).  When dot_out is set (fine A only, one RHS), the
@@ -294,23 +284,15 @@ cudaError_t inverse_group(void* M, int ld, const InversePlan& plan, const int* d
 cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s);
 cudaError_t gauss_jordan_panel(void* M, int N, int k, void* work, cudaStream_t s);
 cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream_t s);
-// y = B x, or y += B x when accumulate (complex64 B, leading dimension ld);
-// x complex128 (N) -> y complex128 (N); FP32 products and accumulation, result
-// widened to FP64.  xtmp: ld complex64.
-cudaError_t dense_gemv_f32(const void* B, const void* x, void* y, int N, int ld, void* xtmp,
-                           bool accumulate, cudaStream_t s);
-
 // Packed Hermitian matrix: the lower-triangular 64 x 64 tiles (I >= J, stored
 // at I (I + 1) / 2 + J) of a dense ld x ld complex64 matrix (ld multiple of
 // 64); diagonal tiles are made Hermitian from their lower halves.
 cudaError_t pack_hermitian(const void* M, void* P, int ld, cudaStream_t s);
 // y = B x (or y += B x) with B Hermitian in packed tiles, for nrhs vectors;
 // x, y complex128 [nrhs][N]; part: nrhs * 2 * 64 * ntiles complex64 scratch.
-// FP32 products and accumulation; each tile is read once for all vectors.
-cudaError_t hermitian_gemv_f32(const void* P, const void* x, void* y, int N, int ld, int nrhs,
-                               void* part, bool accumulate, cudaStream_t s);
-// The two launches of hermitian_gemv_f32: partial products per stored tile,
-// then their fixed-order sum per row into y.
+// FP32 products and accumulation; each tile is read once for all vectors.  Two
+// launches: partial products per stored tile, then their fixed-order sum per row
+// into y (hermitian_gemv_reduce).
 // xscratch (optional, nrhs * ld complex64): with 16..64 vectors the tile
 // products run on tensor cores from an FP32 copy of x held there.
 cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, int nrhs,

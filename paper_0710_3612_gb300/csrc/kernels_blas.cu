@@ -573,45 +573,6 @@ cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, d
   return cudaGetLastError();
 }
 
-__global__ void k_f64_to_f32_scaled(const double2* __restrict__ in, float2* __restrict__ out,
-                                    const double* nrm, long long count, int dependent) {
-  pdl_wait(dependent, in, out, nrm);
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const double n2 = nrm[2 * blockIdx.y];
-  const double sc = n2 > 0.0 ? 1.0 / sqrt(n2) : 0.0;
-  i += (long long)blockIdx.y * count;
-  double2 v = in[i];
-  out[i] = make_float2((float)(v.x * sc), (float)(v.y * sc));
-}
-
-cudaError_t f64_to_f32_scaled(const void* in, void* out, const double* nrm, long long count,
-                              int nrhs, cudaStream_t s) {
-  launch_after(k_f64_to_f32_scaled, grid1(count, nrhs), RT, 0, s, (const double2*)in, (float2*)out, nrm,
-                                                         count); count_launch();
-  return cudaGetLastError();
-}
-
-__global__ void k_f32_acc_scaled(const float2* __restrict__ in, double2* __restrict__ x,
-                                 const double* nrm, long long count, int dependent) {
-  pdl_wait(dependent, in, x, nrm);
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const double sc = nrm ? sqrt(nrm[2 * blockIdx.y]) : 1.0;
-  i += (long long)blockIdx.y * count;
-  float2 v = in[i];
-  double2 xv = x[i];
-  x[i] = make_double2(fma((double)v.x, sc, xv.x), fma((double)v.y, sc, xv.y));
-}
-
-cudaError_t f32_accumulate_scaled(const void* in, void* x, const double* nrm, long long count,
-                                  int nrhs, cudaStream_t s) {
-  launch_after(k_f32_acc_scaled, grid1(count, nrhs), RT, 0, s,
-               (const float2*)in, (double2*)x, nrm, count);
-  count_launch();
-  return cudaGetLastError();
-}
-
 __global__ void k_cvt_64_32(const double2* __restrict__ in, float2* __restrict__ out,
                             long long count, int dependent) {
   pdl_wait(dependent, in, out);
@@ -659,21 +620,6 @@ cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v,
   return cudaGetLastError();
 }
 
-template <typename R>
-__global__ void k_sub_from(const cplx_t<R>* __restrict__ b, cplx_t<R>* __restrict__ r,
-                           long long count, int dependent) {
-  pdl_wait(dependent, b, r);
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < count) r[i] = csub(b[i], r[i]);
-}
-template <typename R>
-cudaError_t sub_from(const void* b, void* r, long long count, cudaStream_t s) {
-  launch_after(k_sub_from<R>, grid1(count, 1), RT, 0, s,
-               (const cplx_t<R>*)b, (cplx_t<R>*)r, count);
-  count_launch();
-  return cudaGetLastError();
-}
-
 #define INST(R)                                                                              \
   template cudaError_t dot<R>(const void*, const void*, long long, int, double*, double*,    \
                               cudaStream_t);                                                 \
@@ -687,7 +633,6 @@ cudaError_t sub_from(const void* b, void* r, long long count, cudaStream_t s) {
                                 cudaStream_t, void*, const CgControl*);                      \
   template cudaError_t cg_p<R>(void*, const void*, const double*, const double*, const int*, \
                                long long, int, cudaStream_t);                                \
-  template cudaError_t sub_from<R>(const void*, void*, long long, cudaStream_t);             \
   template cudaError_t lincomb<R>(void*, double, const void*, double, const void*, double,   \
                                   const void*, long long, int, cudaStream_t);
 INST(double)

@@ -1473,49 +1473,6 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
   return cudaGetLastError();
 }
 
-__global__ void k_x_to_f32(const double2* __restrict__ x, float2* __restrict__ xf, int N, int ld, int dependent) {
-  pdl_wait(dependent, x, xf);
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ld) xf[i] = i < N ? make_float2((float)x[i].x, (float)x[i].y) : make_float2(0.f, 0.f);
-}
-
-__global__ void __launch_bounds__(256) k_gemv(const float2* __restrict__ B,
-                                              const float2* __restrict__ xf,
-                                              double2* __restrict__ y, int N, int ld,
-                                              bool accumulate, int dependent) {
-  pdl_wait(dependent, B, xf, y);
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= N) return;
-  const float4* b4 = (const float4*)(B + (long long)row * ld);
-  const float4* x4 = (const float4*)xf;
-  float2 acc = make_float2(0.f, 0.f);
-  for (int q = lane; q < ld / 2; q += 32) {
-    const float4 bv = b4[q], xv = x4[q];
-    cfma(acc, make_float2(bv.x, bv.y), make_float2(xv.x, xv.y));
-    cfma(acc, make_float2(bv.z, bv.w), make_float2(xv.z, xv.w));
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    acc.x += __shfl_down_sync(0xffffffffu, acc.x, o);
-    acc.y += __shfl_down_sync(0xffffffffu, acc.y, o);
-  }
-  if (lane == 0) {
-    double2 v = make_double2(acc.x, acc.y);
-    if (accumulate) { v.x += y[row].x; v.y += y[row].y; }
-    y[row] = v;
-  }
-}
-
-cudaError_t dense_gemv_f32(const void* B, const void* x, void* y, int N, int ld, void* xtmp,
-                           bool accumulate, cudaStream_t s) {
-  if (ld % 2 || ld < N) return cudaErrorInvalidValue;
-  launch_after(k_x_to_f32, (ld + 255) / 256, 256, 0, s,
-               (const double2*)x, (float2*)xtmp, N, ld);
-  count_launch();
-  launch_after(k_gemv, (N + 7) / 8, 256, 0, s, (const float2*)B, (const float2*)xtmp, (double2*)y, N, ld,
-                                     accumulate); count_launch();
-  return cudaGetLastError();
-}
-
 // Hermitian inverse in packed lower-triangular 64 x 64 tiles.  Tile (I, J),
 // I >= J, is stored at k = I (I + 1) / 2 + J, row-major.  y = B x reads every
 // stored tile once: tile (I, J) contributes B_IJ x_J to rows of block I and,
@@ -1975,13 +1932,6 @@ cudaError_t hermitian_gemv_tiles_f32in(const void* P, const void* x32, int N, in
                                                  nrhs, (float2*)part, (double2*)x64);
   count_launch();
   return cudaGetLastError();
-}
-
-cudaError_t hermitian_gemv_f32(const void* P, const void* x, void* y, int N, int ld, int nrhs,
-                               void* part, bool accumulate, cudaStream_t s) {
-  cudaError_t e = hermitian_gemv_tiles(P, x, N, ld, nrhs, part, s, nullptr);
-  if (e != cudaSuccess) return e;
-  return hermitian_gemv_reduce(part, y, N, ld, nrhs, accumulate, s);
 }
 
 __global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset, int dependent) {

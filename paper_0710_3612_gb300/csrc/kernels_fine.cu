@@ -265,11 +265,11 @@ __global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __res
       const int slot = (r - t0 + 1 + SNB) % SNB;
       const C* ps = in + off + 2LL * (x + Lx * wrap(r + 2, Lt));
       char* dst = (char*)&ring_psi[wl][slot][lane];
-      cp_async(dst, ps, 16);
-      cp_async(dst + 16, ps + 1, 16);
+      cp_async16(dst, ps);
+      cp_async16(dst + 16, ps + 1);
       const int g = x + Lx * wrap(r + 1, Lt);
-      cp_async(&ring_u[wl][slot][lane][0], U + g, 16);
-      cp_async(&ring_u[wl][slot][lane][1], U + V + g, 16);
+      cp_async16(&ring_u[wl][slot][lane][0], U + g);
+      cp_async16(&ring_u[wl][slot][lane][1], U + V + g);
     }
     cp_commit();
   };
@@ -438,11 +438,11 @@ __global__ void __launch_bounds__(128, 4) k_wilson_A_stream2(const float2* __res
     if (r < t1) {
       const int slot = (r - t0 + 1 + SNB) % SNB;
       const float2* ps = col + 2LL * Lx * wrap(r + 2, Lt);
-      cp_async(&ring_psi[wl][slot][0][lane], ps, 16);
-      cp_async(&ring_psi[wl][slot][1][lane], ps + 2, 16);
+      cp_async16(&ring_psi[wl][slot][0][lane], ps);
+      cp_async16(&ring_psi[wl][slot][1][lane], ps + 2);
       const float2* pu = W + x + Lx * wrap(r + 1, Lt);
-      cp_async(&ring_u[wl][slot][0][lane], pu, 16);
-      cp_async(&ring_u[wl][slot][1][lane], pu + V, 16);
+      cp_async16(&ring_u[wl][slot][0][lane], pu);
+      cp_async16(&ring_u[wl][slot][1][lane], pu + V);
     }
     cp_commit();
   };

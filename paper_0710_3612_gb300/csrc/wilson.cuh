@@ -63,12 +63,9 @@ __device__ __forceinline__ int wrap(int g, int L) { return g < 0 ? g + L : (g >=
 // into range.
 __device__ __forceinline__ int wrap_tile(int g, int L) { return min(wrap(g, L), L - 1); }
 
-__device__ __forceinline__ void cp_async(void* smem, const void* gmem, int bytes) {
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  if (bytes == 16)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem));
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
