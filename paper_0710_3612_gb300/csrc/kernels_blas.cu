@@ -69,7 +69,7 @@ cudaError_t dot(const void* a, const void* b, long long count, int nrhs, double*
   if (nrhs > 64) return cudaErrorInvalidValue;
   const int g = reduce_blocks(count, nrhs);
   launch_after(k_dot<R, false>, dim3(g, nrhs), RT, 0, s, (const cplx_t<R>*)a, (const cplx_t<R>*)b, count,
-                                               partials, out);
+               partials, out);
   count_launch();
   return cudaGetLastError();
 }
@@ -104,7 +104,8 @@ template <typename R>
 cudaError_t axpby(double a, const void* x, double b, void* y, long long count, int nrhs,
                   cudaStream_t s) {
   launch_after(k_axpby<R>, grid1(count, nrhs), RT, 0, s, (R)a, (const cplx_t<R>*)x, (R)b, (cplx_t<R>*)y,
-                                                count); count_launch();
+               count);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -130,7 +131,8 @@ template <typename R>
 cudaError_t scale_inv_sqrt(const void* x, void* y, const double* nrm, long long count, int nrhs,
                            cudaStream_t s) {
   launch_after(k_scale_inv_sqrt<R>, grid1(count, nrhs), RT, 0, s, (const cplx_t<R>*)x, (cplx_t<R>*)y, nrm,
-                                                         count); count_launch();
+               count);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -185,8 +187,7 @@ cudaError_t cg_xr(void* x, void* r, const void* p, const void* q, const double* 
   if (nrhs > 64) return cudaErrorInvalidValue;
   const int g = reduce_blocks(count, nrhs);
   launch_after(k_cg_xr<R>, dim3(g, nrhs), RT, 0, s, (cplx_t<R>*)x, (cplx_t<R>*)r, (const cplx_t<R>*)p,
-                                          (const cplx_t<R>*)q, rz, pq, frozen, count, ws, rr,
-                                          (float2*)r32, cc ? *cc : CgControl{});
+               (const cplx_t<R>*)q, rz, pq, frozen, count, ws, rr, (float2*)r32, cc ? *cc : CgControl{});
   count_launch();
   return cudaGetLastError();
 }
@@ -211,8 +212,8 @@ __global__ void __launch_bounds__(RT) k_cg_p(cplx_t<R>* __restrict__ p, const cp
 template <typename R>
 cudaError_t cg_p(void* p, const void* z, const double* rz_new, const double* rz_old,
                  const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  launch_after(k_cg_p<R>, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (cplx_t<R>*)p, (const cplx_t<R>*)z, rz_new, rz_old, frozen, count);
+  launch_after(k_cg_p<R>, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (cplx_t<R>*)p,
+               (const cplx_t<R>*)z, rz_new, rz_old, frozen, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -320,8 +321,8 @@ __global__ void __launch_bounds__(RT) k_dot2_zq_rz(const float2* __restrict__ z,
 cudaError_t dot2_zq_rz(const void* z32, const void* q, const void* r, long long count, int nrhs,
                        double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  launch_after(k_dot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (const float2*)z32, (const double2*)q, (const double2*)r, count, ws, zr);
+  launch_after(k_dot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (const float2*)z32,
+               (const double2*)q, (const double2*)r, count, ws, zr);
   count_launch();
   return cudaGetLastError();
 }
@@ -351,8 +352,8 @@ __global__ void __launch_bounds__(RT) k_cg_p_pr(double2* __restrict__ p, const f
 
 cudaError_t cg_p_pr(void* p, const void* z32, const double* zr, const double* pq, double* rz,
                     const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  launch_after(k_cg_p_pr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (double2*)p, (const float2*)z32, zr, pq, rz, frozen, count);
+  launch_after(k_cg_p_pr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (double2*)p, (const float2*)z32,
+               zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -388,7 +389,7 @@ cudaError_t rdot(const void* a, const void* b, long long count, int nrhs, double
                  cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
   launch_after(k_rdot, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (const float2*)a, (const float2*)b,
-                                                         count, ws, out);
+               count, ws, out);
   count_launch();
   return cudaGetLastError();
 }
@@ -428,9 +429,8 @@ cudaError_t rcg_xr(void* x32, void* r32, const void* p32, const void* q32, const
                    const double* pq, const int* frozen, long long count, int nrhs, double* ws,
                    double* rr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  launch_after(k_rcg_xr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (float2*)x32, (float2*)r32, (const float2*)p32, (const float2*)q32, rz, pq, frozen, count,
-      ws, rr);
+  launch_after(k_rcg_xr, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (float2*)x32, (float2*)r32,
+               (const float2*)p32, (const float2*)q32, rz, pq, frozen, count, ws, rr);
   count_launch();
   return cudaGetLastError();
 }
@@ -457,8 +457,8 @@ __global__ void __launch_bounds__(RT) k_rdot2_zq_rz(const float2* __restrict__ z
 cudaError_t rdot2_zq_rz(const void* z32, const void* q32, const void* r32, long long count,
                         int nrhs, double* ws, double* zr, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  launch_after(k_rdot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (const float2*)z32, (const float2*)q32, (const float2*)r32, count, ws, zr);
+  launch_after(k_rdot2_zq_rz, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (const float2*)z32,
+               (const float2*)q32, (const float2*)r32, count, ws, zr);
   count_launch();
   return cudaGetLastError();
 }
@@ -485,8 +485,8 @@ __global__ void __launch_bounds__(RT) k_rcg_p(float2* __restrict__ p, const floa
 
 cudaError_t rcg_p(void* p32, const void* z32, const double* zr, const double* pq, double* rz,
                   const int* frozen, long long count, int nrhs, cudaStream_t s) {
-  launch_after(k_rcg_p, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-      (float2*)p32, (const float2*)z32, zr, pq, rz, frozen, count);
+  launch_after(k_rcg_p, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (float2*)p32, (const float2*)z32,
+               zr, pq, rz, frozen, count);
   count_launch();
   return cudaGetLastError();
 }
@@ -562,9 +562,8 @@ __global__ void k_copy_slots(const double* src, double* dst, int n2, int depende
 cudaError_t ru_residual(const void* r64, void* r32, long long count, int nrhs, double* ws,
                         double* rr, double* rmax, cudaStream_t s) {
   if (nrhs > 64) return cudaErrorInvalidValue;
-  launch_after(k_ru_residual, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s,
-               (const double2*)r64, (float2*)r32,
-                                                                count, ws, rr);
+  launch_after(k_ru_residual, dim3(reduce_blocks(count, nrhs), nrhs), RT, 0, s, (const double2*)r64,
+               (float2*)r32, count, ws, rr);
   count_launch();
   if (rmax) {
     launch_after(k_copy_slots, 1, 128, 0, s, rr, rmax, 2 * nrhs);
@@ -586,11 +585,13 @@ __global__ void k_cvt_32_64(const float2* __restrict__ in, double2* __restrict__
   if (i < count) out[i] = make_double2(in[i].x, in[i].y);
 }
 cudaError_t convert_f64_f32(const void* in, void* out, long long count, cudaStream_t s) {
-  launch_after(k_cvt_64_32, grid1(count, 1), RT, 0, s, (const double2*)in, (float2*)out, count); count_launch();
+  launch_after(k_cvt_64_32, grid1(count, 1), RT, 0, s, (const double2*)in, (float2*)out, count);
+  count_launch();
   return cudaGetLastError();
 }
 cudaError_t convert_f32_f64(const void* in, void* out, long long count, cudaStream_t s) {
-  launch_after(k_cvt_32_64, grid1(count, 1), RT, 0, s, (const float2*)in, (double2*)out, count); count_launch();
+  launch_after(k_cvt_32_64, grid1(count, 1), RT, 0, s, (const float2*)in, (double2*)out, count);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -615,8 +616,8 @@ template <typename R>
 cudaError_t lincomb(void* out, double a, const void* u, double b, const void* v, double c,
                     const void* w, long long count, int nrhs, cudaStream_t s) {
   launch_after(k_lincomb<R>, grid1(count, nrhs), RT, 0, s, (cplx_t<R>*)out, (R)a, (const cplx_t<R>*)u, (R)b,
-                                                  (const cplx_t<R>*)v, (R)c,
-                                                  (const cplx_t<R>*)w, count); count_launch();
+               (const cplx_t<R>*)v, (R)c, (const cplx_t<R>*)w, count);
+  count_launch();
   return cudaGetLastError();
 }
 

@@ -274,7 +274,7 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
     if (e != cudaSuccess) return e;
     dim3 grid(Lx * Lt, (nrhs + MMA_RC - 1) / MMA_RC);
     launch_after(k_coarse_apply_mma, grid, 64, smem, s, (const float2*)in, (float2*)out,
-                                              (const __nv_bfloat162*)A, Lx, Lt, n, nrhs, ep);
+                 (const __nv_bfloat162*)A, Lx, Lt, n, nrhs, ep);
     count_launch();
     return cudaGetLastError();
   }
@@ -282,13 +282,13 @@ cudaError_t coarse_apply(const void* in, void* out, const void* A, int weights, 
   const int threads = (9 * n + 31) / 32 * 32;
   if (weights == W_F64)
     launch_after(k_coarse_apply<double, double2>, grid, threads, 18 * n * sizeof(double2), s,
-        (const double2*)in, (double2*)out, (const double2*)A, Lx, Lt, n, ep);
+                 (const double2*)in, (double2*)out, (const double2*)A, Lx, Lt, n, ep);
   else if (weights == W_F32)
-    launch_after(k_coarse_apply<float, float2>, grid, threads, 18 * n * sizeof(float2), s,
-        (const float2*)in, (float2*)out, (const float2*)A, Lx, Lt, n, ep);
+    launch_after(k_coarse_apply<float, float2>, grid, threads, 18 * n * sizeof(float2), s, (const float2*)in,
+                 (float2*)out, (const float2*)A, Lx, Lt, n, ep);
   else
     launch_after(k_coarse_apply<float, __nv_bfloat162>, grid, threads, 18 * n * sizeof(float2), s,
-        (const float2*)in, (float2*)out, (const __nv_bfloat162*)A, Lx, Lt, n, ep);
+                 (const float2*)in, (float2*)out, (const __nv_bfloat162*)A, Lx, Lt, n, ep);
   count_launch();
   return cudaGetLastError();
 }
@@ -311,8 +311,8 @@ __global__ void k_coarse_lincomb(double a, const double2* X, double b, const dou
 cudaError_t coarse_lincomb(double a, const void* X, double b, const void* Y, double c, void* out,
                            long long sites, int n, cudaStream_t s) {
   const long long count = sites * 9 * n * n;
-  launch_after(k_coarse_lincomb, (unsigned)((count + 255) / 256), 256, 0, s,
-      a, (const double2*)X, b, (const double2*)Y, c, (double2*)out, count, n);
+  launch_after(k_coarse_lincomb, (unsigned)((count + 255) / 256), 256, 0, s, a, (const double2*)X, b,
+               (const double2*)Y, c, (double2*)out, count, n);
   count_launch();
   return cudaGetLastError();
 }
@@ -351,7 +351,7 @@ cudaError_t probe_vectors(void* out, int Lxc, int Ltc, int nc, int Kx, int Kt, i
                           cudaStream_t s) {
   const long long n = (long long)nc * Lxc * Ltc * nc;
   launch_after(k_probe_vectors, (unsigned)((n + 255) / 256), 256, 0, s, (double2*)out, Lxc, Ltc, nc, Kx, Kt,
-                                                            cx, ct);
+               cx, ct);
   count_launch();
   return cudaGetLastError();
 }
@@ -360,7 +360,7 @@ cudaError_t probe_scatter(const void* y, void* Ac, int Lxc, int Ltc, int nc, int
                           int ct, cudaStream_t s) {
   const long long n = (long long)Lxc * Ltc * 9 * nc * nc;
   launch_after(k_probe_scatter, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)y, (double2*)Ac, Lxc,
-                                                            Ltc, nc, Kx, Kt, cx, ct);
+               Ltc, nc, Kx, Kt, cx, ct);
   count_launch();
   return cudaGetLastError();
 }
@@ -536,15 +536,15 @@ cudaError_t restrict_op(const void* fine, void* coarse, const void* Vst, int Lx,
     static SmemLimit limit;
     const cudaError_t e = limit.raise(k_restrict_multi<R>, 96 * 1024);
     if (e != cudaSuccess) return e;
-    launch_after(k_restrict_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
-        (const cplx_t<R>*)fine, (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
-        nrhs, transfer_group(nrhs * 2 * Nv, bx * bt * h));
+    launch_after(k_restrict_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s, (const cplx_t<R>*)fine,
+                 (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv, nrhs,
+                 transfer_group(nrhs * 2 * Nv, bx * bt * h));
     count_launch();
     return cudaGetLastError();
   }
   const int warps = (Lx / bx) * (Lt / bt) * 2 * Nv;
-  launch_after(k_restrict<R>, dim3((warps + 7) / 8, nrhs), 256, 0, s,
-      (const cplx_t<R>*)fine, (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv);
+  launch_after(k_restrict<R>, dim3((warps + 7) / 8, nrhs), 256, 0, s, (const cplx_t<R>*)fine,
+               (cplx_t<R>*)coarse, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv);
   count_launch();
   return cudaGetLastError();
 }
@@ -579,16 +579,16 @@ cudaError_t prolong_op(const void* coarse, void* fine, const void* Vst, int Lx, 
     static SmemLimit limit;
     const cudaError_t e = limit.raise(k_prolong_multi<R>, 96 * 1024);
     if (e != cudaSuccess) return e;
-    launch_after(k_prolong_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s,
-        (const cplx_t<R>*)coarse, (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
-        nrhs, accumulate, transfer_group(nrhs * bx * bt * 2 * h, Nv));
+    launch_after(k_prolong_multi<R>, (Lx / bx) * (Lt / bt), 256, sm, s, (const cplx_t<R>*)coarse,
+                 (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv, nrhs, accumulate,
+                 transfer_group(nrhs * bx * bt * 2 * h, Nv));
     count_launch();
     return cudaGetLastError();
   }
   const int tot = Lx * Lt * 2 * h;
-  launch_after(k_prolong<R>, dim3((tot + 255) / 256, nrhs), 256, 0, s,
-      (const cplx_t<R>*)coarse, (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv,
-      accumulate); count_launch();
+  launch_after(k_prolong<R>, dim3((tot + 255) / 256, nrhs), 256, 0, s, (const cplx_t<R>*)coarse,
+               (cplx_t<R>*)fine, (const cplx_t<R>*)Vst, Lx, Lt, bx, bt, h, Nv, accumulate);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -688,9 +688,8 @@ cudaError_t block_gram_schmidt(const void* E, void* Vst, int Lx, int Lt, int bx,
     static SmemLimit limit;
     const cudaError_t e = limit.raise(k_block_gs<LPB, NQ>, 160 * 1024);
     if (e != cudaSuccess) return e;
-    launch_after(k_block_gs<LPB, NQ>, (nb + per - 1) / per, 32, smem, s,
-                 (const double2*)E, (double2*)Vst, Lx, Lt, bx,
-                                                              bt, h, Nv, breakdown_tol, flag, nb);
+    launch_after(k_block_gs<LPB, NQ>, (nb + per - 1) / per, 32, smem, s, (const double2*)E, (double2*)Vst, Lx,
+                 Lt, bx, bt, h, Nv, breakdown_tol, flag, nb);
     count_launch();
     return cudaGetLastError();
   };
@@ -842,14 +841,17 @@ cudaError_t galerkin_fine(const void* U64, double diag, const void* Vst, void* W
                           int Lx, int Lt, int bx, int bt, int Nv, cudaStream_t s) {
   const long long Vc = (long long)(Lx / bx) * (Lt / bt), nc = 2 * Nv;
   const long long nW = Vc * nc * (bx + 2) * (bt + 2);
-  launch_after(k_galerkin_W, (unsigned)((nW + 255) / 256), 256, 0, s,
-      (const double2*)U64, diag, (const double2*)Vst, (double2*)Wbuf, Lx, Lt, bx, bt, Nv); count_launch();
+  launch_after(k_galerkin_W, (unsigned)((nW + 255) / 256), 256, 0, s, (const double2*)U64, diag,
+               (const double2*)Vst, (double2*)Wbuf, Lx, Lt, bx, bt, Nv);
+  count_launch();
   const long long nA = Vc * (nc * (nc + 1) / 2 + 4 * nc * nc);
-  launch_after(k_galerkin_WW<false>, (unsigned)((nA + 255) / 256), 256, 0, s,
-      (const double2*)Wbuf, (const double2*)Vst, (double2*)Ac, Lx, Lt, bx, bt, Nv); count_launch();
+  launch_after(k_galerkin_WW<false>, (unsigned)((nA + 255) / 256), 256, 0, s, (const double2*)Wbuf,
+               (const double2*)Vst, (double2*)Ac, Lx, Lt, bx, bt, Nv);
+  count_launch();
   if (G1) {
-    launch_after(k_galerkin_WW<true>, (unsigned)((nA + 255) / 256), 256, 0, s,
-        (const double2*)Wbuf, (const double2*)Vst, (double2*)G1, Lx, Lt, bx, bt, Nv); count_launch();
+    launch_after(k_galerkin_WW<true>, (unsigned)((nA + 255) / 256), 256, 0, s, (const double2*)Wbuf,
+                 (const double2*)Vst, (double2*)G1, Lx, Lt, bx, bt, Nv);
+    count_launch();
   }
   return cudaGetLastError();
 }
@@ -927,8 +929,9 @@ cudaError_t galerkin_coarse(const void* Af, const void* Vst, void* Ac, int Lx, i
   static SmemLimit limit;
   const cudaError_t e = limit.raise(k_galerkin_coarse, 200 * 1024);
   if (e != cudaSuccess) return e;
-  launch_after(k_galerkin_coarse, Vc, 256, smem, s, (const double2*)Af, (const double2*)Vst, (double2*)Ac,
-                                          Lx, Lt, bx, bt, nf, Nv); count_launch();
+  launch_after(k_galerkin_coarse, Vc, 256, smem, s, (const double2*)Af, (const double2*)Vst, (double2*)Ac, Lx,
+               Lt, bx, bt, nf, Nv);
+  count_launch();
   return cudaGetLastError();
 }
 
@@ -966,8 +969,9 @@ cudaError_t coarse_to_dense_f32(const void* A, void* dense, int Lx, int Lt, int 
   cudaError_t e = cudaMemsetAsync(dense, 0, (size_t)(ld * ld * sizeof(float2)), s);
   if (e != cudaSuccess) return e;
   const long long tot = (long long)Lx * Lt * n * n;
-  launch_after(k_coarse_to_dense, (unsigned)((tot + 255) / 256), 256, 0, s, (const double2*)A,
-                                                                  (float2*)dense, Lx, Lt, n, ld); count_launch();
+  launch_after(k_coarse_to_dense, (unsigned)((tot + 255) / 256), 256, 0, s, (const double2*)A, (float2*)dense,
+               Lx, Lt, n, ld);
+  count_launch();
   if (ld > N) {
     launch_after(k_pad_identity, (unsigned)((ld - N + 255) / 256), 256, 0, s, (float2*)dense, N, ld);
     count_launch();
@@ -1437,7 +1441,8 @@ cudaError_t gauss_jordan_begin(void* M, int N, void* work, cudaStream_t s) {
   static SmemLimit limit;
   const cudaError_t e = limit.raise(k_gj_panel, (int)(2 * GJB * GJS * sizeof(float2)));
   if (e != cudaSuccess) return e;
-  launch_after(k_gj_pivot0, 1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s, (const float2*)M, N, Pb[0]);
+  launch_after(k_gj_pivot0, 1, 256, (GJB * GJS + 2 * 16 * 48) * sizeof(float2), s, (const float2*)M, N,
+               Pb[0]);
   count_launch();
   return cudaGetLastError();
 }
@@ -1446,8 +1451,8 @@ cudaError_t gauss_jordan_panel(void* M, int N, int k, void* work, cudaStream_t s
   float2 *Pb[2], *Cold, *Cn, *Rp;
   gj_work_split(work, N, Pb, &Cold, &Cn, &Rp);
   const int nb = N / GJB;
-  launch_after(k_gj_panel, dim3(2 * nb, GJB / 16), 256, 2 * GJB * GJS * sizeof(float2), s,
-      (const float2*)M, N, k, Pb[k & 1], Cold, Cn, Rp);
+  launch_after(k_gj_panel, dim3(2 * nb, GJB / 16), 256, 2 * GJB * GJS * sizeof(float2), s, (const float2*)M,
+               N, k, Pb[k & 1], Cold, Cn, Rp);
   count_launch();
   return cudaGetLastError();
 }
@@ -1468,7 +1473,7 @@ cudaError_t gauss_jordan_update_tc(void* M, int N, int k, void* work, cudaStream
   const cudaError_t e = limit.raise(k_gj_update_tc, (int)sm);
   if (e != cudaSuccess) return e;
   launch_after(k_gj_update_tc, tc_tile_count(nb), 256, sm, s, (float2*)M, N, k, Pb[k & 1], Pb[(k + 1) & 1],
-                                                    Cold, Cn, Rp, (int*)(Rp + (long long)GJB * N));
+               Cold, Cn, Rp, (int*)(Rp + (long long)GJB * N));
   count_launch();
   return cudaGetLastError();
 }
@@ -1865,7 +1870,8 @@ __global__ void __launch_bounds__(256) k_hgemv_reduce(const float2* __restrict__
 
 cudaError_t to_f32_padded(const void* x, void* xs, int N, int ld, int nrhs, cudaStream_t s) {
   const long long n = (long long)ld * nrhs;
-  launch_after(k_x32_pad, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)x, (float2*)xs, N, ld, nrhs);
+  launch_after(k_x32_pad, (unsigned)((n + 255) / 256), 256, 0, s, (const double2*)x, (float2*)xs, N, ld,
+               nrhs);
   count_launch();
   return cudaGetLastError();
 }
@@ -1880,8 +1886,8 @@ cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, in
     cudaError_t e = limit.raise(k_hgemv_mma, (int)sm);
     if (e == cudaSuccess) e = to_f32_padded(x, xscratch, N, ld, nrhs, s);
     if (e != cudaSuccess) return e;
-    launch_after(k_hgemv_mma, ntiles, 256, sm, s, (const float2*)P, (const float2*)xscratch, ld, ntiles,
-                                        nrhs, (float2*)part);
+    launch_after(k_hgemv_mma, ntiles, 256, sm, s, (const float2*)P, (const float2*)xscratch, ld, ntiles, nrhs,
+                 (float2*)part);
     count_launch();
     return cudaGetLastError();
   }
@@ -1889,16 +1895,16 @@ cudaError_t hermitian_gemv_tiles(const void* P, const void* x, int N, int ld, in
     const dim3 grid(ntiles);
     if (nrhs == 1)
       launch_after(k_hgemv_warp<1>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
-                                           (float2*)part, nullptr);
+                   (float2*)part, nullptr);
     else if (nrhs == 2)
       launch_after(k_hgemv_warp<2>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
-                                           (float2*)part, nullptr);
+                   (float2*)part, nullptr);
     else
       launch_after(k_hgemv_warp<4>, grid, 64, 0, s, (const float2*)P, (const double2*)x, N, ntiles, nrhs,
-                                           (float2*)part, nullptr);
+                   (float2*)part, nullptr);
   } else {
     launch_after(k_hgemv_tiles, ntiles, 256, 0, s, (const float2*)P, (const double2*)x, N, nrhs,
-                                         (float2*)part);
+                 (float2*)part);
   }
   count_launch();
   return cudaGetLastError();
@@ -1908,8 +1914,8 @@ cudaError_t hermitian_gemv_reduce(const void* part, void* y, int N, int ld, int 
                                   bool accumulate, cudaStream_t s, void* y32) {
   if (ld % HT || ld < N) return cudaErrorInvalidValue;
   const int nt = ld / HT;
-  launch_after(k_hgemv_reduce, dim3(nt, nrhs), 256, 0, s, (const float2*)part, (double2*)y, N, nt,
-                                                accumulate, (float2*)y32);
+  launch_after(k_hgemv_reduce, dim3(nt, nrhs), 256, 0, s, (const float2*)part, (double2*)y, N, nt, accumulate,
+               (float2*)y32);
   count_launch();
   return cudaGetLastError();
 }
@@ -1923,13 +1929,13 @@ cudaError_t hermitian_gemv_tiles_f32in(const void* P, const void* x32, int N, in
   const dim3 grid(ntiles);
   if (nrhs == 1)
     launch_after(k_hgemv_warp<1, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
-                                                 nrhs, (float2*)part, (double2*)x64);
+                 nrhs, (float2*)part, (double2*)x64);
   else if (nrhs == 2)
     launch_after(k_hgemv_warp<2, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
-                                                 nrhs, (float2*)part, (double2*)x64);
+                 nrhs, (float2*)part, (double2*)x64);
   else
     launch_after(k_hgemv_warp<4, float2>, grid, 64, 0, s, (const float2*)P, (const float2*)x32, N, ntiles,
-                                                 nrhs, (float2*)part, (double2*)x64);
+                 nrhs, (float2*)part, (double2*)x64);
   count_launch();
   return cudaGetLastError();
 }
@@ -1945,7 +1951,8 @@ __global__ void k_block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int
 
 cudaError_t block_map(int Lx, int Lt, int bx, int bt, int32_t* coarse, int32_t* offset,
                       cudaStream_t s) {
-  launch_after(k_block_map, (Lx * Lt + 255) / 256, 256, 0, s, Lx, Lt, bx, bt, coarse, offset); count_launch();
+  launch_after(k_block_map, (Lx * Lt + 255) / 256, 256, 0, s, Lx, Lt, bx, bt, coarse, offset);
+  count_launch();
   return cudaGetLastError();
 }
 

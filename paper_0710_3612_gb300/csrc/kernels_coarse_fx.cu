@@ -274,8 +274,8 @@ cudaError_t launch(const double2* x, double2* y, const double2* A, const int4* W
   static SmemLimit limit;
   const cudaError_t e = limit.raise(k_coarse_fx<RG>, 64 * 1024);
   if (e != cudaSuccess) return e;
-  launch_after(k_coarse_fx<RG>, dim3(Lx * Lt, (nrhs + rpc - 1) / rpc), (NR + 31) & ~31, smem, s,
-      x, y, A, W, E, Lx, Lt, n, nrhs, rpc, ep);
+  launch_after(k_coarse_fx<RG>, dim3(Lx * Lt, (nrhs + rpc - 1) / rpc), (NR + 31) & ~31, smem, s, x, y, A, W,
+               E, Lx, Lt, n, nrhs, rpc, ep);
   return cudaGetLastError();
 }
 
@@ -298,14 +298,11 @@ cudaError_t coarse_finish(const void* G0, const void* G1, double m, void* A64, v
                            : limit0.raise(k_coarse_finish<false>, 160 * 1024);
   if (e != cudaSuccess) return e;
   if (G0)
-    launch_after(k_coarse_finish<true>, (unsigned)sites, 256, smem, s,
-                 (const double2*)G0, (const double2*)G1, m,
-                                                             (double2*)A64, (float2*)A32,
-                                                             (__nv_bfloat162*)A16, W, E, n, P);
+    launch_after(k_coarse_finish<true>, (unsigned)sites, 256, smem, s, (const double2*)G0, (const double2*)G1,
+                 m, (double2*)A64, (float2*)A32, (__nv_bfloat162*)A16, W, E, n, P);
   else
     launch_after(k_coarse_finish<false>, (unsigned)sites, 256, smem, s, nullptr, nullptr, 0.0, (double2*)A64,
-                                                              (float2*)A32, (__nv_bfloat162*)A16, W, E, n,
-                                                              P);
+                 (float2*)A32, (__nv_bfloat162*)A16, W, E, n, P);
   count_launch();
   return cudaGetLastError();
 }

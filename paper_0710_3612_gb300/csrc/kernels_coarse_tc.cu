@@ -479,9 +479,8 @@ cudaError_t launch_tc(const void* in, void* out, const void* A, int Lx, int Lt, 
   // columns before its first site).  Strips of at most 8 sites dealt out in turn left a
   // quarter of the SM time idle at 4096 sites (4 strips for some CTAs, 3 for others).
   const int grid = (int)std::max(1LL, std::min((long long)sms, V / 2));
-  launch_after(k_coarse_apply_tc<NDOF>, grid, C::THREADS, smem, s,
-               map, (float2*)out, (const __nv_bfloat162*)A, Lx,
-                                                        Lt, nrhs, R, ep);
+  launch_after(k_coarse_apply_tc<NDOF>, grid, C::THREADS, smem, s, map, (float2*)out,
+               (const __nv_bfloat162*)A, Lx, Lt, nrhs, R, ep);
   count_launch();
   return cudaGetLastError();
 }

@@ -39,10 +39,10 @@ cudaError_t wilson_D(const void* in, void* out, const void* U, double diag, int 
   dim3 grid((V + 255) / 256, nrhs);
   if (dagger)
     launch_after(k_wilson_D<R, true>, grid, 256, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
-                                             (const cplx_t<R>*)U, (R)diag, Lx, Lt);
+                 (const cplx_t<R>*)U, (R)diag, Lx, Lt);
   else
     launch_after(k_wilson_D<R, false>, grid, 256, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
-                                              (const cplx_t<R>*)U, (R)diag, Lx, Lt);
+                 (const cplx_t<R>*)U, (R)diag, Lx, Lt);
   count_launch();
   return cudaGetLastError();
 }
@@ -335,9 +335,10 @@ __global__ void __launch_bounds__(128, 3) k_wilson_A_stream(const double2* __res
 // row step takes 40 packed operations for two sites where k_wilson_A_stream takes 88, and
 // only one shuffle per component and direction; a warp owns 64 sites of a row, 60 of them
 // outputs.  Its links are stored as -U / 2, so that D is diag psi + the sum of hops and nothing
-// leaves the range that the result has.  The t-backward product of a row is formed when the row is current and carried.  Bound by FMA
-// issue (72% of the heavy pipe) and HBM: 4096^2 128 us (0.93 of the copy bandwidth; 144 us with
-// one site per lane), 1024^2 x 16 119 (146), 256^2 x 64 40 (68 with tiles).
+// leaves the range that the result has.  The t-backward product of a row is formed when the row
+// is current and carried.  Bound by FMA issue (72% of the heavy pipe) and HBM: 4096^2 128 us (0.93
+// of the copy bandwidth; 144 us with one site per lane), 1024^2 x 16 117 (146), 256^2 x 64 40 (68
+// with tiles).
 using P2 = unsigned long long;                       // two floats, low = first site
 
 __device__ __forceinline__ P2 p2(float a, float b) {
@@ -538,15 +539,19 @@ static void launch_wilson_A(const void* in, void* out, const void* U, double dia
                 "tile above the static shared-memory limit");
   dim3 grid((Lx + TX - 1) / TX, (Lt + TY * RPT - 1) / (TY * RPT), nrhs);
   launch_after(k_wilson_A<R, TX, TY, RPT>, grid, TX * TY, 0, s, (const cplx_t<R>*)in, (cplx_t<R>*)out,
-                                                      (const cplx_t<R>*)U, (R)diag, Lx, Lt, ep);
+               (const cplx_t<R>*)U, (R)diag, Lx, Lt, ep);
 }
 
 // ---------------------------------------------------------------------------
-// Launch shapes of the fused A and their autotuner.  Every shape runs the same
-// per-site arithmetic (wilson_site order), so a shape is admitted by the
-// tuner only if it reproduces the default shape's output bit for bit; the
-// tuner then keeps the fastest admitted shape per (precision, Lx, Lt, nrhs)
-// when it beats the default shape by more than 3%.
+// Launch shapes of the fused A and their autotuner.  A shape is admitted by the
+// tuner only if it reproduces the default shape's output bit for bit: the tiles
+// share their per-site arithmetic (wilson_site order), the integer kernel's do not
+// depend on the tile; the FP32 streaming kernel associates its sums otherwise and
+// is admitted only where it is the default (wide lattices and batches, so that an
+// FP32 result's last bits may depend on the number of right-hand sides).  The
+// tuner keeps the fastest admitted shape per (precision, Lx, Lt, nrhs) when it
+// beats the default shape by more than 3%; it takes 62 launches of every admitted
+// shape in the first set-up of a shape in a process.
 // Launches with the fused <in, A in> epilogue keep the default shape (their
 // partial sums depend on the tiling).
 // ---------------------------------------------------------------------------
@@ -611,11 +616,11 @@ static cudaError_t launch_variant(int v, const void* in, void* out, const void* 
         const int rows = stream32_rows(Lx, Lt, nrhs);
         const long long warps = stream32_warps(Lx, Lt, 1, rows);
         launch_after(k_wilson_A_stream2, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
-            (const float2*)in, (float2*)out, (const float2*)W, (float)diag, Lx, Lt, rows, ep);
+                     (const float2*)in, (float2*)out, (const float2*)W, (float)diag, Lx, Lt, rows, ep);
       } else {
         const long long warps = (long long)((Lx + SOUT - 1) / SOUT) * ((Lt + SROWS - 1) / SROWS);
         launch_after(k_wilson_A_stream, dim3((unsigned)((warps + 3) / 4), nrhs), 128, 0, s,
-            (const double2*)in, (double2*)out, (const double2*)U, diag, Lx, Lt, ep);
+                     (const double2*)in, (double2*)out, (const double2*)U, diag, Lx, Lt, ep);
       }
       break;
     }
@@ -686,8 +691,8 @@ cudaError_t wilson_A_tune(const void* in, void* out, void* ref, const void* U, c
     launch_variant<R>(v, in, out, U, W, diag, Lx, Lt, nrhs, none, s);
     int diff = 0;
     cudaMemsetAsync(dflag, 0, sizeof(int), s);
-    launch_after(k_count_diff, 152, 256, 0, s, (const unsigned long long*)out,
-                                     (const unsigned long long*)ref, words, dflag);
+    launch_after(k_count_diff, 152, 256, 0, s, (const unsigned long long*)out, (const unsigned long long*)ref,
+                 words, dflag);
     cudaMemcpyAsync(&diff, dflag, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t err = cudaStreamSynchronize(s);
     if (err != cudaSuccess) {
@@ -795,8 +800,8 @@ __global__ void k_fold_links(const double2* __restrict__ g, cplx_t<R>* __restric
 template <typename R>
 cudaError_t fold_links(const void* gauge, void* U, int Lx, int Lt, cudaStream_t s, double factor) {
   const int n = 2 * Lx * Lt;
-  launch_after(k_fold_links<R>, (n + 255) / 256, 256, 0, s,
-               (const double2*)gauge, (cplx_t<R>*)U, Lx, Lt, factor);
+  launch_after(k_fold_links<R>, (n + 255) / 256, 256, 0, s, (const double2*)gauge, (cplx_t<R>*)U, Lx, Lt,
+               factor);
   count_launch();
   return cudaGetLastError();
 }
@@ -820,7 +825,7 @@ cudaError_t link_unitarity(const void* gauge, long long count, double* out, cuda
   if (e != cudaSuccess) return e;
   const long long g = (count + 255) / 256;
   launch_after(k_link_unitarity, (unsigned)(g < 1216 ? g : 1216), 256, 0, s, (const double2*)gauge, count,
-                                                                 (unsigned long long*)out);
+               (unsigned long long*)out);
   count_launch();
   return cudaGetLastError();
 }

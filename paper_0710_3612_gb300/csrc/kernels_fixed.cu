@@ -149,8 +149,8 @@ struct FxTile {
 // point in shared memory, D psi on the tile plus a 1-site halo, D^dagger on the tile.
 // 905 instructions per site at 32 x 16 (426 of them on the 64-wide ALU pipe: shifts,
 // masks, comparisons), 22 mad.wide per clock: bound by those two pipes.  256^2 x 64:
-// 166 us against 1024 us in FP64 (137 FP64 instructions per site), 128^2 4.2 against
-// 10.2 us, 210 x 90 x 12 12.6 against 71.6 us; with the fused dot 207 against 1254 us.
+// 167 us against 1024 us in FP64 (137 FP64 instructions per site), 128^2 4.2 against
+// 10.2 us, 210 x 90 x 12 12.8 against 71.6 us; with the fused dot 207 against 1254 us.
 // A warp-streaming form (rows in registers, shuffles along x) took 260 us there.  SHIFT: hop
 // terms with k > 0 (1.1% more).
 template <int TX, int TY, int RPT, int MINB, int MODE, bool SHIFT>

@@ -118,9 +118,8 @@ cudaError_t gauge_metropolis(double* theta, int Lx, int Lt, double beta, double 
   for (long long sw = first_sweep; sw < first_sweep + sweeps; ++sw)
     for (int mu = 0; mu < 2; ++mu)
       for (int parity = 0; parity < 2; ++parity) {
-        launch_after(k_metropolis_half, (n + 255) / 256, 256, 0, s,
-            theta, Lx, Lt, beta, eps, mu, parity, (unsigned long long)(4 * sw + 2 * mu + parity),
-            key, accepted);
+        launch_after(k_metropolis_half, (n + 255) / 256, 256, 0, s, theta, Lx, Lt, beta, eps, mu, parity,
+                     (unsigned long long)(4 * sw + 2 * mu + parity), key, accepted);
         count_launch();
       }
   return cudaGetLastError();

@@ -311,12 +311,10 @@ cudaError_t hermitian_gemv_tc(const void* P, const void* x, void* y, int N, int 
   const cudaError_t ex = to_f32_padded(x, xscratch, N, ld, nrhs, s);
   if (ex != cudaSuccess) return ex;
   const int nt = ld / GT_T, splits = gt_splits(nt);
-  launch_after(k_hgemv_tc, dim3((nt + 1) / 2, splits), GT_THREADS, GT_SMEM, s,
-               (const float2*)P, (const float2*)xscratch,
-                                                                     ld, nt, nrhs, (float*)part);
-  launch_after(k_hgemv_tc_sum, dim3((N + 127) / 128, nrhs), 128, 0, s,
-               (const float*)part, (double2*)y, N, ld, splits,
-                                                             accumulate, (float2*)y32);
+  launch_after(k_hgemv_tc, dim3((nt + 1) / 2, splits), GT_THREADS, GT_SMEM, s, (const float2*)P,
+               (const float2*)xscratch, ld, nt, nrhs, (float*)part);
+  launch_after(k_hgemv_tc_sum, dim3((N + 127) / 128, nrhs), 128, 0, s, (const float*)part, (double2*)y, N, ld,
+               splits, accumulate, (float2*)y32);
   count_launch();
   count_launch();
   return cudaGetLastError();
