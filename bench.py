@@ -563,7 +563,7 @@ def gpu_bench(args):
             "clocks": res["clocks"],
             "cpu_baseline": cpu,
         }
-        print(json.dumps(line))
+        report(line, args.details)
     if world > 1:
         dist.destroy_process_group()
 
@@ -1212,6 +1212,34 @@ def reference_arm(args):
     print(json.dumps(line))
 
 
+# What the one line on stdout holds of the full record; a line with every leg (20 KB and more) is
+# cut by programs that keep the end of the output only.
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+             "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks", "solver",
+             "mixed_vs_plain_fp64")
+LINE_MAX = 1500
+
+
+def summary(line):
+    """The record without its legs: the headline, and one number of each part of the metric."""
+    out = {k: line[k] for k in LINE_KEYS if k in line}
+    out["latency_ms"] = {k: line["latency_ms"][k] for k in ("p50", "p99")}
+    out["plain_fp64"] = line["plain_fp64"]["value"]
+    out["stencil_gbs"] = line["stencil"]["gbs"]
+    return out
+
+
+def report(line, details):
+    """Full record to the file `details` or to stderr, then the one line to stdout."""
+    if details:
+        with open(details, "w") as f:
+            json.dump(line, f)
+            f.write("\n")
+    else:
+        print(json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(summary(line)), flush=True)
+
+
 def ncu_case(args):
     """Small cases for kernel-level ncu captures (a few launches of one kernel):
     stencil -- fused FP32 A on a 2048 x 2048 lattice (about 200 MB per launch,
@@ -1303,6 +1331,8 @@ def main():
     ap.add_argument("--serving-only", action="store_true",
                     help="run the serving leg alone and print it as the JSON line")
     ap.add_argument("--serve-budget-gb", type=int, default=128)
+    ap.add_argument("--details", default="",
+                    help="file for the full record of every leg (default: one line on stderr)")
     ap.add_argument("--timed-only", action="store_true",
                     help="skip the plain-FP64, roofline, stencil and end-to-end legs (profiling runs)")
     ap.add_argument("--gj-tcgen05", action="store_true",
