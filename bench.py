@@ -589,6 +589,41 @@ def ncu_traffic():
     return out
 
 
+def inverse_tile_products(Lx, Lt, n):
+    """64 x 64 tile products of the coarsest inverse's updates, and its launches: the order of
+    csrc/kernels_inverse.cu (inverse_plan) on the block graph of the 9-point stencil -- fewest
+    couplings next, up to 8 uncoupled pivots together, a pivot joining the blocks it couples."""
+    nt = (Lx * Lt * n + 63) // 64
+    adj = [1 << b for b in range(nt)]
+    blocks = [range(j * n // 64, (j * n + n - 1) // 64 + 1) for j in range(Lx * Lt)]
+    for j in range(Lx * Lt):
+        for d in range(9):
+            k = (j % Lx + d % 3 - 1) % Lx + Lx * ((j // Lx + d // 3 - 1) % Lt)
+            for a in blocks[j]:
+                for b in blocks[k]:
+                    adj[a] |= 1 << b
+    left, products, groups = set(range(nt)), 0, 0
+    while left:
+        deg = {k: bin(adj[k]).count("1") - 1 for k in left}
+        order = sorted(left, key=lambda k: (deg[k], k))
+        grp, total = [], 0
+        for k in order:
+            if deg[k] > 1.6 * deg[order[0]] + 4.0 or len(grp) == 8:
+                break
+            if grp and (total + deg[k] > nt or any(adj[k] >> p & 1 for p in grp)):
+                continue
+            grp.append(k)
+            total += deg[k]
+        for k in grp:
+            products += deg[k] * (deg[k] + 1) // 2
+            for a in range(nt):
+                if adj[k] >> a & 1 and a != k:
+                    adj[a] |= adj[k]
+            left.remove(k)
+        groups += 1
+    return products, groups
+
+
 def roofline(prof, wl, peaks):
     """Roofline of the dominant kernel of one profiled (eager) step, and of
     the other candidates.  The candidates are the profiling families that time
@@ -604,6 +639,7 @@ def roofline(prof, wl, peaks):
     V2 = V // (b1[0] * b1[1])
     V3 = V2 // (b2[0] * b2[1])
     N3 = V3 * 2 * Nv2
+    shape3 = (Lx // (b1[0] * b2[0]), Lt // (b1[1] * b2[1]), 2 * Nv2)
     ld = (N3 + 63) // 64 * 64
     nt = ld // 64
     ntiles = nt * (nt + 1) // 2
@@ -618,9 +654,10 @@ def roofline(prof, wl, peaks):
         o = {"kernel": cand[fam], "launches": calls, "avg_us": round(per_call_s * 1e6, 3),
              "ms_in_step": round(ms, 3)}
         if fam == 8:
-            # complex rank-64 update of the lower 64 x 64 tiles outside the pivot
-            # row and column: 64^3 complex multiply-adds (8 real flops) per tile
-            flops = (ntiles - nt) * 64.0 ** 3 * 8.0
+            # rank-64 updates of the lower 64 x 64 tiles of coupled blocks: 64^3 complex
+            # multiply-adds (8 real flops) per product, shared by the inverse's launches
+            products, groups = inverse_tile_products(*shape3)
+            flops = products / groups * 64.0 ** 3 * 8.0
             peak = peaks["bf16_tflops_sustained"] * 1.1 / 2.25   # nominal TF32 / BF16 ratio
             o.update({"bound": "tensor", "achieved": round(flops / per_call_s / 1e12, 3),
                       "peak": round(peak, 1), "unit": "TFLOP/s", "flops_per_launch": flops,

@@ -38,6 +38,13 @@ def test_line_is_short_and_complete(capsys, tmp_path):
     assert got["latency_ms"] == {"p50": 1.097, "p99": 77.353} and got["stencil_gbs"] == 6227.6
 
 
+def test_inverse_counts_its_own_tile_products():
+    """The 4096-unknown coarsest level: the counts stated in kernels_inverse.cu.  One site per
+    block (n = 64) on 3 x 3 sites couples every pair: the dense sweep's sum over pivots."""
+    assert bench.inverse_tile_products(16, 16, 16) == (25840, 28)
+    assert bench.inverse_tile_products(3, 3, 64) == (9 * 8 * 9 // 2, 9)
+
+
 def test_record_goes_to_stderr_by_default(capsys):
     rec = _record()
     bench.report(rec, "")
