@@ -352,7 +352,8 @@ mg_status mg_get_refine_rho(const mg_handle* h, double* rho, int max, int* count
  * b, x: device complex128 [nrhs][Lt][Lx][2].  Right-hand sides are solved in
  * batches of params->max_rhs that share one Krylov loop (one operator and
  * V-cycle launch per iteration for the whole batch, per-RHS scalars; a
- * converged RHS is frozen).  Stops each RHS when the true FP64
+ * converged RHS is frozen).  Launches are shaped by the size of the batch, so the
+ * last bits of a solution may depend on how many right-hand sides share it.  Stops each RHS when the true FP64
  * |b - A x| / |b| <= tol.  b = 0 gives x = 0.  info (host, may be NULL)
  * receives nrhs records.  Synchronises the stream.  MG_ERR_NOCONV when
  * maxiter iterations are exhausted. */
